@@ -25,7 +25,7 @@ template <typename T> bool dev_alloc(T **p, size_t count)
 // Every device array of a prepared layer with its size in bytes, in a fixed order (allocation,
 // release, export and import all walk this table).  Needs d.K, d.M, d.Mt.
 struct ArrayRef { void **ptr; size_t bytes; };
-constexpr int kLayerArrays = 19;
+constexpr int kLayerArrays = 21;
 void layer_arrays(LayerDev &d, ArrayRef (&t)[kLayerArrays])
 {
     const size_t MK = (size_t)d.M * d.K, M = (size_t)d.M;
@@ -46,7 +46,9 @@ void layer_arrays(LayerDev &d, ArrayRef (&t)[kLayerArrays])
     t[i++] = {(void **)&d.fxQ, M * 4};
     t[i++] = {(void **)&d.fxB, M * 4};
     t[i++] = {(void **)&d.act, 16};
-    t[i++] = {(void **)&d.w_f32, d.has_f32 ? MK * 4 : 0};
+    t[i++] = {(void **)&d.w_f32, d.has_f32 == 1 ? MK * 4 : 0};
+    t[i++] = {(void **)&d.f_scale, d.has_f32 == 1 ? M * 4 : 0};
+    t[i++] = {(void **)&d.wdig, d.has_f32 == 2 ? 3 * MK : 0}; // two-digit handles leave the last third unused
     t[i++] = {(void **)&d.l1U, d.has_uv ? M * 4 : 0};
     t[i++] = {(void **)&d.l1V, d.has_uv ? M * 4 : 0};
 }
@@ -119,12 +121,12 @@ struct BlobHeader {
     int32_t n_layers, dims[kMaxLayers + 1];
     int32_t w_bits, a_bits, w_gran, a_gran, rotation, activation;
     float omega0, act_s0;
-    int32_t calibrated, calib_layers_done, has_fused;
+    int32_t calibrated, calib_layers_done, has_fused, float_digits;
     int32_t epi_mode[kMaxLayers];
     float phase_bound[kMaxLayers];
     uint64_t payload_bytes, payload_fnv1a;
 };
-constexpr uint32_t kBlobVersion = 4;
+constexpr uint32_t kBlobVersion = 5;
 const char kBlobMagic[8] = {'D', 'H', 'Q', 'B', '2', '0', '0', 0};
 
 uint64_t fnv1a(const uint8_t *p, size_t n)
@@ -230,40 +232,6 @@ dhq_status_t layerwise_forward(dhq_handle_s *h, const float *coords, int64_t n, 
     return DHQ_OK;
 }
 
-// W8A32 / W32A32: one pass of the floating-point layer kernel per layer, in chunks; X dumps optional.
-dhq_status_t float_forward(dhq_handle_s *h, const float *coords, int64_t n, float *out, const dhq_debug_bufs_t *bufs, cudaStream_t st)
-{
-    const int64_t chunk = n < kDebugChunk ? n : kDebugChunk;
-    dhq_status_t s = ensure_scratch(h, chunk);
-    if (s != DHQ_OK) return s;
-    for (int64_t t0 = 0; t0 < n; t0 += chunk) {
-        const int64_t cnt = n - t0 < chunk ? n - t0 : chunk;
-        const float *X = nullptr;
-        for (int l = 1; l <= h->L; ++l) {
-            const LayerDev &d = h->layer[l - 1];
-            FloatLayerArgs a;
-            memset(&a, 0, sizeof(a));
-            a.X = X; a.coords = coords + t0 * 2; a.n = cnt;
-            a.K = d.K; a.M = d.M; a.d_L = h->d_L;
-            a.w8 = h->float_mode == 1;
-            a.rotate = a.w8 && h->cfg.rotation == DHQ_ROT_INPUT;
-            a.qw_k4m = d.qw_k4m; a.w_f32 = reinterpret_cast<const float4 *>(d.w_f32);
-            a.s_w = d.s_w; a.bias = d.bias;
-            a.omega0 = h->cfg.omega0; a.sine = l < h->L;
-            a.Y = h->scratch[(l - 1) & 1];
-            if (l == h->L) a.out = out ? out + t0 * h->d_L : nullptr;
-            if (bufs) {
-                if (bufs->X && bufs->X[l - 1]) a.dX = bufs->X[l - 1] + t0 * d.K;
-                if (bufs->Y && bufs->Y[l - 1]) a.Y = bufs->Y[l - 1] + t0 * d.M;
-            }
-            CK(launch_float_layer(a, st));
-            h->launches++;
-            X = a.Y;
-        }
-    }
-    return DHQ_OK;
-}
-
 // The forward pass of a calibrated handle: the fused kernel, or, for the two-sided transform, the
 // layer-by-layer kernels.
 dhq_status_t run_forward(dhq_handle_s *h, const float *coords, int64_t n, float *out, bool on_host, cudaStream_t st)
@@ -297,6 +265,7 @@ void dhq_destroy(dhq_handle_t h)
     if (!h) return;
     cudaDeviceSynchronize();
     fused_destroy(h);
+    float_destroy(h);
     for (int l = 0; l < kMaxLayers; ++l) free_layer(h->layer[l]);
     cudaFree(h->d_status);
     cudaFree(h->scratch[0]); cudaFree(h->scratch[1]);
@@ -310,6 +279,39 @@ void dhq_destroy(dhq_handle_t h)
         if (h->ev_k[i]) cudaEventDestroy(h->ev_k[i]);
     }
     delete h;
+}
+
+// The floating-point datapaths' own weights.  W8A32: the integer rows q_w H_K need two digits unless a
+// row is close to its largest possible entry (a weight row with one dominant input).
+static dhq_status_t prepare_float(dhq_handle_s *h, const float *const *W, cudaStream_t st)
+{
+    h->float_digits = 3;
+    FloatPrepArgs a;
+    memset(&a, 0, sizeof(a));
+    a.w8 = h->float_mode == 1;
+    a.rotate = a.w8 && h->cfg.rotation == DHQ_ROT_INPUT;
+    a.omega0 = (double)h->cfg.omega0;
+    a.row_max = reinterpret_cast<unsigned int *>(h->d_status) + 12;
+    for (int pass = a.w8 && h->L > 2 ? 0 : 1; pass < 2; ++pass) {
+        for (int l = 1; l <= h->L; ++l) {
+            const LayerDev &d = h->layer[l - 1];
+            a.first = l == 1;
+            a.hidden = l > 1 && l < h->L;
+            if (pass == 0 && !a.hidden) continue;
+            a.digits = pass == 0 ? 0 : h->float_digits;
+            a.W = W[l - 1];
+            a.d_out = d.d_out; a.d_in = d.d_in; a.K = d.K; a.M = d.M;
+            a.dev = d;
+            CK(launch_prep_float(a, st, &h->launches));
+        }
+        if (pass == 0) {
+            unsigned int row_max = 0;
+            CK(cudaMemcpyAsync(&row_max, a.row_max, sizeof(row_max), cudaMemcpyDeviceToHost, st));
+            CK(cudaStreamSynchronize(st));
+            h->float_digits = row_max <= 32639u ? 2 : 3;
+        }
+    }
+    return DHQ_OK;
 }
 
 static dhq_status_t prepare_impl(const dhq_config_t *cfg, const float *const *W, const float *const *b,
@@ -355,11 +357,8 @@ static dhq_status_t prepare_impl(const dhq_config_t *cfg, const float *const *W,
             // coordinates are not bounded by the weights; the wavelet's envelope needs the unwrapped phase
             if (l == 1) d.epi_mode = (per_token || gabor) ? EPI_SINE_WIDE : EPI_SINE_FIXED;
             d.has_uv = both && l == 1;
-            d.has_f32 = h->float_mode == 2;
+            d.has_f32 = !h->float_mode ? 0 : (l == 1 || l == L) ? 1 : 2;
             if (!alloc_layer(d)) { rc = DHQ_ERR_ALLOC; break; }
-            if (d.has_f32 && launch_prep_float_weights(W[l - 1], d.d_out, d.d_in, d.K, d.M, d.w_f32, st) != cudaSuccess) {
-                rc = DHQ_ERR_CUDA; break;
-            }
             if (cudaMemsetAsync(d.act, 0, 16, st) != cudaSuccess) { rc = DHQ_ERR_CUDA; break; }
             PrepArgs a;
             memset(&a, 0, sizeof(a));
@@ -377,12 +376,13 @@ static dhq_status_t prepare_impl(const dhq_config_t *cfg, const float *const *W,
             a.phase_bound = d_bounds + (l - 1);
             a.code_l1 = d_sums + (l - 1);
             if (launch_prepare(a, st, &h->launches) != cudaSuccess) { rc = DHQ_ERR_CUDA; break; }
-            if (per_token &&
-                launch_finalize(d, h->float_mode ? 8 : cfg->a_bits, 1, l < L, (double)cfg->omega0, st, &h->launches) != cudaSuccess) {
+            if (per_token && !h->float_mode &&
+                launch_finalize(d, cfg->a_bits, 1, l < L, (double)cfg->omega0, st, &h->launches) != cudaSuccess) {
                 rc = DHQ_ERR_CUDA; break;
             }
         }
         if (rc != DHQ_OK) break;
+        if (h->float_mode && (rc = prepare_float(h, W, st)) != DHQ_OK) break;
         float bounds[kMaxLayers];
         unsigned long long sums[kMaxLayers];
         if (cudaMemcpyAsync(bounds, d_bounds, sizeof(bounds), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -408,7 +408,8 @@ static dhq_status_t prepare_impl(const dhq_config_t *cfg, const float *const *W,
         h->calibrated = per_token;
         // layer by layer: the fp32 datapaths, the two-sided transform with per-channel weight scales, and the
         // wavelet combined with the two-sided transform
-        if ((!both || both_fused) && !h->float_mode) rc = fused_create(h);
+        if (h->float_mode) rc = float_create(h);
+        else if (!both || both_fused) rc = fused_create(h);
     } while (0);
     cudaFree(d_bounds);
     cudaFree(d_sums);
@@ -691,6 +692,7 @@ dhq_status_t dhq_export(dhq_handle_t h, void *host_buf, int64_t capacity, int64_
     hd.calibrated = h->calibrated ? 1 : 0;
     hd.calib_layers_done = h->calib_layers_done;
     hd.has_fused = h->fused ? 1 : 0;
+    hd.float_digits = h->float_digits;
     for (int l = 0; l < h->L; ++l) {
         hd.epi_mode[l] = h->layer[l].epi_mode;
         hd.phase_bound[l] = h->layer[l].phase_bound;
@@ -726,12 +728,14 @@ dhq_status_t dhq_import(const void *host_buf, int64_t bytes, void *stream, dhq_h
     h->cfg.dims = h->dims;
     h->L = hd.n_layers; h->w = dims[1]; h->d_L = dims[hd.n_layers];
     h->float_mode = float_mode_of(cfg);
+    h->float_digits = hd.float_digits;
+    if (h->float_mode ? (hd.float_digits != 2 && hd.float_digits != 3) : hd.float_digits != 0) { delete h; return DHQ_ERR_INVALID_ARG; }
     h->gabor_s0 = cfg.activation == DHQ_ACT_GABOR ? (double)cfg.act_s0 : 0.0;
     size_t payload = 0;
     for (int l = 1; l <= h->L; ++l) {
         LayerDev &d = h->layer[l - 1];
         set_layer_dims(d, l, h->L, h->w, dims);
-        d.has_f32 = h->float_mode == 2;
+        d.has_f32 = !h->float_mode ? 0 : (l == 1 || l == h->L) ? 1 : 2;
         d.has_uv = cfg.rotation == DHQ_ROT_BOTH && l == 1;
         ArrayRef t[kLayerArrays];
         layer_arrays(d, t);
@@ -766,7 +770,8 @@ dhq_status_t dhq_import(const void *host_buf, int64_t bytes, void *stream, dhq_h
         if (cudaStreamSynchronize(st) != cudaSuccess) { rc = DHQ_ERR_CUDA; break; } // host_buf may go after the call
         h->calibrated = hd.calibrated != 0;
         h->calib_layers_done = hd.calib_layers_done;
-        if (hd.has_fused) rc = fused_create(h);
+        if (h->float_mode) rc = float_create(h);
+        else if (hd.has_fused) rc = fused_create(h);
     } while (0);
     if (rc != DHQ_OK) {
         dhq_destroy(h);

@@ -32,8 +32,11 @@ struct LayerDev {
     float *act = nullptr;      // [4]: frozen absmax (max taken on the bit pattern), s_x, inv, unused
     int has_uv = 0;            // two-sided transform, layer 1: l1U, l1V below
     int32_t *l1U = nullptr, *l1V = nullptr; // [M] H_M applied to u_m = q[m][0]+q[m][2] and v_m = q[m][1]+q[m][3]
-    int has_f32 = 0;           // W32A32 handles keep the unquantized weights too
-    float *w_f32 = nullptr;    // [K/4][M] float4: fp32 weights, zero padded (has_f32 only)
+    int has_f32 = 0;           // floating-point datapaths: 1 first and last layer (w_f32, f_scale), 2 hidden layer (wdig)
+    float *w_f32 = nullptr;    // last layer: [K/4][M] float4 fp32 weights (W8A32: the integers q_w H_K), zero padded;
+                               // first layer: [M] float4 (two weights and the bias in turns of the phase)
+    float *f_scale = nullptr;  // [M] last layer: scale of the rows of w_f32 (W32A32: 1)
+    uint8_t *wdig = nullptr;   // base-256 digits of the rows of a hidden layer in tensor-core order
 };
 
 } // namespace dhq
@@ -61,6 +64,8 @@ struct dhq_handle_s {
     unsigned long long wait_limit_ns = 2000000000ull; // bound of every wait inside the fused kernel (dhq_set_wait_limit)
     bool stall_next_forward = false; // test hook: see dhq_debug_stall_next_forward
     double gabor_s0 = 0.0;          // > 0: wavelet activation (layer-by-layer path)
+    void *float_state = nullptr;    // state of the floating-point datapaths
+    int float_digits = 0;           // base-256 digits per weight of their hidden layers
     int float_mode = 0;             // 0: fully quantized (DHQ); 1: W8A32 (activations fp32); 2: W32A32 (plain fp32 network)
 };
 
@@ -102,25 +107,24 @@ struct LayerArgs {
 
 cudaError_t launch_layer(const LayerArgs &a, cudaStream_t st);
 
-// Arguments of one pass of the floating-point comparison datapaths (W8A32, W32A32).
-struct FloatLayerArgs {
-    const float *X;        // [n][K] layer input, or NULL for layer 1 (built from coords)
-    const float *coords;   // [n][2], layer 1 only
-    int64_t n;
-    int K, M, d_L;
-    int rotate;            // W8A32 with the Hadamard fold: rotate the layer input
-    int w8;                // 1: quantized weights (qw_k4m, s_w); 0: fp32 weights (w_f32)
-    const uint32_t *qw_k4m;
-    const float4 *w_f32;
-    const float *s_w, *bias;
-    float omega0;
-    int sine;
-    float *Y;              // [n][M] or NULL
-    float *out;            // [n][d_L] or NULL (last layer)
-    float *dX;             // dump of the layer input, or NULL
+// The floating-point comparison datapaths (W8A32, W32A32), dhq_float.cu.
+dhq_status_t float_create(dhq_handle_s *h);
+void float_destroy(dhq_handle_s *h);
+// bufs: X and Y dumps only, may be NULL; out may be NULL when bufs is given
+dhq_status_t float_forward(dhq_handle_s *h, const float *coords, int64_t n, float *out, const dhq_debug_bufs_t *bufs, cudaStream_t st);
+struct FloatPrepArgs {
+    const float *W;        // fp32 weights as given, [d_out][d_in]
+    int d_out, d_in, K, M;
+    int w8;                // 1: the row is q_w (H_K), from the codes; 0: the fp32 row
+    int rotate;            // w8: the codes are those of rotated weights
+    int first;             // layer 1: weights and bias in turns of the phase
+    int hidden;            // 1: base-256 digits for the tensor cores; 0: fp32 (last layer)
+    int digits;            // hidden: 2 or 3, or 0 to only take the largest |value| (w8) into *row_max
+    unsigned int *row_max;
+    double omega0;
+    LayerDev dev;
 };
-cudaError_t launch_float_layer(const FloatLayerArgs &a, cudaStream_t st);
-cudaError_t launch_prep_float_weights(const float *W, int d_out, int d_in, int K, int M, float *dst, cudaStream_t st);
+cudaError_t launch_prep_float(const FloatPrepArgs &a, cudaStream_t st, int64_t *launches);
 
 struct PrepArgs {
     const float *W, *b;

@@ -1,0 +1,60 @@
+"""The floating-point datapaths where their fixed-point kernel can go wrong: every width, one and
+several tiles with ragged ends, more tiles than the grid has blocks, no tensor-core layer (L = 2),
+many layers, and integer rows that need a third digit (a weight row with one dominant input: its
+rotated codes are +-127 throughout, so q H has an entry of 127 K).
+
+The reference is the fp64 definition of each layer on the library's own input of that layer, at the
+gate of the other float tests: fp32 phase of the first layer (50 rad, half an ulp 1.9e-6, and the
+rounding of its constants, 3e-6), 24-bit activations and weights of the others (below 2e-6)."""
+import numpy as np
+import pytest
+import torch
+
+import dhq_inputs
+from tests.gpu_util import to_dev
+
+pytestmark = pytest.mark.gpu
+
+dhq = pytest.importorskip("paper_2508_13478_b200")
+from oracle import dhq_oracle as orc  # noqa: E402
+from oracle import odef  # noqa: E402
+
+TOL_FLOAT = 2e-5
+
+
+@pytest.mark.parametrize("width,n_linear,d_out,n,w_bits,sparse", [
+    (64, 2, 1, 1, 32, False), (64, 5, 4, 127, 8, False), (128, 3, 2, 129, 32, False), (128, 4, 3, 300, 8, True),
+    (256, 16, 3, 128, 32, False), (256, 3, 1, 128 * 149 + 5, 8, False), (256, 4, 4, 257, 8, True), (512, 2, 3, 200, 8, False),
+    (512, 3, 3, 128 * 148 + 1, 32, False), (512, 4, 2, 385, 8, True), (512, 5, 3, 1, 4, False)])
+def test_fixed_point_layers(width, n_linear, d_out, n, w_bits, sparse):
+    dims = (2,) + (width,) * (n_linear - 1) + (d_out,)
+    weights, biases = dhq_inputs.siren_init(dims, 30.0, 700 + width + n_linear)
+    if sparse:
+        weights[1][::3] = 0.0
+        weights[1][np.arange(0, width, 3), (7 * np.arange(0, width, 3)) % width] = 0.02
+    coords = dhq_inputs.grid_coords(n // 100 + 1, 100)[:n]
+    h = dhq.dhq_prepare(dims, [to_dev(x) for x in weights], [to_dev(x) for x in biases], 30.0, w_bits, dhq.DHQ_BITS_FLOAT)
+    try:
+        cd = to_dev(coords)
+        X = [torch.empty((n, dhq.dhq_layer_dims(h, l)[0]), device="cuda") for l in range(1, n_linear + 1)]
+        Y = [torch.empty((n, dhq.dhq_layer_dims(h, l)[1]), device="cuda") for l in range(1, n_linear + 1)]
+        dumped = torch.empty((n, d_out), device="cuda")
+        dhq.dhq_forward_debug(h, cd, dumped, {"X": X, "Y": Y})
+        out = torch.full((n, d_out), float("nan"), device="cuda")
+        dhq.dhq_forward(h, cd, out)
+        torch.cuda.synchronize()
+        assert dhq.dhq_last_status(h) == 0
+        assert torch.equal(out.view(torch.int32), dumped.view(torch.int32))
+    finally:
+        dhq.dhq_destroy(h)
+    net = orc.prepare(weights, biases, dims, 30.0, w_bits if w_bits < 32 else 8, 8, 0, 1, rotate=True)
+    for l in range(1, n_linear + 1):
+        x = X[l - 1].cpu().numpy()
+        if w_bits < 32:
+            lay = net.layers[l - 1]
+            want = odef.w8a32_layer(lay.qw, lay.s_w, lay.b_pad, x, True, 30.0, lay.sine)
+        else:
+            z = x.astype(np.float64)[:, : dims[l - 1]] @ weights[l - 1].astype(np.float64).T + biases[l - 1].astype(np.float64)
+            want = np.sin(30.0 * z) if l < n_linear else z
+        got = Y[l - 1].cpu().numpy()[:, : want.shape[1]]
+        assert np.abs(got - want).max() <= TOL_FLOAT, f"layer {l}"
