@@ -86,6 +86,8 @@ def load_library():
     L.dhq_last_status.argtypes = [vp]
     L.dhq_launch_count.argtypes = [vp]
     L.dhq_launch_count.restype = c_i64
+    L.dhq_release_cached_memory.argtypes = []
+    L.dhq_release_cached_memory.restype = None
     L.dhq_destroy.argtypes = [vp]
     L.dhq_destroy.restype = None
     L.dhq_status_string.argtypes = [c_i]
@@ -292,6 +294,11 @@ def dhq_launch_count(handle) -> int:
 
 def dhq_destroy(handle):
     load_library().dhq_destroy(handle)
+
+
+def dhq_release_cached_memory():
+    """Give the device memory kept from destroyed handles back to the device."""
+    load_library().dhq_release_cached_memory()
 
 
 def dhq_measure_pipe(pipe, iters=2000, stream=None):

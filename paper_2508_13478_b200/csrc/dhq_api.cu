@@ -4,6 +4,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include "dhq_internal.cuh"
 
@@ -53,21 +54,101 @@ void layer_arrays(LayerDev &d, ArrayRef (&t)[kLayerArrays])
     t[i++] = {(void **)&d.l1V, d.has_uv ? M * 4 : 0};
 }
 
-bool alloc_layer(LayerDev &d)
+// ------------------------------------------------------------------ device memory of a handle
+//
+// Everything a handle needs from dhq_prepare or dhq_import to dhq_destroy lies in one allocation: with
+// one cudaMalloc per array (21 arrays a layer) opening and closing a 4-layer network spent 1.3 of its
+// 1.5 ms in cudaMalloc and cudaFree, and up to 28 ms on a device with a long allocation history.
+// Released blocks are kept for the next handle of the process, at most kPoolBlocks of them and
+// kPoolBytes together over all devices; what does not fit is freed, and dhq_release_cached_memory or a
+// failed allocation frees all.  dhq_destroy waits for the device before it releases the block, so a
+// block handed out again is not in use on any stream.
+constexpr int kPoolBlocks = 8;
+constexpr size_t kPoolBytes = 128u << 20;
+struct PoolBlock { void *p; size_t bytes; int device; };
+std::mutex g_pool_mutex;
+PoolBlock g_pool[kPoolBlocks];
+int g_pool_count = 0;
+size_t g_pool_bytes = 0;
+
+void pool_free_all()
 {
-    ArrayRef t[kLayerArrays];
-    layer_arrays(d, t);
-    for (const ArrayRef &a : t)
-        if (cudaMalloc(a.ptr, a.bytes < 16 ? 16 : a.bytes) != cudaSuccess) return false;
-    return true;
+    std::lock_guard<std::mutex> lock(g_pool_mutex);
+    for (int i = 0; i < g_pool_count; ++i) cudaFree(g_pool[i].p);
+    g_pool_count = 0;
+    g_pool_bytes = 0;
 }
 
-void free_layer(LayerDev &d)
+// A block of at least `bytes` on the current device `device`; *got receives its size.
+void *pool_take(size_t bytes, int device, size_t *got)
 {
-    ArrayRef t[kLayerArrays];
-    layer_arrays(d, t);
-    for (const ArrayRef &a : t) cudaFree(*a.ptr);
-    d = LayerDev();
+    {
+        std::lock_guard<std::mutex> lock(g_pool_mutex);
+        int best = -1;
+        for (int i = 0; i < g_pool_count; ++i)
+            if (g_pool[i].device == device && g_pool[i].bytes >= bytes && g_pool[i].bytes <= 2 * bytes + 65536 &&
+                (best < 0 || g_pool[i].bytes < g_pool[best].bytes)) best = i;
+        if (best >= 0) {
+            void *p = g_pool[best].p;
+            *got = g_pool[best].bytes;
+            g_pool_bytes -= g_pool[best].bytes;
+            g_pool[best] = g_pool[--g_pool_count];
+            return p;
+        }
+    }
+    void *p = nullptr;
+    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+        (void)cudaGetLastError();
+        pool_free_all();
+        if (cudaMalloc(&p, bytes) != cudaSuccess) return nullptr;
+    }
+    *got = bytes;
+    return p;
+}
+
+void pool_give(void *p, size_t bytes, int device)
+{
+    if (!p) return;
+    {
+        std::lock_guard<std::mutex> lock(g_pool_mutex);
+        if (g_pool_count < kPoolBlocks && g_pool_bytes + bytes <= kPoolBytes) {
+            g_pool[g_pool_count++] = {p, bytes, device};
+            g_pool_bytes += bytes;
+            return;
+        }
+    }
+    cudaFree(p);
+}
+
+// Lays the handle's arrays out in one block (h->device is current).  At its start, zeroed on `st`: the
+// status words, what the preparation accumulates, and the layers' activation scales.
+dhq_status_t alloc_handle(dhq_handle_s *h, cudaStream_t st)
+{
+    auto place = [&](uint8_t *base) {
+        size_t off = 0;
+        auto put = [&](void **ptr, size_t bytes) {
+            *ptr = base + off;
+            off += (bytes + 255) & ~(size_t)255;
+        };
+        put((void **)&h->d_status, 64);
+        put((void **)&h->d_prep, sizeof(PrepSums));
+        void *acts = nullptr;
+        put(&acts, 16 * h->L);
+        h->zero_bytes = off;
+        put((void **)&h->x_scratch, h->float_mode ? float_scratch_bytes(h) : 0);
+        for (int l = 0; l < h->L; ++l) {
+            ArrayRef t[kLayerArrays];
+            layer_arrays(h->layer[l], t);
+            for (const ArrayRef &a : t) put(a.ptr, a.bytes);
+            h->layer[l].act = static_cast<float *>(acts) + 4 * l;
+        }
+        return off;
+    };
+    h->block = pool_take(place(nullptr), h->device, &h->block_bytes);
+    if (!h->block) return DHQ_ERR_ALLOC;
+    place(static_cast<uint8_t *>(h->block));
+    CK(cudaMemsetAsync(h->block, 0, h->zero_bytes, st));
+    return DHQ_OK;
 }
 
 // Padded sizes of layer l (1-based) of a network of hidden width w.
@@ -170,20 +251,21 @@ LayerArgs layer_args(dhq_handle_s *h, int l, const float *coords, const float *X
 }
 
 // One calibration pass: the maximum of |rotated input of layer l| over the given coordinates, with
-// layers < l run as they are frozen, is left in the layer's act[0] (not yet turned into scales).
-dhq_status_t calibrate_layer_pass(dhq_handle_s *h, int l, const float *coords, int64_t n, cudaStream_t st)
+// layers < l run as they are frozen, is left in the layer's act[0].  freeze: act[0] is zero already, and
+// the layer's scales and epilogue constants are formed as well.
+dhq_status_t calibrate_layer_pass(dhq_handle_s *h, int l, const float *coords, int64_t n, bool freeze, cudaStream_t st)
 {
     if (h->fused && ((uintptr_t)coords & 7) == 0) {
         // the fused kernel run up to layer l's rotated input: one launch instead of l layer passes per
         // 64 Ki coordinates; same arithmetic, so the same maximum bit for bit
-        CK(cudaMemsetAsync(h->layer[l - 1].act, 0, 4 * sizeof(float), st));
-        return fused_calibrate_layer(h, l, coords, n, st);
+        if (!freeze) CK(cudaMemsetAsync(h->layer[l - 1].act, 0, 4 * sizeof(float), st));
+        return fused_calibrate_layer(h, l, coords, n, freeze, st);
     }
     const int64_t chunk = n < kDebugChunk ? n : kDebugChunk;
     dhq_status_t s = ensure_scratch(h, chunk);
     if (s != DHQ_OK) return s;
     LayerDev &d = h->layer[l - 1];
-    CK(cudaMemsetAsync(d.act, 0, 4 * sizeof(float), st));
+    if (!freeze) CK(cudaMemsetAsync(d.act, 0, 4 * sizeof(float), st));
     for (int64_t t0 = 0; t0 < n; t0 += chunk) {
         int64_t cnt = n - t0 < chunk ? n - t0 : chunk;
         const float *X = nullptr;
@@ -196,15 +278,16 @@ dhq_status_t calibrate_layer_pass(dhq_handle_s *h, int l, const float *coords, i
             X = a.Y;
         }
     }
+    if (freeze) CK(launch_finalize(d, h->cfg.a_bits, 0, l < h->L, (double)h->cfg.omega0, st, &h->launches));
     return DHQ_OK;
 }
 
 dhq_status_t calibrate_impl(dhq_handle_s *h, const float *coords, int64_t n, cudaStream_t st)
 {
+    CK(cudaMemsetAsync(h->layer[0].act, 0, (size_t)h->L * 16, st)); // the layers' scales lie side by side
     for (int l = 1; l <= h->L; ++l) {
-        dhq_status_t s = calibrate_layer_pass(h, l, coords, n, st);
+        dhq_status_t s = calibrate_layer_pass(h, l, coords, n, true, st);
         if (s != DHQ_OK) return s;
-        CK(launch_finalize(h->layer[l - 1], h->cfg.a_bits, 0, l < h->L, (double)h->cfg.omega0, st, &h->launches));
     }
     h->calibrated = true;
     h->calib_layers_done = h->L;
@@ -266,8 +349,7 @@ void dhq_destroy(dhq_handle_t h)
     cudaDeviceSynchronize();
     fused_destroy(h);
     float_destroy(h);
-    for (int l = 0; l < kMaxLayers; ++l) free_layer(h->layer[l]);
-    cudaFree(h->d_status);
+    pool_give(h->block, h->block_bytes, h->device);
     cudaFree(h->scratch[0]); cudaFree(h->scratch[1]);
     cudaFree(h->stage_in); cudaFree(h->stage_out);
     if (h->copy_in) cudaStreamDestroy(h->copy_in);
@@ -291,7 +373,7 @@ static dhq_status_t prepare_float(dhq_handle_s *h, const float *const *W, cudaSt
     a.w8 = h->float_mode == 1;
     a.rotate = a.w8 && h->cfg.rotation == DHQ_ROT_INPUT;
     a.omega0 = (double)h->cfg.omega0;
-    a.row_max = reinterpret_cast<unsigned int *>(h->d_status) + 12;
+    a.row_max = &h->d_prep->row_max;
     for (int pass = a.w8 && h->L > 2 ? 0 : 1; pass < 2; ++pass) {
         for (int l = 1; l <= h->L; ++l) {
             const LayerDev &d = h->layer[l - 1];
@@ -337,8 +419,6 @@ static dhq_status_t prepare_impl(const dhq_config_t *cfg, const float *const *W,
     h->L = L; h->w = w; h->d_L = d_L;
     cudaStream_t st = (cudaStream_t)stream;
     dhq_status_t rc = DHQ_OK;
-    float *d_bounds = nullptr;
-    unsigned long long *d_sums = nullptr;
     const bool both = cfg->rotation == DHQ_ROT_BOTH;
     h->float_mode = float_mode_of(*cfg);
     h->gabor_s0 = cfg->activation == DHQ_ACT_GABOR ? (double)cfg->act_s0 : 0.0;
@@ -347,60 +427,48 @@ static dhq_status_t prepare_impl(const dhq_config_t *cfg, const float *const *W,
     const bool per_token = cfg->a_gran == DHQ_GRAN_CHANNEL_OR_TOKEN || h->float_mode != 0;
     do {
         if (cudaGetDevice(&h->device) != cudaSuccess) { rc = DHQ_ERR_CUDA; break; }
-        if (!dev_alloc(&h->d_status, 16) || !dev_alloc(&d_bounds, kMaxLayers) || !dev_alloc(&d_sums, kMaxLayers)) { rc = DHQ_ERR_ALLOC; break; }
-        if (cudaMemsetAsync(h->d_status, 0, 64, st) != cudaSuccess ||
-            cudaMemsetAsync(d_bounds, 0, kMaxLayers * sizeof(float), st) != cudaSuccess ||
-            cudaMemsetAsync(d_sums, 0, kMaxLayers * sizeof(unsigned long long), st) != cudaSuccess) { rc = DHQ_ERR_CUDA; break; }
-        for (int l = 1; l <= L && rc == DHQ_OK; ++l) {
+        PrepNet net;
+        memset(&net, 0, sizeof(net));
+        net.L = L; net.w = w;
+        for (int l = 1; l <= L; ++l) {
             LayerDev &d = h->layer[l - 1];
             set_layer_dims(d, l, L, w, cfg->dims);
             // coordinates are not bounded by the weights; the wavelet's envelope needs the unwrapped phase
             if (l == 1) d.epi_mode = (per_token || gabor) ? EPI_SINE_WIDE : EPI_SINE_FIXED;
             d.has_uv = both && l == 1;
             d.has_f32 = !h->float_mode ? 0 : (l == 1 || l == L) ? 1 : 2;
-            if (!alloc_layer(d)) { rc = DHQ_ERR_ALLOC; break; }
-            if (cudaMemsetAsync(d.act, 0, 16, st) != cudaSuccess) { rc = DHQ_ERR_CUDA; break; }
-            PrepArgs a;
-            memset(&a, 0, sizeof(a));
-            a.W = W[l - 1]; a.b = b[l - 1];
-            a.d_out = d.d_out; a.d_in = d.d_in; a.K = d.K; a.M = d.M; a.Mt = d.Mt;
-            // (a W32A32 handle still gets 8-bit codes of the unrotated weights; its forward does not read them)
-            a.bits = h->float_mode == 2 ? 8 : cfg->w_bits;
-            a.a_bits = h->float_mode ? 8 : cfg->a_bits;
-            a.per_channel = cfg->w_gran == DHQ_GRAN_CHANNEL_OR_TOKEN;
-            a.sine = l < L; a.first = l == 1;
-            a.permute_rows = (l > 1 && l < L) ? 1 : 0;
-            a.rotate = h->float_mode == 2 ? 0 : cfg->rotation == DHQ_ROT_INPUT ? 1 : both ? 2 : 0;
-            a.omega0 = (double)cfg->omega0;
-            a.dev = d;
-            a.phase_bound = d_bounds + (l - 1);
-            a.code_l1 = d_sums + (l - 1);
-            if (launch_prepare(a, st, &h->launches) != cudaSuccess) { rc = DHQ_ERR_CUDA; break; }
-            if (per_token && !h->float_mode &&
-                launch_finalize(d, cfg->a_bits, 1, l < L, (double)cfg->omega0, st, &h->launches) != cudaSuccess) {
-                rc = DHQ_ERR_CUDA; break;
-            }
         }
-        if (rc != DHQ_OK) break;
+        if ((rc = alloc_handle(h, st)) != DHQ_OK) break;
+        // (a W32A32 handle still gets 8-bit codes of the unrotated weights; its forward does not read them)
+        net.bits = h->float_mode == 2 ? 8 : cfg->w_bits;
+        net.a_bits = h->float_mode ? 8 : cfg->a_bits;
+        net.per_channel = cfg->w_gran == DHQ_GRAN_CHANNEL_OR_TOKEN;
+        net.finalize = per_token && !h->float_mode;
+        net.rotate = h->float_mode == 2 ? 0 : cfg->rotation == DHQ_ROT_INPUT ? 1 : both ? 2 : 0;
+        net.omega0 = (double)cfg->omega0;
+        net.sums = h->d_prep;
+        for (int l = 1; l <= L; ++l) {
+            net.W[l - 1] = W[l - 1]; net.b[l - 1] = b[l - 1];
+            net.dev[l - 1] = h->layer[l - 1];
+        }
+        if (launch_prepare(net, st, &h->launches) != cudaSuccess) { rc = DHQ_ERR_CUDA; break; }
         if (h->float_mode && (rc = prepare_float(h, W, st)) != DHQ_OK) break;
-        float bounds[kMaxLayers];
-        unsigned long long sums[kMaxLayers];
-        if (cudaMemcpyAsync(bounds, d_bounds, sizeof(bounds), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-            cudaMemcpyAsync(sums, d_sums, sizeof(sums), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        PrepSums sums;
+        if (cudaMemcpyAsync(&sums, h->d_prep, sizeof(sums), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess) { rc = DHQ_ERR_CUDA; break; }
         // Two-sided transform in the fused kernel: the output-side rotation runs on the int32 accumulators,
         // which needs one weight scale per tensor and |H_M acc| <= sum_m |acc_m| <= qmax_a * sum |q_w| < 2^31.
         bool both_fused = both && cfg->w_gran == DHQ_GRAN_TENSOR && !h->float_mode;
         for (int l = 1; l <= L && both_fused; ++l)
-            if (sums[l - 1] * (unsigned long long)((1 << (cfg->a_bits - 1)) - 1) >= (1ull << 31)) both_fused = false;
+            if (sums.code_l1[l - 1] * (unsigned long long)((1 << (cfg->a_bits - 1)) - 1) >= (1ull << 31)) both_fused = false;
         const bool a_per_token = cfg->a_gran == DHQ_GRAN_CHANNEL_OR_TOKEN;
         for (int l = 1; l <= L; ++l) {
             LayerDev &d = h->layer[l - 1];
-            d.phase_bound = bounds[l - 1];
+            d.phase_bound = sums.phase_bound[l - 1];
             if (l == L) d.epi_mode = EPI_LINEAR;
             else if (l == 1) {}
             // (two-sided: the quantization error of all M rows meets in every output; no tight phase bound)
-            else if (bounds[l - 1] <= (a_per_token ? kFastPhaseLimitPerToken : kFastPhaseLimit) && !gabor && !both) d.epi_mode = EPI_SINE_FAST;
+            else if (d.phase_bound <= (a_per_token ? kFastPhaseLimitPerToken : kFastPhaseLimit) && !gabor && !both) d.epi_mode = EPI_SINE_FAST;
             // no bound below the limit: the values that are below it still take the short route (the kernels
             // with a per-token scale and the fused two-sided ones carry that variant)
             else d.epi_mode = (!gabor && !h->float_mode && ((a_per_token && !both) || both_fused)) ? EPI_SINE_MIXED : EPI_SINE_WIDE;
@@ -411,8 +479,6 @@ static dhq_status_t prepare_impl(const dhq_config_t *cfg, const float *const *W,
         if (h->float_mode) rc = float_create(h);
         else if (!both || both_fused) rc = fused_create(h);
     } while (0);
-    cudaFree(d_bounds);
-    cudaFree(d_sums);
     if (rc != DHQ_OK) {
         dhq_destroy(h);
         return rc;
@@ -441,7 +507,7 @@ dhq_status_t dhq_calibrate_layer(dhq_handle_t h, int layer, const float *coords,
         CK(cudaMemsetAsync(h->layer[layer - 1].act, 0, 4 * sizeof(float), (cudaStream_t)stream));
         return DHQ_OK;
     }
-    return calibrate_layer_pass(h, layer, coords, n, (cudaStream_t)stream);
+    return calibrate_layer_pass(h, layer, coords, n, false, (cudaStream_t)stream);
 }
 
 dhq_status_t dhq_get_act_absmax(dhq_handle_t h, int layer, float *absmax, void *stream)
@@ -754,11 +820,9 @@ dhq_status_t dhq_import(const void *host_buf, int64_t bytes, void *stream, dhq_h
     dhq_status_t rc = DHQ_OK;
     do {
         if (cudaGetDevice(&h->device) != cudaSuccess) { rc = DHQ_ERR_CUDA; break; }
-        if (!dev_alloc(&h->d_status, 16)) { rc = DHQ_ERR_ALLOC; break; }
-        if (cudaMemsetAsync(h->d_status, 0, 64, st) != cudaSuccess) { rc = DHQ_ERR_CUDA; break; }
+        if ((rc = alloc_handle(h, st)) != DHQ_OK) break;
         for (int l = 0; l < h->L && rc == DHQ_OK; ++l) {
             LayerDev &d = h->layer[l];
-            if (!alloc_layer(d)) { rc = DHQ_ERR_ALLOC; break; }
             ArrayRef t[kLayerArrays];
             layer_arrays(d, t);
             for (const ArrayRef &a : t) {
@@ -828,6 +892,8 @@ dhq_status_t dhq_last_launch_clock(dhq_handle_t h, double *sm_mhz, double *milli
     if (milliseconds) *milliseconds = ns * 1e-6;
     return DHQ_OK;
 }
+
+void dhq_release_cached_memory(void) { pool_free_all(); }
 
 int64_t dhq_launch_count(dhq_handle_t h) { return h ? h->launches : 0; }
 

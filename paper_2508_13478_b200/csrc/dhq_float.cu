@@ -550,6 +550,14 @@ cudaError_t launch_prep_float(const FloatPrepArgs &a, cudaStream_t st, int64_t *
 
 // ------------------------------------------------------------------- host side
 
+// One tile's activations per SM.
+size_t float_scratch_bytes(const dhq_handle_s *h)
+{
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess) sms = 148;
+    return (size_t)sms * 3 * kTile * h->w;
+}
+
 struct FloatState {
     FloatParams p;
     size_t smem_bytes;
@@ -574,9 +582,9 @@ dhq_status_t float_create(dhq_handle_s *h)
     if (!fs) return DHQ_ERR_ALLOC;
     memset(fs, 0, sizeof(*fs));
     h->float_state = fs;
-    int dev = 0, max_optin = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+    const int dev = h->device;
+    int max_optin = 0;
+    if (cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&fs->sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return DHQ_ERR_CUDA;
     FloatParams &p = fs->p;
@@ -599,18 +607,16 @@ dhq_status_t float_create(dhq_handle_s *h)
     p.n_stages = stages;
     fs->smem_bytes = float_map(h->w, stages, h->L).total + 1024;
     if (fs->smem_bytes < (size_t)kMinSmem) fs->smem_bytes = kMinSmem;
-    if (cudaMalloc((void **)&p.x, (size_t)fs->sm_count * 3 * kTile * h->w) != cudaSuccess) return DHQ_ERR_ALLOC;
+    p.x = h->x_scratch;
     float_fn fns[2] = {pick_float<false>(h->w, h->float_digits), pick_float<true>(h->w, h->float_digits)};
     for (float_fn f : fns)
-        if (!f || cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fs->smem_bytes) != cudaSuccess) return DHQ_ERR_CUDA;
+        if (!allow_smem((const void *)f, dev, max_optin)) return DHQ_ERR_CUDA;
     return DHQ_OK;
 }
 
 void float_destroy(dhq_handle_s *h)
 {
-    FloatState *fs = static_cast<FloatState *>(h->float_state);
-    if (fs) cudaFree(fs->p.x);
-    delete fs;
+    delete static_cast<FloatState *>(h->float_state);
     h->float_state = nullptr;
 }
 

@@ -1,6 +1,9 @@
 // Host side of the fused forward (kernels: dhq_fused.cuh, instantiated per width in
 // dhq_fused_w*.cu): the parameter block of a handle, the choice of the instantiation and the
 // launch; and the kernel's per-element loops run in isolation (micro-benchmark).
+#include <mutex>
+#include <set>
+#include <utility>
 #include "dhq_fused.cuh"
 
 namespace dhq {
@@ -29,7 +32,7 @@ static fused_fn pick_gabor_kernel(int W, bool per_token, bool rot)
     }
     return nullptr;
 }
-static fused_fn pick_calib_kernel(int W, bool rot, bool gabor, bool both)
+static fused_calib_fn pick_calib_kernel(int W, bool rot, bool gabor, bool both)
 {
     switch (W) {
     case 64: return fused_pick_calib_64(rot, gabor, both);
@@ -155,6 +158,20 @@ static fused_dump_fn pick_dump_for(const dhq_handle_s *h, bool per_token)
     return pick_dump_kernel(h->w, per_token, rot);
 }
 
+// Lets a kernel use all of an SM's shared memory; the driver is asked once per kernel and device
+// (8 of these calls per dhq_prepare took 15 us).
+bool allow_smem(const void *fn, int device, int bytes)
+{
+    static std::mutex mutex;
+    static std::set<std::pair<const void *, int>> done;
+    if (!fn) return false;
+    std::lock_guard<std::mutex> lock(mutex);
+    if (done.count({fn, device})) return true;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
+    done.insert({fn, device});
+    return true;
+}
+
 dhq_status_t fused_create(dhq_handle_s *h)
 {
     FusedState *fs = new (std::nothrow) FusedState();
@@ -189,9 +206,9 @@ dhq_status_t fused_create(dhq_handle_s *h)
     p.const_words = words;
     fused_fn fn = pick_for(h, p.per_token, false, false);
     if (!fn) return DHQ_ERR_UNSUPPORTED;
-    int dev = 0, max_optin = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+    const int dev = h->device;
+    int max_optin = 0;
+    if (cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&fs->sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return DHQ_ERR_CUDA;
     // weight ring: as many slab stages as fit beside the A tiles and the constants; all hidden
@@ -209,19 +226,10 @@ dhq_status_t fused_create(dhq_handle_s *h)
     size_t bytes = smem_map(h->w, p.n_stages, words).total + 1024;
     if (bytes < (size_t)kMinSmem) bytes = kMinSmem;
     fs->smem_bytes = bytes;
-    for (int v = 0; v < 4; ++v) { // every variant of this handle's kernel
-        fused_fn f = pick_for(h, p.per_token, (v & 1) != 0, (v & 2) != 0);
-        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
-            return DHQ_ERR_CUDA;
-    }
-    if (!p.per_token) {
-        fused_fn fc = pick_calib_kernel(h->w, h->cfg.rotation == DHQ_ROT_INPUT, gabor, both);
-        if (!fc || cudaFuncSetAttribute(fc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
-            return DHQ_ERR_CUDA;
-    }
-    fused_dump_fn fd = pick_dump_for(h, p.per_token);
-    if (!fd || cudaFuncSetAttribute(fd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
-        return DHQ_ERR_CUDA;
+    for (int v = 0; v < 4; ++v) // every variant of this handle's kernel
+        if (!allow_smem((const void *)pick_for(h, p.per_token, (v & 1) != 0, (v & 2) != 0), dev, max_optin)) return DHQ_ERR_CUDA;
+    if (!p.per_token && !allow_smem((const void *)pick_calib_kernel(h->w, h->cfg.rotation == DHQ_ROT_INPUT, gabor, both), dev, max_optin)) return DHQ_ERR_CUDA;
+    if (!allow_smem((const void *)pick_dump_for(h, p.per_token), dev, max_optin)) return DHQ_ERR_CUDA;
     return DHQ_OK;
 }
 
@@ -273,8 +281,9 @@ dhq_status_t fused_forward(dhq_handle_s *h, const float *coords, int64_t n, floa
 
 // Layer 1's rotated input is H_4 [x, y, 0, 0] = [x+y, x-y, x+y, x-y] (or [x, y, 0, 0] without the
 // rotation): its absmax over the coordinate set needs no network.
-__global__ void calib_l1_kernel(const float *coords, long long n, int rot, float *act)
+__global__ void calib_l1_kernel(const float *coords, long long n, int rot, int freeze, int a_bits, double omega0, LayerDev dev)
 {
+    float *act = dev.act;
     float amax = 0.f;
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
         const float2 xy = __ldg(reinterpret_cast<const float2 *>(coords) + t);
@@ -283,28 +292,37 @@ __global__ void calib_l1_kernel(const float *coords, long long n, int rot, float
     }
     for (int o = 16; o; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
     if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned int *>(act), __float_as_uint(amax));
+    __shared__ int last;
+    if (freeze) freeze_by_last_block(dev, a_bits, 1, omega0, &last);
 }
 
 // One calibration pass by the fused kernel: the maximum of |rotated input of layer l| over the
 // coordinates, with layers < l run as they are frozen, is accumulated into the layer's act[0]
 // (which the caller has cleared).  Per-tensor activation scales; every rotation mode and activation
 // that has a fused kernel.
-dhq_status_t fused_calibrate_layer(dhq_handle_s *h, int l, const float *coords, int64_t n, cudaStream_t st)
+dhq_status_t fused_calibrate_layer(dhq_handle_s *h, int l, const float *coords, int64_t n, bool freeze, cudaStream_t st)
 {
     FusedState *fs = static_cast<FusedState *>(h->fused);
     if (!fs || fs->p.per_token || l < 1 || l > h->L) return DHQ_ERR_INVALID_ARG;
     if (n <= 0) return DHQ_OK;
     if (l == 1) {
         const long long blocks = (n + 255) / 256;
-        calib_l1_kernel<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, st>>>(coords, n, h->cfg.rotation != DHQ_ROT_NONE, h->layer[0].act);
+        calib_l1_kernel<<<(unsigned)(blocks < 1184 ? blocks : 1184), 256, 0, st>>>(coords, n, h->cfg.rotation != DHQ_ROT_NONE,
+                                                                                     freeze, h->cfg.a_bits, (double)h->cfg.omega0, h->layer[0]);
         h->launches++;
         return cudaGetLastError() == cudaSuccess ? DHQ_OK : DHQ_ERR_CUDA;
     }
-    FusedParams p = fs->p;
+    FusedParamsCalib p;
+    static_cast<FusedParams &>(p) = fs->p;
     fill_call(h, p, coords, n, nullptr);
     p.L = l; // the network up to the rotated input of layer l
+    p.freeze = freeze;
+    p.a_bits = h->cfg.a_bits;
+    p.sine = l < h->L;
+    p.omega0 = (double)h->cfg.omega0;
+    p.dev = h->layer[l - 1];
     const int slots = (h->w == 512) ? 1 : 2;
-    fused_fn fn = pick_calib_kernel(h->w, h->cfg.rotation == DHQ_ROT_INPUT, h->gabor_s0 > 0.0, h->cfg.rotation == DHQ_ROT_BOTH);
+    fused_calib_fn fn = pick_calib_kernel(h->w, h->cfg.rotation == DHQ_ROT_INPUT, h->gabor_s0 > 0.0, h->cfg.rotation == DHQ_ROT_BOTH);
     const long long ctas = (p.n_tiles + slots - 1) / slots;
     int grid = (int)(ctas < fs->sm_count ? ctas : fs->sm_count);
     fn<<<grid, h->w == 512 ? kThreads + 32 : kThreads, fs->smem_bytes, st>>>(p);

@@ -37,6 +37,7 @@
 #include <cstring>
 #include <new>
 #include <type_traits>
+#include "dhq_finalize.cuh"
 #include "dhq_internal.cuh"
 #include "dhq_tmem.cuh"
 
@@ -122,7 +123,13 @@ struct FusedParams {
 struct FusedParamsDump : FusedParams {
     DumpPtrs d;
 };
-template <bool DUMP> using ParamsOf = std::conditional_t<DUMP, FusedParamsDump, FusedParams>;
+struct FusedParamsCalib : FusedParams {
+    int freeze;          // the kernel's last block turns the maximum into the layer's scales and constants
+    int a_bits, sine;
+    double omega0;
+    LayerDev dev;        // the calibrated layer
+};
+template <bool DUMP, bool CALIB = false> using ParamsOf = std::conditional_t<DUMP, FusedParamsDump, std::conditional_t<CALIB, FusedParamsCalib, FusedParams>>;
 
 struct FusedState {
     FusedParams p;
@@ -752,7 +759,7 @@ template <int W> __device__ __forceinline__ bool int_butterfly_across(SlotCtx &c
 }
 
 template <int W, bool PER_TOKEN, bool ROT, bool SPREAD, bool AHEAD, bool DUMP, bool BOTH, bool CALIB, bool GABOR, bool MIXED>
-__device__ void epilogue_role(const ParamsOf<DUMP> &p, const SmemMap &sm, uint32_t smem_base, int warp, int lane,
+__device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm, uint32_t smem_base, int warp, int lane,
                               uint32_t tmem_base, volatile int *abort_flag)
 {
     using C = Cfg<W>;
@@ -1234,7 +1241,7 @@ __device__ void xy_role(const FusedParams &p, const SmemMap &sm, uint32_t smem_b
 
 template <int W, bool PER_TOKEN, bool ROT, bool SPREAD, bool AHEAD, bool DUMP = false, bool BOTH = false, bool CALIB = false,
           bool GABOR = false, bool MIXED = false>
-__global__ void __launch_bounds__(Cfg<W>::THREADS, 1) fused_kernel(const __grid_constant__ ParamsOf<DUMP> p)
+__global__ void __launch_bounds__(Cfg<W>::THREADS, 1) fused_kernel(const __grid_constant__ ParamsOf<DUMP, CALIB> p)
 {
     using C = Cfg<W>;
     extern __shared__ uint8_t smem_raw[];
@@ -1338,6 +1345,9 @@ __global__ void __launch_bounds__(Cfg<W>::THREADS, 1) fused_kernel(const __grid_
             }
         }
     }
+    if constexpr (CALIB) {
+        if (p.freeze) freeze_by_last_block(p.dev, p.a_bits, p.sine, p.omega0, abort_flag);
+    }
 }
 
 // ------------------------------------------------------------------- choosing an instantiation
@@ -1387,7 +1397,8 @@ template <int W> fused_dump_fn pick_both_dump_width(bool per_token)
 }
 // Calibration kernels (per-tensor activation scales): the network up to the rotated input of layer
 // p.L, whose absmax they take.
-template <int W> fused_fn pick_calib_width(bool rot, bool gabor, bool both)
+typedef void (*fused_calib_fn)(const FusedParamsCalib);
+template <int W> fused_calib_fn pick_calib_width(bool rot, bool gabor, bool both)
 {
     if (both) return gabor ? fused_kernel<W, false, true, false, false, false, true, true, true> : fused_kernel<W, false, true, false, false, false, true, true, false>;
     if (gabor) return rot ? fused_kernel<W, false, true, false, false, false, false, true, true> : fused_kernel<W, false, false, false, false, false, false, true, true>;
@@ -1450,10 +1461,10 @@ fused_dump_fn fused_pick_gabor_dump_64(bool per_token, bool rot);
 fused_dump_fn fused_pick_gabor_dump_128(bool per_token, bool rot);
 fused_dump_fn fused_pick_gabor_dump_256(bool per_token, bool rot);
 fused_dump_fn fused_pick_gabor_dump_512(bool per_token, bool rot);
-fused_fn fused_pick_calib_64(bool rot, bool gabor, bool both);
-fused_fn fused_pick_calib_128(bool rot, bool gabor, bool both);
-fused_fn fused_pick_calib_256(bool rot, bool gabor, bool both);
-fused_fn fused_pick_calib_512(bool rot, bool gabor, bool both);
+fused_calib_fn fused_pick_calib_64(bool rot, bool gabor, bool both);
+fused_calib_fn fused_pick_calib_128(bool rot, bool gabor, bool both);
+fused_calib_fn fused_pick_calib_256(bool rot, bool gabor, bool both);
+fused_calib_fn fused_pick_calib_512(bool rot, bool gabor, bool both);
 fused_fn fused_pick_both_64(bool per_token);
 fused_fn fused_pick_both_128(bool per_token);
 fused_fn fused_pick_both_256(bool per_token);

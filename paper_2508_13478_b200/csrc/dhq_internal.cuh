@@ -41,6 +41,8 @@ struct LayerDev {
 
 } // namespace dhq
 
+namespace dhq { struct PrepSums; }
+
 struct dhq_handle_s {
     dhq_config_t cfg;
     int dims[dhq::kMaxLayers + 1];
@@ -49,7 +51,11 @@ struct dhq_handle_s {
     bool calibrated = false;
     int calib_layers_done = 0;      // layers whose per-tensor activation scale is frozen (sharded calibration)
     dhq::LayerDev layer[dhq::kMaxLayers];
+    void *block = nullptr;          // the device memory of everything below up to the layers' arrays
+    size_t block_bytes = 0, zero_bytes = 0;
     int *d_status = nullptr;        // device status word
+    dhq::PrepSums *d_prep = nullptr; // accumulated by the preparation kernels
+    uint8_t *x_scratch = nullptr;   // activations of the floating-point datapaths, see FloatParams
     float *scratch[2] = {nullptr, nullptr}; // ping-pong activations of the layer-by-layer path
     int64_t scratch_tokens = 0;
     float *stage_in = nullptr, *stage_out = nullptr; // dhq_forward_host staging
@@ -110,6 +116,7 @@ cudaError_t launch_layer(const LayerArgs &a, cudaStream_t st);
 // The floating-point comparison datapaths (W8A32, W32A32), dhq_float.cu.
 dhq_status_t float_create(dhq_handle_s *h);
 void float_destroy(dhq_handle_s *h);
+size_t float_scratch_bytes(const dhq_handle_s *h);
 // bufs: X and Y dumps only, may be NULL; out may be NULL when bufs is given
 dhq_status_t float_forward(dhq_handle_s *h, const float *coords, int64_t n, float *out, const dhq_debug_bufs_t *bufs, cudaStream_t st);
 struct FloatPrepArgs {
@@ -126,21 +133,25 @@ struct FloatPrepArgs {
 };
 cudaError_t launch_prep_float(const FloatPrepArgs &a, cudaStream_t st, int64_t *launches);
 
-struct PrepArgs {
-    const float *W, *b;
-    int d_out, d_in, K, M, Mt;
+// What the preparation kernels accumulate over a layer for the host.
+struct PrepSums {
+    float phase_bound[kMaxLayers];
+    unsigned long long code_l1[kMaxLayers]; // sum over the layer of |q_w[m][k]| (bounds the rotated accumulators)
+    unsigned int row_max;                   // see FloatPrepArgs
+};
+// The weight side of a whole network: every kernel covers all layers.
+struct PrepNet {
+    int L, w;
     int bits, per_channel;
     int a_bits;            // activation bit-width (enters the phase bound)
     int rotate;            // 0: DHQ_ROT_NONE, weights are quantized as they are; 2: DHQ_ROT_BOTH, columns rotated too
-    int permute_rows;      // 1: rows of the tensor-core image in fused_column order (layers 2 .. L-1)
-    int sine;              // hidden or first layer
-    int first;             // layer 1: no phase bound from the weights (coordinates are unbounded)
+    int finalize;          // per-token activation scales: the epilogue constants too
     double omega0;
-    LayerDev dev;
-    float *phase_bound;    // device scalar
-    unsigned long long *code_l1; // device scalar: sum over the layer of |q_w[m][k]| (bounds the rotated accumulators)
+    PrepSums *sums;        // zeroed
+    const float *W[kMaxLayers], *b[kMaxLayers];
+    LayerDev dev[kMaxLayers];
 };
-cudaError_t launch_prepare(const PrepArgs &a, cudaStream_t st, int64_t *launches);
+cudaError_t launch_prepare(const PrepNet &a, cudaStream_t st, int64_t *launches);
 // Epilogue constants from s_w and (per-tensor) the frozen activation scale.
 cudaError_t launch_finalize(const LayerDev &dev, int a_bits, int per_token, int sine, double omega0,
                             cudaStream_t st, int64_t *launches);
@@ -177,6 +188,8 @@ __host__ __device__ inline int fused_feature(int col, int W)
     const int ch = fused_chunk(W), c = col / ch, j = col % ch;
     return c * ch + (j >> 1) + (j & 1) * (ch / 2);
 }
+// Lets a kernel use `bytes` of dynamic shared memory on `device` (asked of the driver once).
+bool allow_smem(const void *fn, int device, int bytes);
 // Fused tensor-core forward.
 dhq_status_t fused_create(dhq_handle_s *h);
 void fused_destroy(dhq_handle_s *h);
@@ -188,7 +201,8 @@ dhq_status_t fused_forward(dhq_handle_s *h, const float *coords, int64_t n, floa
 // used for layer 1; the input of a later layer is the output of the one before it.
 // One calibration pass of layer l (1-based) by the fused kernel; needs a fused handle with per-tensor
 // activation scales and not the two-sided transform.
-dhq_status_t fused_calibrate_layer(dhq_handle_s *h, int l, const float *coords, int64_t n, cudaStream_t st);
+// (freeze: act[0] is zero already; the kernel's last block forms the scales and epilogue constants)
+dhq_status_t fused_calibrate_layer(dhq_handle_s *h, int l, const float *coords, int64_t n, bool freeze, cudaStream_t st);
 struct DumpPtrs {
     float *X[kMaxLayers];
     int8_t *codes[kMaxLayers];
