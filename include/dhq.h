@@ -79,10 +79,12 @@ typedef enum { DHQ_GRAN_TENSOR = 0, DHQ_GRAN_CHANNEL_OR_TOKEN = 1 } dhq_gran_t;
  * the fused kernel: H_M is applied to the int32 accumulators, exactly (the library checks at
  * prepare time that qmax_a * sum |q_w| < 2^31, so nothing can overflow), then the fp32 epilogue;
  * about 1.6-1.7 times the time of DHQ_ROT_INPUT.  With per-output-channel weight scales the
- * rotation has to act on the dequantized values; that case runs layer by layer (one kernel pass
- * per layer, fp64 rotation), as does dhq_forward_debug for either.  Both routes are within 1e-5 of
- * the definition; they are not bit-identical to each other (fp32 against fp64 epilogue), so for
- * DHQ_ROT_BOTH dhq_forward and dhq_forward_debug need not agree bit for bit;
+ * rotation has to act on the dequantized values.  Widths 128 and 256: H_M diag(s_w) q_W is formed at
+ * prepare time and held in 32-bit fixed point, its product with the activation codes is taken
+ * exactly on the int8 tensor cores (one launch); widths 64 and 512 run layer by layer (fp64
+ * rotation).  Both agree with dhq_forward_debug bit for bit.  With one weight scale per tensor the
+ * two routes are each within 1e-5 of the definition but not bit-identical (fp32 against fp64 epilogue), so there dhq_forward
+ * and dhq_forward_debug need not agree;
  * dhq_forward_fused_debug observes the fused route.  dhq_forward_static_scratch does not take it. */
 typedef enum { DHQ_ROT_INPUT = 0, DHQ_ROT_BOTH = 1, DHQ_ROT_NONE = 2 } dhq_rot_t;
 

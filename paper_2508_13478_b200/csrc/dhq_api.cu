@@ -26,7 +26,7 @@ template <typename T> bool dev_alloc(T **p, size_t count)
 // Every device array of a prepared layer with its size in bytes, in a fixed order (allocation,
 // release, export and import all walk this table).  Needs d.K, d.M, d.Mt.
 struct ArrayRef { void **ptr; size_t bytes; };
-constexpr int kLayerArrays = 21;
+constexpr int kLayerArrays = 26;
 void layer_arrays(LayerDev &d, ArrayRef (&t)[kLayerArrays])
 {
     const size_t MK = (size_t)d.M * d.K, M = (size_t)d.M;
@@ -50,6 +50,11 @@ void layer_arrays(LayerDev &d, ArrayRef (&t)[kLayerArrays])
     t[i++] = {(void **)&d.w_f32, d.has_f32 == 1 ? MK * 4 : 0};
     t[i++] = {(void **)&d.f_scale, d.has_f32 == 1 ? M * 4 : 0};
     t[i++] = {(void **)&d.wdig, d.has_f32 == 2 ? 3 * MK : 0}; // two-digit handles leave the last third unused
+    t[i++] = {(void **)&d.gd_k4m, d.has_digits ? 4 * MK : 0};
+    t[i++] = {(void **)&d.gd_img, d.has_digits && d.K > 4 ? 4 * MK : 0}; // (the last layer's 16 rows are 4 of each digit)
+    t[i++] = {(void **)&d.g_scale, d.has_digits ? M * 8 : 0};
+    t[i++] = {(void **)&d.cN, d.has_digits ? M * 4 : 0};
+    t[i++] = {(void **)&d.cB_lo, d.has_digits ? M * 4 : 0};
     t[i++] = {(void **)&d.l1U, d.has_uv ? M * 4 : 0};
     t[i++] = {(void **)&d.l1V, d.has_uv ? M * 4 : 0};
 }
@@ -120,6 +125,20 @@ void pool_give(void *p, size_t bytes, int device)
     cudaFree(p);
 }
 
+size_t digit_scratch_bytes(const dhq_handle_s *h)
+{
+    size_t b = 0;
+    for (int l = 0; l < h->L; ++l) b += (size_t)h->layer[l].M * h->layer[l].K * sizeof(double);
+    return b;
+}
+
+// The two-sided transform with a weight scale per output channel has a kernel at these widths (at 512 the
+// activations and the digits' sums do not fit tensor memory together; 64 has too few columns per thread).
+bool takes_digits(const dhq_config_t &cfg, int w)
+{
+    return cfg.rotation == DHQ_ROT_BOTH && cfg.w_gran == DHQ_GRAN_CHANNEL_OR_TOKEN && (w == 128 || w == 256);
+}
+
 // Lays the handle's arrays out in one block (h->device is current).  At its start, zeroed on `st`: the
 // status words, what the preparation accumulates, and the layers' activation scales.
 dhq_status_t alloc_handle(dhq_handle_s *h, cudaStream_t st)
@@ -135,6 +154,7 @@ dhq_status_t alloc_handle(dhq_handle_s *h, cudaStream_t st)
         void *acts = nullptr;
         put(&acts, 16 * h->L);
         h->zero_bytes = off;
+        if (h->layer[0].has_digits) put((void **)&h->g_scratch, digit_scratch_bytes(h));
         put((void **)&h->x_scratch, h->float_mode ? float_scratch_bytes(h) : 0);
         for (int l = 0; l < h->L; ++l) {
             ArrayRef t[kLayerArrays];
@@ -207,7 +227,7 @@ struct BlobHeader {
     float phase_bound[kMaxLayers];
     uint64_t payload_bytes, payload_fnv1a;
 };
-constexpr uint32_t kBlobVersion = 5;
+constexpr uint32_t kBlobVersion = 6;
 const char kBlobMagic[8] = {'D', 'H', 'Q', 'B', '2', '0', '0', 0};
 
 uint64_t fnv1a(const uint8_t *p, size_t n)
@@ -245,6 +265,10 @@ LayerArgs layer_args(dhq_handle_s *h, int l, const float *coords, const float *X
     a.rotate = h->cfg.rotation == DHQ_ROT_INPUT ? 1 : h->cfg.rotation == DHQ_ROT_BOTH ? 2 : 0;
     a.s_w = d.s_w; a.bias = d.bias; a.omega0 = (double)h->cfg.omega0; a.sine = l < h->L;
     a.gabor_s0 = h->gabor_s0;
+    if (d.has_digits) {
+        a.gd_k4m = d.gd_k4m; a.g_scale = d.g_scale; a.cN = d.cN; a.cB_lo = d.cB_lo;
+        a.digit_gc = digit_gabor_c(h->gabor_s0, (double)h->cfg.omega0);
+    }
     a.qw_k4m = d.qw_k4m; a.cA = d.cA; a.cA_lo = d.cA_lo; a.cB = d.cB; a.act = d.act;
     a.fxP = d.fxP; a.fxQ = d.fxQ; a.fxB = d.fxB;
     return a;
@@ -320,6 +344,7 @@ dhq_status_t layerwise_forward(dhq_handle_s *h, const float *coords, int64_t n, 
 dhq_status_t run_forward(dhq_handle_s *h, const float *coords, int64_t n, float *out, bool on_host, cudaStream_t st)
 {
     if (h->float_mode) return float_forward(h, coords, n, out, nullptr, st);
+    if (h->digit_state) return digit_forward(h, coords, n, out, st);
     if (!h->fused) return layerwise_forward(h, coords, n, out, st); // wavelet activation; two-sided transform with per-channel weight scales
     return fused_forward(h, coords, n, out, on_host, st);
 }
@@ -349,6 +374,7 @@ void dhq_destroy(dhq_handle_t h)
     cudaDeviceSynchronize();
     fused_destroy(h);
     float_destroy(h);
+    digit_destroy(h);
     pool_give(h->block, h->block_bytes, h->device);
     cudaFree(h->scratch[0]); cudaFree(h->scratch[1]);
     cudaFree(h->stage_in); cudaFree(h->stage_out);
@@ -436,6 +462,7 @@ static dhq_status_t prepare_impl(const dhq_config_t *cfg, const float *const *W,
             // coordinates are not bounded by the weights; the wavelet's envelope needs the unwrapped phase
             if (l == 1) d.epi_mode = (per_token || gabor) ? EPI_SINE_WIDE : EPI_SINE_FIXED;
             d.has_uv = both && l == 1;
+            d.has_digits = takes_digits(*cfg, w);
             d.has_f32 = !h->float_mode ? 0 : (l == 1 || l == L) ? 1 : 2;
         }
         if ((rc = alloc_handle(h, st)) != DHQ_OK) break;
@@ -453,6 +480,18 @@ static dhq_status_t prepare_impl(const dhq_config_t *cfg, const float *const *W,
         }
         if (launch_prepare(net, st, &h->launches) != cudaSuccess) { rc = DHQ_ERR_CUDA; break; }
         if (h->float_mode && (rc = prepare_float(h, W, st)) != DHQ_OK) break;
+        if (h->layer[0].has_digits) {
+            DigitPrep g;
+            memset(&g, 0, sizeof(g));
+            g.L = L; g.w = w; g.finalize = per_token; g.omega0 = (double)cfg->omega0;
+            double *at = h->g_scratch;
+            for (int l = 0; l < L; ++l) {
+                g.dev[l] = h->layer[l];
+                g.g[l] = at;
+                at += (size_t)h->layer[l].M * h->layer[l].K;
+            }
+            if (launch_prep_digits(g, st, &h->launches) != cudaSuccess) { rc = DHQ_ERR_CUDA; break; }
+        }
         PrepSums sums;
         if (cudaMemcpyAsync(&sums, h->d_prep, sizeof(sums), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess) { rc = DHQ_ERR_CUDA; break; }
@@ -477,6 +516,7 @@ static dhq_status_t prepare_impl(const dhq_config_t *cfg, const float *const *W,
         // layer by layer: the fp32 datapaths, the two-sided transform with per-channel weight scales, and the
         // wavelet combined with the two-sided transform
         if (h->float_mode) rc = float_create(h);
+        else if (h->layer[0].has_digits) rc = digit_create(h);
         else if (!both || both_fused) rc = fused_create(h);
     } while (0);
     if (rc != DHQ_OK) {
@@ -648,7 +688,7 @@ static dhq_status_t forward_host_entry(dhq_handle_t h, const float *coords_host,
     // coordinates and writes the result through their device addresses, so the transfers happen
     // inside the kernel, tile by tile, beside the arithmetic.  (Calibration reads the coordinates
     // once per layer: it goes through the staged path below.)
-    if (h->calibrated && h->fused && !((uintptr_t)coords_host & 7) && !((uintptr_t)out_host & 3)) {
+    if (h->calibrated && (h->fused || h->digit_state || h->float_mode) && !((uintptr_t)coords_host & 7) && !((uintptr_t)out_host & 3)) {
         // one query per buffer: for page-locked memory it also gives the device alias (asked on every
         // call on purpose: an answer remembered per address could outlive the buffer it was given for)
         cudaPointerAttributes ai, ao;
@@ -803,6 +843,7 @@ dhq_status_t dhq_import(const void *host_buf, int64_t bytes, void *stream, dhq_h
         set_layer_dims(d, l, h->L, h->w, dims);
         d.has_f32 = !h->float_mode ? 0 : (l == 1 || l == h->L) ? 1 : 2;
         d.has_uv = cfg.rotation == DHQ_ROT_BOTH && l == 1;
+        d.has_digits = takes_digits(cfg, h->w);
         ArrayRef t[kLayerArrays];
         layer_arrays(d, t);
         for (const ArrayRef &a : t) payload += a.bytes;
@@ -835,6 +876,7 @@ dhq_status_t dhq_import(const void *host_buf, int64_t bytes, void *stream, dhq_h
         h->calibrated = hd.calibrated != 0;
         h->calib_layers_done = hd.calib_layers_done;
         if (h->float_mode) rc = float_create(h);
+        else if (h->layer[0].has_digits) rc = digit_create(h);
         else if (hd.has_fused) rc = fused_create(h);
     } while (0);
     if (rc != DHQ_OK) {

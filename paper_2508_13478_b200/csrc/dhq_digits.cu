@@ -1,0 +1,593 @@
+// The two-sided transform (Eq. 4-5 literally) with one weight scale per output channel, widths 128
+// and 256, in one kernel per forward.
+//
+// The layer output is z = H_M (s_w s_x acc) + b with acc = q_W q_x.  The rotation of the outputs acts on
+// numbers that are no longer integers times one scale, so it cannot be taken on the accumulators (as
+// the fused kernel does with one scale per tensor), and an fp32 butterfly of them would cost 1e-7 per
+// radian of phase.  But it is linear, and everything but q_x is known at prepare time:
+//
+//     z = s_x (G q_x) + b,     G = H_M diag(s_w) q_W   (real, M x K; formed in fp64)
+//
+// A row of G is held as 32-bit fixed point relative to its largest entry, in four signed base-256
+// digits, and G q_x is four int8 products with exact int32 sums - the same product for every order of
+// summation, so this kernel and the layer-by-layer one (layer_kernel) give the same bits.  What is
+// lost against fp64 is 2^-32 of the row's largest entry per weight.
+//
+// Layout: one tile of 128 coordinates at a time, 16 epilogue warps; a token is a tensor-memory lane
+// and the four threads of a row own a chunk of W/4 features each.  The outputs come in blocks of 64:
+// block b holds 16 features of every chunk, so that all warps work on every block, the four digits' sums
+// in columns 0-255; activations wait in columns 256-511 until the whole row is there and the rotation
+// of the next layer's input can run through it (stages 1, 2, 4 inside a block, 8 .. W/8 in a thread's
+// chunk, W/4 and W/2 across chunks).  The weights stream from L2 in pieces of 16 KB.
+//
+// What bounds it: the phase of an activation, 24 fp32 operations because it is carried as if in fp64
+// (digit_phase; with the 8 of a plain compensated phase the same launch takes 0.71 ms), beside the
+// butterflies: about 45 issue slots per element against 32 x 51 cycles of MMAs per block of 64 outputs.
+// A block's sums are released as soon as they are in registers, so that the next block's MMAs run
+// beside its phases.  Measured: 2 -> 256 x 5 -> 3, per-channel / per-token, 262,144 coordinates 9.79 -> 0.84 ms
+// (one dp4a pass and an fp64 butterfly per layer before).
+#include "dhq_fused.cuh"
+
+namespace dhq {
+
+constexpr int kDBlock = 64;          // outputs per block
+constexpr int kDActCol = 256;        // first tensor-memory column of the activations
+constexpr int kDThreads = 18 * 32;   // 16 epilogue warps, MMA, weight copies
+constexpr int kDMaxStages = 12;
+
+// Feature of position `i` (0..15) of thread `sub` in block b, chunks of CH = W/4 features: positions 2p and
+// 2p+1 are the features p and p + CH/2 of the chunk, so that a register pair goes through the stages
+// below CH/2 as one packed value.
+__host__ __device__ inline int digit_feature(int W, int b, int sub, int i)
+{
+    const int ch = W / 4;
+    return sub * ch + b * 8 + (i >> 1) + (i & 1) * (ch / 2);
+}
+
+struct DigitLayer {
+    const uint8_t *img;              // [block][digit][K/16][64][16]; last layer: [K/16][16][16], row 4 * digit + output
+    const float *c, *c_lo, *cb, *cb_lo, *cn; // per output: see digit_phase
+    const float *act;
+};
+struct DigitParams {
+    const float *coords;
+    float *out;
+    long long n, n_tiles;
+    int L, d_L, n_stages;
+    float qmaxf, gabor_c;            // gabor_c: s0 / omega0 in turns, 0 for the sine
+    int *status;
+    unsigned long long wait_limit_ns;
+    DigitLayer layer[kMaxLayers];
+    const uint32_t *l1w;             // [4 digits][M] words of four k
+    const double *last_scale;        // [4]
+    const float *last_bias;
+};
+
+struct DigitMap {
+    uint32_t a, ring, last_w, consts, amax, w_full, w_empty, codes_full, acc_full, acc_empty, acc_last, last_full, quad_sync, drain, holder, abort_flag, total;
+};
+__host__ __device__ inline DigitMap digit_map(int W, int n_stages, int L)
+{
+    DigitMap m;
+    uint32_t off = 0;
+    m.a = off; off += kTile * W;
+    m.ring = off; off += (uint32_t)n_stages * kDBlock * W;
+    m.last_w = off; off += 16 * W;
+    m.consts = off; off += (uint32_t)(5 * (L - 1) + 4) * W * 4; // per layer c | c_lo | cb | cb_lo | cn in block order; then layer 1's digits
+    m.amax = off; off += 4 * kTile * 4;
+    m.w_full = off; off += 8 * kDMaxStages;
+    m.w_empty = off; off += 8 * kDMaxStages;
+    m.codes_full = off; off += 8;
+    m.acc_full = off; off += 8;
+    m.acc_empty = off; off += 8;
+    m.acc_last = off; off += 8;
+    m.last_full = off; off += 8;
+    m.quad_sync = off; off += 8 * 4;
+    m.drain = off; off += 8;
+    m.holder = off; off += 8;
+    m.abort_flag = off; off += 16;
+    m.total = off;
+    return m;
+}
+
+// Rotated activations of this thread's quarter of the row -> codes (and, per token, their scale).
+// Chunks of CH columns; the thread takes CH/4 positions of every chunk.
+template <int W, bool PER_TOKEN>
+__device__ __forceinline__ bool digit_finish(SlotCtx &c, float static_s, float static_inv, float &s_out)
+{
+    constexpr int CH = W / 4, G = CH / 4;
+    uint32_t u[4][G];
+    ptx::tmem_wait_st();
+    ptx::tc_fence_before();
+    if (!slot_barrier<true>(c)) return false;
+    ptx::tc_fence_after();
+#pragma unroll
+    for (int ch = 0; ch < 4; ++ch) tmem_ld<G>(c.taddr + ch * CH + c.sub * G, u[ch]);
+    ptx::tmem_wait_ld();
+#pragma unroll
+    for (int h = 1; h < 4; h <<= 1) {
+#pragma unroll
+        for (int ch = 0; ch < 4; ++ch) {
+            if ((ch & h) == 0) {
+#pragma unroll
+                for (int i = 0; i < G; i += 2) {
+                    f32x2 a = pack2u(u[ch][i], u[ch][i + 1]), b = pack2u(u[ch + h][i], u[ch + h][i + 1]);
+                    bfly2(a, b);
+                    unpack2u(a, u[ch][i], u[ch][i + 1]);
+                    unpack2u(b, u[ch + h][i], u[ch + h][i + 1]);
+                }
+            }
+        }
+    }
+    float inv = static_inv;
+    s_out = static_s;
+    if (PER_TOKEN) {
+        float amax = 0.f;
+#pragma unroll
+        for (int ch = 0; ch < 4; ++ch) {
+#pragma unroll
+            for (int i = 0; i < G; ++i) amax = fmaxf(amax, fabsf(__uint_as_float(u[ch][i])));
+        }
+        asm volatile("st.shared.f32 [%0], %1;" ::"r"(c.amax_addr + (c.sub * kTile + c.row) * 4), "f"(amax) : "memory");
+        if (!slot_barrier<true>(c)) return false;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            float o;
+            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(o) : "r"(c.amax_addr + (r * kTile + c.row) * 4));
+            amax = fmaxf(amax, o);
+        }
+        scales_of(amax, c.qmaxf, s_out, inv);
+    }
+#pragma unroll
+    for (int ch = 0; ch < 4; ++ch) quantize_store<G, CH, !PER_TOKEN>(c.a_tile, c.row, ch, c.sub * G, u[ch], inv, c.qmaxf);
+    ptx::fence_proxy_async();
+    ptx::tc_fence_before();
+    ptx::mbar_arrive(c.bar_codes);
+    return true;
+}
+
+template <int W, bool PER_TOKEN, bool GABOR>
+__device__ void digit_epilogue(const DigitParams &p, const DigitMap &sm, uint32_t base, int warp, int lane, uint32_t tmem, volatile int *abort_flag)
+{
+    constexpr int CH = W / 4, NB = W / kDBlock;
+    const int quad = warp & 3, sub = warp >> 2;
+    SlotCtx c;
+    c.row = quad * 32 + lane;
+    c.sub = sub;
+    c.taddr = tmem + kDActCol + ((uint32_t)(quad * 32) << 16);
+    c.a_tile = base + sm.a;
+    c.bar_sync = base + sm.quad_sync + 8 * quad;
+    c.bar_codes = base + sm.codes_full;
+    c.amax_addr = base + sm.amax;
+    c.sync_parity = 0;
+    c.qmaxf = p.qmaxf;
+    c.abort_flag = abort_flag;
+    c.status = p.status;
+    const uint32_t acc = tmem + ((uint32_t)(quad * 32) << 16) + sub * 16;
+    uint32_t use = 0, last_parity = 0;
+    float s_x = 1.0f;
+
+    // four outputs' sums, and constants from shared memory, -> activations
+    auto activations4 = [&](const float *f0, const float *f1, uint32_t at, float *y) {
+        const float4 ca = lds128(at), cl = lds128(at + W * 4), cb = lds128(at + 2 * W * 4), cbl = lds128(at + 3 * W * 4);
+        float4 cn = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (GABOR) cn = lds128(at + 4 * W * 4);
+        const float av[4] = {ca.x, ca.y, ca.z, ca.w}, lv[4] = {cl.x, cl.y, cl.z, cl.w}, bv[4] = {cb.x, cb.y, cb.z, cb.w}, blv[4] = {cbl.x, cbl.y, cbl.z, cbl.w},
+                    nv[4] = {cn.x, cn.y, cn.z, cn.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            float c_hi = av[e], c_lo = lv[e];
+            if (PER_TOKEN) token_const(av[e], lv[e], s_x, c_hi, c_lo);
+            y[e] = sin_approx(digit_phase(f0[e], f1[e], c_hi, c_lo, bv[e], blv[e]));
+            if constexpr (GABOR) y[e] = __fmul_rn(y[e], digit_envelope(f0[e], f1[e], c_hi, bv[e], nv[e], p.gabor_c));
+        }
+    };
+    // stages 1, 2, 4 of 16 finished activations, and into the row's columns
+    auto put_block = [&](int b, const float (&y)[16]) {
+        f32x2 P[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) P[i] = pack2(y[2 * i], y[2 * i + 1]);
+#pragma unroll
+        for (int h = 1; h < 8; h <<= 1) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if ((i & h) == 0) bfly2(P[i], P[i + h]);
+        }
+        uint32_t v[16];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) unpack2u(P[i], v[2 * i], v[2 * i + 1]);
+        ptx::tmem_st16(c.taddr + sub * CH + b * 16, v);
+    };
+    // stages 8 .. CH/2 of the thread's own chunk
+    auto chunk_stages = [&]() {
+        uint32_t v[CH];
+        ptx::tmem_wait_st();
+        tmem_ld<CH>(c.taddr + sub * CH, v);
+        ptx::tmem_wait_ld();
+        f32x2 P[CH / 2];
+#pragma unroll
+        for (int i = 0; i < CH / 2; ++i) P[i] = pack2u(v[2 * i], v[2 * i + 1]);
+#pragma unroll
+        for (int h = 8; h < CH / 2; h <<= 1) {
+#pragma unroll
+            for (int i = 0; i < CH / 2; ++i)
+                if ((i & h) == 0) bfly2(P[i], P[i + h]);
+        }
+#pragma unroll
+        for (int i = 0; i < CH / 2; ++i) {
+            float a, b;
+            unpack2(P[i], a, b);
+            v[2 * i] = __float_as_uint(__fadd_rn(a, b));
+            v[2 * i + 1] = __float_as_uint(__fsub_rn(a, b));
+        }
+        tmem_st<CH>(c.taddr + sub * CH, v);
+    };
+
+    for (long long tile = blockIdx.x; tile < p.n_tiles; tile += gridDim.x) {
+        const long long tok = tile * kTile + c.row;
+        const bool valid = tok < p.n;
+        float x = 0.f, yc = 0.f;
+        if (valid) { x = __ldg(p.coords + 2 * tok); yc = __ldg(p.coords + 2 * tok + 1); }
+        // layer 1: the rotated padded coordinate is [x+y, x-y, x+y, x-y]
+        const float e0 = __fadd_rn(__fadd_rn(x, yc), 0.f), e1 = __fadd_rn(__fsub_rn(x, yc), 0.f);
+        float inv_x;
+        if (PER_TOKEN) {
+            scales_of(fmaxf(fabsf(e0), fabsf(e1)), p.qmaxf, s_x, inv_x);
+        } else {
+            s_x = 1.0f; // the constants hold it
+            inv_x = __ldg(p.layer[0].act + 2);
+        }
+        const uint32_t b0 = code_bits<true>(e0, inv_x, p.qmaxf), b1 = code_bits<true>(e1, inv_x, p.qmaxf);
+        const int qx = (int)pack4(b0, b1, b0, b1);
+        for (int l = 1; l < p.L; ++l) {
+            const uint32_t cbase = base + sm.consts + (uint32_t)((l - 1) * 5 * W * 4);
+            float static_inv = 0.f;
+            if (!PER_TOKEN) static_inv = __ldg(p.layer[l].act + 2);
+#pragma unroll 1
+            for (int b = 0; b < NB; ++b) {
+                const uint32_t at = cbase + (uint32_t)(b * kDBlock + sub * 16) * 4;
+                float f0[16], f1[16];
+                if (l == 1) {
+                    const uint32_t dg = base + sm.consts + (uint32_t)((5 * (p.L - 1) * W + b * kDBlock + sub * 16) * 4);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float4 w0 = lds128(dg + q * 16), w1 = lds128(dg + W * 4 + q * 16), w2 = lds128(dg + 2 * W * 4 + q * 16), w3 = lds128(dg + 3 * W * 4 + q * 16);
+                        const float wv[4][4] = {{w0.x, w0.y, w0.z, w0.w}, {w1.x, w1.y, w1.z, w1.w}, {w2.x, w2.y, w2.z, w2.w}, {w3.x, w3.y, w3.z, w3.w}};
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            digit_sums(__dp4a(qx, (int)__float_as_uint(wv[0][e]), 0), __dp4a(qx, (int)__float_as_uint(wv[1][e]), 0),
+                                       __dp4a(qx, (int)__float_as_uint(wv[2][e]), 0), __dp4a(qx, (int)__float_as_uint(wv[3][e]), 0), f0[4 * q + e], f1[4 * q + e]);
+                    }
+                } else {
+                    if (!wait_bar_warp<true>(base + sm.acc_full, use & 1, abort_flag, p.status)) return;
+                    ++use;
+                    ptx::tc_fence_after();
+#pragma unroll
+                    for (int hf = 0; hf < 2; ++hf) {
+                        uint32_t D[4][8];
+#pragma unroll
+                        for (int d = 0; d < 4; ++d) ptx::tmem_ld8(acc + d * kDBlock + hf * 8, D[d]);
+                        ptx::tmem_wait_ld();
+                        if (hf == 1) { // the sums are free for the next block
+                            ptx::tc_fence_before();
+                            ptx::mbar_arrive(base + sm.acc_empty);
+                        }
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) digit_sums((int)D[0][i], (int)D[1][i], (int)D[2][i], (int)D[3][i], f0[hf * 8 + i], f1[hf * 8 + i]);
+                    }
+                }
+                float y[16];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) activations4(f0 + 4 * q, f1 + 4 * q, at + q * 16, y + 4 * q);
+                put_block(b, y);
+            }
+            chunk_stages();
+            if (!digit_finish<W, PER_TOKEN>(c, 1.0f, static_inv, s_x)) return;
+        }
+        // last layer: the sums of digit d of output m in column 4 d + m
+        if (!wait_bar_warp<true>(base + sm.acc_last, last_parity, abort_flag, p.status)) return;
+        last_parity ^= 1;
+        ptx::tc_fence_after();
+        if (sub == 0) {
+            uint32_t u[16];
+            ptx::tmem_ld16(tmem + ((uint32_t)(quad * 32) << 16), u);
+            ptx::tmem_wait_ld();
+            if (valid) {
+                const double st = PER_TOKEN ? (double)s_x : (double)__ldg(p.layer[p.L - 1].act + 1);
+#pragma unroll
+                for (int m = 0; m < 4; ++m)
+                    if (m < p.d_L) p.out[tok * p.d_L + m] = digit_last((int)u[m], (int)u[4 + m], (int)u[8 + m], (int)u[12 + m], __ldg(p.last_scale + m), st, __ldg(p.last_bias + m));
+            }
+        }
+        ptx::tc_fence_before();
+    }
+}
+
+template <int W>
+__device__ void digit_mma(const DigitParams &p, const DigitMap &sm, uint32_t base, uint32_t tmem, volatile int *abort_flag)
+{
+    constexpr int NB = W / kDBlock, PIECE = kDBlock * W;
+    const uint32_t idesc = ptx::idesc_i8(kTile, kDBlock), idesc_last = ptx::idesc_i8(kTile, 16);
+    constexpr uint32_t kDescHi = (128u >> 4) | (1u << 14);
+    const uint32_t a0 = ((base + sm.a) >> 4) | ((kTile * 16u >> 4) << 16), b0 = ((base + sm.ring) >> 4) | ((kDBlock * 16u >> 4) << 16);
+    const uint32_t l0 = ((base + sm.last_w) >> 4) | ((16u * 16u >> 4) << 16);
+    uint32_t use = 0, codes = 0, wpar = 0;
+    int stage = 0;
+    bool ok = true;
+    for (long long tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
+        for (int l = 2; l < p.L && ok; ++l) {
+            ok = wait_bar<0, kHintNs>(base + sm.codes_full, codes & 1, abort_flag, p.status);
+            ++codes;
+            for (int b = 0; b < NB && ok; ++b, ++use) {
+                if (!wait_bar<0, kHintNs>(base + sm.acc_empty, (use & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
+                ptx::tc_fence_after();
+                for (int d = 0; d < 4; ++d) {
+                    if (!wait_bar<0, kHintNs>(base + sm.w_full + 8 * stage, wpar, abort_flag, p.status)) { ok = false; break; }
+                    const uint32_t bk = b0 + (uint32_t)stage * (PIECE >> 4);
+#pragma unroll
+                    for (int ks = 0; ks < W / 32; ++ks)
+                        ptx::mma_i8_words(tmem + (uint32_t)d * kDBlock, a0 + (ks * 2 * kTile * 16 >> 4), bk + (ks * 2 * kDBlock * 16 >> 4), kDescHi, idesc, ks > 0 ? 1u : 0u);
+                    ptx::mma_commit(base + sm.w_empty + 8 * stage);
+                    if (++stage == p.n_stages) { stage = 0; wpar ^= 1; }
+                }
+                if (ok) ptx::mma_commit(base + sm.acc_full);
+            }
+        }
+        if (!ok) break;
+        if (!wait_bar<0, kHintNs>(base + sm.last_full, 0, abort_flag, p.status) ||
+            !wait_bar<0, kHintNs>(base + sm.codes_full, codes & 1, abort_flag, p.status)) { ok = false; break; }
+        ++codes;
+        ptx::tc_fence_after();
+#pragma unroll
+        for (int ks = 0; ks < W / 32; ++ks)
+            ptx::mma_i8_words(tmem, a0 + (ks * 2 * kTile * 16 >> 4), l0 + (ks * 2 * 16 * 16 >> 4), kDescHi, idesc_last, ks > 0 ? 1u : 0u);
+        ptx::mma_commit(base + sm.acc_last);
+    }
+    if (!ok) { // give the MMAs already issued a bounded time to finish before tensor memory is released
+        ptx::mma_commit(base + sm.drain);
+        const unsigned long long t0 = ptx::globaltimer();
+        while (!ptx::mbar_try_wait(base + sm.drain, 0) && ptx::globaltimer() - t0 < wait_limit_of(abort_flag)) {}
+    }
+}
+
+template <int W>
+__device__ void digit_load(const DigitParams &p, const DigitMap &sm, uint32_t base, volatile int *abort_flag)
+{
+    constexpr int PIECE = kDBlock * W, PIECES = W / kDBlock * 4;
+    ptx::mbar_expect_tx(base + sm.last_full, 16 * W);
+    ptx::bulk_g2s(base + sm.last_w, p.layer[p.L - 1].img, 16 * W, base + sm.last_full);
+    int stage = 0;
+    uint32_t par = 1, issued = 0;
+    bool ok = true;
+    for (long long tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
+        for (int l = 2; l < p.L && ok; ++l) {
+            for (int i = 0; i < PIECES; ++i) {
+                if (!wait_bar<0, kHintNs>(base + sm.w_empty + 8 * stage, par, abort_flag, p.status)) { ok = false; break; }
+                ptx::mbar_expect_tx(base + sm.w_full + 8 * stage, PIECE);
+                ptx::bulk_g2s(base + sm.ring + (uint32_t)stage * PIECE, p.layer[l - 1].img + (size_t)i * PIECE, PIECE, base + sm.w_full + 8 * stage);
+                ++issued;
+                if (++stage == p.n_stages) { stage = 0; par ^= 1; }
+            }
+        }
+    }
+    if (!ok || *abort_flag) { // let copies in flight land before the CTA may exit
+        const unsigned long long t0 = ptx::globaltimer();
+        const uint32_t n = (uint32_t)p.n_stages;
+        for (uint32_t i = issued > n ? issued - n : 0; i < issued; ++i)
+            while (!ptx::mbar_try_wait(base + sm.w_full + 8 * (i % n), (i / n) & 1) && ptx::globaltimer() - t0 < wait_limit_of(abort_flag)) {}
+        while (!ptx::mbar_try_wait(base + sm.last_full, 0) && ptx::globaltimer() - t0 < wait_limit_of(abort_flag)) {}
+    }
+}
+
+template <int W, bool PER_TOKEN, bool GABOR>
+__global__ void __launch_bounds__(kDThreads, 1) digit_kernel(const __grid_constant__ DigitParams p)
+{
+    constexpr int NB = W / kDBlock;
+    extern __shared__ uint8_t smem_raw[];
+    const uint32_t raw = ptx::smem_u32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    uint8_t *gen = smem_raw + (base - raw);
+    const DigitMap sm = digit_map(W, p.n_stages, p.L);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(gen + sm.abort_flag);
+    if (threadIdx.x == 0) {
+        *abort_flag = 0;
+        *reinterpret_cast<volatile unsigned long long *>(abort_flag + 2) = p.wait_limit_ns;
+        for (int i = 0; i < kDMaxStages; ++i) {
+            ptx::mbar_init(base + sm.w_full + 8 * i, 1);
+            ptx::mbar_init(base + sm.w_empty + 8 * i, 1);
+        }
+        ptx::mbar_init(base + sm.codes_full, kEpiWarps * 32);
+        ptx::mbar_init(base + sm.acc_full, 1);
+        ptx::mbar_init(base + sm.acc_empty, kEpiWarps * 32);
+        ptx::mbar_init(base + sm.acc_last, 1);
+        ptx::mbar_init(base + sm.last_full, 1);
+        for (int i = 0; i < 4; ++i) ptx::mbar_init(base + sm.quad_sync + 8 * i, 128);
+        ptx::mbar_init(base + sm.drain, 1);
+        ptx::fence_mbar_init();
+    }
+    if (warp == kMmaWarp) {
+        ptx::tmem_alloc(base + sm.holder, 512);
+        ptx::tmem_relinquish();
+    }
+    float *consts = reinterpret_cast<float *>(gen + sm.consts);
+    for (int i = threadIdx.x; i < W; i += kDThreads) { // i: position in block order, m: its feature
+        const int b = i / kDBlock, m = digit_feature(W, b, (i % kDBlock) >> 4, i & 15);
+        for (int l = 0; l < p.L - 1; ++l) {
+            float *d = consts + l * 5 * W + i;
+            d[0] = __ldg(p.layer[l].c + m);
+            d[W] = __ldg(p.layer[l].c_lo + m);
+            d[2 * W] = __ldg(p.layer[l].cb + m);
+            d[3 * W] = __ldg(p.layer[l].cb_lo + m);
+            d[4 * W] = __ldg(p.layer[l].cn + m);
+        }
+        for (int d = 0; d < 4; ++d) reinterpret_cast<uint32_t *>(consts)[(5 * (p.L - 1) + d) * W + i] = __ldg(p.l1w + d * W + m);
+    }
+    static_assert(NB * kDBlock == W, "whole blocks");
+    ptx::tc_fence_before();
+    __syncthreads();
+    ptx::tc_fence_after();
+    const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(gen + sm.holder);
+    if (warp < kEpiWarps) digit_epilogue<W, PER_TOKEN, GABOR>(p, sm, base, warp, lane, tmem, abort_flag);
+    else if (lane == 0) {
+        if (warp == kMmaWarp) digit_mma<W>(p, sm, base, tmem, abort_flag);
+        else digit_load<W>(p, sm, base, abort_flag);
+    }
+    ptx::tc_fence_before();
+    __syncthreads();
+    if (warp == kMmaWarp) {
+        __syncwarp();
+        ptx::tmem_dealloc(tmem, 512);
+    }
+}
+
+// ------------------------------------------------------------------- weight side, once per network
+
+// G = H_M diag(s_w) q_W, one block per column k of a layer, in fp64 (a 24-bit scale times a 7-bit code,
+// sums of up to 256 of them: exact but for rows whose scales lie more than 2^14 apart).
+__global__ void prep_digit_cols_kernel(const __grid_constant__ DigitPrep a)
+{
+    extern __shared__ double gcol[];
+    const int l = (int)blockIdx.x < 4 ? 0 : 1 + ((int)blockIdx.x - 4) / a.w; // 4 columns, then w per layer
+    const int k = l == 0 ? (int)blockIdx.x : ((int)blockIdx.x - 4) % a.w;
+    const LayerDev &dev = a.dev[l];
+    const int K = dev.K, M = dev.M;
+    for (int m = threadIdx.x; m < M; m += blockDim.x) gcol[m] = (double)dev.s_w[m] * (double)dev.qw[(size_t)m * K + k];
+    for (int h = 1; h < M; h <<= 1) {
+        __syncthreads();
+        for (int p = threadIdx.x; p < M / 2; p += blockDim.x) {
+            const int i = ((p & ~(h - 1)) << 1) | (p & (h - 1));
+            const double x = gcol[i], y = gcol[i + h];
+            gcol[i] = x + y;
+            gcol[i + h] = x - y;
+        }
+    }
+    __syncthreads();
+    for (int m = threadIdx.x; m < M; m += blockDim.x) a.g[l][(size_t)m * K + k] = gcol[m];
+}
+
+// One block per row: 32-bit fixed point relative to the largest entry, four signed base-256 digits in both
+// layouts, and the row's scale (per unit of the integer; hidden layers in turns of the phase, times
+// 2^24 because the first digit's sum is the unit there).
+__global__ void __launch_bounds__(128) prep_digit_rows_kernel(const __grid_constant__ DigitPrep a)
+{
+    __shared__ double red[4];
+    const int l = min((int)blockIdx.x / a.w, a.L - 1), m = (int)blockIdx.x - l * a.w, tid = threadIdx.x;
+    const LayerDev &dev = a.dev[l];
+    const int K = dev.K, M = dev.M;
+    const double *row = a.g[l] + (size_t)m * K;
+    double g = 0.0;
+    for (int k = tid; k < K; k += 128) g = fmax(g, fabs(row[k]));
+    for (int o = 16; o; o >>= 1) g = fmax(g, __shfl_xor_sync(0xffffffffu, g, o));
+    if ((tid & 31) == 0) red[tid >> 5] = g;
+    __syncthreads();
+    g = fmax(fmax(red[0], red[1]), fmax(red[2], red[3]));
+    const double f = g > 0.0 ? 2139062143.0 / g : 0.0; // 127 in every digit
+    size_t at = 0; // place of (m, k = 0, digit 0) in the tensor-core image, and the distance of digits
+    size_t digit_bytes = 0;
+    if (l > 0 && l < a.L - 1) {
+        const int CH = a.w / 4, sub = m / CH, q = m % CH, pr = q % (CH / 2), b = pr / 8, i = 2 * (pr % 8) + q / (CH / 2);
+        digit_bytes = (size_t)kDBlock * K;
+        at = (size_t)b * 4 * digit_bytes + (sub * 16 + i) * 16;
+    }
+    const int rows = l == a.L - 1 ? 16 : kDBlock;
+    for (int k = tid; k < K; k += 128) {
+        const uint32_t v = (uint32_t)((long long)rint(row[k] * f) + 0x80808080ll) ^ 0x80808080u;
+#pragma unroll
+        for (int d = 0; d < 4; ++d) {
+            const uint8_t byte = (uint8_t)(v >> (24 - 8 * d));
+            reinterpret_cast<uint8_t *>(dev.gd_k4m)[(size_t)d * M * K + ((size_t)(k >> 2) * M + m) * 4 + (k & 3)] = byte;
+            if (l > 0) {
+                const size_t o = l == a.L - 1 ? (size_t)(4 * d + m) * 16 : at + d * digit_bytes;
+                dev.gd_img[o + (size_t)(k >> 4) * rows * 16 + (k & 15)] = byte;
+            }
+        }
+    }
+    if (tid == 0) {
+        const bool sine = l < a.L - 1;
+        dev.g_scale[m] = f > 0.0 ? (sine ? a.omega0 * 0.15915494309189533576888 * 16777216.0 : 1.0) / f : 0.0;
+        if (a.finalize) finalize_row(dev, m, 1.0f, 0.f, sine, a.omega0);
+    }
+}
+
+cudaError_t launch_prep_digits(const DigitPrep &a, cudaStream_t st, int64_t *launches)
+{
+    prep_digit_cols_kernel<<<4 + (a.L - 1) * a.w, 128, a.w * sizeof(double), st>>>(a);
+    prep_digit_rows_kernel<<<(a.L - 1) * a.w + 4, 128, 0, st>>>(a);
+    *launches += 2;
+    return cudaGetLastError();
+}
+
+// ------------------------------------------------------------------- host side
+
+struct DigitState {
+    DigitParams p;
+    size_t smem_bytes;
+    int sm_count;
+};
+
+typedef void (*digit_fn)(const DigitParams);
+template <int W> static digit_fn pick_digit(bool per_token, bool gabor)
+{
+    if (gabor) return per_token ? digit_kernel<W, true, true> : digit_kernel<W, false, true>;
+    return per_token ? digit_kernel<W, true, false> : digit_kernel<W, false, false>;
+}
+static digit_fn digit_kernel_of(const dhq_handle_s *h)
+{
+    const bool per_token = h->cfg.a_gran == DHQ_GRAN_CHANNEL_OR_TOKEN, gabor = h->gabor_s0 > 0.0;
+    return h->w == 256 ? pick_digit<256>(per_token, gabor) : h->w == 128 ? pick_digit<128>(per_token, gabor) : nullptr;
+}
+
+dhq_status_t digit_create(dhq_handle_s *h)
+{
+    DigitState *ds = new (std::nothrow) DigitState();
+    if (!ds) return DHQ_ERR_ALLOC;
+    memset(ds, 0, sizeof(*ds));
+    h->digit_state = ds;
+    int max_optin = 0;
+    if (cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device) != cudaSuccess ||
+        cudaDeviceGetAttribute(&ds->sm_count, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess)
+        return DHQ_ERR_CUDA;
+    DigitParams &p = ds->p;
+    p.L = h->L; p.d_L = h->d_L;
+    p.qmaxf = (float)((1 << (h->cfg.a_bits - 1)) - 1);
+    p.gabor_c = digit_gabor_c(h->gabor_s0, (double)h->cfg.omega0);
+    p.status = h->d_status;
+    for (int l = 0; l < h->L; ++l) {
+        const LayerDev &d = h->layer[l];
+        p.layer[l].img = d.gd_img;
+        p.layer[l].c = d.cA; p.layer[l].c_lo = d.cA_lo; p.layer[l].cb = d.cB; p.layer[l].cb_lo = d.cB_lo; p.layer[l].cn = d.cN;
+        p.layer[l].act = d.act;
+    }
+    p.l1w = reinterpret_cast<const uint32_t *>(h->layer[0].gd_k4m);
+    p.last_scale = h->layer[h->L - 1].g_scale;
+    p.last_bias = h->layer[h->L - 1].bias;
+    const size_t piece = (size_t)kDBlock * h->w, fixed = digit_map(h->w, 0, h->L).total + 1024;
+    if (fixed + piece > (size_t)max_optin) return DHQ_ERR_UNSUPPORTED;
+    int stages = (int)(((size_t)max_optin - fixed) / piece);
+    p.n_stages = stages < kDMaxStages ? stages : kDMaxStages;
+    ds->smem_bytes = digit_map(h->w, p.n_stages, h->L).total + 1024;
+    if (ds->smem_bytes < (size_t)kMinSmem) ds->smem_bytes = kMinSmem;
+    return allow_smem((const void *)digit_kernel_of(h), h->device, max_optin) ? DHQ_OK : DHQ_ERR_CUDA;
+}
+
+void digit_destroy(dhq_handle_s *h)
+{
+    delete static_cast<DigitState *>(h->digit_state);
+    h->digit_state = nullptr;
+}
+
+dhq_status_t digit_forward(dhq_handle_s *h, const float *coords, int64_t n, float *out, cudaStream_t st)
+{
+    DigitState *ds = static_cast<DigitState *>(h->digit_state);
+    DigitParams p = ds->p;
+    p.coords = coords; p.out = out; p.n = n;
+    p.n_tiles = (n + kTile - 1) / kTile;
+    p.wait_limit_ns = h->wait_limit_ns;
+    const int grid = (int)(p.n_tiles < ds->sm_count ? p.n_tiles : ds->sm_count);
+    digit_kernel_of(h)<<<grid, kDThreads, ds->smem_bytes, st>>>(p);
+    h->launches++;
+    return cudaGetLastError() == cudaSuccess ? DHQ_OK : DHQ_ERR_CUDA;
+}
+
+} // namespace dhq

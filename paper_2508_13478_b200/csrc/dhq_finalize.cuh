@@ -9,6 +9,16 @@ namespace dhq {
 // last layer.
 __device__ __forceinline__ double finalize_row(const LayerDev &dev, int m, float s_x, float s_w, int sine, double omega0)
 {
+    if (dev.has_digits) { // phases in turns, the bias modulo one turn
+        const double A = dev.g_scale[m] * (double)s_x, b = omega0 * (double)dev.bias[m] * 0.15915494309189533576888, n = rint(b);
+        const float hi = (float)A;
+        dev.cA[m] = hi;
+        dev.cA_lo[m] = (float)(A - (double)hi);
+        dev.cB[m] = (float)(b - n);
+        dev.cB_lo[m] = (float)(b - n - (double)(float)(b - n));
+        dev.cN[m] = (float)n;
+        return A;
+    }
     const double f = sine ? omega0 : 1.0;
     const double A = f * (double)s_w * (double)s_x;
     const float hi = (float)A;

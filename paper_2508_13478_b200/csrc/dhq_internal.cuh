@@ -32,6 +32,11 @@ struct LayerDev {
     float *act = nullptr;      // [4]: frozen absmax (max taken on the bit pattern), s_x, inv, unused
     int has_uv = 0;            // two-sided transform, layer 1: l1U, l1V below
     int32_t *l1U = nullptr, *l1V = nullptr; // [M] H_M applied to u_m = q[m][0]+q[m][2] and v_m = q[m][1]+q[m][3]
+    int has_digits = 0;        // two-sided transform with a weight scale per output channel, see dhq_digits.cu
+    uint32_t *gd_k4m = nullptr; // [4 digits][K/4][M] words of four consecutive k
+    uint8_t *gd_img = nullptr; // the digits in tensor-core order (layers 2 .. L)
+    double *g_scale = nullptr; // [M] value of a unit of the fixed-point row
+    float *cN = nullptr, *cB_lo = nullptr; // [M] bias in turns: integer part, and what cB (the rest) loses
     int has_f32 = 0;           // floating-point datapaths: 1 first and last layer (w_f32, f_scale), 2 hidden layer (wdig)
     float *w_f32 = nullptr;    // last layer: [K/4][M] float4 fp32 weights (W8A32: the integers q_w H_K), zero padded;
                                // first layer: [M] float4 (two weights and the bias in turns of the phase)
@@ -70,6 +75,8 @@ struct dhq_handle_s {
     unsigned long long wait_limit_ns = 2000000000ull; // bound of every wait inside the fused kernel (dhq_set_wait_limit)
     bool stall_next_forward = false; // test hook: see dhq_debug_stall_next_forward
     double gabor_s0 = 0.0;          // > 0: wavelet activation (layer-by-layer path)
+    void *digit_state = nullptr;    // state of the two-sided kernel for per-channel weight scales
+    double *g_scratch = nullptr;    // its matrices in fp64 (used by the preparation only)
     void *float_state = nullptr;    // state of the floating-point datapaths
     int float_digits = 0;           // base-256 digits per weight of their hidden layers
     int float_mode = 0;             // 0: fully quantized (DHQ); 1: W8A32 (activations fp32); 2: W32A32 (plain fp32 network)
@@ -105,6 +112,11 @@ struct LayerArgs {
     const float *s_w, *bias;
     double omega0;
     int sine;
+    // the same with the digits of dhq_digits.cu (gd_k4m not NULL): bit for bit what that kernel computes
+    const uint32_t *gd_k4m;
+    const double *g_scale;
+    const float *cN, *cB_lo;
+    float digit_gc;
     double gabor_s0;       // > 0: hidden layers apply sin(omega0 z) exp(-(s0 z)^2) instead of the sine
     float *Y;              // [n][M] or NULL
     float *out;            // [n][d_L] or NULL (last layer)
@@ -152,6 +164,17 @@ struct PrepNet {
     LayerDev dev[kMaxLayers];
 };
 cudaError_t launch_prepare(const PrepNet &a, cudaStream_t st, int64_t *launches);
+// Two-sided transform, weight scale per output channel (dhq_digits.cu), widths 128 and 256.
+struct DigitPrep {
+    int L, w, finalize;
+    double omega0;
+    double *g[kMaxLayers]; // [M][K] per layer
+    LayerDev dev[kMaxLayers];
+};
+cudaError_t launch_prep_digits(const DigitPrep &a, cudaStream_t st, int64_t *launches);
+dhq_status_t digit_create(dhq_handle_s *h);
+void digit_destroy(dhq_handle_s *h);
+dhq_status_t digit_forward(dhq_handle_s *h, const float *coords, int64_t n, float *out, cudaStream_t st);
 // Epilogue constants from s_w and (per-tensor) the frozen activation scale.
 cudaError_t launch_finalize(const LayerDev &dev, int a_bits, int per_token, int sine, double omega0,
                             cudaStream_t st, int64_t *launches);

@@ -92,6 +92,36 @@ __global__ void __launch_bounds__(LW_THREADS) layer_kernel(LayerArgs a)
             for (int t = 0; t < TB; ++t)
                 acc[t] = __dp4a(((const int *)cs)[t * K4 + k4], w, acc[t]);
         }
+        if (a.gd_k4m) {
+            // two-sided transform by the digits of H_M diag(s_w) q_W (acc above is only for the dump)
+            const float cA = a.cA[m], cAl = a.cA_lo[m], cB = a.cB[m], cBl = a.cB_lo[m], cN = a.cN[m];
+            const int64_t MK4 = (int64_t)M * K4;
+            for (int t = 0; t < TB; ++t) {
+                const int64_t tok = base + t;
+                if (tok >= a.n) break;
+                int D[4] = {0, 0, 0, 0};
+                for (int k4 = 0; k4 < K4; ++k4) {
+                    const int x4 = ((const int *)cs)[t * K4 + k4];
+#pragma unroll
+                    for (int d = 0; d < 4; ++d) D[d] = __dp4a(x4, (int)a.gd_k4m[d * MK4 + (int64_t)k4 * M + m], D[d]);
+                }
+                float y;
+                if (a.sine) {
+                    float c_hi = cA, c_lo = cAl;
+                    if (a.per_token) token_const(cA, cAl, s_tok[t], c_hi, c_lo);
+                    float f0, f1;
+                    digit_sums(D[0], D[1], D[2], D[3], f0, f1);
+                    y = sin_approx(digit_phase(f0, f1, c_hi, c_lo, cB, cBl));
+                    if (a.gabor_s0 > 0.0) y = __fmul_rn(y, digit_envelope(f0, f1, c_hi, cB, cN, a.digit_gc));
+                } else {
+                    y = digit_last(D[0], D[1], D[2], D[3], a.g_scale[m], (double)s_tok[t], a.bias[m]);
+                }
+                if (a.dacc) a.dacc[tok * M + m] = acc[t];
+                if (a.Y) a.Y[tok * M + m] = y;
+                if (a.out && m < a.d_L) a.out[tok * a.d_L + m] = y;
+            }
+            continue;
+        }
         if (a.rotate == 2) {
             // two-sided transform: keep d = s_w s_x acc of every token; the output follows below
             const double sw = (double)a.s_w[m];
@@ -124,7 +154,7 @@ __global__ void __launch_bounds__(LW_THREADS) layer_kernel(LayerArgs a)
             if (a.out && m < a.d_L) a.out[tok * a.d_L + m] = y;
         }
     }
-    if (a.rotate != 2) return;
+    if (a.rotate != 2 || a.gd_k4m) return;
     // z = H_M d + b (H_M H_M = M I, and the 1/M is in the weights): fp64 butterfly over the M outputs.
     // The sum of up to 512 terms reaches phases of tens of radians that must stay within 1e-5 of
     // the fp64 definition; an fp32 butterfly does not (about 1e-7 rms per radian of phase).
@@ -165,7 +195,7 @@ cudaError_t launch_layer(const LayerArgs &a, cudaStream_t st)
     if (a.n <= 0) return cudaSuccess;
     int64_t blocks = (a.n + TB - 1) / TB;
     size_t dyn = 0;
-    if (a.rotate == 2 && !a.calib_only) {
+    if (a.rotate == 2 && !a.calib_only && !a.gd_k4m) {
         dyn = (size_t)TB * a.M * sizeof(double); // up to 64 KB beside the 41 KB of static shared memory
         cudaError_t e = cudaFuncSetAttribute(layer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TB * 512 * (int)sizeof(double));
         if (e != cudaSuccess) return e;

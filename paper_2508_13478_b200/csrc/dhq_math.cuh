@@ -128,6 +128,47 @@ __device__ __forceinline__ float sine_fixed(int qs, int qd, uint32_t P, uint32_t
     return sin_approx(__fmul_rn((float)(int)ph, 1.4629180792671596e-09f)); // 2 pi / 2^32
 }
 
+// Two-sided transform with a weight scale per output channel: the matrix H_M diag(s_w) q_W is held as four
+// base-256 digits per entry and D0 .. D3 are the digits' products with the activation codes (exact;
+// |D| < 2^23 at widths up to 256).  The phase in turns is t = c (D0 + D1 / 2^8 + D2 / 2^16 + D3 / 2^24) + cb with
+// c = c_hi + c_lo and the bias modulo one turn cb + cb_lo.  The result is 2 pi (t - nearest integer) rounded to
+// fp32 as if t had been known in fp64: the product's rounding error, the parts of the sum that an
+// fp32 addition drops and the low part of 2 pi are all carried along (error 0.5 ulp + 2^-31 turns).  That care
+// is for the quantizer that follows, not for the 1e-5 of the output: activations that agree with the fp64
+// evaluation bit for bit are quantized to the same codes.
+__device__ __forceinline__ void digit_sums(int D0, int D1, int D2, int D3, float &f0, float &f1)
+{
+    f0 = (float)D0;
+    f1 = __fmul_rn((float)(D1 * 256 + (D2 + (D3 >> 8))), 0x1p-16f);
+}
+__device__ __forceinline__ float digit_phase(float f0, float f1, float c_hi, float c_lo, float cb, float cb_lo)
+{
+    const float two_pi_hi = 6.2831854820251465f, two_pi_lo = -1.7484555e-07f;
+    const float p = __fmul_rn(f0, c_hi), pe = __fmaf_rn(f0, c_hi, -p);
+    const float r = __fsub_rn(p, __fsub_rn(__fadd_rn(p, 12582912.0f), 12582912.0f)); // exact
+    const float s = __fadd_rn(r, cb), v = __fsub_rn(s, r);
+    const float se = __fadd_rn(__fsub_rn(r, __fsub_rn(s, v)), __fsub_rn(cb, v)); // r + cb = s + se
+    const float t = __fsub_rn(s, __fsub_rn(__fadd_rn(s, 12582912.0f), 12582912.0f)); // exact, |s| <= 1
+    const float lo = __fadd_rn(__fadd_rn(pe, se), __fmaf_rn(f0, c_lo, __fmaf_rn(f1, c_hi, cb_lo)));
+    const float q = __fmul_rn(t, two_pi_hi);
+    return __fadd_rn(q, __fmaf_rn(lo, two_pi_hi, __fmaf_rn(t, two_pi_lo, __fmaf_rn(t, two_pi_hi, -q))));
+}
+// The wavelet's envelope exp(-(s0 z)^2) from the same numbers: cn is the integer part that cb lacks, gc = 2 pi s0 / omega0.
+__device__ __forceinline__ float digit_envelope(float f0, float f1, float c_hi, float cb, float cn, float gc)
+{
+    const float g = __fmul_rn(__fmaf_rn(__fadd_rn(f0, f1), c_hi, __fadd_rn(cb, cn)), gc);
+    float e;
+    asm("ex2.approx.f32 %0, %1;" : "=f"(e) : "f"(__fmul_rn(__fmul_rn(g, g), -1.4426950408889634f)));
+    return e;
+}
+inline float digit_gabor_c(double s0, double omega0) { return omega0 != 0.0 ? (float)(s0 / omega0 * 6.283185307179586476925287) : 0.f; }
+// Last layer: z = scale s_x (the digits' number) + b, in fp64, rounded once.
+__device__ __forceinline__ float digit_last(int D0, int D1, int D2, int D3, double scale, double s_x, float b)
+{
+    const long long t = ((((long long)D0 * 256 + D1) * 256 + D2) * 256) + D3;
+    return (float)(scale * s_x * (double)t + (double)b);
+}
+
 // Per-token activation scales: the per-channel constant cA (+ remainder cA_lo) times the
 // token's s_x.  c_lo collects the rounding error of that product and the remainder term.
 __device__ __forceinline__ void token_const(float cA, float cA_lo, float s_x, float &c_hi, float &c_lo)

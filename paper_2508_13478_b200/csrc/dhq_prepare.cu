@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(128) prep_quant_kernel(const __grid_constant__
     const float bound = (float)a.omega0 * (dev.row_l1[m] + slack) * 1.0001f;
     if (bound > 0.f) atomicMax(reinterpret_cast<unsigned int *>(&a.sums->phase_bound[l]), __float_as_uint(bound));
     atomicAdd(&a.sums->code_l1[l], (unsigned long long)qsum);
-    if (a.finalize) finalize_row(dev, m, 1.0f, s, l < a.L - 1, a.omega0);
+    if (a.finalize && !dev.has_digits) finalize_row(dev, m, 1.0f, s, l < a.L - 1, a.omega0);
 }
 
 // Two-sided transform, layer 1 (K = 4): the rotated padded coordinate has the codes [qs, qd, qs, qd],

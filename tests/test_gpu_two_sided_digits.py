@@ -1,0 +1,45 @@
+"""The two-sided transform with a weight scale per output channel, widths 128 and 256: the fixed-point
+kernel of dhq_forward at the ends of its tiles and grid, both activation granularities, no and many
+tensor-core layers, rows of very different scale (2^-12 to 1 of each other), sine and wavelet.  The
+layer-by-layer dumps must satisfy the definition (codes, scales and accumulators exactly, outputs within the
+1e-5 of every fused path; measured 7e-7) and dhq_forward must return their bits, since both evaluate
+the same exact sums."""
+import numpy as np
+import pytest
+import torch
+
+import dhq_inputs
+from tests.gpu_util import check_layers_against_oracle, check_weights, prepare_pair, run_debug, to_dev
+
+pytestmark = pytest.mark.gpu
+
+dhq = pytest.importorskip("paper_2508_13478_b200")
+
+
+@pytest.mark.parametrize("width,n_linear,d_out,a_gran,n,s0", [
+    (128, 2, 1, 1, 1, 0.0), (128, 5, 3, 0, 129, 0.0), (128, 4, 2, 1, 148 * 128 + 1, 0.0), (256, 2, 4, 0, 127, 0.0),
+    (256, 3, 3, 1, 128, 9.0), (256, 16, 3, 1, 130, 0.0), (256, 4, 3, 0, 148 * 128 + 129, 9.0)])
+def test_two_sided_per_channel(width, n_linear, d_out, a_gran, n, s0):
+    dims = (2,) + (width,) * (n_linear - 1) + (d_out,)
+    weights, biases = dhq_inputs.siren_init(dims, 30.0, 40 + width + n_linear)
+    weights[-1] = weights[-1] * np.float32(2.0) ** -np.arange(d_out, dtype=np.float32)[:, None] ** 2
+    if n_linear > 2:
+        weights[1] = weights[1] * (np.float32(2.0) ** -(np.arange(width) % 13).astype(np.float32))[:, None]
+    coords = dhq_inputs.grid_coords(n // 150 + 1, 150)[:n]
+    h, net = prepare_pair(dims, weights, biases, 30.0, 8, 8, 1, a_gran, rotate="both", gabor_s0=s0)
+    try:
+        check_weights(h, net)
+        cd = to_dev(coords)
+        if a_gran == 0:
+            dhq.dhq_calibrate(h, cd)
+        dumped, bufs = run_debug(h, net, cd)
+        worst = check_layers_against_oracle(h, net, coords, dumped, bufs)
+        out = torch.full((n, d_out), float("nan"), device="cuda")
+        before = dhq.dhq_launch_count(h)
+        dhq.dhq_forward(h, cd, out)
+        torch.cuda.synchronize()
+        assert dhq.dhq_launch_count(h) - before == 1 and dhq.dhq_last_status(h) == 0
+        assert torch.equal(out.view(torch.int32), dumped.view(torch.int32))
+        print(f"two-sided per channel, width {width}: outputs within {worst:.2e}")
+    finally:
+        dhq.dhq_destroy(h)
