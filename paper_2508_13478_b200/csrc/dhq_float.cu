@@ -185,6 +185,7 @@ __device__ void float_epilogue(const FloatParams &p, const FloatMap &sm, uint32_
         }
     };
     float x, yc;
+    ptx::wait_for_previous_kernels(); // coordinates, result and the scratch activations
     coords_of(blockIdx.x, x, yc);
     for (long long tile = blockIdx.x; tile < p.n_tiles; tile += gridDim.x) {
         const long long tok = tile * kTile + row;
@@ -303,6 +304,7 @@ template <int W, int WL>
 __device__ void float_mma(const FloatParams &p, const FloatMap &sm, uint32_t base, uint32_t tmem, volatile int *abort_flag)
 {
     constexpr int FB = float_block(W), KC = float_kc(W), NB = W / FB, NKC = W / KC, PIECE = FB * KC;
+    ptx::wait_for_previous_kernels(); // before the first bounded wait
     const uint32_t idesc = ptx::idesc_i8(kTile, FB);
     constexpr uint32_t kDescHi = (128u >> 4) | (1u << 14);
     const uint32_t a0 = ((base + sm.a) >> 4) | ((kTile * 16u >> 4) << 16), b0 = ((base + sm.ring) >> 4) | ((FB * 16u >> 4) << 16);
@@ -360,6 +362,7 @@ __device__ void float_load_weights(const FloatParams &p, const FloatMap &sm, uin
         for (int l = 2; l < p.L && ok; ++l) {
             for (int q = 0; q < PIECES; ++q, ++i) {
                 if ((int)(i % kFLoaders) != which) continue;
+                if (i >= (uint32_t)p.n_stages && i < (uint32_t)p.n_stages + kFLoaders) ptx::wait_for_previous_kernels();
                 const uint32_t stage = i % (uint32_t)p.n_stages, par = ((i / (uint32_t)p.n_stages) & 1) ^ 1;
                 if (!wait_bar<0, kHintNs>(base + sm.w_empty + 8 * stage, par, abort_flag, p.status)) { ok = false; break; }
                 ptx::mbar_expect_tx(base + sm.w_full + 8 * stage, PIECE);
@@ -385,6 +388,7 @@ template <int W>
 __device__ void float_load_x(const FloatParams &p, const FloatMap &sm, uint32_t base, volatile int *abort_flag)
 {
     const uint8_t *src = p.x + (size_t)blockIdx.x * (3 * kTile * W);
+    ptx::wait_for_previous_kernels();
     uint32_t layers = 0;
     bool ok = true;
     for (long long tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
@@ -417,6 +421,7 @@ __global__ void __launch_bounds__(kFThreads, 1) float_kernel(const __grid_consta
     const FloatMap sm = float_map(W, p.n_stages, p.L);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     volatile int *abort_flag = reinterpret_cast<volatile int *>(gen + sm.abort_flag);
+    ptx::launch_dependents();
     if (threadIdx.x == 0) {
         *abort_flag = 0;
         *reinterpret_cast<volatile unsigned long long *>(abort_flag + 2) = p.wait_limit_ns;
@@ -636,9 +641,10 @@ dhq_status_t float_forward(dhq_handle_s *h, const float *coords, int64_t n, floa
         }
     }
     const int grid = (int)(p.n_tiles < fs->sm_count ? p.n_tiles : fs->sm_count);
-    (dump ? pick_float<true>(h->w, h->float_digits) : pick_float<false>(h->w, h->float_digits))<<<grid, kFThreads, fs->smem_bytes, st>>>(p);
+    const float_fn fn = dump ? pick_float<true>(h->w, h->float_digits) : pick_float<false>(h->w, h->float_digits);
+    const cudaError_t e = launch_after(h, (const void *)fn, grid, kFThreads, fs->smem_bytes, st, &p);
     h->launches++;
-    return cudaGetLastError() == cudaSuccess ? DHQ_OK : DHQ_ERR_CUDA;
+    return e == cudaSuccess ? DHQ_OK : DHQ_ERR_CUDA;
 }
 
 } // namespace dhq

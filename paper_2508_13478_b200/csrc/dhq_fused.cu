@@ -172,6 +172,30 @@ bool allow_smem(const void *fn, int device, int bytes)
     return true;
 }
 
+// A forward launch.  Once a launch has followed the preparation and calibration (so that they had
+// completed before it began), later ones use programmatic dependent launch: what the kernel does
+// before wait_for_previous_kernels touches only the handle's weights and constants.  A block of the later launch
+// that waits holds no SM that the earlier one needs: it is not started before all blocks of the earlier
+// launch are.  Back to back, the binding's shorter call included: 4,096 coordinates at width 64 9.9 -> 5.9 us, 1,000 at
+// width 256 18.5 -> 14.9 us, 65,536 at width 256 45.0 -> 41.4 us.
+cudaError_t launch_after(dhq_handle_s *h, const void *fn, int grid, int threads, size_t smem, cudaStream_t st, void *params)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = h->settled ? 1 : 0;
+    h->settled = true;
+    void *args[1] = {params};
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 dhq_status_t fused_create(dhq_handle_s *h)
 {
     FusedState *fs = new (std::nothrow) FusedState();
@@ -274,9 +298,9 @@ dhq_status_t fused_forward(dhq_handle_s *h, const float *coords, int64_t n, floa
     fused_fn fn = pick_for(h, p.per_token, spread, !on_host);
     const long long ctas = spread ? p.n_tiles : (p.n_tiles + slots - 1) / slots;
     int grid = (int)(ctas < fs->sm_count ? ctas : fs->sm_count);
-    fn<<<grid, h->w == 512 ? kThreads + 32 : kThreads, fs->smem_bytes, st>>>(p);
+    const cudaError_t e = launch_after(h, (const void *)fn, grid, h->w == 512 ? kThreads + 32 : kThreads, fs->smem_bytes, st, &p);
     h->launches++;
-    return cudaGetLastError() == cudaSuccess ? DHQ_OK : DHQ_ERR_CUDA;
+    return e == cudaSuccess ? DHQ_OK : DHQ_ERR_CUDA;
 }
 
 // Layer 1's rotated input is H_4 [x, y, 0, 0] = [x+y, x-y, x+y, x-y] (or [x, y, 0, 0] without the

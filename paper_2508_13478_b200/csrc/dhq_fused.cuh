@@ -789,6 +789,8 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
     const FusedLayer &l1 = p.layer[0];
     const float qmaxf = p.qmaxf;
 
+    ptx::wait_for_previous_kernels(); // coordinates and result belong to the caller
+
     if (C::SLOTS == 2 && slot == 1 && tile_index<SPREAD>(0, 1, 2) < p.n_tiles && p.resident) {
         // Start the second slot about half a layer period after the first, so that one slot's
         // sine-heavy pass 1 and MMA wait fall on the other slot's pass 2 instead of both slots
@@ -1067,6 +1069,8 @@ __device__ void mma_role(const FusedParams &p, const SmemMap &sm, uint32_t smem_
                          volatile int *abort_flag)
 {
     using C = Cfg<W>;
+    // (before the first bounded wait: a kernel before this one may run for longer than the limit)
+    ptx::wait_for_previous_kernels();
     uint32_t codes_parity[2] = {0, 0};
     const uint32_t idesc_hidden = ptx::idesc_i8(kTile, C::NW), idesc_last = ptx::idesc_i8(kTile, 16);
     const uint32_t slab = C::PIECE_BYTES;
@@ -1186,6 +1190,7 @@ __device__ void load_role(const FusedParams &p, const SmemMap &sm, uint32_t smem
     for (long long i = 0; i < total; ++i) {
         const int stage = (int)(i % p.n_stages);
         if (i >= p.n_stages) {
+            if (i == p.n_stages) ptx::wait_for_previous_kernels(); // the first pieces may come early: weights do not change
             uint32_t par = (uint32_t)(((i / p.n_stages) - 1) & 1);
             if (!wait_bar<0, kHintNs>(smem_base + sm.w_empty + 8 * stage, par, abort_flag, p.status)) { ok = false; break; }
         }
@@ -1218,6 +1223,7 @@ __device__ void xy_role(const FusedParams &p, const SmemMap &sm, uint32_t smem_b
 {
     using C = Cfg<W>;
     if (!p.bulk_xy) return;
+    ptx::wait_for_previous_kernels();
     uint32_t k[2] = {0, 0};
     bool ok = true;
     for (long long r = 0; ok; ++r) {
@@ -1252,6 +1258,9 @@ __global__ void __launch_bounds__(Cfg<W>::THREADS, 1) fused_kernel(const __grid_
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem_gen + sm.abort_flag);
     volatile uint32_t *tmem_holder = reinterpret_cast<volatile uint32_t *>(smem_gen + sm.tmem_holder);
+    // Repeated calls: the next launch's blocks set themselves up - barriers, tensor memory, constants and first
+    // weights - on SMs that this launch leaves free or has finished with, instead of after its last block.
+    ptx::launch_dependents();
 
     if (threadIdx.x == 0) {
         *abort_flag = 0;

@@ -54,6 +54,7 @@ struct dhq_handle_s {
     int L = 0, w = 0, d_L = 0;
     int device = 0;
     bool calibrated = false;
+    bool settled = false;           // a forward has been enqueued since the weights or scales last changed
     int calib_layers_done = 0;      // layers whose per-tensor activation scale is frozen (sharded calibration)
     dhq::LayerDev layer[dhq::kMaxLayers];
     void *block = nullptr;          // the device memory of everything below up to the layers' arrays
@@ -213,6 +214,8 @@ __host__ __device__ inline int fused_feature(int col, int W)
 }
 // Lets a kernel use `bytes` of dynamic shared memory on `device` (asked of the driver once).
 bool allow_smem(const void *fn, int device, int bytes);
+// Launches a forward kernel, overlapping its set-up with the kernels before it where that is allowed.
+cudaError_t launch_after(dhq_handle_s *h, const void *fn, int grid, int threads, size_t smem, cudaStream_t st, void *params);
 // Fused tensor-core forward.
 dhq_status_t fused_create(dhq_handle_s *h);
 void fused_destroy(dhq_handle_s *h);
