@@ -138,6 +138,8 @@ static bool runs_mixed(const dhq_handle_s *h)
     return false;
 }
 
+static int threads_for(const dhq_handle_s *h) { return fused_threads(h->w, h->cfg.rotation == DHQ_ROT_BOTH, h->gabor_s0 > 0.0); }
+
 // The kernel a handle's forward launches (spread, ahead: see pick_kernel; the other families have one mapping).
 static fused_fn pick_for(const dhq_handle_s *h, bool per_token, bool spread, bool ahead)
 {
@@ -146,6 +148,13 @@ static fused_fn pick_for(const dhq_handle_s *h, bool per_token, bool spread, boo
     if (both) return pick_both_kernel(h->w, per_token);
     if (runs_mixed(h)) return pick_mixed_kernel(h->w, rot, ahead);
     return pick_kernel(h->w, per_token, rot, spread, ahead);
+}
+
+// The same for a launch of at most one tile per SM; NULL where the width has no such kernel.
+static fused_fn pick_narrow_for(const dhq_handle_s *h, bool per_token)
+{
+    const bool both = h->cfg.rotation == DHQ_ROT_BOTH, rot = h->cfg.rotation == DHQ_ROT_INPUT;
+    return h->w == 256 ? fused_pick_narrow_256(per_token, rot, both, h->gabor_s0 > 0.0, runs_mixed(h)) : nullptr;
 }
 
 // Its observing instantiation.
@@ -159,14 +168,17 @@ static fused_dump_fn pick_dump_for(const dhq_handle_s *h, bool per_token)
 }
 
 // Lets a kernel use all of an SM's shared memory; the driver is asked once per kernel and device
-// (8 of these calls per dhq_prepare took 15 us).
-bool allow_smem(const void *fn, int device, int bytes)
+// (8 of these calls per dhq_prepare took 15 us).  A kernel whose warpgroups split its registers must have been
+// launched with at least min_regs a thread, or the split would wait for registers that do not exist.
+bool allow_smem(const void *fn, int device, int bytes, int min_regs)
 {
     static std::mutex mutex;
     static std::set<std::pair<const void *, int>> done;
     if (!fn) return false;
     std::lock_guard<std::mutex> lock(mutex);
     if (done.count({fn, device})) return true;
+    cudaFuncAttributes at;
+    if (min_regs > 0 && (cudaFuncGetAttributes(&at, fn) != cudaSuccess || at.numRegs < min_regs)) return false;
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
     done.insert({fn, device});
     return true;
@@ -250,10 +262,13 @@ dhq_status_t fused_create(dhq_handle_s *h)
     size_t bytes = smem_map(h->w, p.n_stages, words).total + 1024;
     if (bytes < (size_t)kMinSmem) bytes = kMinSmem;
     fs->smem_bytes = bytes;
+    const int min_regs = splits_registers(h->w, both, gabor) ? kLaunchRegs : 0;
     for (int v = 0; v < 4; ++v) // every variant of this handle's kernel
-        if (!allow_smem((const void *)pick_for(h, p.per_token, (v & 1) != 0, (v & 2) != 0), dev, max_optin)) return DHQ_ERR_CUDA;
-    if (!p.per_token && !allow_smem((const void *)pick_calib_kernel(h->w, h->cfg.rotation == DHQ_ROT_INPUT, gabor, both), dev, max_optin)) return DHQ_ERR_CUDA;
-    if (!allow_smem((const void *)pick_dump_for(h, p.per_token), dev, max_optin)) return DHQ_ERR_CUDA;
+        if (!allow_smem((const void *)pick_for(h, p.per_token, (v & 1) != 0, (v & 2) != 0), dev, max_optin, min_regs)) return DHQ_ERR_CUDA;
+    const fused_fn narrow = pick_narrow_for(h, p.per_token);
+    if (narrow && !allow_smem((const void *)narrow, dev, max_optin, min_regs)) return DHQ_ERR_CUDA;
+    if (!p.per_token && !allow_smem((const void *)pick_calib_kernel(h->w, h->cfg.rotation == DHQ_ROT_INPUT, gabor, both), dev, max_optin, min_regs)) return DHQ_ERR_CUDA;
+    if (!allow_smem((const void *)pick_dump_for(h, p.per_token), dev, max_optin, min_regs)) return DHQ_ERR_CUDA;
     return DHQ_OK;
 }
 
@@ -295,10 +310,11 @@ dhq_status_t fused_forward(dhq_handle_s *h, const float *coords, int64_t n, floa
     const bool both = h->cfg.rotation == DHQ_ROT_BOTH;
     const bool gabor = h->gabor_s0 > 0.0;
     const bool spread = !both && !gabor && !runs_mixed(h) && slots > 1 && p.n_tiles < (long long)fs->sm_count * slots;
-    fused_fn fn = pick_for(h, p.per_token, spread, !on_host);
-    const long long ctas = spread ? p.n_tiles : (p.n_tiles + slots - 1) / slots;
+    const fused_fn narrow = p.n_tiles <= (long long)fs->sm_count ? pick_narrow_for(h, p.per_token) : nullptr;
+    const fused_fn fn = narrow ? narrow : pick_for(h, p.per_token, spread, !on_host);
+    const long long ctas = spread || narrow ? p.n_tiles : (p.n_tiles + slots - 1) / slots;
     int grid = (int)(ctas < fs->sm_count ? ctas : fs->sm_count);
-    const cudaError_t e = launch_after(h, (const void *)fn, grid, h->w == 512 ? kThreads + 32 : kThreads, fs->smem_bytes, st, &p);
+    const cudaError_t e = launch_after(h, (const void *)fn, grid, threads_for(h), fs->smem_bytes, st, &p);
     h->launches++;
     return e == cudaSuccess ? DHQ_OK : DHQ_ERR_CUDA;
 }
@@ -349,7 +365,7 @@ dhq_status_t fused_calibrate_layer(dhq_handle_s *h, int l, const float *coords, 
     fused_calib_fn fn = pick_calib_kernel(h->w, h->cfg.rotation == DHQ_ROT_INPUT, h->gabor_s0 > 0.0, h->cfg.rotation == DHQ_ROT_BOTH);
     const long long ctas = (p.n_tiles + slots - 1) / slots;
     int grid = (int)(ctas < fs->sm_count ? ctas : fs->sm_count);
-    fn<<<grid, h->w == 512 ? kThreads + 32 : kThreads, fs->smem_bytes, st>>>(p);
+    fn<<<grid, threads_for(h), fs->smem_bytes, st>>>(p);
     h->launches++;
     return cudaGetLastError() == cudaSuccess ? DHQ_OK : DHQ_ERR_CUDA;
 }
@@ -368,7 +384,7 @@ dhq_status_t fused_forward_dump(dhq_handle_s *h, const float *coords, int64_t n,
     fused_dump_fn fn = pick_dump_for(h, p.per_token);
     const long long ctas = (p.n_tiles + slots - 1) / slots;
     int grid = (int)(ctas < fs->sm_count ? ctas : fs->sm_count);
-    fn<<<grid, h->w == 512 ? kThreads + 32 : kThreads, fs->smem_bytes, st>>>(p);
+    fn<<<grid, threads_for(h), fs->smem_bytes, st>>>(p);
     h->launches++;
     return cudaGetLastError() == cudaSuccess ? DHQ_OK : DHQ_ERR_CUDA;
 }

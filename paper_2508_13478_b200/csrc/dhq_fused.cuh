@@ -1,7 +1,7 @@
 // Fused forward kernel: the whole quantized INR (Sections III-B and III-C of the paper) for
 // tiles of 128 coordinates without activations leaving the SM between layers.
 //
-// One persistent CTA per SM, 18 warps (19 at width 512):
+// One persistent CTA per SM, 18 to 20 warps (fused_threads):
 //   warps 0-15  epilogue warps.  Width <= 256: two "slots" of 8 warps, each slot has one tile of
 //               128 tokens in flight (its own A operand tile and 256 tensor-memory columns), so
 //               that one slot's CUDA-core work overlaps the other slot's MMA; the second slot
@@ -46,14 +46,25 @@ namespace dhq {
 constexpr int kTile = 128;
 constexpr int kEpiWarps = 16;
 constexpr int kMmaWarp = 16, kLoadWarp = 17, kXyWarp = 18;
-constexpr int kThreads = 18 * 32; // width 512 runs one more warp (Cfg::THREADS)
+// Register split: 20 warps, four warpgroups of epilogue warps and one with the MMA and copy warps.  The
+// launch gives every thread 96 registers; the fifth warpgroup then hands 40 of its own back and the other four
+// take 8 more each, 512 * 104 + 128 * 56 <= 640 * 96.  Measured per kernel: width 256, 1,048,576 coordinates, 4
+// layers 515 -> 499 us; width 128 96 -> 85; two-sided at width 512 768 -> 742; but the plain kernels of
+// width 512 lost 2 to 5 % and those of width 64 2 %, so they keep 18 warps (19 at width 512).
+__host__ __device__ constexpr bool splits_registers(int W, bool both, bool gabor) { return W == 128 || W == 256 || (W == 512 && (both || gabor)); }
+__host__ __device__ constexpr int fused_threads(int W, bool both, bool gabor) { return splits_registers(W, both, gabor) ? 20 * 32 : W == 512 ? 19 * 32 : 18 * 32; }
+constexpr int kEpiRegs = 104, kRoleRegs = 56, kLaunchRegs = 96;
+static_assert(kEpiWarps * kEpiRegs + (20 - kEpiWarps) * kRoleRegs <= 20 * kLaunchRegs, "more registers than the launch has");
 constexpr int kMaxStages = 32;
 constexpr uint32_t kCopyBytes = 8192; // bytes per bulk copy of a weight slab
 constexpr int kMinSmem = 120 * 1024; // more than half an SM's shared memory: one CTA per SM
 
-// Work split for a hidden width W.
-template <int W> struct Cfg {
-    static constexpr int SLOTS = (W == 512) ? 1 : 2;
+// Work split for a hidden width W.  NARROW: all 16 epilogue warps on one tile, for launches with at most one
+// tile per SM, where the time of a tile is what counts (a slot of 8 warps alone on an SM needs 24
+// cycles per 32 elements and scheduler, 16 warps 18).
+template <int W_, bool NARROW = false> struct Cfg {
+    static constexpr int W = W_;
+    static constexpr int SLOTS = (W == 512 || NARROW) ? 1 : 2;
     static constexpr int R = kEpiWarps / (4 * SLOTS);          // threads per row: 2 or 4
     static constexpr int CH = (W == 64) ? 32 : 64;             // columns per register chunk (= fused_chunk(W))
     static constexpr int NCH = W / CH;                         // chunks per row
@@ -62,15 +73,17 @@ template <int W> struct Cfg {
     static constexpr int GPT = CH / (G * R);                   // groups per thread
     static constexpr int KSLABS = (W == 512) ? 4 : 1;          // weight slabs per layer along K
     static constexpr int SLABK = W / KSLABS;                   // k per slab (= fused_slab_k)
-    static constexpr int NHALF = (W == 512) ? 2 : 1;           // MMAs along N (an MMA has N <= 256)
+    // A layer's products are finished in two halves of the output columns, each with its own barrier, so
+    // that the first half's epilogue starts while the second half's MMAs run (width 256, 1,048,576
+    // coordinates, per-tensor scales, 4 layers: 545 -> 515 us).
+    static constexpr int NHALF = (W >= 256) ? 2 : 1;
     static constexpr int NW = W / NHALF;                       // N of one MMA
-    static constexpr int PIECES = KSLABS * NHALF;              // weight pieces per layer (ring units)
-    static constexpr int PIECE_BYTES = SLABK * NW;             // 64 KB (width 256), 32 KB (width 512)
+    static constexpr int PIECES = (W == 512) ? KSLABS * NHALF : 1; // weight pieces per layer (ring units)
+    static constexpr int PIECE_BYTES = (W == 512) ? SLABK * NW : W * W; // 64 KB (width 256), 32 KB (width 512)
     static constexpr int SLOT_THREADS = R * kTile;
     // Width 512: the coordinates of a whole tile arrive by one bulk copy issued by a 19th warp (measured:
     // 2.6 % faster, 6.7 % from mapped host memory; narrower networks lost 4-7 % to the extra barrier).
     static constexpr bool BULK_XY = (W == 512);
-    static constexpr int THREADS = kThreads + (BULK_XY ? 32 : 0);
     static constexpr int TMEM_COLS_PER_SLOT = 512 / SLOTS;
 };
 
@@ -84,12 +97,12 @@ template <bool SPREAD> __device__ __forceinline__ long long tile_index(long long
                   : ((long long)blockIdx.x + r * gridDim.x) * slots + slot;
 }
 
-// Chunk cc of the thread with index `sub` among the R threads of a row.  Width 512 gives every
-// thread one chunk in each half of the columns (the halves' accumulators complete one after the
-// other); otherwise a thread's chunks are adjacent.
-template <int W> __device__ __forceinline__ int chunk_of(int sub, int cc)
+// Chunk cc of the thread with index `sub` among the R threads of a row.  Where the halves of the columns
+// complete one after the other, every thread has one chunk in each; otherwise a thread's chunks are
+// adjacent.
+template <class C> __device__ __forceinline__ int chunk_of(int sub, int cc)
 {
-    return (W == 512) ? cc * Cfg<W>::R + sub : sub * Cfg<W>::CPT + cc;
+    return (C::NHALF == 2) ? cc * C::R + sub : sub * C::CPT + cc;
 }
 
 struct FusedLayer {
@@ -546,10 +559,9 @@ template <bool SUSPEND> __device__ __forceinline__ bool slot_barrier(SlotCtx &c)
 // Passes 2 and 3: remaining butterfly stages across chunks, quantizer, store of the codes, and the
 // arrival on the "codes ready" barrier.  Returns false if a wait ran out.  s_out receives the
 // token's activation scale of the next layer.
-template <int W, bool PER_TOKEN, bool ROT, bool DUMP = false>
+template <class C, bool PER_TOKEN, bool ROT, bool DUMP = false>
 __device__ __forceinline__ bool finish_layer(SlotCtx &c, float static_s, float static_inv, float &s_out, int8_t *dump_codes = nullptr)
 {
-    using C = Cfg<W>;
     constexpr int NCH = C::NCH, G = C::G, CH = C::CH;
     ptx::tmem_wait_st();
     ptx::tc_fence_before();
@@ -630,9 +642,8 @@ __device__ __forceinline__ bool finish_layer(SlotCtx &c, float static_s, float s
 // once): in place of the quantizer, the maximum of |x~| over the tile's valid tokens goes to the
 // calibrated layer's act[0] (atomic maximum on the bit pattern: non-negative floats order as
 // integers).  Same barrier, loads and butterfly stages as finish_layer up to that point.
-template <int W, bool ROT> __device__ __forceinline__ bool calib_finish(SlotCtx &c, bool valid, float *act)
+template <class C, bool ROT> __device__ __forceinline__ bool calib_finish(SlotCtx &c, bool valid, float *act)
 {
-    using C = Cfg<W>;
     constexpr int NCH = C::NCH, G = C::G, CH = C::CH;
     ptx::tmem_wait_st();
     ptx::tc_fence_before();
@@ -719,9 +730,8 @@ template <int CH> __device__ __forceinline__ void int_butterfly_chunk(uint32_t (
 // ... then the stages across chunks, on groups of G positions of every chunk (as pass 2 does for
 // the forward rotation), in place in tensor memory.  Both sides of it are barriers of the R warps
 // that share the rows.  Returns false if a wait ran out.
-template <int W> __device__ __forceinline__ bool int_butterfly_across(SlotCtx &c)
+template <class C> __device__ __forceinline__ bool int_butterfly_across(SlotCtx &c)
 {
-    using C = Cfg<W>;
     constexpr int NCH = C::NCH, G = C::G, CH = C::CH;
     ptx::tmem_wait_st();
     ptx::tc_fence_before();
@@ -758,12 +768,11 @@ template <int W> __device__ __forceinline__ bool int_butterfly_across(SlotCtx &c
     return true;
 }
 
-template <int W, bool PER_TOKEN, bool ROT, bool SPREAD, bool AHEAD, bool DUMP, bool BOTH, bool CALIB, bool GABOR, bool MIXED>
+template <class C, bool PER_TOKEN, bool ROT, bool SPREAD, bool AHEAD, bool DUMP, bool BOTH, bool CALIB, bool GABOR, bool MIXED>
 __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm, uint32_t smem_base, int warp, int lane,
                               uint32_t tmem_base, volatile int *abort_flag)
 {
-    using C = Cfg<W>;
-    constexpr int CH = C::CH;
+    constexpr int W = C::W, CH = C::CH;
     const int slot = warp / (4 * C::R);
     const int quad = warp & 3;
     const int sub = (warp % (4 * C::R)) >> 2;
@@ -872,7 +881,7 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
         }
 #pragma unroll
         for (int cc = 0; cc < C::CPT; ++cc) {
-            const int ch = chunk_of<W>(sub, cc);
+            const int ch = chunk_of<C>(sub, cc);
             uint32_t v[CH];
             if constexpr (DUMP) {
                 // the first layer's accumulators are never formed on the fixed-point route (the phase is
@@ -890,11 +899,11 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
         if constexpr (CALIB) {
             // calibration of layer p.L: the network is run up to that layer's rotated input
             if (p.L == 2) {
-                if (!calib_finish<W, ROT>(c, valid, const_cast<float *>(p.layer[1].act))) return;
+                if (!calib_finish<C, ROT>(c, valid, const_cast<float *>(p.layer[1].act))) return;
                 continue;
             }
         }
-        if (!finish_layer<W, PER_TOKEN, ROT, DUMP>(c, next_s, next_inv, s_x, dC)) return;
+        if (!finish_layer<C, PER_TOKEN, ROT, DUMP>(c, next_s, next_inv, s_x, dC)) return;
         if constexpr (DUMP) {
             if (valid && sub == 0 && p.d.s_x[1]) p.d.s_x[1][tok] = s_x;
         }
@@ -913,8 +922,9 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
         // ---------------- layers 2 .. L on the tensor core
         for (int l = 2; l < p.L; ++l) {
             const FusedLayer &ly = p.layer[l - 1];
-            if (!wait_bar_warp<PER_TOKEN>(bar_acc, acc_parity, abort_flag, p.status)) return;
-            if constexpr (C::NHALF == 1) acc_parity ^= 1;
+            // (one chunk per thread: the barrier of the half that it lies in)
+            if (!wait_bar_warp<PER_TOKEN>(C::NHALF == 2 && C::CPT == 1 ? bar_acc + 8 * (sub / (C::R / 2)) : bar_acc, acc_parity, abort_flag, p.status)) return;
+            if constexpr (C::NHALF == 1 || C::CPT == 1) acc_parity ^= 1;
             ptx::tc_fence_after();
             if (!PER_TOKEN) {
                 next_s = __ldg(p.layer[l].act + 1);
@@ -926,8 +936,8 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
                 // pass 0: acc' = H_W acc on the integers, in place in tensor memory
 #pragma unroll
                 for (int cc = 0; cc < C::CPT; ++cc) {
-                    const int ch = chunk_of<W>(sub, cc);
-                    if constexpr (C::NHALF == 2) {
+                    const int ch = chunk_of<C>(sub, cc);
+                    if constexpr (C::NHALF == 2 && C::CPT == 2) {
                         if (cc == 1) {
                             if (!wait_bar_warp<PER_TOKEN>(bar_acc + 8, acc_parity, abort_flag, p.status)) return;
                             acc_parity ^= 1;
@@ -941,13 +951,13 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
                     int_butterfly_chunk<CH>(v);
                     tmem_st<CH>(c.taddr + ch * CH, v);
                 }
-                if (!int_butterfly_across<W>(c)) return;
+                if (!int_butterfly_across<C>(c)) return;
             }
 #pragma unroll
             for (int cc = 0; cc < C::CPT; ++cc) {
-                const int ch = chunk_of<W>(sub, cc);
-                if constexpr (C::NHALF == 2 && !BOTH) {
-                    // width 512: the thread's second chunk lies in the second half of the output columns,
+                const int ch = chunk_of<C>(sub, cc);
+                if constexpr (C::NHALF == 2 && C::CPT == 2 && !BOTH) {
+                    // the thread's second chunk lies in the second half of the output columns,
                     // whose MMAs run while the first chunk is worked on
                     if (cc == 1) {
                         if (!wait_bar_warp<PER_TOKEN>(bar_acc + 8, acc_parity, abort_flag, p.status)) return;
@@ -990,11 +1000,11 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
             if constexpr (DUMP) dC = (valid && p.d.codes[l]) ? p.d.codes[l] + tok * W : nullptr;
             if constexpr (CALIB) {
                 if (l == p.L - 1) {
-                    if (!calib_finish<W, ROT>(c, valid, const_cast<float *>(p.layer[l].act))) return;
+                    if (!calib_finish<C, ROT>(c, valid, const_cast<float *>(p.layer[l].act))) return;
                     continue;
                 }
             }
-            if (!finish_layer<W, PER_TOKEN, ROT, DUMP>(c, next_s, next_inv, s_x, dC)) return;
+            if (!finish_layer<C, PER_TOKEN, ROT, DUMP>(c, next_s, next_inv, s_x, dC)) return;
             if constexpr (DUMP) {
                 if (valid && sub == 0 && p.d.s_x[l]) p.d.s_x[l][tok] = s_x;
             }
@@ -1064,11 +1074,11 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
     if (!AHEAD && !C::BULK_XY && sub == 0 && c.row == 0) ptx::bulk_wait_all(); // the last tiles' stores
 }
 
-template <int W, bool SPREAD, bool CALIB>
+template <class C, bool SPREAD, bool CALIB>
 __device__ void mma_role(const FusedParams &p, const SmemMap &sm, uint32_t smem_base, uint32_t tmem_base,
                          volatile int *abort_flag)
 {
-    using C = Cfg<W>;
+    constexpr int W = C::W;
     // (before the first bounded wait: a kernel before this one may run for longer than the limit)
     ptx::wait_for_previous_kernels();
     uint32_t codes_parity[2] = {0, 0};
@@ -1083,7 +1093,7 @@ __device__ void mma_role(const FusedParams &p, const SmemMap &sm, uint32_t smem_
         if (tile_index<SPREAD>(r, 0, C::SLOTS) >= p.n_tiles) break;
         const int active = (C::SLOTS == 2 && tile_index<SPREAD>(r, 1, C::SLOTS) < p.n_tiles) ? 2 : 1;
         for (int l = 2; l < p.L && ok; ++l) {
-            if constexpr (C::NHALF == 2) {
+            if constexpr (W == 512) {
                 // width 512: eight pieces per layer, the four k-pieces of output columns 0..255 first;
                 // each half of the accumulator is committed on its own barrier as soon as it is complete
                 for (int pc = 0; pc < C::PIECES && ok; ++pc) {
@@ -1131,8 +1141,8 @@ __device__ void mma_role(const FusedParams &p, const SmemMap &sm, uint32_t smem_
 #pragma unroll
                         for (int ks = 0; ks < C::SLABK / 32; ++ks)
                             ptx::mma_i8(d, ad0 + ks * a_step, bd0 + ks * b_step, idesc_hidden, (ksl > 0 || ks > 0) ? 1u : 0u);
+                        if (ksl == C::KSLABS - 1) ptx::mma_commit(smem_base + sm.acc_full + 8 * (s * 4 + half));
                     }
-                    if (ksl == C::KSLABS - 1) ptx::mma_commit(smem_base + sm.acc_full + 8 * (s * 4));
                 }
                 if (!ok) break;
                 if (!p.resident) {
@@ -1166,10 +1176,10 @@ __device__ void mma_role(const FusedParams &p, const SmemMap &sm, uint32_t smem_
     }
 }
 
-template <int W, bool SPREAD, bool CALIB>
+template <class C, bool SPREAD, bool CALIB>
 __device__ void load_role(const FusedParams &p, const SmemMap &sm, uint32_t smem_base, volatile int *abort_flag)
 {
-    using C = Cfg<W>;
+    constexpr int W = C::W;
     const uint32_t slab = C::PIECE_BYTES;
     // (test hook: with skip_last_weights set the copy is left out and nothing ever completes
     // last_full, so the waits for it run out, the abort path runs and the kernel returns)
@@ -1218,10 +1228,9 @@ __device__ void load_role(const FusedParams &p, const SmemMap &sm, uint32_t smem
 
 // Width 512.  Coordinates: one bulk copy per whole tile (1 KB) into the slot's buffer, issued as
 // soon as the slot's threads have taken the previous tile's coordinates out of it.
-template <int W, bool SPREAD>
+template <class C, bool SPREAD>
 __device__ void xy_role(const FusedParams &p, const SmemMap &sm, uint32_t smem_base, volatile int *abort_flag)
 {
-    using C = Cfg<W>;
     if (!p.bulk_xy) return;
     ptx::wait_for_previous_kernels();
     uint32_t k[2] = {0, 0};
@@ -1246,10 +1255,10 @@ __device__ void xy_role(const FusedParams &p, const SmemMap &sm, uint32_t smem_b
 }
 
 template <int W, bool PER_TOKEN, bool ROT, bool SPREAD, bool AHEAD, bool DUMP = false, bool BOTH = false, bool CALIB = false,
-          bool GABOR = false, bool MIXED = false>
-__global__ void __launch_bounds__(Cfg<W>::THREADS, 1) fused_kernel(const __grid_constant__ ParamsOf<DUMP, CALIB> p)
+          bool GABOR = false, bool MIXED = false, bool NARROW = false>
+__global__ void __launch_bounds__(fused_threads(W, BOTH, GABOR), 1) fused_kernel(const __grid_constant__ ParamsOf<DUMP, CALIB> p)
 {
-    using C = Cfg<W>;
+    using C = Cfg<W, NARROW>;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = ptx::smem_u32(smem_raw);
     const uint32_t smem_base = (raw + 1023u) & ~1023u;
@@ -1303,7 +1312,7 @@ __global__ void __launch_bounds__(Cfg<W>::THREADS, 1) fused_kernel(const __grid_
             const uint32_t *srcB = fixed ? ly.fxB : reinterpret_cast<const uint32_t *>(ly.cB);
             const uint32_t *srcC = fixed ? ly.fxQ : reinterpret_cast<const uint32_t *>(ly.cA_lo);
             const int areas = (l == 0) ? (fixed ? 3 : (BOTH ? 5 : 4)) : ((ly.epi_mode == EPI_SINE_WIDE || ly.epi_mode == EPI_SINE_MIXED) ? 3 : 2);
-            for (int i = threadIdx.x; i < W; i += C::THREADS) { // i: tensor-memory column, m: its feature
+            for (int i = threadIdx.x; i < W; i += fused_threads(W, BOTH, GABOR)) { // i: tensor-memory column, m: its feature
                 const int m = fused_feature(i, W);
                 d[i] = __ldg(srcA + m);
                 d[W + i] = __ldg(srcB + m);
@@ -1321,12 +1330,16 @@ __global__ void __launch_bounds__(Cfg<W>::THREADS, 1) fused_kernel(const __grid_
     ptx::tc_fence_after();
     const uint32_t tmem_base = *tmem_holder;
 
+    if constexpr (splits_registers(W, BOTH, GABOR)) {
+        if (warp < kEpiWarps) ptx::take_registers<kEpiRegs>();
+        else ptx::give_registers<kRoleRegs>();
+    }
     if (warp < kEpiWarps) {
-        epilogue_role<W, PER_TOKEN, ROT, SPREAD, AHEAD, DUMP, BOTH, CALIB, GABOR, MIXED>(p, sm, smem_base, warp, lane, tmem_base, abort_flag);
+        epilogue_role<C, PER_TOKEN, ROT, SPREAD, AHEAD, DUMP, BOTH, CALIB, GABOR, MIXED>(p, sm, smem_base, warp, lane, tmem_base, abort_flag);
     } else if (warp == kMmaWarp) {
-        if (lane == 0) mma_role<W, SPREAD, CALIB>(p, sm, smem_base, tmem_base, abort_flag);
+        if (lane == 0) mma_role<C, SPREAD, CALIB>(p, sm, smem_base, tmem_base, abort_flag);
     } else if (warp == kLoadWarp) {
-        if (lane == 0) load_role<W, SPREAD, CALIB>(p, sm, smem_base, abort_flag);
+        if (lane == 0) load_role<C, SPREAD, CALIB>(p, sm, smem_base, abort_flag);
         if constexpr (DUMP) {
             // Observing instantiation only (in the timed kernels these few instructions cost 3-4 %): an
             // otherwise idle lane of CTA 0 notes the SM's cycle counter and the global nanosecond timer
@@ -1339,7 +1352,7 @@ __global__ void __launch_bounds__(Cfg<W>::THREADS, 1) fused_kernel(const __grid_
         }
     } else {
         if constexpr (C::BULK_XY) {
-            if (lane == 0) xy_role<W, SPREAD>(p, sm, smem_base, abort_flag);
+            if (warp == kXyWarp && lane == 0) xy_role<C, SPREAD>(p, sm, smem_base, abort_flag);
         }
     }
     ptx::tc_fence_before();
@@ -1372,6 +1385,19 @@ template <int W, bool AHEAD_OK> fused_fn pick_width(bool per_token, bool rot, bo
 {
     if (AHEAD_OK && ahead) return spread ? pick_flags<W, true, AHEAD_OK>(per_token, rot) : pick_flags<W, false, AHEAD_OK>(per_token, rot);
     return spread ? pick_flags<W, true, false>(per_token, rot) : pick_flags<W, false, false>(per_token, rot);
+}
+// At most one tile per SM, widths with such a split.
+template <int W> fused_fn pick_narrow_width(bool per_token, bool rot, bool both, bool gabor, bool mixed)
+{
+    if (gabor) {
+        if (both) return per_token ? fused_kernel<W, true, true, false, false, false, true, false, true, false, true> : fused_kernel<W, false, true, false, false, false, true, false, true, false, true>;
+        if (rot) return per_token ? fused_kernel<W, true, true, false, false, false, false, false, true, false, true> : fused_kernel<W, false, true, false, false, false, false, false, true, false, true>;
+        return per_token ? fused_kernel<W, true, false, false, false, false, false, false, true, false, true> : fused_kernel<W, false, false, false, false, false, false, false, true, false, true>;
+    }
+    if (both) return per_token ? fused_kernel<W, true, true, false, false, false, true, false, false, false, true> : fused_kernel<W, false, true, false, false, false, true, false, false, false, true>;
+    if (mixed) return rot ? fused_kernel<W, true, true, false, false, false, false, false, false, true, true> : fused_kernel<W, true, false, false, false, false, false, false, false, true, true>;
+    if (rot) return per_token ? fused_kernel<W, true, true, false, false, false, false, false, false, false, true> : fused_kernel<W, false, true, false, false, false, false, false, false, false, true>;
+    return per_token ? fused_kernel<W, true, false, false, false, false, false, false, false, false, true> : fused_kernel<W, false, false, false, false, false, false, false, false, false, true>;
 }
 typedef void (*fused_dump_fn)(const FusedParamsDump);
 // The observing instantiation of a width: the tile mapping and coordinate fetch of the large
@@ -1446,6 +1472,7 @@ fused_dump_fn fused_pick_dump_64(bool per_token, bool rot);
 fused_dump_fn fused_pick_dump_128(bool per_token, bool rot);
 fused_dump_fn fused_pick_dump_256(bool per_token, bool rot);
 fused_dump_fn fused_pick_dump_512(bool per_token, bool rot);
+fused_fn fused_pick_narrow_256(bool per_token, bool rot, bool both, bool gabor, bool mixed);
 fused_fn fused_pick_gabor_64(bool per_token, bool rot);
 fused_fn fused_pick_gabor_128(bool per_token, bool rot);
 fused_fn fused_pick_gabor_256(bool per_token, bool rot);

@@ -56,6 +56,9 @@ __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontr
 // ... and waits here until the kernels before it have completed and their writes are visible (nothing
 // to wait for in a kernel that was launched the ordinary way).
 __device__ __forceinline__ void wait_for_previous_kernels() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Register split between warpgroups: every warp of the warpgroup executes it once.
+template <int N> __device__ __forceinline__ void take_registers() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N> __device__ __forceinline__ void give_registers() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 // Generic-proxy writes to shared memory become visible to the async proxy (tensor core, bulk copy).
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void fence_mbar_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
