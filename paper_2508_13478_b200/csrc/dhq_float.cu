@@ -27,7 +27,8 @@
 // remaining 32 KB of shared memory keep too few weight bytes in flight (105 cycles per MMA); at
 // width 256 the sines and digits of the block behind take as long as the MMAs.
 // Measured: 2 -> 256 x 3 -> 3, fp32, 65,536 coordinates 940 -> 92 us; 2 -> 512 x 4 -> 3, 8-bit
-// weights, 262,144 coordinates 17.2 -> 1.22 ms (one fp32 CUDA-core pass per layer before).
+// weights, 262,144 coordinates 17.2 -> 1.11 ms (one fp32 CUDA-core pass per layer before; 1.21 ms without the
+// register split of the warpgroups).
 #include "dhq_fused.cuh"
 
 namespace dhq {
@@ -457,6 +458,8 @@ __global__ void __launch_bounds__(kFThreads, 1) float_kernel(const __grid_consta
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(gen + sm.holder);
+    if (warp < kEpiWarps) ptx::take_registers<kEpiRegs>(); // see splits_registers
+    else ptx::give_registers<kRoleRegs>();
     if (warp < kEpiWarps) float_epilogue<W, WL, DUMP>(p, sm, base, warp, lane, tmem, abort_flag);
     else if (lane == 0) {
         if (warp == kMmaWarp) float_mma<W, WL>(p, sm, base, tmem, abort_flag);
@@ -615,7 +618,7 @@ dhq_status_t float_create(dhq_handle_s *h)
     p.x = h->x_scratch;
     float_fn fns[2] = {pick_float<false>(h->w, h->float_digits), pick_float<true>(h->w, h->float_digits)};
     for (float_fn f : fns)
-        if (!allow_smem((const void *)f, dev, max_optin)) return DHQ_ERR_CUDA;
+        if (!allow_smem((const void *)f, dev, max_optin, kLaunchRegs)) return DHQ_ERR_CUDA;
     return DHQ_OK;
 }
 

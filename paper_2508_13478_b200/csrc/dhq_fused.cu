@@ -154,7 +154,13 @@ static fused_fn pick_for(const dhq_handle_s *h, bool per_token, bool spread, boo
 static fused_fn pick_narrow_for(const dhq_handle_s *h, bool per_token)
 {
     const bool both = h->cfg.rotation == DHQ_ROT_BOTH, rot = h->cfg.rotation == DHQ_ROT_INPUT;
-    return h->w == 256 ? fused_pick_narrow_256(per_token, rot, both, h->gabor_s0 > 0.0, runs_mixed(h)) : nullptr;
+    const bool gabor = h->gabor_s0 > 0.0, mixed = runs_mixed(h);
+    switch (h->w) {
+    case 64: return !(both || gabor || mixed) ? nullptr : fused_pick_narrow_64(per_token, rot, both, gabor, mixed);
+    case 128: return !(both || gabor || mixed) ? nullptr : fused_pick_narrow_128(per_token, rot, both, gabor, mixed);
+    case 256: return fused_pick_narrow_256(per_token, rot, both, gabor, mixed);
+    }
+    return nullptr;
 }
 
 // Its observing instantiation.
@@ -286,12 +292,13 @@ int64_t fused_round_tokens(const dhq_handle_s *h)
 }
 
 // The per-call part of the parameter block.
-static void fill_call(const dhq_handle_s *h, FusedParams &p, const float *coords, int64_t n, float *out)
+static void fill_call(const dhq_handle_s *h, FusedParams &p, const float *coords, int64_t n, float *out, bool on_host)
 {
     p.coords = coords; p.out = out; p.n = n;
     p.n_tiles = (n + kTile - 1) / kTile;
     p.bulk_xy = (((uintptr_t)coords) & 15) == 0;
-    p.bulk_out = (((uintptr_t)out) & 15) == 0 && (smem_map(h->w, p.n_stages, p.const_words).out_tile & 15) == 0;
+    // (two more barriers per tile: worth it over the host link only)
+    p.bulk_out = on_host && (((uintptr_t)out) & 15) == 0 && (smem_map(h->w, p.n_stages, p.const_words).out_tile & 15) == 0;
     p.wait_limit_ns = h->wait_limit_ns;
     p.skip_last_weights = 0;
 }
@@ -301,7 +308,7 @@ dhq_status_t fused_forward(dhq_handle_s *h, const float *coords, int64_t n, floa
     FusedState *fs = static_cast<FusedState *>(h->fused);
     if (!fs) return DHQ_ERR_INVALID_ARG;
     FusedParams p = fs->p;
-    fill_call(h, p, coords, n, out);
+    fill_call(h, p, coords, n, out, on_host);
     if (h->stall_next_forward) { // test hook, one launch only
         p.skip_last_weights = 1;
         h->stall_next_forward = false;
@@ -354,7 +361,7 @@ dhq_status_t fused_calibrate_layer(dhq_handle_s *h, int l, const float *coords, 
     }
     FusedParamsCalib p;
     static_cast<FusedParams &>(p) = fs->p;
-    fill_call(h, p, coords, n, nullptr);
+    fill_call(h, p, coords, n, nullptr, false);
     p.L = l; // the network up to the rotated input of layer l
     p.freeze = freeze;
     p.a_bits = h->cfg.a_bits;
@@ -378,7 +385,7 @@ dhq_status_t fused_forward_dump(dhq_handle_s *h, const float *coords, int64_t n,
     if (!fs) return DHQ_ERR_INVALID_ARG;
     FusedParamsDump p;
     static_cast<FusedParams &>(p) = fs->p;
-    fill_call(h, p, coords, n, out);
+    fill_call(h, p, coords, n, out, false);
     p.d = d;
     const int slots = (h->w == 512) ? 1 : 2;
     fused_dump_fn fn = pick_dump_for(h, p.per_token);

@@ -1386,18 +1386,21 @@ template <int W, bool AHEAD_OK> fused_fn pick_width(bool per_token, bool rot, bo
     if (AHEAD_OK && ahead) return spread ? pick_flags<W, true, AHEAD_OK>(per_token, rot) : pick_flags<W, false, AHEAD_OK>(per_token, rot);
     return spread ? pick_flags<W, true, false>(per_token, rot) : pick_flags<W, false, false>(per_token, rot);
 }
-// At most one tile per SM, widths with such a split.
+// At most one tile per SM: NARROW at width 256; at widths 64 and 128, for the families that pick_width does not
+// spread, the plain split with the tiles on as many SMs as there are tiles.
 template <int W> fused_fn pick_narrow_width(bool per_token, bool rot, bool both, bool gabor, bool mixed)
 {
+    constexpr bool N = W == 256, SP = !N;
     if (gabor) {
-        if (both) return per_token ? fused_kernel<W, true, true, false, false, false, true, false, true, false, true> : fused_kernel<W, false, true, false, false, false, true, false, true, false, true>;
-        if (rot) return per_token ? fused_kernel<W, true, true, false, false, false, false, false, true, false, true> : fused_kernel<W, false, true, false, false, false, false, false, true, false, true>;
-        return per_token ? fused_kernel<W, true, false, false, false, false, false, false, true, false, true> : fused_kernel<W, false, false, false, false, false, false, false, true, false, true>;
+        if (both) return per_token ? fused_kernel<W, true, true, SP, false, false, true, false, true, false, N> : fused_kernel<W, false, true, SP, false, false, true, false, true, false, N>;
+        if (rot) return per_token ? fused_kernel<W, true, true, SP, false, false, false, false, true, false, N> : fused_kernel<W, false, true, SP, false, false, false, false, true, false, N>;
+        return per_token ? fused_kernel<W, true, false, SP, false, false, false, false, true, false, N> : fused_kernel<W, false, false, SP, false, false, false, false, true, false, N>;
     }
-    if (both) return per_token ? fused_kernel<W, true, true, false, false, false, true, false, false, false, true> : fused_kernel<W, false, true, false, false, false, true, false, false, false, true>;
-    if (mixed) return rot ? fused_kernel<W, true, true, false, false, false, false, false, false, true, true> : fused_kernel<W, true, false, false, false, false, false, false, false, true, true>;
-    if (rot) return per_token ? fused_kernel<W, true, true, false, false, false, false, false, false, false, true> : fused_kernel<W, false, true, false, false, false, false, false, false, false, true>;
-    return per_token ? fused_kernel<W, true, false, false, false, false, false, false, false, false, true> : fused_kernel<W, false, false, false, false, false, false, false, false, false, true>;
+    if (both) return per_token ? fused_kernel<W, true, true, SP, false, false, true, false, false, false, N> : fused_kernel<W, false, true, SP, false, false, true, false, false, false, N>;
+    if (mixed) return rot ? fused_kernel<W, true, true, SP, false, false, false, false, false, true, N> : fused_kernel<W, true, false, SP, false, false, false, false, false, true, N>;
+    if constexpr (!N) return nullptr;
+    else if (rot) return per_token ? fused_kernel<W, true, true, SP, false, false, false, false, false, false, N> : fused_kernel<W, false, true, SP, false, false, false, false, false, false, N>;
+    else return per_token ? fused_kernel<W, true, false, SP, false, false, false, false, false, false, N> : fused_kernel<W, false, false, SP, false, false, false, false, false, false, N>;
 }
 typedef void (*fused_dump_fn)(const FusedParamsDump);
 // The observing instantiation of a width: the tile mapping and coordinate fetch of the large
@@ -1472,6 +1475,8 @@ fused_dump_fn fused_pick_dump_64(bool per_token, bool rot);
 fused_dump_fn fused_pick_dump_128(bool per_token, bool rot);
 fused_dump_fn fused_pick_dump_256(bool per_token, bool rot);
 fused_dump_fn fused_pick_dump_512(bool per_token, bool rot);
+fused_fn fused_pick_narrow_64(bool per_token, bool rot, bool both, bool gabor, bool mixed);
+fused_fn fused_pick_narrow_128(bool per_token, bool rot, bool both, bool gabor, bool mixed);
 fused_fn fused_pick_narrow_256(bool per_token, bool rot, bool both, bool gabor, bool mixed);
 fused_fn fused_pick_gabor_64(bool per_token, bool rot);
 fused_fn fused_pick_gabor_128(bool per_token, bool rot);
