@@ -163,6 +163,19 @@ static fused_fn pick_narrow_for(const dhq_handle_s *h, bool per_token)
     return nullptr;
 }
 
+// The same for a launch of at most one tile of 64 tokens per SM.
+static fused_fn pick_dup_for(const dhq_handle_s *h, bool per_token)
+{
+    const bool both = h->cfg.rotation == DHQ_ROT_BOTH, rot = h->cfg.rotation == DHQ_ROT_INPUT, gabor = h->gabor_s0 > 0.0, mixed = runs_mixed(h);
+    switch (h->w) {
+    case 64: return fused_pick_dup_64(per_token, rot, both, gabor, mixed);
+    case 128: return fused_pick_dup_128(per_token, rot, both, gabor, mixed);
+    case 256: return fused_pick_dup_256(per_token, rot, both, gabor, mixed);
+    case 512: return fused_pick_dup_512(per_token, rot, both, gabor, mixed);
+    }
+    return nullptr;
+}
+
 // Its observing instantiation.
 static fused_dump_fn pick_dump_for(const dhq_handle_s *h, bool per_token)
 {
@@ -272,6 +285,7 @@ dhq_status_t fused_create(dhq_handle_s *h)
     for (int v = 0; v < 4; ++v) // every variant of this handle's kernel
         if (!allow_smem((const void *)pick_for(h, p.per_token, (v & 1) != 0, (v & 2) != 0), dev, max_optin, min_regs)) return DHQ_ERR_CUDA;
     const fused_fn narrow = pick_narrow_for(h, p.per_token);
+    if (!allow_smem((const void *)pick_dup_for(h, p.per_token), dev, max_optin, min_regs)) return DHQ_ERR_CUDA;
     if (narrow && !allow_smem((const void *)narrow, dev, max_optin, min_regs)) return DHQ_ERR_CUDA;
     if (!p.per_token && !allow_smem((const void *)pick_calib_kernel(h->w, h->cfg.rotation == DHQ_ROT_INPUT, gabor, both), dev, max_optin, min_regs)) return DHQ_ERR_CUDA;
     if (!allow_smem((const void *)pick_dump_for(h, p.per_token), dev, max_optin, min_regs)) return DHQ_ERR_CUDA;
@@ -317,7 +331,10 @@ dhq_status_t fused_forward(dhq_handle_s *h, const float *coords, int64_t n, floa
     const bool both = h->cfg.rotation == DHQ_ROT_BOTH;
     const bool gabor = h->gabor_s0 > 0.0;
     const bool spread = !both && !gabor && !runs_mixed(h) && slots > 1 && p.n_tiles < (long long)fs->sm_count * slots;
-    const fused_fn narrow = p.n_tiles <= (long long)fs->sm_count ? pick_narrow_for(h, p.per_token) : nullptr;
+    constexpr int kHalfTile = kTile / 2;
+    const fused_fn dup = n <= (int64_t)fs->sm_count * kHalfTile ? pick_dup_for(h, p.per_token) : nullptr;
+    if (dup) p.n_tiles = (n + kHalfTile - 1) / kHalfTile;
+    const fused_fn narrow = dup ? dup : p.n_tiles <= (long long)fs->sm_count ? pick_narrow_for(h, p.per_token) : nullptr;
     const fused_fn fn = narrow ? narrow : pick_for(h, p.per_token, spread, !on_host);
     const long long ctas = spread || narrow ? p.n_tiles : (p.n_tiles + slots - 1) / slots;
     int grid = (int)(ctas < fs->sm_count ? ctas : fs->sm_count);

@@ -62,15 +62,25 @@ constexpr int kMinSmem = 120 * 1024; // more than half an SM's shared memory: on
 // Work split for a hidden width W.  NARROW: all 16 epilogue warps on one tile, for launches with at most one
 // tile per SM, where the time of a tile is what counts (a slot of 8 warps alone on an SM needs 24
 // cycles per 32 elements and scheduler, 16 warps 18).
-template <int W_, bool NARROW = false> struct Cfg {
+// DUP: tiles of 64 tokens, for launches with at most one such tile per SM.  Every token sits in two rows of the
+// operand tile, 16 apart (lanes i and i + 16 of one warp), and the two threads take one half each of every
+// chunk's columns: a thread's share of a layer's elements halves.  The stage whose pairs lie in different
+// halves is a shuffle; everything after it stays in the own half, because the later stages pair equal
+// positions of different chunks.
+// Measured back to back, 1,600 coordinates: width 512 36.0 -> 30.2 us (per token 44.6 -> 35.8, wavelet 54.9 ->
+// 37.9), 256 12.7 -> 10.9 (15.8 -> 12.2), 128 10.4 -> 8.0, 64 6.9 -> 5.8.
+template <int W_, bool NARROW = false, bool DUP_ = false> struct Cfg {
     static constexpr int W = W_;
-    static constexpr int SLOTS = (W == 512 || NARROW) ? 1 : 2;
-    static constexpr int R = kEpiWarps / (4 * SLOTS);          // threads per row: 2 or 4
+    static constexpr bool DUP = DUP_;
+    static constexpr int TOK = DUP ? kTile / 2 : kTile;        // tokens per tile
+    static constexpr int SLOTS = (W == 512 || NARROW || DUP) ? 1 : 2;
+    static constexpr int R = (W == 512 || NARROW) ? 4 : 2;     // warps that share a row
     static constexpr int CH = (W == 64) ? 32 : 64;             // columns per register chunk (= fused_chunk(W))
     static constexpr int NCH = W / CH;                         // chunks per row
     static constexpr int CPT = NCH / R;                        // chunks per thread
-    static constexpr int G = (64 / NCH < CH / R) ? 64 / NCH : CH / R; // positions per pass-2 group
-    static constexpr int GPT = CH / (G * R);                   // groups per thread
+    static constexpr int HC = DUP ? CH / 2 : CH;               // columns of a chunk that a thread takes
+    static constexpr int G = (64 / NCH < HC / R) ? 64 / NCH : HC / R; // positions per pass-2 group
+    static constexpr int GPT = HC / (G * R);                   // groups per thread
     static constexpr int KSLABS = (W == 512) ? 4 : 1;          // weight slabs per layer along K
     static constexpr int SLABK = W / KSLABS;                   // k per slab (= fused_slab_k)
     // A layer's products are finished in two halves of the output columns, each with its own barrier, so
@@ -321,7 +331,7 @@ template <int N> __device__ __forceinline__ void store_code_words(uint32_t a_til
 }
 // Quantize G consecutive tensor-memory columns of chunk `ch` starting at column position p0 (even
 // positions hold features p0/2 + k, odd positions features CH/2 + p0/2 + k) and store the codes.
-template <int G, int CH, bool CLAMP, bool DUMP = false>
+template <int G, int CH, bool CLAMP, bool DUMP = false, bool DUP = false>
 __device__ __forceinline__ void quantize_store(uint32_t a_tile, int row, int ch, int p0, const uint32_t *u, float inv, float qmaxf,
                                                int8_t *dump_row = nullptr)
 {
@@ -337,6 +347,10 @@ __device__ __forceinline__ void quantize_store(uint32_t a_tile, int row, int ch,
     }
     store_code_words<G / 2>(a_tile, row, ch * CH + p0 / 2, we);
     store_code_words<G / 2>(a_tile, row, ch * CH + CH / 2 + p0 / 2, wo);
+    if constexpr (DUP) {
+        store_code_words<G / 2>(a_tile, row ^ 16, ch * CH + p0 / 2, we);
+        store_code_words<G / 2>(a_tile, row ^ 16, ch * CH + CH / 2 + p0 / 2, wo);
+    }
     if constexpr (DUMP) {
         // the very words that went into the A operand tile, at their feature positions k
         if (dump_row) {
@@ -381,7 +395,9 @@ __device__ __forceinline__ float4 lds128(uint32_t addr)
 // butterflies follow every fourth group - so that the special-function unit (one sine per 8 issue
 // cycles and scheduler) is fed evenly instead of in one burst per chunk.  Each element still goes
 // through the stages in the order 1, 2, 4, ...: the sums are unchanged.
-template <int CH, bool ROT, class Sine8> __device__ __forceinline__ void chunk_pipeline(uint32_t (&v)[CH], Sine8 sine8)
+// DUP: v holds the thread's half of a chunk of 2 CH columns; the stage before the last one exchanges it with
+// lane ^ 16 (the lower half keeps the sums, the upper one the differences: other + (-own)).
+template <int CH, bool ROT, bool DUP, class Sine8> __device__ __forceinline__ void chunk_pipeline(uint32_t (&v)[CH], Sine8 sine8)
 {
     constexpr int NP = CH / 2;
     f32x2 P[NP];
@@ -411,10 +427,20 @@ template <int CH, bool ROT, class Sine8> __device__ __forceinline__ void chunk_p
         }
     }
 #pragma unroll
-    for (int h = 16; h < NP; h <<= 1) {
+    for (int h = NP < 16 ? 4 : 16; h < NP; h <<= 1) {
 #pragma unroll
         for (int i = 0; i < NP; ++i)
             if ((i & h) == 0) bfly2(P[i], P[i + h]);
+    }
+    if constexpr (DUP) {
+        const uint32_t flip = (threadIdx.x & 16) << 27; // sign bit of the upper half's own values
+#pragma unroll
+        for (int i = 0; i < NP; ++i) {
+            uint32_t a, b;
+            unpack2u(P[i], a, b);
+            const uint32_t oa = __shfl_xor_sync(0xffffffffu, a, 16), ob = __shfl_xor_sync(0xffffffffu, b, 16);
+            P[i] = add2(pack2u(oa, ob), pack2u(a ^ flip, b ^ flip));
+        }
     }
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
@@ -441,12 +467,12 @@ template <int W> __device__ __forceinline__ void dump_y4(float *yrow, int col, f
 // from shared memory in column order: area A = cA, B = cB, C = cA_lo, each W words.
 // TRACK (with EPI_SINE_FAST): *xmax receives the largest |phase| the thread met, for the caller's decision
 // whether the chunk has to be redone under EPI_SINE_MIXED.  LIMIT: the limit of EPI_SINE_MIXED.
-template <int W, int CH, bool PER_TOKEN, bool ROT, int MODE, bool DUMP = false, bool GABOR = false, bool TRACK = false>
+template <int W, int CH, bool PER_TOKEN, bool ROT, int MODE, bool DUMP = false, bool GABOR = false, bool TRACK = false, bool DUP = false>
 __device__ __forceinline__ void hidden_chunk(uint32_t cbase, int m0, float s_x, uint32_t (&v)[CH], float *dump_y = nullptr,
                                              float gabor_c = 0.f, [[maybe_unused]] float *xmax = nullptr, [[maybe_unused]] float limit = 0.f)
 {
     [[maybe_unused]] float xm = 0.f;
-    chunk_pipeline<CH, ROT>(v, [&](int j, f32x2 *out) {
+    chunk_pipeline<CH, ROT, DUP>(v, [&](int j, f32x2 *out) {
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int i = 8 * j + 4 * q; // four columns = two pairs
@@ -492,11 +518,11 @@ __device__ __forceinline__ void hidden_chunk(uint32_t cbase, int m0, float s_x, 
 // Layer 1 for the CH columns starting at column m0.  Fixed-point mode: areas A = P, B = B, C = Q.
 // Float mode (per-token scales): A = cA, B = cB, C = cA_lo, D = the weight codes, one word per
 // column, and acc = dp4a(codes of the token, codes of the column's feature).
-template <int W, int CH, bool PER_TOKEN, bool ROT, bool DUMP = false, bool BOTH = false, bool GABOR = false>
+template <int W, int CH, bool PER_TOKEN, bool ROT, bool DUMP = false, bool BOTH = false, bool GABOR = false, bool DUP = false>
 __device__ __forceinline__ void layer1_chunk(uint32_t cbase, int m0, int qs, int qd, uint32_t qx, float s_x, uint32_t (&v)[CH],
                                              float *dump_y = nullptr, float gabor_c = 0.f)
 {
-    chunk_pipeline<CH, ROT>(v, [&](int j, f32x2 *out) {
+    chunk_pipeline<CH, ROT, DUP>(v, [&](int j, f32x2 *out) {
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int i = 8 * j + 4 * q;
@@ -563,6 +589,7 @@ template <class C, bool PER_TOKEN, bool ROT, bool DUMP = false>
 __device__ __forceinline__ bool finish_layer(SlotCtx &c, float static_s, float static_inv, float &s_out, int8_t *dump_codes = nullptr)
 {
     constexpr int NCH = C::NCH, G = C::G, CH = C::CH;
+    const int half = C::DUP && (c.row & 16) ? C::HC : 0; // (the half lies in the chunk's first columns of this lane)
     ptx::tmem_wait_st();
     ptx::tc_fence_before();
     if (!slot_barrier<PER_TOKEN>(c)) return false;
@@ -600,13 +627,14 @@ __device__ __forceinline__ bool finish_layer(SlotCtx &c, float static_s, float s
             }
         } else {
 #pragma unroll
-            for (int ch = 0; ch < NCH; ++ch) quantize_store<G, CH, true, DUMP>(c.a_tile, c.row, ch, g * G, u[ch], static_inv, c.qmaxf, dump_codes);
+            for (int ch = 0; ch < NCH; ++ch) quantize_store<G, CH, true, DUMP, C::DUP>(c.a_tile, c.row, ch, half + g * G, u[ch], static_inv, c.qmaxf, dump_codes);
         }
     }
     if (!PER_TOKEN) {
         s_out = static_s;
     } else {
-        // combine the row's absmax over the R threads that share it
+        // combine the row's absmax over the threads that share it
+        if constexpr (C::DUP) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 16));
         asm volatile("st.shared.f32 [%0], %1;" ::"r"(c.amax_addr + (c.sub * kTile + c.row) * 4), "f"(amax) : "memory");
         ptx::tmem_wait_st();
         ptx::tc_fence_before();
@@ -629,7 +657,7 @@ __device__ __forceinline__ bool finish_layer(SlotCtx &c, float static_s, float s
             for (int ch = 0; ch < NCH; ++ch) tmem_ld<G>(c.taddr + ch * CH + g * G, u[ch]);
             ptx::tmem_wait_ld();
 #pragma unroll
-            for (int ch = 0; ch < NCH; ++ch) quantize_store<G, CH, false, DUMP>(c.a_tile, c.row, ch, g * G, u[ch], inv, c.qmaxf, dump_codes);
+            for (int ch = 0; ch < NCH; ++ch) quantize_store<G, CH, false, DUMP, C::DUP>(c.a_tile, c.row, ch, half + g * G, u[ch], inv, c.qmaxf, dump_codes);
         }
     }
     ptx::fence_proxy_async();
@@ -732,14 +760,14 @@ template <int CH> __device__ __forceinline__ void int_butterfly_chunk(uint32_t (
 // that share the rows.  Returns false if a wait ran out.
 template <class C> __device__ __forceinline__ bool int_butterfly_across(SlotCtx &c)
 {
-    constexpr int NCH = C::NCH, G = C::G, CH = C::CH;
+    constexpr int NCH = C::NCH, G = C::G, CH = C::CH, GPT = CH / (G * C::R); // (all columns, with DUP too)
     ptx::tmem_wait_st();
     ptx::tc_fence_before();
     if (!slot_barrier<false>(c)) return false;
     ptx::tc_fence_after();
 #pragma unroll 1
-    for (int gg = 0; gg < C::GPT; ++gg) {
-        const int g = c.sub * C::GPT + gg;
+    for (int gg = 0; gg < GPT; ++gg) {
+        const int g = c.sub * GPT + gg;
         uint32_t u[NCH][G];
 #pragma unroll
         for (int ch = 0; ch < NCH; ++ch) tmem_ld<G>(c.taddr + ch * CH + g * G, u[ch]);
@@ -768,6 +796,23 @@ template <class C> __device__ __forceinline__ bool int_butterfly_across(SlotCtx 
     return true;
 }
 
+// A thread's columns of the chunk at `taddr` (a tensor-memory load takes the same columns in every lane: with
+// DUP the warp loads both halves and each thread keeps its own).
+template <class C> __device__ __forceinline__ void load_part(uint32_t taddr, uint32_t (&v)[C::HC])
+{
+    tmem_ld<C::HC>(taddr, v);
+    if constexpr (C::DUP) {
+        uint32_t up[C::HC];
+        tmem_ld<C::HC>(taddr + C::HC, up);
+        ptx::tmem_wait_ld();
+        const bool upper = threadIdx.x & 16;
+#pragma unroll
+        for (int i = 0; i < C::HC; ++i) v[i] = upper ? up[i] : v[i];
+    } else {
+        ptx::tmem_wait_ld();
+    }
+}
+
 template <class C, bool PER_TOKEN, bool ROT, bool SPREAD, bool AHEAD, bool DUMP, bool BOTH, bool CALIB, bool GABOR, bool MIXED>
 __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm, uint32_t smem_base, int warp, int lane,
                               uint32_t tmem_base, volatile int *abort_flag)
@@ -777,7 +822,10 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
     const int quad = warp & 3;
     const int sub = (warp % (4 * C::R)) >> 2;
     SlotCtx c;
+    if (C::DUP && slot >= C::SLOTS) return; // widths 64 and 128 have eight warps' worth of chunks
     c.row = quad * 32 + lane;
+    const int trow = C::DUP ? quad * 16 + (lane & 15) : c.row; // token of the tile
+    const int chalf = C::DUP && (lane & 16) ? C::HC : 0;       // first column of the thread's part of a chunk
     c.sub = sub;
     c.taddr = tmem_base + (uint32_t)(slot * C::TMEM_COLS_PER_SLOT) + ((uint32_t)(quad * 32) << 16);
     c.a_tile = smem_base + sm.a_tile[slot];
@@ -811,17 +859,17 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
     for (long long r = 0;; ++r) {
         const long long tile = tile_index<SPREAD>(r, slot, C::SLOTS);
         if (tile >= p.n_tiles) break;
-        const long long tok = tile * kTile + c.row;
+        const long long tok = tile * C::TOK + trow;
         const bool valid = tok < p.n;
 
         // ---------------- layer 1 on the CUDA cores: x~ = H_4 [x, y, 0, 0]
         float x = 0.f, y = 0.f;
         if constexpr (C::BULK_XY) {
-            if (p.bulk_xy && (tile + 1) * kTile <= p.n) {
+            if (p.bulk_xy && (tile + 1) * C::TOK <= p.n) {
                 // the whole tile was brought to shared memory by one bulk copy, a tile ahead
                 if (!wait_bar_warp<PER_TOKEN>(smem_base + sm.xy_full + 8 * slot, xy_k & 1u, abort_flag, p.status)) return;
                 ++xy_k;
-                asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(x), "=f"(y) : "r"(smem_base + sm.xy + (uint32_t)((slot * kTile + c.row) * 8)));
+                asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(x), "=f"(y) : "r"(smem_base + sm.xy + (uint32_t)((slot * kTile + trow) * 8)));
                 // The arrival below hands the buffer back to the copy warp, whose next bulk copy (async
                 // proxy) overwrites it.  The arrival does not wait for this thread's load to have been
                 // performed: with the load/store unit backed up (the observing instantiation's stores) the
@@ -882,7 +930,7 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
 #pragma unroll
         for (int cc = 0; cc < C::CPT; ++cc) {
             const int ch = chunk_of<C>(sub, cc);
-            uint32_t v[CH];
+            uint32_t v[C::HC];
             if constexpr (DUMP) {
                 // the first layer's accumulators are never formed on the fixed-point route (the phase is
                 // built from the two distinct codes directly); the dump states them: codes . weight codes
@@ -893,8 +941,8 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
                     }
                 }
             }
-            layer1_chunk<W, CH, PER_TOKEN, ROT, DUMP, BOTH, GABOR>(consts + l1.c_off * 4, ch * CH, qs, qd, qx, s_x, v, dY, p.gabor_c);
-            tmem_st<CH>(c.taddr + ch * CH, v);
+            layer1_chunk<W, C::HC, PER_TOKEN, ROT, DUMP, BOTH, GABOR, C::DUP>(consts + l1.c_off * 4, ch * CH + chalf, qs, qd, qx, s_x, v, dY, p.gabor_c);
+            tmem_st<C::HC>(c.taddr + ch * CH, v);
         }
         if constexpr (CALIB) {
             // calibration of layer p.L: the network is run up to that layer's rotated input
@@ -914,7 +962,7 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
             // it occupies).  Not earlier than this: at the start of a launch every tile's first fetch
             // is under way.  Only for coordinates in device memory: from mapped host memory the
             // 8-byte asynchronous copies were slower than the plain load at the tile's start.
-            const long long tok_next = tile_index<SPREAD>(r + 1, slot, C::SLOTS) * kTile + c.row;
+            const long long tok_next = tile_index<SPREAD>(r + 1, slot, C::SLOTS) * C::TOK + trow;
             if (tok_next < p.n)
                 asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(xy_addr), "l"(reinterpret_cast<const float2 *>(p.coords) + tok_next) : "memory");
         }
@@ -965,15 +1013,14 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
                         ptx::tc_fence_after();
                     }
                 }
-                uint32_t v[CH];
-                tmem_ld<CH>(c.taddr + ch * CH, v);
-                ptx::tmem_wait_ld();
+                uint32_t v[C::HC];
+                load_part<C>(c.taddr + ch * CH, v);
                 if constexpr (DUMP) {
                     dY = (valid && p.d.Y[l - 1]) ? p.d.Y[l - 1] + tok * W : nullptr;
-                    if constexpr (!BOTH) dump_acc_chunk<W, CH>((valid && p.d.acc[l - 1]) ? p.d.acc[l - 1] + tok * W : nullptr, ch * CH, v);
+                    if constexpr (!BOTH && !C::DUP) dump_acc_chunk<W, CH>((valid && p.d.acc[l - 1]) ? p.d.acc[l - 1] + tok * W : nullptr, ch * CH, v);
                 }
                 if (fast) {
-                    hidden_chunk<W, CH, PER_TOKEN, ROT, EPI_SINE_FAST, DUMP>(cbase, ch * CH, s_x, v, dY);
+                    hidden_chunk<W, C::HC, PER_TOKEN, ROT, EPI_SINE_FAST, DUMP, false, false, C::DUP>(cbase, ch * CH + chalf, s_x, v, dY);
                 } else {
                     [[maybe_unused]] bool done = false;
                     if constexpr ((MIXED || BOTH) && !GABOR) {
@@ -984,18 +1031,17 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
                             // beyond the limit.  The per-value rule gives the same bits either way.
                             constexpr float kLimit = BOTH ? kMixedPhaseLimitBoth : PER_TOKEN ? kFastPhaseLimitPerToken : kFastPhaseLimit;
                             float xm = 0.f;
-                            hidden_chunk<W, CH, PER_TOKEN, ROT, EPI_SINE_FAST, DUMP, false, true>(cbase, ch * CH, s_x, v, dY, 0.f, &xm);
+                            hidden_chunk<W, C::HC, PER_TOKEN, ROT, EPI_SINE_FAST, DUMP, false, true, C::DUP>(cbase, ch * CH + chalf, s_x, v, dY, 0.f, &xm);
                             if (!__all_sync(0xffffffffu, xm <= kLimit)) {
-                                tmem_ld<CH>(c.taddr + ch * CH, v);
-                                ptx::tmem_wait_ld();
-                                hidden_chunk<W, CH, PER_TOKEN, ROT, EPI_SINE_MIXED, DUMP>(cbase, ch * CH, s_x, v, dY, 0.f, nullptr, kLimit);
+                                load_part<C>(c.taddr + ch * CH, v);
+                                hidden_chunk<W, C::HC, PER_TOKEN, ROT, EPI_SINE_MIXED, DUMP, false, false, C::DUP>(cbase, ch * CH + chalf, s_x, v, dY, 0.f, nullptr, kLimit);
                             }
                             done = true;
                         }
                     }
-                    if (!done) hidden_chunk<W, CH, PER_TOKEN, ROT, EPI_SINE_WIDE, DUMP, GABOR>(cbase, ch * CH, s_x, v, dY, p.gabor_c);
+                    if (!done) hidden_chunk<W, C::HC, PER_TOKEN, ROT, EPI_SINE_WIDE, DUMP, GABOR, false, C::DUP>(cbase, ch * CH + chalf, s_x, v, dY, p.gabor_c);
                 }
-                tmem_st<CH>(c.taddr + ch * CH, v);
+                tmem_st<C::HC>(c.taddr + ch * CH, v);
             }
             if constexpr (DUMP) dC = (valid && p.d.codes[l]) ? p.d.codes[l] + tok * W : nullptr;
             if constexpr (CALIB) {
@@ -1028,7 +1074,7 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
                 // write instead of 128 x d_L four-byte ones.  The slot's 128 sub-0 threads meet on an
                 // mbarrier (bounded wait, like every other) before and after filling the buffer; its
                 // first thread issues the store.
-                const bool by_bulk = !AHEAD && !C::BULK_XY && p.bulk_out && (tile + 1) * kTile <= p.n;
+                const bool by_bulk = !AHEAD && !C::BULK_XY && p.bulk_out && (tile + 1) * C::TOK <= p.n;
                 const uint32_t ot = smem_base + sm.out_tile + (uint32_t)(slot * kTile * 16);
                 if (by_bulk) {
                     if (c.row == 0) ptx::bulk_wait_read(); // the previous tile's store has read the buffer
@@ -1048,14 +1094,14 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
                         }
                     }
                 }
-                if (valid) {
+                if (valid && (!C::DUP || lane < 16)) {
 #pragma unroll
                     for (int m = 0; m < 4; ++m) {
                         if (m < p.d_L) {
                             float c_hi = __ldg(ly.cA + m), c_lo = 0.f;
                             if (PER_TOKEN) c_hi = __fmul_rn(c_hi, s_x);
                             const float yv = epilogue(EPI_LINEAR, (float)(int)u[m], c_hi, c_lo, __ldg(ly.cB + m));
-                            if (by_bulk) asm volatile("st.shared.f32 [%0], %1;" ::"r"(ot + (uint32_t)((c.row * p.d_L + m) * 4)), "f"(yv) : "memory");
+                            if (by_bulk) asm volatile("st.shared.f32 [%0], %1;" ::"r"(ot + (uint32_t)((trow * p.d_L + m) * 4)), "f"(yv) : "memory");
                             else p.out[tok * p.d_L + m] = yv;
                         }
                     }
@@ -1065,7 +1111,7 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
                     ptx::mbar_arrive(smem_base + sm.out_sync + 8 * slot);
                     if (!wait_bar_warp<PER_TOKEN>(smem_base + sm.out_sync + 8 * slot, out_parity, abort_flag, p.status)) return;
                     out_parity ^= 1;
-                    if (c.row == 0) ptx::bulk_s2g(p.out + tile * kTile * p.d_L, ot, (uint32_t)(kTile * p.d_L * 4));
+                    if (c.row == 0) ptx::bulk_s2g(p.out + tile * C::TOK * p.d_L, ot, (uint32_t)(C::TOK * p.d_L * 4));
                 }
             }
             ptx::tc_fence_before();
@@ -1239,10 +1285,10 @@ __device__ void xy_role(const FusedParams &p, const SmemMap &sm, uint32_t smem_b
         if (tile_index<SPREAD>(r, 0, C::SLOTS) >= p.n_tiles) break;
         for (int s = 0; s < C::SLOTS && ok; ++s) {
             const long long tile = tile_index<SPREAD>(r, s, C::SLOTS);
-            if (tile >= p.n_tiles || (tile + 1) * kTile > p.n) continue; // none, or ragged: the threads load it themselves
+            if (tile >= p.n_tiles || (tile + 1) * C::TOK > p.n) continue; // none, or ragged: the threads load it themselves
             if (k[s] > 0 && !wait_bar<0, kHintNs>(smem_base + sm.xy_empty + 8 * s, (k[s] - 1) & 1u, abort_flag, p.status)) { ok = false; break; }
-            ptx::mbar_expect_tx(smem_base + sm.xy_full + 8 * s, kTile * 8);
-            ptx::bulk_g2s(smem_base + sm.xy + (uint32_t)(s * kTile * 8), p.coords + tile * kTile * 2, kTile * 8, smem_base + sm.xy_full + 8 * s);
+            ptx::mbar_expect_tx(smem_base + sm.xy_full + 8 * s, C::TOK * 8);
+            ptx::bulk_g2s(smem_base + sm.xy + (uint32_t)(s * kTile * 8), p.coords + tile * C::TOK * 2, C::TOK * 8, smem_base + sm.xy_full + 8 * s);
             ++k[s];
         }
     }
@@ -1255,10 +1301,10 @@ __device__ void xy_role(const FusedParams &p, const SmemMap &sm, uint32_t smem_b
 }
 
 template <int W, bool PER_TOKEN, bool ROT, bool SPREAD, bool AHEAD, bool DUMP = false, bool BOTH = false, bool CALIB = false,
-          bool GABOR = false, bool MIXED = false, bool NARROW = false>
+          bool GABOR = false, bool MIXED = false, bool NARROW = false, bool DUP = false>
 __global__ void __launch_bounds__(fused_threads(W, BOTH, GABOR), 1) fused_kernel(const __grid_constant__ ParamsOf<DUMP, CALIB> p)
 {
-    using C = Cfg<W, NARROW>;
+    using C = Cfg<W, NARROW, DUP>;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = ptx::smem_u32(smem_raw);
     const uint32_t smem_base = (raw + 1023u) & ~1023u;
@@ -1402,6 +1448,20 @@ template <int W> fused_fn pick_narrow_width(bool per_token, bool rot, bool both,
     else if (rot) return per_token ? fused_kernel<W, true, true, SP, false, false, false, false, false, false, N> : fused_kernel<W, false, true, SP, false, false, false, false, false, false, N>;
     else return per_token ? fused_kernel<W, true, false, SP, false, false, false, false, false, false, N> : fused_kernel<W, false, false, SP, false, false, false, false, false, false, N>;
 }
+// At most one tile of 64 tokens per SM.
+template <int W> fused_fn pick_dup_width(bool per_token, bool rot, bool both, bool gabor, bool mixed)
+{
+    constexpr bool N = W == 256;
+    if (gabor) {
+        if (both) return per_token ? fused_kernel<W, true, true, false, false, false, true, false, true, false, N, true> : fused_kernel<W, false, true, false, false, false, true, false, true, false, N, true>;
+        if (rot) return per_token ? fused_kernel<W, true, true, false, false, false, false, false, true, false, N, true> : fused_kernel<W, false, true, false, false, false, false, false, true, false, N, true>;
+        return per_token ? fused_kernel<W, true, false, false, false, false, false, false, true, false, N, true> : fused_kernel<W, false, false, false, false, false, false, false, true, false, N, true>;
+    }
+    if (both) return per_token ? fused_kernel<W, true, true, false, false, false, true, false, false, false, N, true> : fused_kernel<W, false, true, false, false, false, true, false, false, false, N, true>;
+    if (mixed) return rot ? fused_kernel<W, true, true, false, false, false, false, false, false, true, N, true> : fused_kernel<W, true, false, false, false, false, false, false, false, true, N, true>;
+    if (rot) return per_token ? fused_kernel<W, true, true, false, false, false, false, false, false, false, N, true> : fused_kernel<W, false, true, false, false, false, false, false, false, false, N, true>;
+    return per_token ? fused_kernel<W, true, false, false, false, false, false, false, false, false, N, true> : fused_kernel<W, false, false, false, false, false, false, false, false, false, N, true>;
+}
 typedef void (*fused_dump_fn)(const FusedParamsDump);
 // The observing instantiation of a width: the tile mapping and coordinate fetch of the large
 // device-memory launches (not spread; fetched ahead where the width has that variant).
@@ -1475,6 +1535,10 @@ fused_dump_fn fused_pick_dump_64(bool per_token, bool rot);
 fused_dump_fn fused_pick_dump_128(bool per_token, bool rot);
 fused_dump_fn fused_pick_dump_256(bool per_token, bool rot);
 fused_dump_fn fused_pick_dump_512(bool per_token, bool rot);
+fused_fn fused_pick_dup_64(bool per_token, bool rot, bool both, bool gabor, bool mixed);
+fused_fn fused_pick_dup_128(bool per_token, bool rot, bool both, bool gabor, bool mixed);
+fused_fn fused_pick_dup_256(bool per_token, bool rot, bool both, bool gabor, bool mixed);
+fused_fn fused_pick_dup_512(bool per_token, bool rot, bool both, bool gabor, bool mixed);
 fused_fn fused_pick_narrow_64(bool per_token, bool rot, bool both, bool gabor, bool mixed);
 fused_fn fused_pick_narrow_128(bool per_token, bool rot, bool both, bool gabor, bool mixed);
 fused_fn fused_pick_narrow_256(bool per_token, bool rot, bool both, bool gabor, bool mixed);

@@ -8,6 +8,7 @@ fused_fn fused_pick_512(bool per_token, bool rot, bool spread, bool ahead) { ret
 fused_dump_fn fused_pick_dump_512(bool per_token, bool rot) { return pick_dump_width<512, false>(per_token, rot); }
 fused_fn fused_pick_both_512(bool per_token) { return pick_both_width<512>(per_token); }
 fused_dump_fn fused_pick_both_dump_512(bool per_token) { return pick_both_dump_width<512>(per_token); }
+fused_fn fused_pick_dup_512(bool per_token, bool rot, bool both, bool gabor, bool mixed) { return pick_dup_width<512>(per_token, rot, both, gabor, mixed); }
 fused_calib_fn fused_pick_calib_512(bool rot, bool gabor, bool both) { return pick_calib_width<512>(rot, gabor, both); }
 fused_fn fused_pick_mixed_512(bool rot, bool ahead) { return pick_mixed_width<512, false>(rot, ahead); }
 fused_dump_fn fused_pick_mixed_dump_512(bool rot) { return pick_mixed_dump_width<512, false>(rot); }

@@ -1,5 +1,5 @@
-"""Launches of at most one tile per SM take kernels of their own (all epilogue warps on one tile): on
-either side of that border and at ragged ends dhq_forward must return the bits of the observed fused
+"""Launches of at most one tile per SM take kernels of their own (all epilogue warps on one tile; up to 64
+tokens per SM tiles of 64): on either side of these borders and at ragged ends dhq_forward must return the bits of the observed fused
 kernel, whose per-layer values the other tests compare with the definition."""
 import numpy as np
 import pytest
@@ -18,7 +18,7 @@ KINDS = [dict(), dict(w_gran=1, a_gran=1), dict(rotation=2), dict(rotation=2, a_
 
 
 @pytest.mark.parametrize("kind", range(len(KINDS)))
-@pytest.mark.parametrize("width", [128, 256])
+@pytest.mark.parametrize("width", [64, 128, 256, 512])
 def test_small_launches_return_the_observed_kernels_bits(width, kind):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     n_linear, d_out = (4, 3) if kind % 2 else (8, 2)   # resident and streamed weights at width 256
@@ -30,7 +30,7 @@ def test_small_launches_return_the_observed_kernels_bits(width, kind):
         dhq.dhq_calibrate(h, grid)
         want = torch.empty((grid.shape[0], d_out), device="cuda")
         dhq.dhq_forward_fused_debug(h, grid, want)
-        for n in (1, 31, 128, 129, 1000, (sms - 1) * 128 + 1, sms * 128, sms * 128 + 1):
+        for n in (1, 31, 64, 65, 129, 1000, sms * 64 - 63, sms * 64, sms * 64 + 1, (sms - 1) * 128 + 1, sms * 128, sms * 128 + 1):
             got = torch.full((n, d_out), float("nan"), device="cuda")
             dhq.dhq_forward(h, grid[:n], got)
             ch, oh = grid[:n].cpu().pin_memory(), torch.zeros((n, d_out)).pin_memory()
