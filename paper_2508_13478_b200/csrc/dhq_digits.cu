@@ -20,12 +20,12 @@
 // of the next layer's input can run through it (stages 1, 2, 4 inside a block, 8 .. W/8 in a thread's
 // chunk, W/4 and W/2 across chunks).  The weights stream from L2 in pieces of 16 KB.
 //
-// What bounds it: the phase of an activation, 24 fp32 operations because it is carried as if in fp64
-// (digit_phase; with the 8 of a plain compensated phase the same launch takes 0.71 ms), beside the
-// butterflies: about 45 issue slots per element against 32 x 51 cycles of MMAs per block of 64 outputs.
-// A block's sums are released as soon as they are in registers, so that the next block's MMAs run
-// beside its phases.  Measured: 2 -> 256 x 5 -> 3, per-channel / per-token, 262,144 coordinates 9.79 -> 0.84 ms
-// (one dp4a pass and an fp64 butterfly per layer before).
+// What bounds it: issue slots of the epilogue, about 35 per element (13 of them the phase, carried as if in
+// fp64: digit_phase), beside 32 x 51 cycles of MMAs per block of 64 outputs.  A block's sums are released as
+// soon as they are in registers, so that the next block's MMAs run beside its phases; the first block's MMAs
+// and the stages across chunks are exposed (one tile fills tensor memory).  Measured: 2 -> 256 x 5 -> 3,
+// per-channel / per-token, 262,144 coordinates 9.79 -> 0.74 ms (one dp4a pass and an fp64 butterfly per layer
+// before).
 #include "dhq_fused.cuh"
 
 namespace dhq {
