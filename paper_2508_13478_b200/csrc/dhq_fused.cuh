@@ -856,6 +856,11 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
         const unsigned long long t0 = ptx::globaltimer(), delay = (3500ull * W * W) / (256 * 256);
         while (ptx::globaltimer() - t0 < delay) __nanosleep(64);
     }
+    // LATE: no coordinate fetch of its own (host buffers, wavelet, two-sided): the next tile's coordinates are
+    // loaded before the last layer's wait, early enough for part of their latency and late enough not to hold
+    // registers during the layers.
+    constexpr bool LATE = !AHEAD && !C::BULK_XY && !CALIB && !DUMP && C::SLOTS == 2;
+    [[maybe_unused]] float2 xy_next = make_float2(0.f, 0.f);
     for (long long r = 0;; ++r) {
         const long long tile = tile_index<SPREAD>(r, slot, C::SLOTS);
         if (tile >= p.n_tiles) break;
@@ -882,7 +887,9 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
                 x = xy.x; y = xy.y;
             }
         } else
-        if (!AHEAD || r == 0) {
+        if (LATE && r > 0) {
+            x = xy_next.x; y = xy_next.y;
+        } else if (!AHEAD || r == 0) {
             if (valid) {
                 float2 xy = __ldg(reinterpret_cast<const float2 *>(p.coords) + tok);
                 x = xy.x; y = xy.y;
@@ -1057,6 +1064,10 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
         }
         if constexpr (!CALIB) {
             const FusedLayer &ly = p.layer[p.L - 1];
+            if constexpr (LATE) {
+                const long long tok_next = tile_index<SPREAD>(r + 1, slot, C::SLOTS) * C::TOK + trow;
+                xy_next = tok_next < p.n ? __ldg(reinterpret_cast<const float2 *>(p.coords) + tok_next) : make_float2(0.f, 0.f);
+            }
             if (!wait_bar_warp<PER_TOKEN>(bar_last, last_parity, abort_flag, p.status)) return;
             last_parity ^= 1;
             ptx::tc_fence_after();
