@@ -20,13 +20,13 @@
 // largest layer error against fp64 4.3e-6 (the first layer's; 5.6e-6 with fp32 multiply-adds).
 //
 // What bounds it.  The digits of a tile of 128 activations stay in shared memory for a whole layer
-// (192 KB at width 512), the weights stream past them from L2.  An MMA takes 67 cycles at N = 128
-// and 51 at N = 64 (operands leave shared memory at 128 B per cycle), hence blocks of 128 outputs
+// (192 KB at width 512; below that from layer to layer), the weights stream past them from L2.  An MMA takes
+// 67 cycles at N = 128 and 51 at N = 64 (operands leave shared memory at 128 B per cycle), hence blocks of 128 outputs
 // and a single set of 3 x 128 accumulator columns: the epilogue releases it as soon as the phases
 // are in registers and computes sines and digits beside the next block's MMAs.  At width 512 the
 // remaining 32 KB of shared memory keep too few weight bytes in flight (105 cycles per MMA); at
 // width 256 the sines and digits of the block behind take as long as the MMAs.
-// Measured: 2 -> 256 x 3 -> 3, fp32, 65,536 coordinates 940 -> 92 us; 2 -> 512 x 4 -> 3, 8-bit
+// Measured: 2 -> 256 x 3 -> 3, fp32, 65,536 coordinates 940 -> 67 us (88 with the digits through L2); 2 -> 512 x 4 -> 3, 8-bit
 // weights, 262,144 coordinates 17.2 -> 1.11 ms (one fp32 CUDA-core pass per layer before; 1.21 ms without the
 // register split of the warpgroups).
 #include "dhq_fused.cuh"
@@ -57,6 +57,15 @@ struct FloatParams {
     float *dX[kMaxLayers], *dY[kMaxLayers];  // dumps (DUMP instantiation)
 };
 
+// Below width 512 the activations' digits never leave shared memory.  The operand area is cut into parts of KC
+// features (the outputs of one block), one more than a layer has: part k of the t-th tensor-core layer of the
+// CTA lies in buffer (t NB + k) mod (NB + 1).  Block 0's outputs go to the buffer that this layer does not
+// read, block 1's (the last) to the one of this layer's part 0, whose MMAs have all completed with that block's
+// sums.  So the next layer's MMAs begin on part 0 while block 1's outputs are still being formed.  At width 512 one layer's
+// digits fill 192 KB and go through L2 instead.
+__host__ __device__ constexpr bool float_x_in_smem(int W) { return W < 512; }
+__host__ __device__ constexpr uint32_t float_part_bytes(int W) { return 3u * kTile * (W < 128 ? W : 128); }
+
 // At width 512 the activations leave no room for the epilogue constants: they are read through L1.
 __host__ __device__ constexpr bool float_consts_in_smem(int W) { return W < 512; }
 
@@ -67,7 +76,7 @@ __host__ __device__ inline FloatMap float_map(int W, int n_stages, int L)
 {
     FloatMap m;
     uint32_t off = 0;
-    m.a = off; off += 3u * kTile * W;
+    m.a = off; off += float_x_in_smem(W) ? (uint32_t)(W / float_block(W) + 1) * float_part_bytes(W) : 3u * kTile * W;
     m.ring = off; off += (uint32_t)n_stages * float_block(W) * float_kc(W);
     m.consts = off; off += float_consts_in_smem(W) ? (uint32_t)(4 + 3 * (L - 2)) * W * 4 : 0; // first layer, then c0 | c0_lo | cb per hidden layer
     m.w_full = off; off += 8 * kFMaxStages;
@@ -123,6 +132,8 @@ __device__ void float_epilogue(const FloatParams &p, const FloatMap &sm, uint32_
                                volatile int *abort_flag)
 {
     constexpr int FB = float_block(W), NB = W / FB, GPB = FB / 64; // GPB groups of 16 outputs per thread and block
+    constexpr bool XS = float_x_in_smem(W);
+    uint32_t tlayer = 0, x_addr = 0; // tensor-core layers so far; where the block's digits go (XS)
     const int quad = warp & 3, sub = warp >> 2, row = quad * 32 + lane;
     const uint32_t taddr = tmem + ((uint32_t)(quad * 32) << 16);
     uint8_t *xrow = p.x + (size_t)blockIdx.x * (3 * kTile * W) + row * 16;
@@ -148,8 +159,12 @@ __device__ void float_epilogue(const FloatParams &p, const FloatMap &sm, uint32_
                 digits4(v, j, d);
             }
 #pragma unroll
-            for (int i = 0; i < 3; ++i)
-                *reinterpret_cast<uint4 *>(xrow + i * (kTile * W) + (k0 / 16) * (kTile * 16)) = make_uint4(d.w[i][0], d.w[i][1], d.w[i][2], d.w[i][3]);
+            for (int i = 0; i < 3; ++i) {
+                if constexpr (XS)
+                    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(x_addr + (uint32_t)(i * kTile * FB + (k0 % FB) * kTile + row * 16)),
+                                 "r"(d.w[i][0]), "r"(d.w[i][1]), "r"(d.w[i][2]), "r"(d.w[i][3]) : "memory");
+                else *reinterpret_cast<uint4 *>(xrow + i * (kTile * W) + (k0 / 16) * (kTile * 16)) = make_uint4(d.w[i][0], d.w[i][1], d.w[i][2], d.w[i][3]);
+            }
         } else {
             // last layer (at most four outputs): fp32 multiply-adds here, this thread's share of the K products
 #pragma unroll
@@ -169,6 +184,17 @@ __device__ void float_epilogue(const FloatParams &p, const FloatMap &sm, uint32_
         const long long tok = tile * kTile + row;
         x = yc = 0.f;
         if (tile < p.n_tiles && tok < p.n) { x = __ldg(p.coords + 2 * tok); yc = __ldg(p.coords + 2 * tok + 1); }
+    };
+    // block b of the outputs is about to be formed / is complete: the inputs of tensor-core layer t
+    auto begin_part = [&](uint32_t t, int b) {
+        if constexpr (XS) x_addr = base + sm.a + (t * NB + b) % (NB + 1) * float_part_bytes(W);
+    };
+    auto end_part = [&](int b) {
+        if constexpr (XS) {
+            ptx::fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(base + sm.a_full + 8 * b);
+        }
     };
     // layer 1, two products per output: block b of a tile
     auto first_layer = [&](int b, float x, float yc, long long tok, bool valid) {
@@ -202,19 +228,27 @@ __device__ void float_epilogue(const FloatParams &p, const FloatMap &sm, uint32_
         // (with hidden layers, the first layer of every tile but the first was done beside the tile before)
         if (tile == blockIdx.x || p.L == 2) {
 #pragma unroll 1
-            for (int b = 0; b < NB; ++b) first_layer(b, x, yc, tok, valid);
+            for (int b = 0; b < NB; ++b) {
+                begin_part(tlayer, b);
+                first_layer(b, x, yc, tok, valid);
+                if (p.L > 2) end_part(b);
+            }
         }
         coords_of(tile + gridDim.x, x, yc);
         for (int l = 2; l < p.L; ++l) {
-            // the activations in device memory become visible to the bulk copies of this CTA
-            asm volatile("fence.proxy.async;" ::: "memory");
-            ptx::mbar_arrive(base + sm.x_ready);
+            ++tlayer;
+            if constexpr (!XS) {
+                // the activations in device memory become visible to the bulk copies of this CTA
+                asm volatile("fence.proxy.async;" ::: "memory");
+                ptx::mbar_arrive(base + sm.x_ready);
+            }
 #pragma unroll 1
             for (int b = 0; b < NB; ++b, ++use) {
                 const int k0 = b * FB + sub * GPB * 16;
                 const uint32_t t = taddr + sub * GPB * 16;
                 if (!wait_bar_warp<true>(base + sm.acc_full, use & 1, abort_flag, p.status)) return;
                 ptx::tc_fence_after();
+                begin_part(tlayer, b);
                 f32x2 r[GPB * 8];
 #pragma unroll
                 for (int g = 0; g < GPB; ++g) {
@@ -254,9 +288,10 @@ __device__ void float_epilogue(const FloatParams &p, const FloatMap &sm, uint32_
                     emit(l, k0 + g * 16, y, tok, valid);
                 }
                 // Beside the last tensor-core layer, which writes no activations: the first layer of the CTA's next
-                // tile, whose digits go where this tile's were (they are all in shared memory by now).
+                // tile, whose digits go where this tile's were (at width 512 those are all in shared memory by now).
                 if (l == p.L - 1 && tile + gridDim.x < p.n_tiles)
                     first_layer(b, x, yc, tok + gridDim.x * (long long)kTile, (tok + gridDim.x * (long long)kTile) < p.n);
+                if (l < p.L - 1 || tile + gridDim.x < p.n_tiles) end_part(b);
             }
         }
         // last layer: the four threads of a row exchange their partial sums through tensor memory
@@ -308,6 +343,8 @@ __device__ void float_mma(const FloatParams &p, const FloatMap &sm, uint32_t bas
     ptx::wait_for_previous_kernels(); // before the first bounded wait
     const uint32_t idesc = ptx::idesc_i8(kTile, FB);
     constexpr uint32_t kDescHi = (128u >> 4) | (1u << 14);
+    constexpr bool XS = float_x_in_smem(W);
+    constexpr int DIGIT = kTile * (XS ? FB : W); // bytes between the digits of an activation
     const uint32_t a0 = ((base + sm.a) >> 4) | ((kTile * 16u >> 4) << 16), b0 = ((base + sm.ring) >> 4) | ((FB * 16u >> 4) << 16);
     uint32_t use = 0, layers = 0;
     int stage = 0;
@@ -320,6 +357,12 @@ __device__ void float_mma(const FloatParams &p, const FloatMap &sm, uint32_t bas
                 ptx::tc_fence_after();
                 uint32_t ak = a0;
                 for (int kc = 0; kc < NKC; ++kc, ak += (KC / 16) * (kTile * 16) >> 4) {
+                    if constexpr (XS) {
+                        static_assert(KC == FB && NB <= 2, "a part is a weight piece's k range; see float_x_in_smem");
+                        ak = a0 + (((layers * NB + kc) % (NB + 1) * float_part_bytes(W)) >> 4);
+                        if (b == 0) ok = wait_bar<0, kHintNs>(base + sm.a_full + 8 * kc, layers & 1, abort_flag, p.status);
+                        if (b == 0 && ok) ptx::tc_fence_after();
+                    } else
                     for (int c = 0; b == 0 && c < KC / 64 && ok; ++c)
                         ok = wait_bar<0, kHintNs>(base + sm.a_full + 8 * (kc * (KC / 64) + c), layers & 1, abort_flag, p.status);
                     if (!ok) break;
@@ -331,7 +374,7 @@ __device__ void float_mma(const FloatParams &p, const FloatMap &sm, uint32_t bas
                         for (int i = 0; i + j < 3; ++i) {
 #pragma unroll
                             for (int ks = 0; ks < KC / 32; ++ks)
-                                ptx::mma_i8_words(tmem + (uint32_t)(i + j) * FB, ak + ((i * kTile * W + ks * 2 * kTile * 16) >> 4), bk + (ks * 2 * FB * 16 >> 4),
+                                ptx::mma_i8_words(tmem + (uint32_t)(i + j) * FB, ak + ((i * DIGIT + ks * 2 * kTile * 16) >> 4), bk + (ks * 2 * FB * 16 >> 4),
                                                   kDescHi, idesc, (j > 0 || ks > 0) ? 1u : (uint32_t)kc);
                         }
                         ptx::mma_commit(base + sm.w_empty + 8 * stage);
@@ -430,7 +473,7 @@ __global__ void __launch_bounds__(kFThreads, 1) float_kernel(const __grid_consta
             ptx::mbar_init(base + sm.w_full + 8 * i, 1);
             ptx::mbar_init(base + sm.w_empty + 8 * i, 1);
         }
-        for (int i = 0; i < 8; ++i) ptx::mbar_init(base + sm.a_full + 8 * i, 1);
+        for (int i = 0; i < 8; ++i) ptx::mbar_init(base + sm.a_full + 8 * i, float_x_in_smem(W) ? kEpiWarps : 1);
         ptx::mbar_init(base + sm.x_ready, kEpiWarps * 32);
         ptx::mbar_init(base + sm.acc_full, 1);
         ptx::mbar_init(base + sm.acc_empty, kEpiWarps * 32);
@@ -464,7 +507,7 @@ __global__ void __launch_bounds__(kFThreads, 1) float_kernel(const __grid_consta
     else if (lane == 0) {
         if (warp == kMmaWarp) float_mma<W, WL>(p, sm, base, tmem, abort_flag);
         else if (warp < kLoadWarp + kFLoaders) float_load_weights<W, WL>(p, sm, base, warp - kLoadWarp, abort_flag);
-        else float_load_x<W>(p, sm, base, abort_flag);
+        else if constexpr (!float_x_in_smem(W)) float_load_x<W>(p, sm, base, abort_flag);
     }
     ptx::tc_fence_before();
     __syncthreads();
@@ -563,7 +606,7 @@ size_t float_scratch_bytes(const dhq_handle_s *h)
 {
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess) sms = 148;
-    return (size_t)sms * 3 * kTile * h->w;
+    return float_x_in_smem(h->w) ? 0 : (size_t)sms * 3 * kTile * h->w;
 }
 
 struct FloatState {
