@@ -134,8 +134,8 @@ __device__ __forceinline__ float sine_fixed(int qs, int qd, uint32_t P, uint32_t
 // c = c_hi + c_lo and the bias modulo one turn cb + cb_lo (cb a multiple of 2^-17).  The result is
 // 2 pi (t - nearest integer) rounded to fp32 as if t had been known in fp64.  Adding 96 = 1.5 * 2^6 cuts the
 // product at 2^-17 (|c D0| < 32; the grid moves by a factor of two beyond), so that the parts above, added to cb
-// and freed of whole turns, stay exact, and so does their product with 6.28125, the first eight bits of 2 pi; all
-// parts below are gathered in `lo` (error 0.5 ulp + 2^-35 turns).  That care is for the quantizer that follows,
+// and freed of whole turns, stay exact until the last fma; all parts below are gathered in `lo` (error 0.5 ulp +
+// 2^-42 turns).  That care is for the quantizer that follows,
 // not for the 1e-5 of the output: activations that agree with the fp64 evaluation bit for bit are quantized to the
 // same codes.  (13 operations; carrying the rounding errors of fp32 sums along took 23, and the kernel of
 // dhq_digits.cu 0.83 ms for 262,144 coordinates in place of 0.74.)
@@ -146,12 +146,12 @@ __device__ __forceinline__ void digit_sums(int D0, int D1, int D2, int D3, float
 }
 __device__ __forceinline__ float digit_phase(float f0, float f1, float c_hi, float c_lo, float cb, float cb_lo)
 {
-    const float two_pi = 6.2831853071795865f, two_pi_a = 6.28125f, two_pi_b = 0.0019353071795865f;
+    const float two_pi = 6.2831853071795865f, two_pi_lo = -1.7484555e-07f; // fl32(2 pi) and what it lacks
     const float q = __fsub_rn(__fmaf_rn(f0, c_hi, 96.0f), 96.0f);
     const float s = __fadd_rn(q, cb);
     const float t = __fsub_rn(s, __fsub_rn(__fadd_rn(s, 12582912.0f), 12582912.0f));
     const float lo = __fadd_rn(__fmaf_rn(f0, c_hi, -q), __fmaf_rn(f0, c_lo, __fmaf_rn(f1, c_hi, cb_lo)));
-    return __fmaf_rn(t, two_pi_a, __fmaf_rn(lo, two_pi, __fmul_rn(t, two_pi_b)));
+    return __fmaf_rn(t, two_pi, __fmaf_rn(lo, two_pi, __fmul_rn(t, two_pi_lo)));
 }
 // The wavelet's envelope exp(-(s0 z)^2) from the same numbers: cn is the part of the bias that cb lacks, gc = 2 pi s0 / omega0.
 __device__ __forceinline__ float digit_envelope(float f0, float f1, float c_hi, float cb, float cn, float gc)
