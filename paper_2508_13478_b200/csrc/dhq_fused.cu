@@ -209,7 +209,7 @@ bool allow_smem(const void *fn, int device, int bytes, int min_regs)
 // that waits holds no SM that the earlier one needs: it is not started before all blocks of the earlier
 // launch are.  Back to back, the binding's shorter call included: 4,096 coordinates at width 64 9.9 -> 5.9 us, 1,000 at
 // width 256 18.5 -> 14.9 us, 65,536 at width 256 45.0 -> 41.4 us.
-cudaError_t launch_after(dhq_handle_s *h, const void *fn, int grid, int threads, size_t smem, cudaStream_t st, void *params)
+static cudaError_t launch_early(const void *fn, int grid, int threads, size_t smem, cudaStream_t st, void *params, bool early)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
@@ -220,11 +220,16 @@ cudaError_t launch_after(dhq_handle_s *h, const void *fn, int grid, int threads,
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
-    cfg.numAttrs = h->settled ? 1 : 0;
-    h->settled = true;
+    cfg.numAttrs = early ? 1 : 0;
     void *args[1] = {params};
     const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
     return e != cudaSuccess ? e : cudaGetLastError();
+}
+cudaError_t launch_after(dhq_handle_s *h, const void *fn, int grid, int threads, size_t smem, cudaStream_t st, void *params)
+{
+    const bool early = h->settled;
+    h->settled = true;
+    return launch_early(fn, grid, threads, smem, st, params, early);
 }
 
 dhq_status_t fused_create(dhq_handle_s *h)
@@ -288,7 +293,8 @@ dhq_status_t fused_create(dhq_handle_s *h)
     if (!allow_smem((const void *)pick_dup_for(h, p.per_token), dev, max_optin, min_regs)) return DHQ_ERR_CUDA;
     if (narrow && !allow_smem((const void *)narrow, dev, max_optin, min_regs)) return DHQ_ERR_CUDA;
     if (!p.per_token && !allow_smem((const void *)pick_calib_kernel(h->w, h->cfg.rotation == DHQ_ROT_INPUT, gabor, both), dev, max_optin, min_regs)) return DHQ_ERR_CUDA;
-    if (!allow_smem((const void *)pick_dump_for(h, p.per_token), dev, max_optin, min_regs)) return DHQ_ERR_CUDA;
+    fs->max_smem = max_optin;
+    fs->min_regs = min_regs; // (the observing kernel is loaded by its first call: that takes milliseconds)
     return DHQ_OK;
 }
 
@@ -385,13 +391,12 @@ dhq_status_t fused_calibrate_layer(dhq_handle_s *h, int l, const float *coords, 
     p.sine = l < h->L;
     p.omega0 = (double)h->cfg.omega0;
     p.dev = h->layer[l - 1];
-    const int slots = (h->w == 512) ? 1 : 2;
     fused_calib_fn fn = pick_calib_kernel(h->w, h->cfg.rotation == DHQ_ROT_INPUT, h->gabor_s0 > 0.0, h->cfg.rotation == DHQ_ROT_BOTH);
-    const long long ctas = (p.n_tiles + slots - 1) / slots;
-    int grid = (int)(ctas < fs->sm_count ? ctas : fs->sm_count);
-    fn<<<grid, threads_for(h), fs->smem_bytes, st>>>(p);
+    const int grid = (int)(p.n_tiles < fs->sm_count ? p.n_tiles : fs->sm_count);
+    // set up beside the pass before it; reads nothing of that pass before wait_for_previous_kernels
+    const cudaError_t e = launch_early((const void *)fn, grid, threads_for(h), fs->smem_bytes, st, &p, true);
     h->launches++;
-    return cudaGetLastError() == cudaSuccess ? DHQ_OK : DHQ_ERR_CUDA;
+    return e == cudaSuccess ? DHQ_OK : DHQ_ERR_CUDA;
 }
 
 // The same forward by the observing instantiation of the kernel: every per-layer value the
@@ -406,6 +411,7 @@ dhq_status_t fused_forward_dump(dhq_handle_s *h, const float *coords, int64_t n,
     p.d = d;
     const int slots = (h->w == 512) ? 1 : 2;
     fused_dump_fn fn = pick_dump_for(h, p.per_token);
+    if (!allow_smem((const void *)fn, h->device, fs->max_smem, fs->min_regs)) return DHQ_ERR_CUDA;
     const long long ctas = (p.n_tiles + slots - 1) / slots;
     int grid = (int)(ctas < fs->sm_count ? ctas : fs->sm_count);
     fn<<<grid, threads_for(h), fs->smem_bytes, st>>>(p);

@@ -157,7 +157,7 @@ template <bool DUMP, bool CALIB = false> using ParamsOf = std::conditional_t<DUM
 struct FusedState {
     FusedParams p;
     size_t smem_bytes;
-    int sm_count;
+    int sm_count, max_smem, min_regs;
 };
 
 // Shared-memory map (byte offsets from a 1024-byte aligned base).
@@ -1358,6 +1358,7 @@ __global__ void __launch_bounds__(fused_threads(W, BOTH, GABOR), 1) fused_kernel
         ptx::tmem_alloc(smem_base + sm.tmem_holder, 512);
         ptx::tmem_relinquish();
     }
+    if constexpr (CALIB) ptx::wait_for_previous_kernels(); // the constants below come from the pass before this one
     // per-layer epilogue constants -> shared memory
     {
         uint32_t *dst = reinterpret_cast<uint32_t *>(smem_gen + sm.consts);
@@ -1505,13 +1506,13 @@ template <int W> fused_dump_fn pick_both_dump_width(bool per_token)
     return per_token ? fused_kernel<W, true, true, false, false, true, true> : fused_kernel<W, false, true, false, false, true, true>;
 }
 // Calibration kernels (per-tensor activation scales): the network up to the rotated input of layer
-// p.L, whose absmax they take.
+// p.L, whose absmax they take.  Spread: a small coordinate set takes as many SMs as it has tiles.
 typedef void (*fused_calib_fn)(const FusedParamsCalib);
 template <int W> fused_calib_fn pick_calib_width(bool rot, bool gabor, bool both)
 {
-    if (both) return gabor ? fused_kernel<W, false, true, false, false, false, true, true, true> : fused_kernel<W, false, true, false, false, false, true, true, false>;
-    if (gabor) return rot ? fused_kernel<W, false, true, false, false, false, false, true, true> : fused_kernel<W, false, false, false, false, false, false, true, true>;
-    return rot ? fused_kernel<W, false, true, false, false, false, false, true> : fused_kernel<W, false, false, false, false, false, false, true>;
+    if (both) return gabor ? fused_kernel<W, false, true, true, false, false, true, true, true> : fused_kernel<W, false, true, true, false, false, true, true, false>;
+    if (gabor) return rot ? fused_kernel<W, false, true, true, false, false, false, true, true> : fused_kernel<W, false, false, true, false, false, false, true, true>;
+    return rot ? fused_kernel<W, false, true, true, false, false, false, true> : fused_kernel<W, false, false, true, false, false, false, true>;
 }
 // The wavelet activation's kernels: not spread, coordinates not fetched ahead.
 template <int W> fused_fn pick_gabor_width(bool per_token, bool rot)
