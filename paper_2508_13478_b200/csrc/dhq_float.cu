@@ -35,7 +35,7 @@ namespace dhq {
 
 __host__ __device__ constexpr int float_block(int W) { return W < 128 ? W : 128; } // outputs per accumulator set, three times as many columns
 __host__ __device__ constexpr int float_kc(int W) { return W == 256 || W == 128 ? 128 : 64; }   // k per weight piece (4 to 16 KB)
-constexpr int kFPartCol = 3 * 128;           // first tensor-memory column of the last layer's partial sums
+constexpr int kFPartCol = 3 * 128;           // first tensor-memory column of the last layer's partial sums: two sets of 16 columns
 constexpr int kFLoaders = 2;                 // warps that copy weights, see float_load_weights
 constexpr int kFThreads = (18 + kFLoaders) * 32; // 16 epilogue warps, MMA, weight copies, activation copies
 constexpr int kFMaxStages = 16;
@@ -294,10 +294,14 @@ __device__ void float_epilogue(const FloatParams &p, const FloatMap &sm, uint32_
                 if (l < p.L - 1 || tile + gridDim.x < p.n_tiles) end_part(b);
             }
         }
-        // last layer: the four threads of a row exchange their partial sums through tensor memory
+        // last layer: the four threads of a row exchange their partial sums through tensor memory.  Tiles use two sets of
+        // columns in turn: a thread may write the next tile's sums while a slower one still reads this tile's (with three
+        // layers and one block of outputs nothing else orders the two), but to come back to this set it has to pass the
+        // next tile's barrier, where the reader arrives after its reads.
         {
+            const uint32_t part_col = taddr + kFPartCol + 16 * qpar;
             const uint32_t u[4] = {__float_as_uint(part[0]), __float_as_uint(part[1]), __float_as_uint(part[2]), __float_as_uint(part[3])};
-            ptx::tmem_st4(taddr + kFPartCol + 4 * sub, u);
+            ptx::tmem_st4(part_col + 4 * sub, u);
             ptx::tmem_wait_st();
             ptx::tc_fence_before();
             ptx::mbar_arrive(base + sm.quad_sync + 8 * quad);
@@ -306,7 +310,7 @@ __device__ void float_epilogue(const FloatParams &p, const FloatMap &sm, uint32_
             ptx::tc_fence_after();
             if (sub == 0) {
                 uint32_t v[16];
-                ptx::tmem_ld16(taddr + kFPartCol, v);
+                ptx::tmem_ld16(part_col, v);
                 ptx::tmem_wait_ld();
                 if (valid) {
 #pragma unroll
@@ -321,13 +325,6 @@ __device__ void float_epilogue(const FloatParams &p, const FloatMap &sm, uint32_
                     }
                 }
                 ptx::tc_fence_before();
-            }
-            // without a tensor-core layer nothing else keeps the next tile's partial sums from overtaking that read
-            if (p.L == 2) {
-                ptx::mbar_arrive(base + sm.quad_sync + 8 * quad);
-                if (!wait_bar_warp<true>(base + sm.quad_sync + 8 * quad, qpar, abort_flag, p.status)) return;
-                qpar ^= 1;
-                ptx::tc_fence_after();
             }
         }
     }

@@ -58,3 +58,26 @@ def test_fixed_point_layers(width, n_linear, d_out, n, w_bits, sparse):
             want = np.sin(30.0 * z) if l < n_linear else z
         got = Y[l - 1].cpu().numpy()[:, : want.shape[1]]
         assert np.abs(got - want).max() <= TOL_FLOAT, f"layer {l}"
+
+
+@pytest.mark.parametrize("width,n_linear", [(64, 3), (128, 3), (64, 2), (128, 4), (256, 3)])
+def test_tiles_of_one_block_do_not_disturb_each_other(width, n_linear):
+    # several tiles per block of the grid: the next tile's last-layer sums must not reach the columns of this tile's
+    # (the ordering differs with the number of layers and of output blocks); every tile alone gives the bits to expect
+    dims = (2,) + (width,) * (n_linear - 1) + (3,)
+    weights, biases = dhq_inputs.siren_init(dims, 30.0, 900 + width + n_linear)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = 128 * (3 * sms + 1) + 77
+    cd = to_dev(dhq_inputs.grid_coords(n // 240 + 1, 240)[:n])
+    h = dhq.dhq_prepare(dims, [to_dev(x) for x in weights], [to_dev(x) for x in biases], 30.0, 32, dhq.DHQ_BITS_FLOAT)
+    try:
+        want = torch.empty((n, 3), device="cuda")
+        for t in range(0, n, 128 * sms):   # one tile per block
+            dhq.dhq_forward(h, cd[t:t + 128 * sms], want[t:t + 128 * sms])
+        for _ in range(20):
+            got = torch.full((n, 3), float("nan"), device="cuda")
+            dhq.dhq_forward(h, cd, got)
+            assert torch.equal(got.view(torch.int32), want.view(torch.int32))
+        assert dhq.dhq_last_status(h) == 0
+    finally:
+        dhq.dhq_destroy(h)
