@@ -203,9 +203,9 @@ bool allow_smem(const void *fn, int device, int bytes, int min_regs)
     return true;
 }
 
-// A forward launch.  Once a launch has followed the preparation and calibration (so that they had
-// completed before it began), later ones use programmatic dependent launch: what the kernel does
-// before wait_for_previous_kernels touches only the handle's weights and constants.  A block of the later launch
+// A forward launch.  Once an ordinary launch has followed the preparation and calibration in a stream (so that
+// they had completed before it began), later ones in that stream use programmatic dependent launch: what the kernel
+// does before wait_for_previous_kernels touches only the handle's weights and constants.  A block of the later launch
 // that waits holds no SM that the earlier one needs: it is not started before all blocks of the earlier
 // launch are.  Back to back, the binding's shorter call included: 4,096 coordinates at width 64 9.9 -> 5.9 us, 1,000 at
 // width 256 18.5 -> 14.9 us, 65,536 at width 256 45.0 -> 41.4 us.
@@ -227,9 +227,19 @@ static cudaError_t launch_early(const void *fn, int grid, int threads, size_t sm
 }
 cudaError_t launch_after(dhq_handle_s *h, const void *fn, int grid, int threads, size_t smem, cudaStream_t st, void *params)
 {
-    const bool early = h->settled;
-    h->settled = true;
-    return launch_early(fn, grid, threads, smem, st, params, early);
+    const bool early = h->settled && st == h->settled_stream;
+    const cudaError_t e = launch_early(fn, grid, threads, smem, st, params, early);
+    if (!early && e == cudaSuccess && st != cudaStreamPerThread) {
+        // A launch that stream capture only recorded has followed nothing yet; neither has one in another stream
+        // than the next (the calibration passes let the launch behind them begin before they are done).
+        cudaStreamCaptureStatus capture;
+        if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) (void)cudaGetLastError();
+        else if (capture == cudaStreamCaptureStatusNone) {
+            h->settled = true;
+            h->settled_stream = st;
+        }
+    }
+    return e;
 }
 
 dhq_status_t fused_create(dhq_handle_s *h)

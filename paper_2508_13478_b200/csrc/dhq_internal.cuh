@@ -54,7 +54,8 @@ struct dhq_handle_s {
     int L = 0, w = 0, d_L = 0;
     int device = 0;
     bool calibrated = false;
-    bool settled = false;           // a forward has been enqueued since the weights or scales last changed
+    bool settled = false;           // since the weights or scales last changed a forward was launched the ordinary way ...
+    cudaStream_t settled_stream = nullptr; // ... in this stream (see launch_after)
     int calib_layers_done = 0;      // layers whose per-tensor activation scale is frozen (sharded calibration)
     dhq::LayerDev layer[dhq::kMaxLayers];
     void *block = nullptr;          // the device memory of everything below up to the layers' arrays
