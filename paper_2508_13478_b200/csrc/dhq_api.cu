@@ -66,8 +66,8 @@ void layer_arrays(LayerDev &d, ArrayRef (&t)[kLayerArrays])
 // 1.5 ms in cudaMalloc and cudaFree, and up to 28 ms on a device with a long allocation history.
 // Released blocks are kept for the next handle of the process, at most kPoolBlocks of them and
 // kPoolBytes together over all devices; what does not fit is freed, and dhq_release_cached_memory or a
-// failed allocation frees all.  dhq_destroy waits for the device before it releases the block, so a
-// block handed out again is not in use on any stream.
+// failed allocation frees all.  dhq_destroy waits for the handle's device before it releases the block (and
+// frees it if that wait fails), so a block handed out again is not in use on any stream.
 constexpr int kPoolBlocks = 8;
 constexpr size_t kPoolBytes = 128u << 20;
 struct PoolBlock { void *p; size_t bytes; int device; };
@@ -372,11 +372,16 @@ const char *dhq_status_string(dhq_status_t s)
 void dhq_destroy(dhq_handle_t h)
 {
     if (!h) return;
-    cudaDeviceSynchronize();
+    // the handle's own device, whichever is current: its kernels have to be done before the block is used again
+    int current = -1;
+    const bool elsewhere = h->device >= 0 && cudaGetDevice(&current) == cudaSuccess && current != h->device;
+    if (elsewhere) cudaSetDevice(h->device);
+    const bool idle = cudaDeviceSynchronize() == cudaSuccess;
     fused_destroy(h);
     float_destroy(h);
     digit_destroy(h);
-    pool_give(h->block, h->block_bytes, h->device);
+    if (idle) pool_give(h->block, h->block_bytes, h->device);
+    else cudaFree(h->block);
     cudaFree(h->scratch[0]); cudaFree(h->scratch[1]);
     cudaFree(h->stage_in); cudaFree(h->stage_out);
     if (h->copy_in) cudaStreamDestroy(h->copy_in);
@@ -387,6 +392,7 @@ void dhq_destroy(dhq_handle_t h)
         if (h->ev_in[i]) cudaEventDestroy(h->ev_in[i]);
         if (h->ev_k[i]) cudaEventDestroy(h->ev_k[i]);
     }
+    if (elsewhere) cudaSetDevice(current);
     delete h;
 }
 

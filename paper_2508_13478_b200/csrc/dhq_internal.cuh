@@ -52,7 +52,7 @@ struct dhq_handle_s {
     dhq_config_t cfg;
     int dims[dhq::kMaxLayers + 1];
     int L = 0, w = 0, d_L = 0;
-    int device = 0;
+    int device = -1;
     bool calibrated = false;
     bool settled = false;           // since the weights or scales last changed a forward was launched the ordinary way ...
     cudaStream_t settled_stream = nullptr; // ... in this stream (see launch_after)

@@ -1,0 +1,77 @@
+"""Host side of the library against a CUDA runtime without a device (fake_cudart.c), so that what needs a second
+GPU, a failing call or a capture in progress is looked at on the CPU.  Each test is a child process with the
+runtime preloaded."""
+import os
+import subprocess
+import sys
+import textwrap
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+PRELUDE = r"""
+import ctypes as C, sys
+F = C.CDLL(sys.argv[1]); D = C.CDLL(sys.argv[2])
+F.fake_log.restype = C.c_char_p
+vp = C.c_void_p
+class Cfg(C.Structure):
+    _fields_ = [("n_layers", C.c_int), ("dims", C.POINTER(C.c_int)), ("w_bits", C.c_int), ("a_bits", C.c_int), ("omega0", C.c_float),
+                ("w_gran", C.c_int), ("a_gran", C.c_int), ("rotation", C.c_int), ("activation", C.c_int), ("act_s0", C.c_float)]
+D.dhq_forward.argtypes = [vp, vp, C.c_int64, vp, vp]; D.dhq_calibrate.argtypes = [vp, vp, C.c_int64, vp]
+D.dhq_destroy.argtypes = [vp]; D.dhq_destroy.restype = None; D.dhq_release_cached_memory.restype = None
+mem = (C.c_float * 4096)()                      # stands for every buffer of the caller
+ptr = C.addressof(mem)
+def prepare(width=64, w_bits=8, a_bits=8, w_gran=0, a_gran=0, rotation=0, expect=0):
+    dims = (C.c_int * 5)(2, width, width, width, 3)
+    cfg = Cfg(4, dims, w_bits, a_bits, 30.0, w_gran, a_gran, rotation, 0, 0.0)
+    W = (vp * 4)(*[ptr] * 4); h = vp()
+    rc = D.dhq_prepare(C.byref(cfg), W, W, None, C.byref(h))
+    assert rc == expect, rc
+    return h
+def forward(h, stream=0, n=100, expect=0):
+    rc = D.dhq_forward(h, ptr, n, ptr, stream)
+    assert rc == expect, rc
+def calibrate(h, stream=0, n=100, expect=0):
+    rc = D.dhq_calibrate(h, ptr, n, stream)
+    assert rc == expect, rc
+def log():
+    lines = F.fake_log().decode().split(); F.fake_clear()
+    return [(w, int(d), int(a)) for w, d, a in (x.split(":") for x in lines)]
+def set_(what, v): F.fake_set(what.encode(), v)
+def early(): return [a for w, _, a in log() if w == "forward"][-1]
+"""
+
+
+@pytest.fixture(scope="module")
+def run(tmp_path_factory):
+    from paper_2508_13478_b200 import build
+    lib = build.build()
+    fake = str(tmp_path_factory.mktemp("fake") / "libfake.so")
+    subprocess.run(["gcc", "-O1", "-shared", "-fPIC", "-o", fake, os.path.join(HERE, "fake_cudart.c")], check=True)
+
+    def child(body):
+        r = subprocess.run([sys.executable, "-c", PRELUDE + textwrap.dedent(body), fake, lib], capture_output=True, text=True,
+                           timeout=120, env=dict(os.environ, LD_PRELOAD=fake))
+        assert r.returncode == 0, r.stdout + r.stderr
+    return child
+
+
+def test_destroy_waits_for_the_handles_device(run):
+    run("""
+    h = prepare(); log()
+    F.cudaSetDevice(1); log()
+    D.dhq_destroy(h)
+    got = log()
+    assert ("sync", 0, 0) in got and not any(w == "sync" and d == 1 for w, d, _ in got), got
+    assert got[-1] == ("set_device", 1, 1), got           # the caller's device is current again
+    F.cudaSetDevice(0); log()
+    h = prepare()
+    assert not any(w == "malloc" for w, _, _ in log())     # the block of the first handle
+    set_("fail_sync", 1); log()
+    D.dhq_destroy(h)                                       # could not wait: the block is not kept
+    assert any(w == "free" for w, _, _ in log())
+    set_("fail_sync", 0)
+    prepare()
+    assert any(w == "malloc" for w, _, _ in log())
+    """)
