@@ -228,7 +228,7 @@ __device__ void digit_epilogue(const DigitParams &p, const DigitMap &sm, uint32_
         const long long tok = tile * kTile + c.row;
         const bool valid = tok < p.n;
         float x = 0.f, yc = 0.f;
-        if (valid) { x = __ldg(p.coords + 2 * tok); yc = __ldg(p.coords + 2 * tok + 1); }
+        if (valid) { const float2 xy = load_coords(p.coords, tok); x = xy.x; yc = xy.y; }
         // layer 1: the rotated padded coordinate is [x+y, x-y, x+y, x-y]
         const float e0 = __fadd_rn(__fadd_rn(x, yc), 0.f), e1 = __fadd_rn(__fsub_rn(x, yc), 0.f);
         float inv_x;

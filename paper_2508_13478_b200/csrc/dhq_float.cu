@@ -183,7 +183,7 @@ __device__ void float_epilogue(const FloatParams &p, const FloatMap &sm, uint32_
     auto coords_of = [&](long long tile, float &x, float &yc) {
         const long long tok = tile * kTile + row;
         x = yc = 0.f;
-        if (tile < p.n_tiles && tok < p.n) { x = __ldg(p.coords + 2 * tok); yc = __ldg(p.coords + 2 * tok + 1); }
+        if (tile < p.n_tiles && tok < p.n) { x = p.coords[2 * tok]; yc = p.coords[2 * tok + 1]; } // plain loads: see load_coords (dhq_forward_debug takes any 4-byte aligned coords)
     };
     // block b of the outputs is about to be formed / is complete: the inputs of tensor-core layer t
     auto begin_part = [&](uint32_t t, int b) {

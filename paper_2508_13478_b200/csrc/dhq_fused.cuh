@@ -378,6 +378,11 @@ template <int N> __device__ __forceinline__ void tmem_st(uint32_t taddr, const u
     else ptx::tmem_st64(taddr, v);
 }
 
+// A launch may be resident before the kernel in front of it has written the caller's coordinates or, in a
+// calibration pass, the scales and constants of the layers before: no non-coherent loads of those (__ldg promises
+// that nothing writes them while the kernel runs).  A forward's scales and constants were there before it began.
+__device__ __forceinline__ float2 load_coords(const float *coords, long long tok) { return *(reinterpret_cast<const float2 *>(coords) + tok); }
+template <bool CALIB, typename T> __device__ __forceinline__ T load_frozen(const T *p) { return CALIB ? __ldcg(p) : __ldg(p); }
 __device__ __forceinline__ float4 lds128(uint32_t addr)
 {
     float4 v;
@@ -883,7 +888,7 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
                 ptx::fence_proxy_async();
                 ptx::mbar_arrive(smem_base + sm.xy_empty + 8 * slot);
             } else if (valid) { // ragged last tile, or coordinates not 16-byte aligned
-                float2 xy = __ldg(reinterpret_cast<const float2 *>(p.coords) + tok);
+                float2 xy = load_coords(p.coords, tok);
                 x = xy.x; y = xy.y;
             }
         } else
@@ -891,7 +896,7 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
             x = xy_next.x; y = xy_next.y;
         } else if (!AHEAD || r == 0) {
             if (valid) {
-                float2 xy = __ldg(reinterpret_cast<const float2 *>(p.coords) + tok);
+                float2 xy = load_coords(p.coords, tok);
                 x = xy.x; y = xy.y;
             }
         } else {
@@ -909,16 +914,16 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
             float a = fmaxf(fmaxf(fabsf(e0), fabsf(e1)), fmaxf(fabsf(e2), fabsf(e3)));
             scales_of(a, qmaxf, s_x, inv_x);
         } else {
-            s_x = __ldg(l1.act + 1);
-            inv_x = __ldg(l1.act + 2);
+            s_x = load_frozen<CALIB>(l1.act + 1);
+            inv_x = load_frozen<CALIB>(l1.act + 2);
         }
         const uint32_t b0 = code_bits<true>(e0, inv_x, qmaxf), b1 = code_bits<true>(e1, inv_x, qmaxf);
         const uint32_t qx = pack4(b0, b1, code_bits<true>(e2, inv_x, qmaxf), code_bits<true>(e3, inv_x, qmaxf));
         const int qs = (int)b0 - 0x4B400000, qd = (int)b1 - 0x4B400000;
         float next_s = 1.f, next_inv = 0.f;
         if (!PER_TOKEN) {
-            next_s = __ldg(p.layer[1].act + 1);
-            next_inv = __ldg(p.layer[1].act + 2);
+            next_s = load_frozen<CALIB>(p.layer[1].act + 1);
+            next_inv = load_frozen<CALIB>(p.layer[1].act + 2);
         }
         // Observing instantiation: where this thread's token writes its per-layer values (null: skip)
         [[maybe_unused]] float *dY = nullptr;
@@ -982,8 +987,8 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
             if constexpr (C::NHALF == 1 || C::CPT == 1) acc_parity ^= 1;
             ptx::tc_fence_after();
             if (!PER_TOKEN) {
-                next_s = __ldg(p.layer[l].act + 1);
-                next_inv = __ldg(p.layer[l].act + 2);
+                next_s = load_frozen<CALIB>(p.layer[l].act + 1);
+                next_inv = load_frozen<CALIB>(p.layer[l].act + 2);
             }
             const uint32_t cbase = consts + ly.c_off * 4;
             const bool fast = ly.epi_mode == EPI_SINE_FAST;
@@ -1066,7 +1071,7 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
             const FusedLayer &ly = p.layer[p.L - 1];
             if constexpr (LATE) {
                 const long long tok_next = tile_index<SPREAD>(r + 1, slot, C::SLOTS) * C::TOK + trow;
-                xy_next = tok_next < p.n ? __ldg(reinterpret_cast<const float2 *>(p.coords) + tok_next) : make_float2(0.f, 0.f);
+                xy_next = tok_next < p.n ? load_coords(p.coords, tok_next) : make_float2(0.f, 0.f);
             }
             if (!wait_bar_warp<PER_TOKEN>(bar_last, last_parity, abort_flag, p.status)) return;
             last_parity ^= 1;
@@ -1372,9 +1377,9 @@ __global__ void __launch_bounds__(fused_threads(W, BOTH, GABOR), 1) fused_kernel
             const int areas = (l == 0) ? (fixed ? 3 : (BOTH ? 5 : 4)) : ((ly.epi_mode == EPI_SINE_WIDE || ly.epi_mode == EPI_SINE_MIXED) ? 3 : 2);
             for (int i = threadIdx.x; i < W; i += fused_threads(W, BOTH, GABOR)) { // i: tensor-memory column, m: its feature
                 const int m = fused_feature(i, W);
-                d[i] = __ldg(srcA + m);
-                d[W + i] = __ldg(srcB + m);
-                if (areas >= 3) d[2 * W + i] = __ldg(srcC + m);
+                d[i] = load_frozen<CALIB>(srcA + m);
+                d[W + i] = load_frozen<CALIB>(srcB + m);
+                if (areas >= 3) d[2 * W + i] = load_frozen<CALIB>(srcC + m);
                 if (areas == 4) d[3 * W + i] = __ldg(ly.qw_k4m + m);
                 if (areas == 5) {
                     d[3 * W + i] = (uint32_t)__ldg(ly.l1U + m);
