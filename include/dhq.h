@@ -244,8 +244,8 @@ DHQ_API dhq_status_t dhq_forward_host(dhq_handle_t h, const float *coords_host, 
  * dhq_debug_bufs_t), for checking each stage against a reference.  Same arithmetic as
  * dhq_forward, operation for operation, so `out` and Y[L-1] equal dhq_forward's output bit for
  * bit; activations go through device memory between layers, in chunks, using scratch memory
- * owned by the handle.  `out` and `bufs` may each be NULL.  Requires frozen scales when
- * a_gran = per tensor (NOT_CALIBRATED otherwise).
+ * owned by the handle.  `out` and `bufs` may each be NULL; every buffer needs the alignment of its
+ * element type and no more.  Requires frozen scales when a_gran = per tensor (NOT_CALIBRATED otherwise).
  */
 DHQ_API dhq_status_t dhq_forward_debug(dhq_handle_t h, const float *coords, int64_t n, float *out,
                                        const dhq_debug_bufs_t *bufs, void *stream);

@@ -143,11 +143,11 @@ __device__ void float_epilogue(const FloatParams &p, const FloatMap &sm, uint32_
     auto emit = [&](int l, int k0, const float (&y)[16], long long tok, bool valid) {
         if constexpr (DUMP) {
             if (valid) {
+                // (one float at a time: the caller's buffers are 4-byte aligned and no more)
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float4 v = make_float4(y[4 * q], y[4 * q + 1], y[4 * q + 2], y[4 * q + 3]);
-                    if (p.dY[l - 1]) *reinterpret_cast<float4 *>(p.dY[l - 1] + tok * W + k0 + 4 * q) = v;
-                    if (p.dX[l]) *reinterpret_cast<float4 *>(p.dX[l] + tok * W + k0 + 4 * q) = v;
+                for (int j = 0; j < 16; ++j) {
+                    if (p.dY[l - 1]) p.dY[l - 1][tok * W + k0 + j] = y[j];
+                    if (p.dX[l]) p.dX[l][tok * W + k0 + j] = y[j];
                 }
             }
         }

@@ -81,3 +81,27 @@ def test_tiles_of_one_block_do_not_disturb_each_other(width, n_linear):
         assert dhq.dhq_last_status(h) == 0
     finally:
         dhq.dhq_destroy(h)
+
+
+@pytest.mark.parametrize("width", [64, 256, 512])
+def test_dump_buffers_and_coordinates_need_no_more_than_float_alignment(width):
+    dims, n = (2, width, width, width, 3), 300
+    weights, biases = dhq_inputs.siren_init(dims, 30.0, 950 + width)
+    coords = to_dev(dhq_inputs.grid_coords(3, 100))
+    h = dhq.dhq_prepare(dims, [to_dev(x) for x in weights], [to_dev(x) for x in biases], 30.0, 32, dhq.DHQ_BITS_FLOAT)
+    try:
+        def run(shift):  # every buffer `shift` floats past a 256-byte boundary
+            def buf(cols):
+                return torch.full((n * cols + 4,), float("nan"), device="cuda")[shift:shift + n * cols].view(n, cols)
+            X = [buf(dhq.dhq_layer_dims(h, l)[0]) for l in range(1, 5)]
+            Y = [buf(dhq.dhq_layer_dims(h, l)[1]) for l in range(1, 5)]
+            c, out = buf(2), buf(3)
+            c.copy_(coords)
+            dhq.dhq_forward_debug(h, c, out, {"X": X, "Y": Y})
+            torch.cuda.synchronize()
+            assert dhq.dhq_last_status(h) == 0
+            return X + Y + [out]
+        for got, want in zip(run(1), run(0)):
+            assert torch.equal(got.view(torch.int32), want.view(torch.int32))
+    finally:
+        dhq.dhq_destroy(h)
