@@ -168,7 +168,8 @@ def dhq_set_act_absmax(handle, layer, absmax, stream=None):
 
 
 _fast = {}
-_raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+# (a build of torch without CUDA has neither; the package imports and checks arguments there all the same)
+_raw_stream, _current_device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
 _f32 = torch.float32
 
 
@@ -182,7 +183,10 @@ def dhq_forward(handle, coords, out, stream=None):
     # and the stream (6.2 -> 1.7 us of host time before the launch).
     if _is_f32(coords) and _is_f32(out):
         fn = _fast.get("forward") or _fast.setdefault("forward", load_library().dhq_forward)
-        st = _raw_stream(_current_device()) if stream is None else stream.cuda_stream
+        if stream is None and _raw_stream and _current_device:
+            st = _raw_stream(_current_device())
+        else:
+            st = (torch.cuda.current_stream() if stream is None else stream).cuda_stream
         code = fn(handle, coords.data_ptr(), coords.size(0), out.data_ptr(), st)
     else:                                       # no tensor, or not of this kind: the error says which
         code = load_library().dhq_forward(handle, _dev_ptr(coords, torch.float32, "coords"), coords.shape[0],

@@ -54,3 +54,24 @@ def test_oracle_and_product_do_not_import_each_other():
             if f.endswith((".py", ".cu", ".cuh", ".h")):
                 text = open(os.path.join(base, f)).read()
                 assert "oracle" not in text.lower(), f"{f} mentions the oracle"
+
+
+def test_package_imports_where_torch_has_no_cuda_functions(lib_path):
+    # a CPU build of torch lacks the private stream functions: importing and argument checks must not need them
+    code = """
+import torch
+for name in ("_cuda_getCurrentRawStream", "_cuda_getDevice"):
+    if hasattr(torch._C, name): delattr(torch._C, name)
+import paper_2508_13478_b200 as dhq
+t = torch.zeros(4, 2)
+try: dhq.dhq_forward(None, t, t)
+except TypeError as e: assert "coords" in str(e)
+else: raise SystemExit("host tensors were taken")
+try: dhq.dhq_forward_host(None, t, t)
+except dhq.DhqError as e: assert e.code == 1
+else: raise SystemExit("no handle, no error")
+"""
+    import subprocess
+    import sys
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
