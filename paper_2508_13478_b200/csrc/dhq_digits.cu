@@ -20,11 +20,11 @@
 // of the next layer's input can run through it (stages 1, 2, 4 inside a block, 8 .. W/8 in a thread's
 // chunk, W/4 and W/2 across chunks).  The weights stream from L2 in pieces of 16 KB.
 //
-// What bounds it: issue slots of the epilogue, about 35 per element (13 of them the phase, carried as if in
+// What bounds it: issue slots of the epilogue, about 38 per element (14 of them the phase, carried as if in
 // fp64: digit_phase), beside 32 x 51 cycles of MMAs per block of 64 outputs.  A block's sums are released as
 // soon as they are in registers, so that the next block's MMAs run beside its phases; the first block's MMAs
 // and the stages across chunks are exposed (one tile fills tensor memory).  Measured: 2 -> 256 x 5 -> 3,
-// per-channel / per-token, 262,144 coordinates 9.79 -> 0.74 ms (one dp4a pass and an fp64 butterfly per layer
+// per-channel / per-token, 262,144 coordinates 9.79 -> 0.77 ms (one dp4a pass and an fp64 butterfly per layer
 // before).
 #include "dhq_fused.cuh"
 

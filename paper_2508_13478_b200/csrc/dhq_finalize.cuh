@@ -14,7 +14,7 @@ __device__ __forceinline__ double finalize_row(const LayerDev &dev, int m, float
         const float hi = (float)A;
         dev.cA[m] = hi;
         dev.cA_lo[m] = (float)(A - (double)hi);
-        const double hi_b = rint((b - n) * 131072.0) * (1.0 / 131072.0); // see digit_phase
+        const double hi_b = rint((b - n) * 2048.0) * (1.0 / 2048.0); // see digit_phase
         dev.cB[m] = (float)hi_b;
         dev.cB_lo[m] = (float)(b - n - hi_b);
         dev.cN[m] = (float)(b - hi_b); // the wavelet's envelope needs the whole bias

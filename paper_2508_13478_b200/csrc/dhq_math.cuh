@@ -130,27 +130,31 @@ __device__ __forceinline__ float sine_fixed(int qs, int qd, uint32_t P, uint32_t
 
 // Two-sided transform with a weight scale per output channel: the matrix H_M diag(s_w) q_W is held as four
 // base-256 digits per entry and D0 .. D3 are the digits' products with the activation codes (exact;
-// |D| < 2^23 at widths up to 256).  The phase in turns is t = c (D0 + D1 / 2^8 + D2 / 2^16 + D3 / 2^24) + cb with
-// c = c_hi + c_lo and the bias modulo one turn cb + cb_lo (cb a multiple of 2^-17).  The result is
-// 2 pi (t - nearest integer) rounded to fp32 as if t had been known in fp64.  Adding 96 = 1.5 * 2^6 cuts the
-// product at 2^-17 (|c D0| < 32; the grid moves by a factor of two beyond), so that the parts above, added to cb
-// and freed of whole turns, stay exact until the last fma; all parts below are gathered in `lo` (error 0.5 ulp +
-// 2^-42 turns).  That care is for the quantizer that follows,
-// not for the 1e-5 of the output: activations that agree with the fp64 evaluation bit for bit are quantized to the
-// same codes.  (13 operations; carrying the rounding errors of fp32 sums along took 23, and the kernel of
-// dhq_digits.cu 0.83 ms for 262,144 coordinates in place of 0.74.)
+// |D| < 2^22 at widths up to 256).  Their carries go into the first, so that the number is f0 + f1 with f0 an
+// integer (exact in fp32) and -1/4 < f1 < 5/4, f1 rounded to 2^-25.
 __device__ __forceinline__ void digit_sums(int D0, int D1, int D2, int D3, float &f0, float &f1)
 {
-    f0 = (float)D0;
-    f1 = __fmul_rn((float)(D1 * 256 + (D2 + (D3 >> 8))), 0x1p-16f);
+    const int u = D1 * 256 + D2; // in units of 2^-16 of D0's
+    f0 = (float)(D0 + (u >> 16));
+    f1 = __fmul_rn((float)((u & 65535) * 256 + D3), 0x1p-24f);
 }
+// The phase in turns is c (f0 + f1) + cb with c = c_hi + c_lo and the bias modulo one turn cb + cb_lo (cb a multiple
+// of 2^-11).  The result is 2 pi (phase - nearest integer) rounded to fp32 as if the phase had been known in fp64.  Adding
+// 6144 = 1.5 * 2^12 cuts the product at 2^-11, so that the parts above, added to cb and freed of whole
+// turns, stay exact until the last fma (below 2^12 turns); all parts below, 2^-10 turns or less, are gathered in `lo`
+// (error 0.5 ulp + 2^-36 turns).  `lo` takes part in the choice of the integer: the hardware sine rounds its
+// argument twice as coarsely beyond pi.  That care is for the quantizer that follows, not for the 1e-5 of the
+// output: activations that agree with the fp64 evaluation bit for bit are quantized to the same codes.
+// Largest error of a hidden output against fp64 3.6e-7 (rms 1.0e-7) up to phases of 500 rad, as with an fp64 butterfly and
+// phase; the entries' 2^-32 adds 2^-32 of the phase beyond.  (Without the carries above and with the cut at 2^-17,
+// 0.735 in place of 0.769 ms for 262,144 coordinates, width 256, 5 layers: 7e-7, and 1e-4 from 128 turns on.)
 __device__ __forceinline__ float digit_phase(float f0, float f1, float c_hi, float c_lo, float cb, float cb_lo)
 {
     const float two_pi = 6.2831853071795865f, two_pi_lo = -1.7484555e-07f; // fl32(2 pi) and what it lacks
-    const float q = __fsub_rn(__fmaf_rn(f0, c_hi, 96.0f), 96.0f);
+    const float q = __fsub_rn(__fmaf_rn(f0, c_hi, 6144.0f), 6144.0f);
     const float s = __fadd_rn(q, cb);
-    const float t = __fsub_rn(s, __fsub_rn(__fadd_rn(s, 12582912.0f), 12582912.0f));
     const float lo = __fadd_rn(__fmaf_rn(f0, c_hi, -q), __fmaf_rn(f0, c_lo, __fmaf_rn(f1, c_hi, cb_lo)));
+    const float t = __fsub_rn(s, __fsub_rn(__fadd_rn(__fadd_rn(s, lo), 12582912.0f), 12582912.0f));
     return __fmaf_rn(t, two_pi, __fmaf_rn(lo, two_pi, __fmul_rn(t, two_pi_lo)));
 }
 // The wavelet's envelope exp(-(s0 z)^2) from the same numbers: cn is the part of the bias that cb lacks, gc = 2 pi s0 / omega0.

@@ -14,6 +14,7 @@ from tests.gpu_util import check_layers_against_oracle, check_weights, prepare_p
 pytestmark = pytest.mark.gpu
 
 dhq = pytest.importorskip("paper_2508_13478_b200")
+from oracle import odef  # noqa: E402
 
 
 @pytest.mark.parametrize("width,n_linear,d_out,a_gran,n,s0", [
@@ -41,5 +42,32 @@ def test_two_sided_per_channel(width, n_linear, d_out, a_gran, n, s0):
         assert dhq.dhq_launch_count(h) - before == 1 and dhq.dhq_last_status(h) == 0
         assert torch.equal(out.view(torch.int32), dumped.view(torch.int32))
         print(f"two-sided per channel, width {width}: outputs within {worst:.2e}")
+    finally:
+        dhq.dhq_destroy(h)
+
+
+@pytest.mark.parametrize("width,a_gran,scale", [(128, 1, 1.0), (256, 0, 1.0), (256, 1, 20.0), (128, 0, 300.0)])
+def test_phases_are_rounded_once(width, a_gran, scale):
+    # The hidden outputs against fp64 on the kernel's own accumulators, phases of 50 to 10,000 rad.  Bound: the hardware
+    # sine on [-pi, pi] (2^-21.41 = 3.6e-7) and the phase rounded to fp32 there (half an ulp, 1.2e-7); the entries of a row
+    # are multiples of 2^-31 of the largest, so that a sum of them is off by at most that part of the largest phase.
+    dims, n = (2, width, width, width, 3), 1500
+    weights, biases = dhq_inputs.siren_init(dims, 30.0, 45 + width)
+    coords = dhq_inputs.grid_coords(30, 50) * np.float32(scale)
+    h, net = prepare_pair(dims, weights, biases, 30.0, 8, 8, 1, a_gran, rotate="both")
+    try:
+        cd = to_dev(coords)
+        dhq.dhq_calibrate(h, cd)
+        _, bufs = run_debug(h, net, cd)
+        H = odef.hadamard(width)
+        worst, excess = [], []
+        for l in (1, 2, 3):
+            s_w = dhq.dhq_get_layer(h, l)[1].astype(np.float64)
+            acc, s_x = bufs["acc"][l - 1].cpu().numpy().astype(np.float64), bufs["s_x"][l - 1].cpu().numpy().astype(np.float64)
+            z = (acc * s_w[None, :] * s_x[:, None]) @ H + biases[l - 1].astype(np.float64)[None, :]
+            worst.append(np.abs(bufs["Y"][l - 1].cpu().numpy() - np.sin(30.0 * z)).max())
+            excess.append(worst[-1] - 2.0 ** -31 * np.abs(30.0 * z).max())
+        print(f"two-sided per channel, width {width}, coordinates x {scale}: " + " ".join(f"{x:.2e}" for x in worst))
+        assert max(excess) <= 5e-7
     finally:
         dhq.dhq_destroy(h)
