@@ -881,6 +881,10 @@ dhq_status_t dhq_import(const void *host_buf, int64_t bytes, void *stream, dhq_h
             }
         }
         if (rc != DHQ_OK) break;
+        // (the same constants again from the same scales: a block of an earlier build splits the bias differently)
+        for (int l = 1; l <= h->L && h->layer[0].has_digits && hd.calibrated; ++l)
+            if (launch_finalize(h->layer[l - 1], cfg.a_bits, cfg.a_gran == DHQ_GRAN_CHANNEL_OR_TOKEN, l < h->L, (double)cfg.omega0, st, &h->launches) != cudaSuccess) rc = DHQ_ERR_CUDA;
+        if (rc != DHQ_OK) break;
         if (cudaStreamSynchronize(st) != cudaSuccess) { rc = DHQ_ERR_CUDA; break; } // host_buf may go after the call
         h->calibrated = hd.calibrated != 0;
         h->calib_layers_done = hd.calib_layers_done;

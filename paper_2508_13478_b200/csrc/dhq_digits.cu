@@ -54,7 +54,8 @@ struct DigitParams {
     float *out;
     long long n, n_tiles;
     int L, d_L, n_stages;
-    float qmaxf, gabor_c;            // gabor_c: s0 / omega0 in turns, 0 for the sine
+    float qmaxf;
+    double gabor_c;                  // see digit_envelope; 0 for the sine
     int *status;
     unsigned long long wait_limit_ns;
     DigitLayer layer[kMaxLayers];
@@ -178,8 +179,9 @@ __device__ void digit_epilogue(const DigitParams &p, const DigitMap &sm, uint32_
         for (int e = 0; e < 4; ++e) {
             float c_hi = av[e], c_lo = lv[e];
             if (PER_TOKEN) token_const(av[e], lv[e], s_x, c_hi, c_lo);
-            y[e] = sin_approx(digit_phase(f0[e], f1[e], c_hi, c_lo, bv[e], blv[e]));
-            if constexpr (GABOR) y[e] = __fmul_rn(y[e], digit_envelope(f0[e], f1[e], c_hi, bv[e], nv[e], p.gabor_c));
+            float s, lo;
+            y[e] = sin_approx(digit_phase(f0[e], f1[e], c_hi, c_lo, bv[e], blv[e], s, lo));
+            if constexpr (GABOR) y[e] = __fmul_rn(y[e], digit_envelope(s, lo, nv[e], p.gabor_c));
         }
     };
     // stages 1, 2, 4 of 16 finished activations, and into the row's columns

@@ -17,7 +17,7 @@ __device__ __forceinline__ double finalize_row(const LayerDev &dev, int m, float
         const double hi_b = rint((b - n) * 2048.0) * (1.0 / 2048.0); // see digit_phase
         dev.cB[m] = (float)hi_b;
         dev.cB_lo[m] = (float)(b - n - hi_b);
-        dev.cN[m] = (float)(b - hi_b); // the wavelet's envelope needs the whole bias
+        dev.cN[m] = (float)n; // the wavelet's envelope needs the whole bias
         return A;
     }
     const double f = sine ? omega0 : 1.0;

@@ -36,7 +36,7 @@ struct LayerDev {
     uint32_t *gd_k4m = nullptr; // [4 digits][K/4][M] words of four consecutive k
     uint8_t *gd_img = nullptr; // the digits in tensor-core order (layers 2 .. L)
     double *g_scale = nullptr; // [M] value of a unit of the fixed-point row
-    float *cN = nullptr, *cB_lo = nullptr; // [M] bias in turns: all but cB, and the same modulo one turn
+    float *cN = nullptr, *cB_lo = nullptr; // [M] bias in turns: its whole turns, and what cB and they lack
     int has_f32 = 0;           // floating-point datapaths: 1 first and last layer (w_f32, f_scale), 2 hidden layer (wdig)
     float *w_f32 = nullptr;    // last layer: [K/4][M] float4 fp32 weights (W8A32: the integers q_w H_K), zero padded;
                                // first layer: [M] float4 (two weights and the bias in turns of the phase)
@@ -118,7 +118,7 @@ struct LayerArgs {
     const uint32_t *gd_k4m;
     const double *g_scale;
     const float *cN, *cB_lo;
-    float digit_gc;
+    double digit_gc;
     double gabor_s0;       // > 0: hidden layers apply sin(omega0 z) exp(-(s0 z)^2) instead of the sine
     float *Y;              // [n][M] or NULL
     float *out;            // [n][d_L] or NULL (last layer)

@@ -111,8 +111,9 @@ __global__ void __launch_bounds__(LW_THREADS) layer_kernel(LayerArgs a)
                     if (a.per_token) token_const(cA, cAl, s_tok[t], c_hi, c_lo);
                     float f0, f1;
                     digit_sums(D[0], D[1], D[2], D[3], f0, f1);
-                    y = sin_approx(digit_phase(f0, f1, c_hi, c_lo, cB, cBl));
-                    if (a.gabor_s0 > 0.0) y = __fmul_rn(y, digit_envelope(f0, f1, c_hi, cB, cN, a.digit_gc));
+                    float s, lo;
+                    y = sin_approx(digit_phase(f0, f1, c_hi, c_lo, cB, cBl, s, lo));
+                    if (a.gabor_s0 > 0.0) y = __fmul_rn(y, digit_envelope(s, lo, cN, a.digit_gc));
                 } else {
                     y = digit_last(D[0], D[1], D[2], D[3], a.g_scale[m], (double)s_tok[t], a.bias[m]);
                 }

@@ -148,24 +148,25 @@ __device__ __forceinline__ void digit_sums(int D0, int D1, int D2, int D3, float
 // Largest error of a hidden output against fp64 3.6e-7 (rms 1.0e-7) up to phases of 500 rad, as with an fp64 butterfly and
 // phase; the entries' 2^-32 adds 2^-32 of the phase beyond.  (Without the carries above and with the cut at 2^-17,
 // 0.735 in place of 0.769 ms for 262,144 coordinates, width 256, 5 layers: 7e-7, and 1e-4 from 128 turns on.)
-__device__ __forceinline__ float digit_phase(float f0, float f1, float c_hi, float c_lo, float cb, float cb_lo)
+// s, lo: the parts of the phase before whole turns are taken off.
+__device__ __forceinline__ float digit_phase(float f0, float f1, float c_hi, float c_lo, float cb, float cb_lo, float &s, float &lo)
 {
     const float two_pi = 6.2831853071795865f, two_pi_lo = -1.7484555e-07f; // fl32(2 pi) and what it lacks
     const float q = __fsub_rn(__fmaf_rn(f0, c_hi, 6144.0f), 6144.0f);
-    const float s = __fadd_rn(q, cb);
-    const float lo = __fadd_rn(__fmaf_rn(f0, c_hi, -q), __fmaf_rn(f0, c_lo, __fmaf_rn(f1, c_hi, cb_lo)));
+    s = __fadd_rn(q, cb);
+    lo = __fadd_rn(__fmaf_rn(f0, c_hi, -q), __fmaf_rn(f0, c_lo, __fmaf_rn(f1, c_hi, cb_lo)));
     const float t = __fsub_rn(s, __fsub_rn(__fadd_rn(__fadd_rn(s, lo), 12582912.0f), 12582912.0f));
     return __fmaf_rn(t, two_pi, __fmaf_rn(lo, two_pi, __fmul_rn(t, two_pi_lo)));
 }
-// The wavelet's envelope exp(-(s0 z)^2) from the same numbers: cn is the part of the bias that cb lacks, gc = 2 pi s0 / omega0.
-__device__ __forceinline__ float digit_envelope(float f0, float f1, float c_hi, float cb, float cn, float gc)
+// The wavelet's envelope exp(-(s0 z)^2) in fp64 from the parts of the phase that digit_phase leaves (all but `lo` exact), rounded
+// once: an fp32 square loses (s0 z)^2 units in the last place of the result, and the activations go to a quantizer.
+// n: the whole turns of the bias; gc = 2 pi s0 / omega0.
+__device__ __forceinline__ float digit_envelope(float s, float lo, float n, double gc)
 {
-    const float g = __fmul_rn(__fmaf_rn(__fadd_rn(f0, f1), c_hi, __fadd_rn(cb, cn)), gc);
-    float e;
-    asm("ex2.approx.f32 %0, %1;" : "=f"(e) : "f"(__fmul_rn(__fmul_rn(g, g), -1.4426950408889634f)));
-    return e;
+    const double g = ((double)__fadd_rn(s, n) + (double)lo) * gc;
+    return (float)exp(-(g * g));
 }
-inline float digit_gabor_c(double s0, double omega0) { return omega0 != 0.0 ? (float)(s0 / omega0 * 6.283185307179586476925287) : 0.f; }
+inline double digit_gabor_c(double s0, double omega0) { return omega0 != 0.0 ? s0 / omega0 * 6.283185307179586476925287 : 0.0; }
 // Last layer: z = scale s_x (the digits' number) + b, in fp64, rounded once.
 __device__ __forceinline__ float digit_last(int D0, int D1, int D2, int D3, double scale, double s_x, float b)
 {

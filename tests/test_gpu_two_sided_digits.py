@@ -71,3 +71,31 @@ def test_phases_are_rounded_once(width, a_gran, scale):
         assert max(excess) <= 5e-7
     finally:
         dhq.dhq_destroy(h)
+
+
+@pytest.mark.parametrize("width,a_gran,s0", [(128, 0, 10.0), (256, 1, 10.0), (256, 0, 3.0), (128, 1, 40.0)])
+def test_wavelet_envelope_is_rounded_once(width, a_gran, s0):
+    # As above for sin(omega0 z) exp(-(s0 z)^2): the sine's bound times the envelope, half an ulp each (6e-8 of the result)
+    # for the envelope and the product, and the entries' rounding through both factors (2^-31 of the largest phase).
+    dims, n = (2, width, width, width, 3), 1500
+    weights, biases = dhq_inputs.siren_init(dims, 30.0, 46 + width)
+    coords = dhq_inputs.grid_coords(30, 50)
+    h, net = prepare_pair(dims, weights, biases, 30.0, 8, 8, 1, a_gran, rotate="both", gabor_s0=s0)
+    try:
+        cd = to_dev(coords)
+        dhq.dhq_calibrate(h, cd)
+        _, bufs = run_debug(h, net, cd)
+        H = odef.hadamard(width)
+        for l in (1, 2, 3):
+            s_w = dhq.dhq_get_layer(h, l)[1].astype(np.float64)
+            acc, s_x = bufs["acc"][l - 1].cpu().numpy().astype(np.float64), bufs["s_x"][l - 1].cpu().numpy().astype(np.float64)
+            z = (acc * s_w[None, :] * s_x[:, None]) @ H + biases[l - 1].astype(np.float64)[None, :]
+            env = np.exp(-(s0 * z) ** 2)
+            want = np.sin(30.0 * z) * env
+            dz = 2.0 ** -31 * np.abs(z).max()
+            bound = 4.8e-7 * env + 1.2e-7 * np.abs(want) + dz * env * (30.0 + 2.0 * s0 * s0 * np.abs(z)) + 1e-37
+            err = np.abs(bufs["Y"][l - 1].cpu().numpy() - want)
+            print(f"two-sided wavelet, width {width}, s0 {s0}, layer {l}: rms {np.sqrt((err ** 2).mean()):.2e}, of the bound {(err / bound).max():.2f}")
+            assert (err <= bound).all()
+    finally:
+        dhq.dhq_destroy(h)
