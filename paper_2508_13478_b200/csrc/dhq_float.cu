@@ -68,6 +68,7 @@ __host__ __device__ constexpr uint32_t float_part_bytes(int W) { return 3u * kTi
 
 // At width 512 the activations leave no room for the epilogue constants: they are read through L1.
 __host__ __device__ constexpr bool float_consts_in_smem(int W) { return W < 512; }
+__host__ __device__ constexpr int float_areas(int W) { return W <= 128 ? 4 : 3; } // per hidden layer, see digit_phase2
 
 struct FloatMap {
     uint32_t a, ring, consts, w_full, w_empty, a_full, x_ready, acc_full, acc_empty, quad_sync, drain, holder, abort_flag, total;
@@ -78,7 +79,7 @@ __host__ __device__ inline FloatMap float_map(int W, int n_stages, int L)
     uint32_t off = 0;
     m.a = off; off += float_x_in_smem(W) ? (uint32_t)(W / float_block(W) + 1) * float_part_bytes(W) : 3u * kTile * W;
     m.ring = off; off += (uint32_t)n_stages * float_block(W) * float_kc(W);
-    m.consts = off; off += float_consts_in_smem(W) ? (uint32_t)(4 + 3 * (L - 2)) * W * 4 : 0; // first layer, then c0 | c0_lo | cb per hidden layer
+    m.consts = off; off += float_consts_in_smem(W) ? (uint32_t)(4 + float_areas(W) * (L - 2)) * W * 4 : 0; // first layer, then c0 | c0_lo | cb (| cb_lo) per hidden layer
     m.w_full = off; off += 8 * kFMaxStages;
     m.w_empty = off; off += 8 * kFMaxStages;
     m.a_full = off; off += 8 * 8;
@@ -113,17 +114,35 @@ __device__ __forceinline__ void digits4(const float (&y)[4], int j, Digits16 &d)
     d.w[2][j] = __byte_perm(a, b, 0x5410) ^ 0x80808080u;
 }
 
-// The phases of two hidden outputs in turns, less whole turns: c0 (D0 + D1 / 256 + D2 / 65536) + cb with
-// c0 = fl32 value plus remainder c0_lo, cb = omega0 b / (2 pi) modulo 1.  The integer part of c0 D0 is
-// taken off inside an fma, before anything is rounded, so that the error does not grow with the phase.
-__device__ __forceinline__ f32x2 digit_phase2(const uint32_t *D0, const uint32_t *D1, const uint32_t *D2, f32x2 c0, f32x2 c0_lo, f32x2 cb)
+// The phases of two hidden outputs in radians, less whole turns: 2 pi (c0 (D0 + D1 / 256 + D2 / 65536) + cb) with
+// c0 = fl32 value plus remainder c0_lo, cb = omega0 b / (2 pi) modulo 1.  The integer is taken off inside an fma, before
+// anything is rounded, so that the error does not grow with the phase, and it is the one nearest to the whole phase: the
+// hardware sine rounds its argument twice as coarsely beyond pi.  Up to width 128, where the fp32 sums of few
+// products are themselves exact to 1.5e-7, the phase is rounded only once, as digit_phase of dhq_math.cuh does it (cb is
+// the part on its 2^-11 grid, cb_lo the rest).
+// Error of the hidden outputs of the second layer against fp64, rms relative to theirs, default initialisation, widths 64 and 256:
+// with fp32 multiply-adds 2.1e-7 and 3.3e-7; here 1.9e-7 and 2.0e-7.
+__host__ __device__ constexpr bool float_rounds_once(int W) { return W <= 128; }
+template <int W>
+__device__ __forceinline__ f32x2 digit_phase2(const uint32_t *D0, const uint32_t *D1, const uint32_t *D2, f32x2 c0, f32x2 c0_lo, f32x2 cb, f32x2 cb_lo)
 {
-    const f32x2 magic = pack2(12582912.0f, 12582912.0f);
+    const f32x2 magic = pack2(12582912.0f, 12582912.0f), two_pi = pack2(6.2831853071795865f, 6.2831853071795865f);
     const f32x2 f0 = pack2((float)(int)D0[0], (float)(int)D0[1]); // |D0| < 2^24: exact
-    // (D2 enters to 1/256 of a unit of D1: 2^-16 of one of D0)
-    const f32x2 f1 = mul2(pack2((float)((int)D1[0] + ((int)D2[0] >> 8)), (float)((int)D1[1] + ((int)D2[1] >> 8))), pack2(0x1p-8f, 0x1p-8f));
-    const f32x2 k = sub2(magic, fma2(f0, c0, magic)); // minus the nearest integer
-    return add2(fma2(f0, c0, k), fma2(f0, c0_lo, fma2(f1, c0, cb)));
+    // (D1 < 2^24 at width 512: 256 times that and D2 are still an int32 at width 256)
+    constexpr int S = W == 512 ? 1 : 0;
+    const f32x2 f1 = mul2(pack2((float)((int)D1[0] * (256 >> S) + ((int)D2[0] >> S)), (float)((int)D1[1] * (256 >> S) + ((int)D2[1] >> S))),
+                          pack2(S ? 0x1p-15f : 0x1p-16f, S ? 0x1p-15f : 0x1p-16f));
+    if constexpr (float_rounds_once(W)) {
+        const f32x2 grid = pack2(6144.0f, 6144.0f), two_pi_lo = pack2(-1.7484555e-07f, -1.7484555e-07f);
+        const f32x2 nq = sub2(grid, fma2(f0, c0, grid)), s = sub2(cb, nq); // minus the product's part on the grid
+        const f32x2 lo = add2(fma2(f0, c0, nq), fma2(f0, c0_lo, fma2(f1, c0, cb_lo)));
+        const f32x2 t = sub2(s, sub2(add2(add2(s, lo), magic), magic));
+        return fma2(t, two_pi, fma2(lo, two_pi, mul2(t, two_pi_lo)));
+    } else {
+        const f32x2 w = fma2(f0, c0_lo, fma2(f1, c0, cb));
+        const f32x2 k = sub2(magic, add2(fma2(f0, c0, w), magic)); // minus the nearest integer
+        return mul2(add2(fma2(f0, c0, k), w), two_pi);
+    }
 }
 __device__ __forceinline__ float sine_of_turns(float r) { return sin_approx(__fmul_rn(r, 6.2831853071795865f)); }
 
@@ -262,17 +281,18 @@ __device__ void float_epilogue(const FloatParams &p, const FloatMap &sm, uint32_
                     }
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
-                        float4 c, e, o;
+                        float4 c, e, o, ol = make_float4(0.f, 0.f, 0.f, 0.f);
                         if constexpr (float_consts_in_smem(W)) {
-                            const uint32_t at = base + sm.consts + (uint32_t)(((4 + 3 * (l - 2)) * W + k0 + g * 16 + 4 * q) * 4);
+                            const uint32_t at = base + sm.consts + (uint32_t)(((4 + float_areas(W) * (l - 2)) * W + k0 + g * 16 + 4 * q) * 4);
                             c = lds128(at); e = lds128(at + W * 4); o = lds128(at + 2 * W * 4);
+                            if constexpr (float_rounds_once(W)) ol = lds128(at + 3 * W * 4);
                         } else {
                             c = __ldg(reinterpret_cast<const float4 *>(p.c0[l - 1] + k0 + g * 16) + q);
                             e = __ldg(reinterpret_cast<const float4 *>(p.c0_lo[l - 1] + k0 + g * 16) + q);
                             o = __ldg(reinterpret_cast<const float4 *>(p.cb[l - 1] + k0 + g * 16) + q);
                         }
-                        r[g * 8 + 2 * q] = digit_phase2(&D[0][4 * q], &D[1][4 * q], &D[2][4 * q], pack2(c.x, c.y), pack2(e.x, e.y), pack2(o.x, o.y));
-                        r[g * 8 + 2 * q + 1] = digit_phase2(&D[0][4 * q + 2], &D[1][4 * q + 2], &D[2][4 * q + 2], pack2(c.z, c.w), pack2(e.z, e.w), pack2(o.z, o.w));
+                        r[g * 8 + 2 * q] = digit_phase2<W>(&D[0][4 * q], &D[1][4 * q], &D[2][4 * q], pack2(c.x, c.y), pack2(e.x, e.y), pack2(o.x, o.y), pack2(ol.x, ol.y));
+                        r[g * 8 + 2 * q + 1] = digit_phase2<W>(&D[0][4 * q + 2], &D[1][4 * q + 2], &D[2][4 * q + 2], pack2(c.z, c.w), pack2(e.z, e.w), pack2(o.z, o.w), pack2(ol.z, ol.w));
                     }
                 }
 #pragma unroll
@@ -282,8 +302,8 @@ __device__ void float_epilogue(const FloatParams &p, const FloatMap &sm, uint32_
                     for (int q = 0; q < 8; ++q) {
                         float u, v;
                         unpack2(r[g * 8 + q], u, v);
-                        y[2 * q] = sine_of_turns(u);
-                        y[2 * q + 1] = sine_of_turns(v);
+                        y[2 * q] = sin_approx(u);
+                        y[2 * q + 1] = sin_approx(v);
                     }
                     emit(l, k0 + g * 16, y, tok, valid);
                 }
@@ -486,11 +506,13 @@ __global__ void __launch_bounds__(kFThreads, 1) float_kernel(const __grid_consta
         float4 *dst = reinterpret_cast<float4 *>(gen + sm.consts);
         for (int i = threadIdx.x; i < W; i += kFThreads) dst[i] = __ldg(p.l1 + i);
         for (int l = 1; l < p.L - 1; ++l) {
-            float *c = reinterpret_cast<float *>(dst) + (4 + 3 * (l - 1)) * W;
+            float *c = reinterpret_cast<float *>(dst) + (4 + float_areas(W) * (l - 1)) * W;
             for (int i = threadIdx.x; i < W; i += kFThreads) {
                 c[i] = __ldg(p.c0[l] + i);
                 c[W + i] = __ldg(p.c0_lo[l] + i);
-                c[2 * W + i] = __ldg(p.cb[l] + i);
+                const float b = __ldg(p.cb[l] + i), on_grid = float_rounds_once(W) ? __fsub_rn(__fadd_rn(b, 6144.0f), 6144.0f) : b;
+                c[2 * W + i] = on_grid;
+                if constexpr (float_rounds_once(W)) c[3 * W + i] = __fsub_rn(b, on_grid);
             }
         }
     }
@@ -546,9 +568,10 @@ __global__ void prep_float_kernel(FloatPrepArgs a)
     const float row_scale = a.w8 ? a.dev.s_w[m] : 1.0f;
     const double turns = a.omega0 * 0.15915494309189533576888;
     if (a.first) {
+        const double b = turns * (double)a.dev.bias[m];
         if (tid == 0)
             reinterpret_cast<float4 *>(a.dev.w_f32)[m] = make_float4((float)(turns * (double)row_scale * value(0)), (float)(turns * (double)row_scale * value(1)),
-                                                                     (float)(turns * (double)a.dev.bias[m]), 0.f);
+                                                                     (float)(b - rint(b)), 0.f); // whole turns would cost the bias bits
         return;
     }
     if (!a.hidden) {

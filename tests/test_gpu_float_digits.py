@@ -105,3 +105,31 @@ def test_dump_buffers_and_coordinates_need_no_more_than_float_alignment(width):
             assert torch.equal(got.view(torch.int32), want.view(torch.int32))
     finally:
         dhq.dhq_destroy(h)
+
+
+@pytest.mark.parametrize("width,w_bits,hidden", [(64, 32, 2.1e-7), (64, 8, 2.2e-7), (128, 32, 2.5e-7), (128, 8, 2.6e-7), (256, 32, 3.2e-7),
+                                                 (256, 8, 3.2e-7), (512, 32, 4.2e-7), (512, 8, 4.3e-7)])
+def test_no_less_exact_than_fp32_multiply_adds(width, w_bits, hidden):
+    # rms error of a layer's outputs relative to their rms, against fp64 on the kernel's own inputs of the layer.  Bounds: what
+    # fp32 multiply-adds with an fp32 phase give for these networks (5.6e-7 for the first layer).
+    dims, n = (2, width, width, width, 3), 2048
+    weights, biases = dhq_inputs.siren_init(dims, 30.0, 11)
+    coords = np.ascontiguousarray(np.random.default_rng(5).random((n, 2)) * 2 - 1).astype(np.float32)
+    h = dhq.dhq_prepare(dims, [to_dev(x) for x in weights], [to_dev(x) for x in biases], 30.0, w_bits, dhq.DHQ_BITS_FLOAT)
+    try:
+        X = [torch.empty((n, dhq.dhq_layer_dims(h, l)[0]), device="cuda") for l in range(1, 5)]
+        Y = [torch.empty((n, dhq.dhq_layer_dims(h, l)[1]), device="cuda") for l in range(1, 5)]
+        dhq.dhq_forward_debug(h, to_dev(coords), None, {"X": X, "Y": Y})
+        torch.cuda.synchronize()
+        layers = [dhq.dhq_get_layer(h, l) for l in (1, 2, 3)]
+    finally:
+        dhq.dhq_destroy(h)
+    for l, (codes, scales, _) in enumerate(layers, start=1):
+        x = X[l - 1].cpu().numpy()
+        if w_bits < 32:
+            want = odef.w8a32_layer(codes, scales, biases[l - 1], x, True, 30.0, True)
+        else:
+            want = np.sin(30.0 * (x.astype(np.float64)[:, : dims[l - 1]] @ weights[l - 1].astype(np.float64).T + biases[l - 1].astype(np.float64)))
+        rel = np.linalg.norm(Y[l - 1].cpu().numpy() - want) / np.linalg.norm(want)
+        print(f"W{w_bits}A32 width {width} layer {l}: {rel:.2e}")
+        assert rel <= (5.6e-7 if l == 1 else hidden)
