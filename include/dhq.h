@@ -97,11 +97,14 @@ typedef enum { DHQ_ROT_INPUT = 0, DHQ_ROT_BOTH = 1, DHQ_ROT_NONE = 2 } dhq_rot_t
  *   both DHQ_BITS_FLOAT                 W32A32: the plain fp32 network, z = W x + b (rotation ignored)
  * The two floating-point datapaths run in one kernel: hidden layers on the int8 tensor cores with
  * activations and weights as 24-bit fixed-point numbers in base-256 digits (exact int32 sums, fp32
- * epilogue), first and last layer as fp32 multiply-adds.  They need no calibration; the
+ * epilogue), first and last layer as fp32 multiply-adds.  Networks for which that would be less exact than
+ * fp32 multiply-adds (small activations, weight rows of wide range: decided at prepare time from the weights and
+ * biases) and weights that are not finite run layer by layer with fp32 multiply-adds instead, one launch per
+ * layer.  They need no calibration; the
  * calibration calls are no-ops for them.  dhq_forward_debug dumps only X and Y for them;
  * dhq_forward_fused_debug, dhq_forward_static_scratch and DHQ_ROT_BOTH are UNSUPPORTED.
- * Their layer outputs carry the rounding of activations and weights to 24 bits and of the phase: they
- * are checked against the fp64 definition within 2e-5 per layer (measured: 4.3e-6), not 1e-5. */
+ * Their layer outputs carry the rounding of activations and weights (24 bits) or of the sums (fp32) and of the phase: they
+ * are checked against the fp64 definition within 2e-5 per layer (measured: 3.9e-6), not 1e-5. */
 #define DHQ_BITS_FLOAT 32
 
 /* Activation of layers 1..L-1.  DHQ_ACT_SINE: sin(omega0 z), the SIREN of the paper's method

@@ -47,7 +47,7 @@ void layer_arrays(LayerDev &d, ArrayRef (&t)[kLayerArrays])
     t[i++] = {(void **)&d.fxQ, M * 4};
     t[i++] = {(void **)&d.fxB, M * 4};
     t[i++] = {(void **)&d.act, 16};
-    t[i++] = {(void **)&d.w_f32, d.has_f32 == 1 ? MK * 4 : 0};
+    t[i++] = {(void **)&d.w_f32, d.has_f32 == 1 || d.has_f32 == 3 ? MK * 4 : 0};
     t[i++] = {(void **)&d.f_scale, d.has_f32 == 1 ? M * 4 : 0};
     t[i++] = {(void **)&d.wdig, d.has_f32 == 2 ? 3 * MK : 0}; // two-digit handles leave the last third unused
     t[i++] = {(void **)&d.gd_k4m, d.has_digits ? 4 * MK : 0};
@@ -214,6 +214,14 @@ int float_mode_of(const dhq_config_t &cfg)
     return cfg.w_bits == DHQ_BITS_FLOAT ? 2 : 1;
 }
 
+// Which arrays a layer of a floating-point handle has (digits 0: layer by layer; W8A32 then needs the codes only).
+int float_arrays(int mode, int digits, int l, int L)
+{
+    if (!mode) return 0;
+    if (digits == 0) return mode == 2 ? 3 : 0;
+    return l == 1 || l == L ? 1 : 2;
+}
+
 // Serialized handle (dhq_export / dhq_import): this header, then every array of every layer in
 // the order of layer_arrays.
 struct BlobHeader {
@@ -340,11 +348,45 @@ dhq_status_t layerwise_forward(dhq_handle_s *h, const float *coords, int64_t n, 
     return DHQ_OK;
 }
 
-// The forward pass of a calibrated handle: the fused kernel, or, for the two-sided transform, the
-// layer-by-layer kernels.
+// W8A32 / W32A32 layer by layer: one pass of the fp32 kernel per layer, in chunks; X and Y dumps optional.
+dhq_status_t float_layers_forward(dhq_handle_s *h, const float *coords, int64_t n, float *out, const dhq_debug_bufs_t *bufs, cudaStream_t st)
+{
+    const int64_t chunk = n < kDebugChunk ? n : kDebugChunk;
+    dhq_status_t s = ensure_scratch(h, chunk);
+    if (s != DHQ_OK) return s;
+    for (int64_t t0 = 0; t0 < n; t0 += chunk) {
+        const int64_t cnt = n - t0 < chunk ? n - t0 : chunk;
+        const float *X = nullptr;
+        for (int l = 1; l <= h->L; ++l) {
+            const LayerDev &d = h->layer[l - 1];
+            FloatLayerArgs a;
+            memset(&a, 0, sizeof(a));
+            a.X = X; a.coords = coords + t0 * 2; a.n = cnt;
+            a.K = d.K; a.M = d.M; a.d_L = h->d_L;
+            a.w8 = h->float_mode == 1;
+            a.rotate = a.w8 && h->cfg.rotation == DHQ_ROT_INPUT;
+            a.qw_k4m = d.qw_k4m; a.w_f32 = reinterpret_cast<const float4 *>(d.w_f32);
+            a.s_w = d.s_w; a.bias = d.bias;
+            a.omega0 = h->cfg.omega0; a.sine = l < h->L;
+            a.Y = h->scratch[(l - 1) & 1];
+            if (l == h->L) a.out = out ? out + t0 * h->d_L : nullptr;
+            if (bufs) {
+                if (bufs->X && bufs->X[l - 1]) a.dX = bufs->X[l - 1] + t0 * d.K;
+                if (bufs->Y && bufs->Y[l - 1]) a.Y = bufs->Y[l - 1] + t0 * d.M;
+            }
+            CK(launch_float_layer(a, st));
+            h->launches++;
+            X = a.Y;
+        }
+    }
+    return DHQ_OK;
+}
+
+// The forward pass of a calibrated handle: its kernel for all layers, or the layer-by-layer kernels.
 dhq_status_t run_forward(dhq_handle_s *h, const float *coords, int64_t n, float *out, bool on_host, cudaStream_t st)
 {
-    if (h->float_mode) return float_forward(h, coords, n, out, nullptr, st);
+    if (h->float_state) return float_forward(h, coords, n, out, nullptr, st);
+    if (h->float_mode) return float_layers_forward(h, coords, n, out, nullptr, st);
     if (h->digit_state) return digit_forward(h, coords, n, out, st);
     if (!h->fused) return layerwise_forward(h, coords, n, out, st); // wavelet activation; two-sided transform with per-channel weight scales
     return fused_forward(h, coords, n, out, on_host, st);
@@ -396,18 +438,42 @@ void dhq_destroy(dhq_handle_t h)
     delete h;
 }
 
+// Whether fixed point holds a floating-point network's numbers with as many bits as fp32 multiply-adds would keep.
+// An activation is a multiple of 2^-23 and a weight of 2^-23 of its row's largest, so the error of a layer's phases
+// grows with 1 / r, r the rms of its input, and with c, the ratio of a row's largest weight to its rms; that of an fp32
+// sum grows with sqrt(K).  Measured at widths 64 to 512 (rms error of the layer's outputs, phases of order 1, r
+// from 0.9 down and c from 1.7 up): equal at c / r = 3.6, 5.2, 7.3 and 10, which is 0.45 sqrt(K); the rule asks for 0.436 sqrt(K) over a
+// layer's rows together and allows a single row 1.5 times that.  The default initialisation has c / r = 2.5, bell-shaped weights
+// about 4.3.  r is what the biases and the spread of the phases give: r_1^2 = mean sin^2(omega0 b_m) (coordinates may
+// lie anywhere), r_l^2 = (1 - mean cos(2 omega0 b_m) exp(-2 v)) / 2 with v = omega0^2 r_{l-1}^2 mean |W_m|^2.
+static bool fixed_point_serves(const PrepSums &p, int L, int w, double omega0)
+{
+    if (!p.finite) return false;
+    double r2 = 0.0;
+    for (int l = 1; l < L; ++l) {
+        double v = 0.0;
+        if (l > 1) {
+            const double limit = 0.19 * w * r2, n = (double)w;
+            if (p.row_sq[l - 1] > 0.0 && (p.row_top[l - 1] / p.row_sq[l - 1] * n > limit || p.worst_top[l - 1] * n > 2.25 * limit)) return false;
+            v = omega0 * omega0 * r2 * p.row_sq[l - 1] / n;
+        }
+        r2 = 0.5 * (1.0 - p.cos_bias[l - 1] / w * std::exp(-2.0 * v));
+    }
+    return true;
+}
+
 // The floating-point datapaths' own weights.  W8A32: the integer rows q_w H_K need two digits unless a
-// row is close to its largest possible entry (a weight row with one dominant input).
+// row is close to its largest possible entry (a weight row with one dominant input).  h->float_digits != 0 on entry: it is
+// set here, to 0 if the network is to run layer by layer (the arrays for that are not laid out yet).
 static dhq_status_t prepare_float(dhq_handle_s *h, const float *const *W, cudaStream_t st)
 {
-    h->float_digits = 3;
     FloatPrepArgs a;
     memset(&a, 0, sizeof(a));
     a.w8 = h->float_mode == 1;
     a.rotate = a.w8 && h->cfg.rotation == DHQ_ROT_INPUT;
     a.omega0 = (double)h->cfg.omega0;
     a.row_max = &h->d_prep->row_max;
-    for (int pass = a.w8 && h->L > 2 ? 0 : 1; pass < 2; ++pass) {
+    for (int pass = 0; pass < 2; ++pass) {
         for (int l = 1; l <= h->L; ++l) {
             const LayerDev &d = h->layer[l - 1];
             a.first = l == 1;
@@ -420,10 +486,12 @@ static dhq_status_t prepare_float(dhq_handle_s *h, const float *const *W, cudaSt
             CK(launch_prep_float(a, st, &h->launches));
         }
         if (pass == 0) {
-            unsigned int row_max = 0;
-            CK(cudaMemcpyAsync(&row_max, a.row_max, sizeof(row_max), cudaMemcpyDeviceToHost, st));
+            PrepSums sums;
+            CK(launch_prep_float_sums(h->L, a.omega0, h->layer, h->d_prep, st, &h->launches));
+            CK(cudaMemcpyAsync(&sums, h->d_prep, sizeof(sums), cudaMemcpyDeviceToHost, st));
             CK(cudaStreamSynchronize(st));
-            h->float_digits = row_max <= 32639u ? 2 : 3;
+            h->float_digits = !fixed_point_serves(sums, h->L, h->w, a.omega0) ? 0 : a.w8 && sums.row_max <= 32639u ? 2 : 3;
+            if (h->float_digits == 0) return DHQ_OK;
         }
     }
     return DHQ_OK;
@@ -454,11 +522,14 @@ static dhq_status_t prepare_impl(const dhq_config_t *cfg, const float *const *W,
     dhq_status_t rc = DHQ_OK;
     const bool both = cfg->rotation == DHQ_ROT_BOTH;
     h->float_mode = float_mode_of(*cfg);
+    h->float_digits = h->float_mode ? 3 : 0;
     h->gabor_s0 = cfg->activation == DHQ_ACT_GABOR ? (double)cfg->act_s0 : 0.0;
     const bool gabor = h->gabor_s0 > 0.0;
     // the floating-point datapaths have no activation quantizer: nothing to calibrate
     const bool per_token = cfg->a_gran == DHQ_GRAN_CHANNEL_OR_TOKEN || h->float_mode != 0;
+    bool again; // a floating-point network that fixed point does not serve is laid out twice
     do {
+        again = false;
         if (cudaGetDevice(&h->device) != cudaSuccess) { rc = DHQ_ERR_CUDA; break; }
         PrepNet net;
         memset(&net, 0, sizeof(net));
@@ -470,7 +541,7 @@ static dhq_status_t prepare_impl(const dhq_config_t *cfg, const float *const *W,
             if (l == 1) d.epi_mode = (per_token || gabor) ? EPI_SINE_WIDE : EPI_SINE_FIXED;
             d.has_uv = both && l == 1;
             d.has_digits = takes_digits(*cfg, w);
-            d.has_f32 = !h->float_mode ? 0 : (l == 1 || l == L) ? 1 : 2;
+            d.has_f32 = float_arrays(h->float_mode, h->float_digits, l, L);
         }
         if ((rc = alloc_handle(h, st)) != DHQ_OK) break;
         // (a W32A32 handle still gets 8-bit codes of the unrotated weights; its forward does not read them)
@@ -486,7 +557,22 @@ static dhq_status_t prepare_impl(const dhq_config_t *cfg, const float *const *W,
             net.dev[l - 1] = h->layer[l - 1];
         }
         if (launch_prepare(net, st, &h->launches) != cudaSuccess) { rc = DHQ_ERR_CUDA; break; }
-        if (h->float_mode && (rc = prepare_float(h, W, st)) != DHQ_OK) break;
+        if (h->float_mode) {
+            const int laid_out_for = h->float_digits;
+            if (laid_out_for && (rc = prepare_float(h, W, st)) != DHQ_OK) break;
+            if (laid_out_for && h->float_digits == 0) { // once more, with the arrays of the layer-by-layer route
+                pool_give(h->block, h->block_bytes, h->device); // (the stream is idle: prepare_float has waited for it)
+                h->block = nullptr;
+                again = true;
+                continue;
+            }
+            for (int l = 1; l <= L && !h->float_digits && h->float_mode == 2 && rc == DHQ_OK; ++l) {
+                const LayerDev &d = h->layer[l - 1];
+                if (launch_prep_float_weights(W[l - 1], d.d_out, d.d_in, d.K, d.M, d.w_f32, st) != cudaSuccess) rc = DHQ_ERR_CUDA;
+                h->launches++;
+            }
+            if (rc != DHQ_OK) break;
+        }
         if (h->layer[0].has_digits) {
             DigitPrep g;
             memset(&g, 0, sizeof(g));
@@ -522,10 +608,10 @@ static dhq_status_t prepare_impl(const dhq_config_t *cfg, const float *const *W,
         h->calibrated = per_token;
         // layer by layer: the fp32 datapaths, the two-sided transform with per-channel weight scales, and the
         // wavelet combined with the two-sided transform
-        if (h->float_mode) rc = float_create(h);
+        if (h->float_mode) rc = h->float_digits ? float_create(h) : DHQ_OK;
         else if (h->layer[0].has_digits) rc = digit_create(h);
         else if (!both || both_fused) rc = fused_create(h);
-    } while (0);
+    } while (again);
     if (rc != DHQ_OK) {
         dhq_destroy(h);
         return rc;
@@ -589,7 +675,8 @@ dhq_status_t dhq_forward_debug(dhq_handle_t h, const float *coords, int64_t n, f
     if (!h || n < 0 || (n > 0 && !coords)) return DHQ_ERR_INVALID_ARG;
     if (!on_own_device(h)) return DHQ_ERR_INVALID_ARG;
     if (n == 0) return DHQ_OK;
-    if (h->float_mode) return float_forward(h, coords, n, out, bufs, (cudaStream_t)stream); // X and Y dumps only
+    if (h->float_state) return float_forward(h, coords, n, out, bufs, (cudaStream_t)stream); // X and Y dumps only
+    if (h->float_mode) return float_layers_forward(h, coords, n, out, bufs, (cudaStream_t)stream);
     if (!h->calibrated) return DHQ_ERR_NOT_CALIBRATED;
     cudaStream_t st = (cudaStream_t)stream;
     const int64_t chunk = n < kDebugChunk ? n : kDebugChunk;
@@ -696,7 +783,7 @@ static dhq_status_t forward_host_entry(dhq_handle_t h, const float *coords_host,
     // coordinates and writes the result through their device addresses, so the transfers happen
     // inside the kernel, tile by tile, beside the arithmetic.  (Calibration reads the coordinates
     // once per layer: it goes through the staged path below.)
-    if (h->calibrated && (h->fused || h->digit_state || h->float_mode) && !((uintptr_t)coords_host & 7) && !((uintptr_t)out_host & 3)) {
+    if (h->calibrated && (h->fused || h->digit_state || h->float_state) && !((uintptr_t)coords_host & 7) && !((uintptr_t)out_host & 3)) {
         // one query per buffer: for page-locked memory it also gives the device alias (asked on every
         // call on purpose: an answer remembered per address could outlive the buffer it was given for)
         cudaPointerAttributes ai, ao;
@@ -844,13 +931,13 @@ dhq_status_t dhq_import(const void *host_buf, int64_t bytes, void *stream, dhq_h
     h->L = hd.n_layers; h->w = dims[1]; h->d_L = dims[hd.n_layers];
     h->float_mode = float_mode_of(cfg);
     h->float_digits = hd.float_digits;
-    if (h->float_mode ? (hd.float_digits != 2 && hd.float_digits != 3) : hd.float_digits != 0) { delete h; return DHQ_ERR_INVALID_ARG; }
+    if (h->float_mode ? (hd.float_digits != 0 && hd.float_digits != 2 && hd.float_digits != 3) : hd.float_digits != 0) { delete h; return DHQ_ERR_INVALID_ARG; }
     h->gabor_s0 = cfg.activation == DHQ_ACT_GABOR ? (double)cfg.act_s0 : 0.0;
     size_t payload = 0;
     for (int l = 1; l <= h->L; ++l) {
         LayerDev &d = h->layer[l - 1];
         set_layer_dims(d, l, h->L, h->w, dims);
-        d.has_f32 = !h->float_mode ? 0 : (l == 1 || l == h->L) ? 1 : 2;
+        d.has_f32 = float_arrays(h->float_mode, h->float_digits, l, h->L);
         d.has_uv = cfg.rotation == DHQ_ROT_BOTH && l == 1;
         d.has_digits = takes_digits(cfg, h->w);
         ArrayRef t[kLayerArrays];
@@ -888,7 +975,7 @@ dhq_status_t dhq_import(const void *host_buf, int64_t bytes, void *stream, dhq_h
         if (cudaStreamSynchronize(st) != cudaSuccess) { rc = DHQ_ERR_CUDA; break; } // host_buf may go after the call
         h->calibrated = hd.calibrated != 0;
         h->calib_layers_done = hd.calib_layers_done;
-        if (h->float_mode) rc = float_create(h);
+        if (h->float_mode) rc = h->float_digits ? float_create(h) : DHQ_OK;
         else if (h->layer[0].has_digits) rc = digit_create(h);
         else if (hd.has_fused) rc = fused_create(h);
     } while (0);

@@ -16,8 +16,8 @@
 // is exact, and the three accumulators of an output meet in fp32 in the epilogue.  Products with
 // i + j > 2 are left out (they are below 2^-23 of the largest product).  The error of an output is
 // that of rounding x and W to 24 bits of their range, which does not grow along the sum the way a
-// chain of K fp32 additions does, and the phase is reduced modulo one turn before it is rounded:
-// largest layer error against fp64 4.3e-6 (the first layer's; 5.6e-6 with fp32 multiply-adds).
+// chain of K fp32 additions does, and the phase is reduced modulo one turn before it is rounded.  Networks whose
+// activations or weights use little of that range go to dhq_float_layers.cu (fixed_point_serves).
 //
 // What bounds it.  The digits of a tile of 128 activations stay in shared memory for a whole layer
 // (192 KB at width 512; below that from layer to layer), the weights stream past them from L2.  An MMA takes
@@ -26,7 +26,7 @@
 // are in registers and computes sines and digits beside the next block's MMAs.  At width 512 the
 // remaining 32 KB of shared memory keep too few weight bytes in flight (105 cycles per MMA); at
 // width 256 the sines and digits of the block behind take as long as the MMAs.
-// Measured: 2 -> 256 x 3 -> 3, fp32, 65,536 coordinates 940 -> 67 us (88 with the digits through L2); 2 -> 512 x 4 -> 3, 8-bit
+// Measured: 2 -> 256 x 3 -> 3, fp32, 65,536 coordinates 940 -> 68 us (88 with the digits through L2); 2 -> 512 x 4 -> 3, 8-bit
 // weights, 262,144 coordinates 17.2 -> 1.11 ms (one fp32 CUDA-core pass per layer before; 1.21 ms without the
 // register split of the warpgroups).
 #include "dhq_fused.cuh"
@@ -587,7 +587,19 @@ __global__ void prep_float_kernel(FloatPrepArgs a)
     __syncthreads();
     for (int i = 0; i < (int)(blockDim.x + 31) / 32; ++i) g = fmax(g, red[i]);
     if (a.digits == 0) { // measuring pass
-        if (tid == 0) atomicMax(a.row_max, (unsigned int)g);
+        double sq = 0.0;
+        for (int k = tid; k < K; k += blockDim.x) sq += value(k) * value(k);
+        for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+        __syncthreads();
+        if ((tid & 31) == 0) red[tid >> 5] = sq;
+        __syncthreads();
+        if (tid == 0) {
+            sq = 0.0;
+            for (int i = 0; i < (int)(blockDim.x + 31) / 32; ++i) sq += red[i];
+            a.dev.cA[m] = (float)(sq * (double)row_scale * (double)row_scale);
+            a.dev.cA_lo[m] = (float)(g * g * (double)row_scale * (double)row_scale);
+            if (a.w8) atomicMax(a.row_max, (unsigned int)g);
+        }
         return;
     }
     const double top = a.digits == 2 ? 32639.0 : 8355711.0; // 127 in every digit
@@ -612,6 +624,60 @@ __global__ void prep_float_kernel(FloatPrepArgs a)
     }
 }
 
+// One block for the network, so that the sums, and what is decided by them, do not depend on an order of arrival.
+struct FloatSumsArgs { int L; double omega0; PrepSums *sums; LayerDev dev[kMaxLayers]; };
+__global__ void __launch_bounds__(256) prep_float_sums_kernel(const __grid_constant__ FloatSumsArgs a)
+{
+    __shared__ double red[8][4];
+    __shared__ int bad;
+    const int tid = threadIdx.x;
+    if (tid == 0) bad = 0;
+    for (int l = 0; l < a.L; ++l) {
+        const LayerDev &d = a.dev[l];
+        const bool hidden = l > 0 && l < a.L - 1;
+        double v[4] = {0.0, 0.0, 0.0, 0.0};
+        int nonfinite = 0;
+        for (int m = tid; m < d.M; m += 256) {
+            if (!isfinite(d.row_l1[m]) || !isfinite(d.s_w[m])) nonfinite = 1; // sum |W_mk| + |b_m|
+            if (l < a.L - 1) v[2] += cos(2.0 * a.omega0 * (double)d.bias[m]);
+            if (hidden) {
+                const double sq = (double)d.cA[m], top = (double)d.cA_lo[m];
+                v[0] += sq;
+                v[1] += top;
+                if (sq > 0.0) v[3] = fmax(v[3], top / sq);
+            }
+        }
+        __syncthreads(); // (the words of the layer before have been read)
+        for (int i = 0; i < 4; ++i) {
+            for (int o = 16; o; o >>= 1) {
+                const double u = __shfl_xor_sync(0xffffffffu, v[i], o);
+                v[i] = i == 3 ? fmax(v[i], u) : v[i] + u;
+            }
+            if ((tid & 31) == 0) red[tid >> 5][i] = v[i];
+        }
+        if (nonfinite) bad = 1;
+        __syncthreads();
+        if (tid == 0) {
+            for (int w = 1; w < 8; ++w)
+                for (int i = 0; i < 4; ++i) v[i] = i == 3 ? fmax(v[i], red[w][i]) : v[i] + red[w][i];
+            a.sums->row_sq[l] = v[0];
+            a.sums->row_top[l] = v[1];
+            a.sums->cos_bias[l] = v[2];
+            a.sums->worst_top[l] = v[3];
+            if (l == a.L - 1) a.sums->finite = !bad;
+        }
+    }
+}
+cudaError_t launch_prep_float_sums(int L, double omega0, const LayerDev *layers, PrepSums *sums, cudaStream_t st, int64_t *launches)
+{
+    FloatSumsArgs a;
+    a.L = L; a.omega0 = omega0; a.sums = sums;
+    for (int l = 0; l < L; ++l) a.dev[l] = layers[l];
+    prep_float_sums_kernel<<<1, 256, 0, st>>>(a);
+    *launches += 1;
+    return cudaGetLastError();
+}
+
 cudaError_t launch_prep_float(const FloatPrepArgs &a, cudaStream_t st, int64_t *launches)
 {
     prep_float_kernel<<<a.M, 128, a.K * sizeof(int), st>>>(a);
@@ -626,7 +692,7 @@ size_t float_scratch_bytes(const dhq_handle_s *h)
 {
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess) sms = 148;
-    return float_x_in_smem(h->w) ? 0 : (size_t)sms * 3 * kTile * h->w;
+    return float_x_in_smem(h->w) || h->float_digits == 0 ? 0 : (size_t)sms * 3 * kTile * h->w;
 }
 
 struct FloatState {

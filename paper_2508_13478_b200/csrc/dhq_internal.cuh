@@ -37,7 +37,8 @@ struct LayerDev {
     uint8_t *gd_img = nullptr; // the digits in tensor-core order (layers 2 .. L)
     double *g_scale = nullptr; // [M] value of a unit of the fixed-point row
     float *cN = nullptr, *cB_lo = nullptr; // [M] bias in turns: its whole turns, and what cB and they lack
-    int has_f32 = 0;           // floating-point datapaths: 1 first and last layer (w_f32, f_scale), 2 hidden layer (wdig)
+    int has_f32 = 0;           // floating-point datapaths: 1 first and last layer (w_f32, f_scale), 2 hidden layer (wdig);
+                               // 3 any layer of W32A32 layer by layer (w_f32: [K/4][M] float4 fp32 weights, zero padded)
     float *w_f32 = nullptr;    // last layer: [K/4][M] float4 fp32 weights (W8A32: the integers q_w H_K), zero padded;
                                // first layer: [M] float4 (two weights and the bias in turns of the phase)
     float *f_scale = nullptr;  // [M] last layer: scale of the rows of w_f32 (W32A32: 1)
@@ -80,7 +81,7 @@ struct dhq_handle_s {
     void *digit_state = nullptr;    // state of the two-sided kernel for per-channel weight scales
     double *g_scratch = nullptr;    // its matrices in fp64 (used by the preparation only)
     void *float_state = nullptr;    // state of the floating-point datapaths
-    int float_digits = 0;           // base-256 digits per weight of their hidden layers
+    int float_digits = 0;           // base-256 digits per weight of their hidden layers; 0: layer by layer in fp32
     int float_mode = 0;             // 0: fully quantized (DHQ); 1: W8A32 (activations fp32); 2: W32A32 (plain fp32 network)
 };
 
@@ -133,6 +134,25 @@ void float_destroy(dhq_handle_s *h);
 size_t float_scratch_bytes(const dhq_handle_s *h);
 // bufs: X and Y dumps only, may be NULL; out may be NULL when bufs is given
 dhq_status_t float_forward(dhq_handle_s *h, const float *coords, int64_t n, float *out, const dhq_debug_bufs_t *bufs, cudaStream_t st);
+// The same layer by layer with fp32 multiply-adds, dhq_float_layers.cu.
+struct FloatLayerArgs {
+    const float *X;        // [n][K] layer input, or NULL for layer 1 (built from coords)
+    const float *coords;   // [n][2], layer 1 only
+    int64_t n;
+    int K, M, d_L;
+    int rotate;            // W8A32 with the Hadamard fold: rotate the layer input
+    int w8;                // 1: quantized weights (qw_k4m, s_w); 0: fp32 weights (w_f32)
+    const uint32_t *qw_k4m;
+    const float4 *w_f32;
+    const float *s_w, *bias;
+    float omega0;
+    int sine;
+    float *Y;              // [n][M] or NULL
+    float *out;            // [n][d_L] or NULL (last layer)
+    float *dX;             // dump of the layer input, or NULL
+};
+cudaError_t launch_float_layer(const FloatLayerArgs &a, cudaStream_t st);
+cudaError_t launch_prep_float_weights(const float *W, int d_out, int d_in, int K, int M, float *dst, cudaStream_t st);
 struct FloatPrepArgs {
     const float *W;        // fp32 weights as given, [d_out][d_in]
     int d_out, d_in, K, M;
@@ -140,7 +160,8 @@ struct FloatPrepArgs {
     int rotate;            // w8: the codes are those of rotated weights
     int first;             // layer 1: weights and bias in turns of the phase
     int hidden;            // 1: base-256 digits for the tensor cores; 0: fp32 (last layer)
-    int digits;            // hidden: 2 or 3, or 0 to only take the largest |value| (w8) into *row_max
+    int digits;            // hidden: 2 or 3, or 0 to only take the largest |value| (w8) into *row_max, and per row the
+                           // sum of squares and the largest square of the weights into dev.cA and dev.cA_lo
     unsigned int *row_max;
     double omega0;
     LayerDev dev;
@@ -152,7 +173,12 @@ struct PrepSums {
     float phase_bound[kMaxLayers];
     unsigned long long code_l1[kMaxLayers]; // sum over the layer of |q_w[m][k]| (bounds the rotated accumulators)
     unsigned int row_max;                   // see FloatPrepArgs
+    // floating-point datapaths, per layer (see fixed_point_serves): sums over the rows of |W_m|^2, of max W_m^2 and of
+    // cos(2 omega0 b_m), the largest max W_m^2 / |W_m|^2, and whether all weights and biases are finite
+    double row_sq[kMaxLayers], row_top[kMaxLayers], cos_bias[kMaxLayers], worst_top[kMaxLayers];
+    int finite;
 };
+cudaError_t launch_prep_float_sums(int L, double omega0, const LayerDev *layers, PrepSums *sums, cudaStream_t st, int64_t *launches);
 // The weight side of a whole network: every kernel covers all layers.
 struct PrepNet {
     int L, w;

@@ -77,7 +77,7 @@ def test_destroy_waits_for_the_handles_device(run):
     """)
 
 
-@pytest.mark.parametrize("kw", ["", "w_bits=32, a_bits=32", "width=128, w_gran=1, a_gran=1, rotation=1"])
+@pytest.mark.parametrize("kw", ["", "width=512, w_gran=1, a_gran=1", "width=128, w_gran=1, a_gran=1, rotation=1"])
 def test_only_a_launch_behind_an_ordinary_one_in_its_stream_is_early(run, kw):
     run(f"""
     h = prepare({kw})
@@ -86,7 +86,7 @@ def test_only_a_launch_behind_an_ordinary_one_in_its_stream_is_early(run, kw):
     forward(h, 32); assert early() == 0                    # another stream: not behind those
     forward(h, 32); assert early() == 1
     forward(h, 16); assert early() == 0
-    if {'w_bits' not in kw and 'a_gran=1' not in kw}:
+    if {"a_gran=1" not in kw}:
         calibrate(h, 16); set_("capturing", 1); forward(h, 48); assert early() == 0   # only recorded
         set_("capturing", 0); forward(h, 48); assert early() == 0
         calibrate(h, 16); set_("fail_launch", 1); forward(h, 16, expect=4)             # enqueued nothing
