@@ -139,8 +139,9 @@ bool takes_digits(const dhq_config_t &cfg, int w)
     return cfg.rotation == DHQ_ROT_BOTH && cfg.w_gran == DHQ_GRAN_CHANNEL_OR_TOKEN && (w == 128 || w == 256);
 }
 
-// Lays the handle's arrays out in one block (h->device is current).  At its start, zeroed on `st`: the
-// status words, what the preparation accumulates, and the layers' activation scales.
+// Lays the handle's arrays out in one block (h->device is current) and zeroes it on `st`: the status words, what the
+// preparation accumulates and the layers' activation scales begin at zero, and parts of arrays that a handle does not
+// use must not carry another network's numbers from a block used before into dhq_export.
 dhq_status_t alloc_handle(dhq_handle_s *h, cudaStream_t st)
 {
     auto place = [&](uint8_t *base) {
@@ -153,7 +154,6 @@ dhq_status_t alloc_handle(dhq_handle_s *h, cudaStream_t st)
         put((void **)&h->d_prep, sizeof(PrepSums));
         void *acts = nullptr;
         put(&acts, 16 * h->L);
-        h->zero_bytes = off;
         if (h->layer[0].has_digits) put((void **)&h->g_scratch, digit_scratch_bytes(h));
         put((void **)&h->x_scratch, h->float_mode ? float_scratch_bytes(h) : 0);
         for (int l = 0; l < h->L; ++l) {
@@ -164,10 +164,11 @@ dhq_status_t alloc_handle(dhq_handle_s *h, cudaStream_t st)
         }
         return off;
     };
-    h->block = pool_take(place(nullptr), h->device, &h->block_bytes);
+    const size_t bytes = place(nullptr);
+    h->block = pool_take(bytes, h->device, &h->block_bytes);
     if (!h->block) return DHQ_ERR_ALLOC;
     place(static_cast<uint8_t *>(h->block));
-    CK(cudaMemsetAsync(h->block, 0, h->zero_bytes, st));
+    CK(cudaMemsetAsync(h->block, 0, bytes, st));
     return DHQ_OK;
 }
 

@@ -60,7 +60,7 @@ struct dhq_handle_s {
     int calib_layers_done = 0;      // layers whose per-tensor activation scale is frozen (sharded calibration)
     dhq::LayerDev layer[dhq::kMaxLayers];
     void *block = nullptr;          // the device memory of everything below up to the layers' arrays
-    size_t block_bytes = 0, zero_bytes = 0;
+    size_t block_bytes = 0;
     int *d_status = nullptr;        // device status word
     dhq::PrepSums *d_prep = nullptr; // accumulated by the preparation kernels
     uint8_t *x_scratch = nullptr;   // activations of the floating-point datapaths, see FloatParams

@@ -92,3 +92,14 @@ def test_only_a_launch_behind_an_ordinary_one_in_its_stream_is_early(run, kw):
         calibrate(h, 16); set_("fail_launch", 1); forward(h, 16, expect=4)             # enqueued nothing
         set_("fail_launch", 0); forward(h, 16); assert early() == 0
     """)
+
+
+def test_device_memory_is_cleared_before_a_handle_uses_it(run):
+    run("""
+    for kw in (dict(), dict(width=512, a_gran=1), dict(width=128, w_gran=1, a_gran=1, rotation=1)):
+        D.dhq_release_cached_memory(); log()
+        prepare(**kw)
+        got = log()
+        blocks, cleared = [a for w, _, a in got if w == "malloc"], [a for w, _, a in got if w == "memset"]
+        assert cleared[0] == blocks[0] and len(cleared) == len(blocks), got
+    """)

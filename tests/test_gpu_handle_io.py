@@ -118,3 +118,25 @@ def test_call_log_is_written_when_asked_for():
         assert ("[dhq] dhq_prepare" in r.stderr) == expect
         if expect:
             assert "-> ok" in r.stderr and "fused" in r.stderr
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kw,other", [(dict(a_bits=32), dict(w_bits=32, a_bits=32)), (dict(w_gran=1, a_gran=1, rotation=1), dict(w_gran=1, a_gran=1, rotation=1)),
+                                      (dict(), dict(a_gran=1)), (dict(w_bits=32, a_bits=32), dict(w_bits=32, a_bits=32))])
+def test_exported_bytes_hold_this_network_only(kw, other):
+    # device memory goes from a destroyed handle to the next one: what the next one does not write must not be in its block
+    dims = (2, 256, 256, 256, 3)
+    nets = [[[to_dev(x) for x in part] for part in dhq_inputs.siren_init(dims, 30.0, seed)] for seed in (1, 2)]
+
+    def export(net, options):
+        h = dhq.dhq_prepare(dims, *net, 30.0, **options)
+        try:
+            return dhq.dhq_export(h)
+        finally:
+            dhq.dhq_destroy(h)
+    dhq.dhq_release_cached_memory()
+    first = export(nets[0], kw)
+    for options in (other, kw):
+        for _ in range(3):
+            export(nets[1], options)
+        assert export(nets[0], kw) == first
