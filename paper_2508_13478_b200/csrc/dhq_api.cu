@@ -318,6 +318,11 @@ dhq_status_t calibrate_layer_pass(dhq_handle_s *h, int l, const float *coords, i
 
 dhq_status_t calibrate_impl(dhq_handle_s *h, const float *coords, int64_t n, cudaStream_t st)
 {
+    // what can run out of memory comes first: a call that fails with ALLOC leaves the scales as they were
+    if (!h->fused || ((uintptr_t)coords & 7)) {
+        const dhq_status_t s = ensure_scratch(h, n < kDebugChunk ? n : kDebugChunk);
+        if (s != DHQ_OK) return s;
+    }
     CK(cudaMemsetAsync(h->layer[0].act, 0, (size_t)h->L * 16, st)); // the layers' scales lie side by side
     for (int l = 1; l <= h->L; ++l) {
         dhq_status_t s = calibrate_layer_pass(h, l, coords, n, true, st);

@@ -103,3 +103,17 @@ def test_device_memory_is_cleared_before_a_handle_uses_it(run):
         blocks, cleared = [a for w, _, a in got if w == "malloc"], [a for w, _, a in got if w == "memset"]
         assert cleared[0] == blocks[0] and len(cleared) == len(blocks), got
     """)
+
+
+def test_a_calibration_that_cannot_allocate_leaves_the_scales(run):
+    run("""
+    h = prepare(width=128, w_gran=1, rotation=1)           # calibrates layer by layer, through scratch memory
+    D.dhq_get_act_absmax.argtypes = [vp, C.c_int, C.POINTER(C.c_float), vp]
+    D.dhq_set_act_absmax.argtypes = [vp, C.c_int, C.c_float, vp]
+    for l in range(1, 5):
+        assert D.dhq_set_act_absmax(h, l, 3.0, None) == 0
+    set_("fail_malloc", 1); calibrate(h, 16, expect=3); set_("fail_malloc", 0)
+    a = C.c_float()
+    for l in range(1, 5):
+        assert D.dhq_get_act_absmax(h, l, C.byref(a), None) == 0 and a.value == 3.0, (l, a.value)
+    """)
