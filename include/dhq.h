@@ -376,7 +376,9 @@ DHQ_API dhq_status_t dhq_last_status(dhq_handle_t h);
 DHQ_API dhq_status_t dhq_last_launch_clock(dhq_handle_t h, double *sm_mhz, double *milliseconds);
 
 /* The device memory of destroyed handles is kept for the next dhq_prepare / dhq_import of the process (at
- * most 8 blocks and 128 MiB in all).  This call gives it back to the device.  Safe from any thread. */
+ * most 8 blocks and 128 MiB in all).  This call gives it back to the device, and forgets which kernels the driver has
+ * been told about: a program that resets a device (cudaDeviceReset) destroys its handles and makes this call first.
+ * Safe from any thread. */
 DHQ_API void dhq_release_cached_memory(void);
 
 /* Number of kernels the library has launched for this handle since it was created. */

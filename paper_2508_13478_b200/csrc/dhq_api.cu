@@ -1041,7 +1041,11 @@ dhq_status_t dhq_last_launch_clock(dhq_handle_t h, double *sm_mhz, double *milli
     return DHQ_OK;
 }
 
-void dhq_release_cached_memory(void) { pool_free_all(); }
+void dhq_release_cached_memory(void)
+{
+    pool_free_all();
+    forget_allowed();
+}
 
 int64_t dhq_launch_count(dhq_handle_t h) { return h ? h->launches : 0; }
 

@@ -2,8 +2,6 @@
 // dhq_fused_w*.cu): the parameter block of a handle, the choice of the instantiation and the
 // launch; and the kernel's per-element loops run in isolation (micro-benchmark).
 #include <mutex>
-#include <set>
-#include <utility>
 #include "dhq_fused.cuh"
 
 namespace dhq {
@@ -187,20 +185,29 @@ static fused_dump_fn pick_dump_for(const dhq_handle_s *h, bool per_token)
 }
 
 // Lets a kernel use all of an SM's shared memory; the driver is asked once per kernel and device
-// (8 of these calls per dhq_prepare took 15 us).  A kernel whose warpgroups split its registers must have been
-// launched with at least min_regs a thread, or the split would wait for registers that do not exist.
+// (8 of these calls per dhq_prepare took 15 us; when the table is full, every time).  A kernel whose warpgroups split
+// its registers must have been launched with at least min_regs a thread, or the split would wait for registers that do
+// not exist.
+constexpr int kMaxAllowed = 512;
+static std::mutex g_allowed_mutex;
+static struct { const void *fn; int device; } g_allowed[kMaxAllowed];
+static int g_allowed_count = 0;
 bool allow_smem(const void *fn, int device, int bytes, int min_regs)
 {
-    static std::mutex mutex;
-    static std::set<std::pair<const void *, int>> done;
     if (!fn) return false;
-    std::lock_guard<std::mutex> lock(mutex);
-    if (done.count({fn, device})) return true;
+    std::lock_guard<std::mutex> lock(g_allowed_mutex);
+    for (int i = 0; i < g_allowed_count; ++i)
+        if (g_allowed[i].fn == fn && g_allowed[i].device == device) return true;
     cudaFuncAttributes at;
     if (min_regs > 0 && (cudaFuncGetAttributes(&at, fn) != cudaSuccess || at.numRegs < min_regs)) return false;
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
-    done.insert({fn, device});
+    if (g_allowed_count < kMaxAllowed) g_allowed[g_allowed_count++] = {fn, device};
     return true;
+}
+void forget_allowed()
+{
+    std::lock_guard<std::mutex> lock(g_allowed_mutex);
+    g_allowed_count = 0;
 }
 
 // A forward launch.  Once an ordinary launch has followed the preparation and calibration in a stream (so that

@@ -241,6 +241,7 @@ __host__ __device__ inline int fused_feature(int col, int W)
 }
 // Lets a kernel use `bytes` of dynamic shared memory on `device` (asked of the driver once).
 bool allow_smem(const void *fn, int device, int bytes, int min_regs = 0);
+void forget_allowed();
 // Launches a forward kernel, overlapping its set-up with the kernels before it where that is allowed.
 cudaError_t launch_after(dhq_handle_s *h, const void *fn, int grid, int threads, size_t smem, cudaStream_t st, void *params);
 // Fused tensor-core forward.

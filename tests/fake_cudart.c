@@ -35,7 +35,7 @@ int cudaMemset(void *d, int v, size_t n) { memset(d, v, n); return 0; }
 int cudaMemsetAsync(void *d, int v, size_t n, void *st) { (void)st; memset(d, v, n); note("memset", (long)n); return 0; }
 int cudaStreamSynchronize(void *st) { (void)st; return 0; }
 int cudaStreamIsCapturing(void *st, int *v) { (void)st; *v = g_capturing; return 0; }
-int cudaFuncSetAttribute(const void *f, int a, int v) { (void)f; (void)a; (void)v; return 0; }
+int cudaFuncSetAttribute(const void *f, int a, int v) { (void)f; (void)a; note("attribute", v); return 0; }
 struct attributes { size_t a, b, c; int max_threads, regs; char rest[256]; };
 int cudaFuncGetAttributes(struct attributes *at, const void *f) { (void)f; at->regs = 96; return 0; }
 int cudaLaunchKernel(const void *f, unsigned long long g0, unsigned g1, unsigned long long b0, unsigned b1, void **args, size_t smem, void *st)

@@ -117,3 +117,16 @@ def test_a_calibration_that_cannot_allocate_leaves_the_scales(run):
     for l in range(1, 5):
         assert D.dhq_get_act_absmax(h, l, C.byref(a), None) == 0 and a.value == 3.0, (l, a.value)
     """)
+
+
+def test_releasing_cached_memory_forgets_what_a_device_was_told(run):
+    # a program that resets the device starts from nothing: no kept block, no kernel attribute taken for granted
+    run("""
+    h = prepare(); first = [w for w, _, _ in log()].count("attribute")
+    assert first > 0
+    D.dhq_destroy(h); prepare(); assert "attribute" not in [w for w, _, _ in log()]
+    D.dhq_release_cached_memory(); log()
+    prepare()
+    names = [w for w, _, _ in log()]
+    assert names.count("attribute") == first and "malloc" in names, names
+    """)
