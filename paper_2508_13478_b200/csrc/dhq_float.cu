@@ -242,8 +242,10 @@ __device__ void float_epilogue(const FloatParams &p, const FloatMap &sm, uint32_
                 q[0] = x; q[1] = yc; q[2] = 0.f; q[3] = 0.f;
             }
         }
+        // (NaN where a coordinate is not finite: digits cannot carry it to the result)
+        const float zero = __fadd_rn(fabsf(__fmul_rn(x, 0.f)), fabsf(__fmul_rn(yc, 0.f)));
 #pragma unroll
-        for (int m = 0; m < 4; ++m) part[m] = 0.f;
+        for (int m = 0; m < 4; ++m) part[m] = zero;
         // (with hidden layers, the first layer of every tile but the first was done beside the tile before)
         if (tile == blockIdx.x || p.L == 2) {
 #pragma unroll 1

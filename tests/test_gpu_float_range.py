@@ -116,3 +116,25 @@ def test_weights_that_are_not_finite_reach_the_result(w_bits, value):
             assert not torch.isfinite(out[:, 0]).any()
         finally:
             dhq.dhq_destroy(h)
+
+
+@pytest.mark.parametrize("width,w_bits,n_hidden", [(64, 32, 3), (128, 8, 2), (256, 32, 1), (512, 8, 3)])
+def test_coordinates_that_are_not_finite_reach_the_result(width, w_bits, n_hidden):
+    dims, W, B = _network("default", width, n_hidden)
+    coords = dhq_inputs.grid_coords(200, 150)
+    bad = coords.copy()
+    rows = np.arange(5, len(bad), 997)
+    bad[rows, rows % 2] = np.where(rows % 3 == 0, np.nan, np.where(rows % 3 == 1, np.inf, -np.inf)).astype(np.float32)
+    h = _prepare(dims, W, B, w_bits)
+    try:
+        out, want = torch.zeros((len(bad), 3), device="cuda"), torch.zeros((len(bad), 3), device="cuda")
+        dhq.dhq_forward(h, to_dev(coords), want)
+        dhq.dhq_forward(h, to_dev(bad), out)
+        torch.cuda.synchronize()
+        assert dhq.dhq_last_status(h) == 0
+    finally:
+        dhq.dhq_destroy(h)
+    got, want = out.cpu().numpy(), want.cpu().numpy()
+    assert np.isnan(got[rows]).all()
+    rest = np.setdiff1d(np.arange(len(bad)), rows)
+    assert np.array_equal(got[rest].view(np.uint32), want[rest].view(np.uint32))
