@@ -274,7 +274,7 @@ DHQ_API dhq_status_t dhq_forward_fused_debug(dhq_handle_t h, const float *coords
                                              const dhq_debug_bufs_t *bufs, void *stream);
 
 /*
- * Bound of the waits inside the fused kernel.  Its warps hand tiles to each other through
+ * Bound of the waits inside the one-launch kernels.  Their warps hand tiles to each other through
  * barriers in shared memory; every such wait gives up after this long, the kernel then records
  * DHQ_ERR_TIMEOUT in the handle's status word (dhq_last_status), releases what it holds and
  * returns, so that a stall never holds the GPU.  Default 2 s; at least 1000 ns.  Takes effect
@@ -284,12 +284,12 @@ DHQ_API dhq_status_t dhq_forward_fused_debug(dhq_handle_t h, const float *coords
 DHQ_API dhq_status_t dhq_set_wait_limit(dhq_handle_t h, int64_t nanoseconds);
 
 /*
- * Test hook for that bound: the next fused-kernel launch of this handle (dhq_forward or the
- * pinned route of dhq_forward_host) leaves out the copy of the last layer's weights into shared
- * memory.  Nothing is in flight for the missing piece; the warps that wait for it run into the
+ * Test hook for that bound: the next forward launch of this handle's one-launch kernel (dhq_forward or the
+ * pinned route of dhq_forward_host) leaves out one copy of weights into shared memory (the last layer's; the
+ * floating-point kernel, which has none there: the first of a hidden layer).  Nothing is in flight for the missing piece; the warps that wait for it run into the
  * wait limit, the kernel returns, `out` holds unspecified values and dhq_last_status reports
  * DHQ_ERR_TIMEOUT.  Later launches are normal.  Set a short limit first (dhq_set_wait_limit).
- * UNSUPPORTED for a handle without a fused kernel (one that runs layer by layer).
+ * UNSUPPORTED for a handle that runs layer by layer or, floating-point, has no hidden layer but the first.
  */
 DHQ_API dhq_status_t dhq_debug_stall_next_forward(dhq_handle_t h);
 

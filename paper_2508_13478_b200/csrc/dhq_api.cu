@@ -759,7 +759,7 @@ dhq_status_t dhq_set_wait_limit(dhq_handle_t h, int64_t nanoseconds)
 dhq_status_t dhq_debug_stall_next_forward(dhq_handle_t h)
 {
     if (!h) return DHQ_ERR_INVALID_ARG;
-    if (!h->fused) return DHQ_ERR_UNSUPPORTED;
+    if (!h->fused && !h->digit_state && !(h->float_state && h->L > 2)) return DHQ_ERR_UNSUPPORTED; // no weight copies to leave out
     h->stall_next_forward = true;
     return DHQ_OK;
 }

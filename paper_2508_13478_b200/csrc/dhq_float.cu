@@ -46,6 +46,7 @@ struct FloatParams {
     float *out;
     long long n, n_tiles;
     int L, d_L, n_stages;
+    int skip_first_weights;                  // test hook: see dhq_debug_stall_next_forward
     int *status;
     unsigned long long wait_limit_ns;
     uint8_t *x;                              // [gridDim.x][3][W/16][128][16]: the digits of a tile's activations
@@ -424,7 +425,7 @@ __device__ void float_load_weights(const FloatParams &p, const FloatMap &sm, uin
     for (long long tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
         for (int l = 2; l < p.L && ok; ++l) {
             for (int q = 0; q < PIECES; ++q, ++i) {
-                if ((int)(i % kFLoaders) != which) continue;
+                if ((int)(i % kFLoaders) != which || (p.skip_first_weights && i == 0)) continue;
                 if (i >= (uint32_t)p.n_stages && i < (uint32_t)p.n_stages + kFLoaders) ptx::wait_for_previous_kernels();
                 const uint32_t stage = i % (uint32_t)p.n_stages, par = ((i / (uint32_t)p.n_stages) & 1) ^ 1;
                 if (!wait_bar<0, kHintNs>(base + sm.w_empty + 8 * stage, par, abort_flag, p.status)) { ok = false; break; }
@@ -767,6 +768,10 @@ dhq_status_t float_forward(dhq_handle_s *h, const float *coords, int64_t n, floa
     p.coords = coords; p.out = out; p.n = n;
     p.n_tiles = (n + kTile - 1) / kTile;
     p.wait_limit_ns = h->wait_limit_ns;
+    if (!bufs && h->stall_next_forward) { // test hook, one launch only
+        p.skip_first_weights = 1;
+        h->stall_next_forward = false;
+    }
     bool dump = !out;
     if (bufs) {
         for (int l = 0; l < h->L; ++l) {
