@@ -133,7 +133,7 @@ size_t digit_scratch_bytes(const dhq_handle_s *h)
 }
 
 // The two-sided transform with a weight scale per output channel has a kernel at these widths (at 512 the
-// activations and the digits' sums do not fit tensor memory together; 64 has too few columns per thread).
+// activations and the digits' sums do not fit tensor memory together; for 64 it is not built).
 bool takes_digits(const dhq_config_t &cfg, int w)
 {
     return cfg.rotation == DHQ_ROT_BOTH && cfg.w_gran == DHQ_GRAN_CHANNEL_OR_TOKEN && (w == 128 || w == 256);
@@ -394,7 +394,7 @@ dhq_status_t run_forward(dhq_handle_s *h, const float *coords, int64_t n, float 
     if (h->float_state) return float_forward(h, coords, n, out, nullptr, st);
     if (h->float_mode) return float_layers_forward(h, coords, n, out, nullptr, st);
     if (h->digit_state) return digit_forward(h, coords, n, out, st);
-    if (!h->fused) return layerwise_forward(h, coords, n, out, st); // wavelet activation; two-sided transform with per-channel weight scales
+    if (!h->fused) return layerwise_forward(h, coords, n, out, st); // two-sided transform where no kernel for all layers takes it
     return fused_forward(h, coords, n, out, on_host, st);
 }
 
@@ -612,8 +612,8 @@ static dhq_status_t prepare_impl(const dhq_config_t *cfg, const float *const *W,
             else d.epi_mode = (!gabor && !h->float_mode && ((a_per_token && !both) || both_fused)) ? EPI_SINE_MIXED : EPI_SINE_WIDE;
         }
         h->calibrated = per_token;
-        // layer by layer: the fp32 datapaths, the two-sided transform with per-channel weight scales, and the
-        // wavelet combined with the two-sided transform
+        // layer by layer: the two-sided transform with per-channel weight scales at widths 64 and 512 or with sums that
+        // could overflow, and the floating-point networks that fixed point does not serve
         if (h->float_mode) rc = h->float_digits ? float_create(h) : DHQ_OK;
         else if (h->layer[0].has_digits) rc = digit_create(h);
         else if (!both || both_fused) rc = fused_create(h);
@@ -1065,7 +1065,7 @@ static void log_call(const char *fn, dhq_handle_t h, int64_t n, int64_t launches
     if (!h) { fprintf(stderr, "[dhq] %s n=%lld -> %s\n", fn, (long long)n, dhq_status_string(s)); return; }
     fprintf(stderr, "[dhq] %s n=%lld (L=%d w=%d d_L=%d W%dA%d rot=%d gran=%d/%d%s) -> %s, %lld kernel(s)\n", fn, (long long)n,
             h->L, h->w, h->d_L, h->cfg.w_bits, h->cfg.a_bits, (int)h->cfg.rotation, (int)h->cfg.w_gran, (int)h->cfg.a_gran,
-            h->fused ? ", fused" : ", layer by layer", dhq_status_string(s), (long long)(h->launches - launches_before));
+            h->fused ? ", fused" : h->digit_state || h->float_state ? ", one launch" : ", layer by layer", dhq_status_string(s), (long long)(h->launches - launches_before));
 }
 
 dhq_status_t dhq_prepare(const dhq_config_t *cfg, const float *const *W, const float *const *b, void *stream, dhq_handle_t *out)

@@ -75,9 +75,9 @@ struct dhq_handle_s {
     bool pipe_ready = false;
     int64_t launches = 0;
     void *fused = nullptr;          // state of the fused path (device parameter block)
-    unsigned long long wait_limit_ns = 2000000000ull; // bound of every wait inside the fused kernel (dhq_set_wait_limit)
+    unsigned long long wait_limit_ns = 2000000000ull; // bound of every wait inside the one-launch kernels (dhq_set_wait_limit)
     bool stall_next_forward = false; // test hook: see dhq_debug_stall_next_forward
-    double gabor_s0 = 0.0;          // > 0: wavelet activation (layer-by-layer path)
+    double gabor_s0 = 0.0;          // > 0: wavelet activation
     void *digit_state = nullptr;    // state of the two-sided kernel for per-channel weight scales
     double *g_scratch = nullptr;    // its matrices in fp64 (used by the preparation only)
     void *float_state = nullptr;    // state of the floating-point datapaths
