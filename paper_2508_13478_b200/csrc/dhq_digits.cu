@@ -141,7 +141,7 @@ __device__ __forceinline__ bool digit_finish(SlotCtx &c, float static_s, float s
         scales_of(amax, c.qmaxf, s_out, inv);
     }
 #pragma unroll
-    for (int ch = 0; ch < 4; ++ch) quantize_store<G, CH, !PER_TOKEN>(c.a_tile, c.row, ch, c.sub * G, u[ch], inv, c.qmaxf);
+    for (int ch = 0; ch < 4; ++ch) quantize_store<G, !PER_TOKEN>(c.a_tile, c.row, ch * CH + c.sub * G, u[ch], inv, c.qmaxf);
     ptx::fence_proxy_async();
     ptx::tc_fence_before();
     ptx::mbar_arrive(c.bar_codes);
@@ -201,7 +201,7 @@ __device__ void digit_epilogue(const DigitParams &p, const DigitMap &sm, uint32_
         for (int i = 0; i < 8; ++i) unpack2u(P[i], v[2 * i], v[2 * i + 1]);
         ptx::tmem_st16(c.taddr + sub * CH + b * 16, v);
     };
-    // stages 8 .. CH/2 of the thread's own chunk
+    // stages 8 .. CH/2 of the thread's own chunk, which is then in feature order
     auto chunk_stages = [&]() {
         uint32_t v[CH];
         ptx::tmem_wait_st();
@@ -220,8 +220,8 @@ __device__ void digit_epilogue(const DigitParams &p, const DigitMap &sm, uint32_
         for (int i = 0; i < CH / 2; ++i) {
             float a, b;
             unpack2(P[i], a, b);
-            v[2 * i] = __float_as_uint(__fadd_rn(a, b));
-            v[2 * i + 1] = __float_as_uint(__fsub_rn(a, b));
+            v[i] = __float_as_uint(__fadd_rn(a, b));
+            v[i + CH / 2] = __float_as_uint(__fsub_rn(a, b));
         }
         tmem_st<CH>(c.taddr + sub * CH, v);
     };

@@ -513,7 +513,7 @@ template <int WHICH> __global__ void __launch_bounds__(512, 1) pass_rate_kernel(
                 }
 #pragma unroll
                 for (int ch = 0; ch < NCH; ++ch)
-                    quantize_store<G, CH, true>(base + slot * (kTile * W), quad * 32 + lane, ch, g * G, u[ch], 1e-3f, 127.f);
+                    quantize_store<G, true>(base + slot * (kTile * W), quad * 32 + lane, ch * CH + g * G, u[ch], 1e-3f, 127.f);
             }
         }
     }
