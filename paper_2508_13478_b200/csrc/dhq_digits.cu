@@ -56,6 +56,7 @@ struct DigitParams {
     int L, d_L, n_stages;
     int skip_last_weights;           // test hook: see dhq_debug_stall_next_forward
     float qmaxf;
+    float2 one2;                     // {1, 1}: see code_bits2
     double gabor_c;                  // see digit_envelope; 0 for the sine
     int *status;
     unsigned long long wait_limit_ns;
@@ -128,7 +129,7 @@ __device__ __forceinline__ bool digit_finish(SlotCtx &c, float static_s, float s
 #pragma unroll
         for (int ch = 0; ch < 4; ++ch) {
 #pragma unroll
-            for (int i = 0; i < G; ++i) amax = fmaxf(amax, fabsf(__uint_as_float(u[ch][i])));
+            for (int i = 0; i < G; i += 2) amax = max_abs(amax, __uint_as_float(u[ch][i]), __uint_as_float(u[ch][i + 1]));
         }
         asm volatile("st.shared.f32 [%0], %1;" ::"r"(c.amax_addr + (c.sub * kTile + c.row) * 4), "f"(amax) : "memory");
         if (!slot_barrier<true>(c)) return false;
@@ -141,7 +142,7 @@ __device__ __forceinline__ bool digit_finish(SlotCtx &c, float static_s, float s
         scales_of(amax, c.qmaxf, s_out, inv);
     }
 #pragma unroll
-    for (int ch = 0; ch < 4; ++ch) quantize_store<G, !PER_TOKEN>(c.a_tile, c.row, ch * CH + c.sub * G, u[ch], inv, c.qmaxf);
+    for (int ch = 0; ch < 4; ++ch) quantize_store<G, !PER_TOKEN>(c.a_tile, c.row, ch * CH + c.sub * G, u[ch], inv, c.qmaxf, c.one2);
     ptx::fence_proxy_async();
     ptx::tc_fence_before();
     ptx::mbar_arrive(c.bar_codes);
@@ -163,6 +164,7 @@ __device__ void digit_epilogue(const DigitParams &p, const DigitMap &sm, uint32_
     c.amax_addr = base + sm.amax;
     c.sync_parity = 0;
     c.qmaxf = p.qmaxf;
+    c.one2 = pack2(p.one2.x, p.one2.y);
     c.abort_flag = abort_flag;
     c.status = p.status;
     const uint32_t acc = tmem + ((uint32_t)(quad * 32) << 16) + sub * 16;
@@ -560,6 +562,7 @@ dhq_status_t digit_create(dhq_handle_s *h)
     DigitParams &p = ds->p;
     p.L = h->L; p.d_L = h->d_L;
     p.qmaxf = (float)((1 << (h->cfg.a_bits - 1)) - 1);
+    p.one2 = make_float2(1.0f, 1.0f);
     p.gabor_c = digit_gabor_c(h->gabor_s0, (double)h->cfg.omega0);
     p.status = h->d_status;
     for (int l = 0; l < h->L; ++l) {

@@ -259,6 +259,7 @@ dhq_status_t fused_create(dhq_handle_s *h)
     p.L = h->L; p.W = h->w; p.d_L = h->d_L;
     p.per_token = h->cfg.a_gran == DHQ_GRAN_CHANNEL_OR_TOKEN;
     p.qmaxf = (float)((1 << (h->cfg.a_bits - 1)) - 1);
+    p.one2 = make_float2(1.0f, 1.0f);
     p.status = h->d_status;
     const bool both = h->cfg.rotation == DHQ_ROT_BOTH;
     const bool gabor = h->gabor_s0 > 0.0;
@@ -513,7 +514,7 @@ template <int WHICH> __global__ void __launch_bounds__(512, 1) pass_rate_kernel(
                 }
 #pragma unroll
                 for (int ch = 0; ch < NCH; ++ch)
-                    quantize_store<G, true>(base + slot * (kTile * W), quad * 32 + lane, ch * CH + g * G, u[ch], 1e-3f, 127.f);
+                    quantize_store<G, true>(base + slot * (kTile * W), quad * 32 + lane, ch * CH + g * G, u[ch], 1e-3f, 127.f, 0);
             }
         }
     }

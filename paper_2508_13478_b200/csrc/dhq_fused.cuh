@@ -132,6 +132,7 @@ struct FusedParams {
     long long n, n_tiles;
     int L, W, d_L, per_token;
     float qmaxf;
+    float2 one2;         // {1, 1}: see code_bits2
     int n_stages, resident;
     int bulk_xy;         // coords 16-byte aligned: whole tiles may arrive by bulk copy (width 512)
     int bulk_out;        // out 16-byte aligned: whole tiles may leave by bulk store (host-buffer variant)
@@ -283,26 +284,66 @@ __device__ __forceinline__ void bfly2(f32x2 &a, f32x2 &b)
     b = sub2(x, y);
 }
 
+// max(m, |a|, |b|), one instruction (NaN is dropped, as by fmaxf).
+__device__ __forceinline__ float max_abs(float m, float a, float b)
+{
+    asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(m) : "f"(a), "f"(b));
+    return m;
+}
+
+// The epilogues of dhq_math.cuh on two columns at once: packed multiplies, additions and fused multiply-adds in the
+// same order give the same bits with half the issue slots.  Per-token scales at width 256, with the one-instruction maxima
+// and the group kept in registers by finish_layer: 262,144 coordinates, 5 layers 260 -> 244 us, 1,048,576 in 4-bit
+// codes 1,031 -> 972; wavelet without rotation at width 128, 267,007 coordinates, 4 layers 147 -> 126.
+__device__ __forceinline__ f32x2 sine2(f32x2 x)
+{
+    float a, b;
+    unpack2(x, a, b);
+    return pack2(sin_approx(a), sin_approx(b));
+}
+__device__ __forceinline__ f32x2 sin_wide2(f32x2 x)
+{
+    const f32x2 magic = pack2(12582912.0f, 12582912.0f);
+    const f32x2 k = sub2(fma2(x, pack2(0.15915494309189535f, 0.15915494309189535f), magic), magic);
+    f32x2 r = fma2(k, pack2(-6.2831854820251465f, -6.2831854820251465f), x);
+    r = fma2(k, pack2(1.7484555e-07f, 1.7484555e-07f), r);
+    return sine2(r);
+}
+__device__ __forceinline__ void token_const2(f32x2 cA, f32x2 cA_lo, f32x2 s_x, f32x2 neg_s_x, f32x2 &c_hi, f32x2 &c_lo)
+{
+    c_hi = mul2(cA, s_x);
+    c_lo = fma2(cA_lo, s_x, fma2(cA, s_x, mul2(cA, neg_s_x))); // (cA times -s_x is -c_hi)
+}
+__device__ __forceinline__ f32x2 gabor_wide2(f32x2 x, float c)
+{
+    const f32x2 g = mul2(x, pack2(c, c));
+    float a, b;
+    unpack2(mul2(mul2(g, g), pack2(-1.4426950408889634f, -1.4426950408889634f)), a, b);
+    float y0, y1;
+    unpack2(sin_wide2(x), y0, y1);
+    // (scalar products: additions follow, see code_bits2)
+    return pack2(__fmul_rn(y0, gabor_envelope(a)), __fmul_rn(y1, gabor_envelope(b)));
+}
+
 // Round-half-even of two values to integer codes held in the low bytes: multiply by inv,
 // (clamp,) add 1.5 * 2^23 - the sum rounds to the integer grid, ties to even, and its low
 // mantissa bits are the two's complement code.  Same integers as
 // __float2int_rn(clamp(v * inv, -qmax, qmax)).  With a per-token scale |v * inv| <= qmax
 // (1 + 2^-23) already, so the clamp is skipped.  The clamp is sign(t) * min(|t|, qmax).
-template <bool CLAMP> __device__ __forceinline__ void code_bits2(f32x2 v, f32x2 inv2, float qmaxf, uint32_t &b0, uint32_t &b1)
+template <bool CLAMP> __device__ __forceinline__ void code_bits2(f32x2 v, f32x2 inv2, float qmaxf, f32x2 one2, uint32_t &b0, uint32_t &b1)
 {
     f32x2 t = mul2(v, inv2);
-    float lo, hi;
-    unpack2(t, lo, hi);
     if (CLAMP) {
+        float lo, hi;
+        unpack2(t, lo, hi);
         asm("min.xorsign.abs.f32 %0, %0, %1;" : "+f"(lo) : "f"(qmaxf));
         asm("min.xorsign.abs.f32 %0, %0, %1;" : "+f"(hi) : "f"(qmaxf));
         unpack2u(add2(pack2(lo, hi), pack2(12582912.0f, 12582912.0f)), b0, b1);
     } else {
-        // Scalar adds here: a packed multiply directly followed by a packed add was observed to be
-        // merged into one fused multiply-add by the assembler, which rounds v * inv only once and
-        // turns exact ties (x.5) the wrong way.  The product must be rounded to fp32 first.
-        b0 = __float_as_uint(__fadd_rn(lo, 12582912.0f));
-        b1 = __float_as_uint(__fadd_rn(hi, 12582912.0f));
+        // A packed multiply directly followed by a packed add was observed to be merged into one fused multiply-add by the
+        // assembler, which rounds v * inv only once and turns exact ties (x.5) the wrong way.  The product must be rounded
+        // to fp32 first: a multiply-add with a one that the assembler does not know takes the place of the addition.
+        unpack2u(fma2(t, one2, pack2(12582912.0f, 12582912.0f)), b0, b1);
     }
 }
 template <bool CLAMP> __device__ __forceinline__ uint32_t code_bits(float v, float inv, float qmaxf)
@@ -334,7 +375,7 @@ template <int N> __device__ __forceinline__ void store_code_words(uint32_t a_til
 // sixteen consecutive codes of a row are one conflict-free 16-byte store, where two runs of eight cost the same
 // wavefronts each (pass 2 alone at width 256 5.66 -> 4.91 cycles per 32 elements and scheduler).
 template <int G, bool CLAMP, bool DUMP = false, bool DUP = false>
-__device__ __forceinline__ void quantize_store(uint32_t a_tile, int row, int k0, const uint32_t *u, float inv, float qmaxf,
+__device__ __forceinline__ void quantize_store(uint32_t a_tile, int row, int k0, const uint32_t *u, float inv, float qmaxf, f32x2 one2,
                                                int8_t *dump_row = nullptr)
 {
     constexpr int N = G < 16 ? G : 16;
@@ -343,7 +384,7 @@ __device__ __forceinline__ void quantize_store(uint32_t a_tile, int row, int k0,
     for (int s = 0; s < G; s += N) {
         uint32_t b[N], w[N / 4];
 #pragma unroll
-        for (int k = 0; k < N; k += 2) code_bits2<CLAMP>(pack2u(u[s + k], u[s + k + 1]), inv2, qmaxf, b[k], b[k + 1]);
+        for (int k = 0; k < N; k += 2) code_bits2<CLAMP>(pack2u(u[s + k], u[s + k + 1]), inv2, qmaxf, one2, b[k], b[k + 1]);
 #pragma unroll
         for (int j = 0; j < N / 4; ++j) w[j] = pack4(b[4 * j], b[4 * j + 1], b[4 * j + 2], b[4 * j + 3]);
         store_code_words<N>(a_tile, row, k0 + s, w);
@@ -472,42 +513,50 @@ __device__ __forceinline__ void hidden_chunk(uint32_t cbase, int m0, float s_x, 
                                              float gabor_c = 0.f, [[maybe_unused]] float *xmax = nullptr, [[maybe_unused]] float limit = 0.f)
 {
     [[maybe_unused]] float xm = 0.f;
+    [[maybe_unused]] const f32x2 s2 = pack2(s_x, s_x), ns2 = pack2(-s_x, -s_x);
     chunk_pipeline<CH, ROT, DUP>(v, [&](int j, f32x2 *out) {
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int i = 8 * j + 4 * q; // four columns = two pairs
             const float4 a = lds128(cbase + (m0 + i) * 4);
             const float4 b = lds128(cbase + (W + m0 + i) * 4);
-            if (MODE == EPI_SINE_FAST && !PER_TOKEN) {
-                // x = fma(acc, cA, cB) for two columns at once, then the sine of each
-                float x0, x1, x2, x3;
-                unpack2(fma2(pack2((float)(int)v[i], (float)(int)v[i + 1]), pack2(a.x, a.y), pack2(b.x, b.y)), x0, x1);
-                unpack2(fma2(pack2((float)(int)v[i + 2], (float)(int)v[i + 3]), pack2(a.z, a.w), pack2(b.z, b.w)), x2, x3);
-                if constexpr (TRACK) xm = fmaxf(xm, fmaxf(fmaxf(fabsf(x0), fabsf(x1)), fmaxf(fabsf(x2), fabsf(x3))));
-                out[2 * q] = pack2(sin_approx(x0), sin_approx(x1));
-                out[2 * q + 1] = pack2(sin_approx(x2), sin_approx(x3));
-            } else {
-                float4 lo = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (MODE == EPI_SINE_WIDE || MODE == EPI_SINE_MIXED) lo = lds128(cbase + (2 * W + m0 + i) * 4);
+            const f32x2 acc01 = pack2((float)(int)v[i], (float)(int)v[i + 1]), acc23 = pack2((float)(int)v[i + 2], (float)(int)v[i + 3]);
+            f32x2 c01 = pack2(a.x, a.y), c23 = pack2(a.z, a.w);
+            const f32x2 b01 = pack2(b.x, b.y), b23 = pack2(b.z, b.w);
+            if constexpr (MODE == EPI_SINE_FAST) {
+                // x = fma(acc, c, cB) for two columns at once, then the sine of each
+                if constexpr (PER_TOKEN) { c01 = mul2(c01, s2); c23 = mul2(c23, s2); }
+                const f32x2 x01 = fma2(acc01, c01, b01), x23 = fma2(acc23, c23, b23);
+                out[2 * q] = sine2(x01);
+                out[2 * q + 1] = sine2(x23);
+                if constexpr (TRACK) {
+                    float x0, x1, x2, x3;
+                    unpack2(x01, x0, x1);
+                    unpack2(x23, x2, x3);
+                    xm = max_abs(max_abs(xm, x0, x1), x2, x3);
+                }
+            } else if constexpr (MODE == EPI_SINE_MIXED) {
+                const float4 lo = lds128(cbase + (2 * W + m0 + i) * 4);
                 const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w}, lv[4] = {lo.x, lo.y, lo.z, lo.w};
                 float y[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     float c_hi = av[e], c_lo = lv[e];
                     if (PER_TOKEN) token_const(av[e], lv[e], s_x, c_hi, c_lo);
-                    if constexpr (TRACK) { // EPI_SINE_FAST, keeping the phase
-                        const float x = __fmaf_rn((float)(int)v[i + e], c_hi, bv[e]);
-                        xm = fmaxf(xm, fabsf(x));
-                        y[e] = sin_approx(x);
-                    } else if constexpr (MODE == EPI_SINE_MIXED) {
-                        y[e] = epilogue_mixed((float)(int)v[i + e], c_hi, c_lo, bv[e], limit);
-                    } else {
-                        y[e] = GABOR ? gabor_epilogue((float)(int)v[i + e], c_hi, c_lo, bv[e], gabor_c)
-                                     : epilogue(MODE, (float)(int)v[i + e], c_hi, c_lo, bv[e]);
-                    }
+                    y[e] = epilogue_mixed((float)(int)v[i + e], c_hi, c_lo, bv[e], limit);
                 }
                 out[2 * q] = pack2(y[0], y[1]);
                 out[2 * q + 1] = pack2(y[2], y[3]);
+            } else {
+                const float4 lo = lds128(cbase + (2 * W + m0 + i) * 4);
+                f32x2 l01 = pack2(lo.x, lo.y), l23 = pack2(lo.z, lo.w);
+                if constexpr (PER_TOKEN) {
+                    token_const2(c01, l01, s2, ns2, c01, l01);
+                    token_const2(c23, l23, s2, ns2, c23, l23);
+                }
+                const f32x2 x01 = fma2(acc01, l01, fma2(acc01, c01, b01)), x23 = fma2(acc23, l23, fma2(acc23, c23, b23));
+                out[2 * q] = GABOR ? gabor_wide2(x01, gabor_c) : sin_wide2(x01);
+                out[2 * q + 1] = GABOR ? gabor_wide2(x23, gabor_c) : sin_wide2(x23);
             }
             if constexpr (DUMP) dump_y4<W>(dump_y, m0 + i, out[2 * q], out[2 * q + 1]);
         }
@@ -522,6 +571,7 @@ template <int W, int CH, bool PER_TOKEN, bool ROT, bool DUMP = false, bool BOTH 
 __device__ __forceinline__ void layer1_chunk(uint32_t cbase, int m0, int qs, int qd, uint32_t qx, float s_x, uint32_t (&v)[CH],
                                              float *dump_y = nullptr, float gabor_c = 0.f)
 {
+    [[maybe_unused]] const f32x2 s2 = pack2(s_x, s_x), ns2 = pack2(-s_x, -s_x);
     chunk_pipeline<CH, ROT, DUP>(v, [&](int j, f32x2 *out) {
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
@@ -530,11 +580,13 @@ __device__ __forceinline__ void layer1_chunk(uint32_t cbase, int m0, int qs, int
             const float4 B = lds128(cbase + (W + m0 + i) * 4);
             const float4 Cc = lds128(cbase + (2 * W + m0 + i) * 4);
             const float Av[4] = {A.x, A.y, A.z, A.w}, Bv[4] = {B.x, B.y, B.z, B.w}, Cv[4] = {Cc.x, Cc.y, Cc.z, Cc.w};
-            float y[4];
             if constexpr (!PER_TOKEN && !GABOR) {
+                float y[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
                     y[e] = sine_fixed(qs, qd, __float_as_uint(Av[e]), __float_as_uint(Cv[e]), __float_as_uint(Bv[e]));
+                out[2 * q] = pack2(y[0], y[1]);
+                out[2 * q + 1] = pack2(y[2], y[3]);
             } else {
                 const float4 wq = lds128(cbase + (3 * W + m0 + i) * 4);
                 const float wv[4] = {wq.x, wq.y, wq.z, wq.w};
@@ -542,19 +594,21 @@ __device__ __forceinline__ void layer1_chunk(uint32_t cbase, int m0, int qs, int
                 if constexpr (BOTH) wq2 = lds128(cbase + (4 * W + m0 + i) * 4);
                 const float wv2[4] = {wq2.x, wq2.y, wq2.z, wq2.w};
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    float c_hi = Av[e], c_lo = Cv[e]; // per-tensor scale (wavelet route): the constants hold s_x already
-                    if (PER_TOKEN) token_const(Av[e], Cv[e], s_x, c_hi, c_lo);
-                    // two-sided transform: areas D, E hold U' = H_M u and V' = H_M v (u, v: the sums of the weight
-                    // codes that meet the two distinct input codes), so acc' = qs U' + qd V' needs no butterfly
-                    const int acc = BOTH ? qs * (int)__float_as_uint(wv[e]) + qd * (int)__float_as_uint(wv2[e])
-                                         : __dp4a((int)qx, (int)__float_as_uint(wv[e]), 0);
+                for (int e = 0; e < 4; e += 2) {
+                    // per-tensor scale (wavelet route): the constants hold s_x already
+                    f32x2 c_hi = pack2(Av[e], Av[e + 1]), c_lo = pack2(Cv[e], Cv[e + 1]);
+                    if constexpr (PER_TOKEN) token_const2(c_hi, c_lo, s2, ns2, c_hi, c_lo);
+                    float acc[2];
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) // two-sided transform: areas D, E hold U' = H_M u and V' = H_M v (u, v: the sums of the
+                        // weight codes that meet the two distinct input codes), so acc' = qs U' + qd V' needs no butterfly
+                        acc[k] = (float)(BOTH ? qs * (int)__float_as_uint(wv[e + k]) + qd * (int)__float_as_uint(wv2[e + k])
+                                              : __dp4a((int)qx, (int)__float_as_uint(wv[e + k]), 0));
+                    const f32x2 a2 = pack2(acc[0], acc[1]), x = fma2(a2, c_lo, fma2(a2, c_hi, pack2(Bv[e], Bv[e + 1])));
                     // (the wavelet's envelope needs the unwrapped phase, which the fixed-point route does not have)
-                    y[e] = GABOR ? gabor_epilogue((float)acc, c_hi, c_lo, Bv[e], gabor_c) : epilogue(EPI_SINE_WIDE, (float)acc, c_hi, c_lo, Bv[e]);
+                    out[2 * q + e / 2] = GABOR ? gabor_wide2(x, gabor_c) : sin_wide2(x);
                 }
             }
-            out[2 * q] = pack2(y[0], y[1]);
-            out[2 * q + 1] = pack2(y[2], y[3]);
             if constexpr (DUMP) dump_y4<W>(dump_y, m0 + i, out[2 * q], out[2 * q + 1]);
         }
     });
@@ -570,6 +624,7 @@ struct SlotCtx {
     uint32_t sync_parity;
     int row, sub;
     float qmaxf;
+    f32x2 one2;          // {1, 1}, see code_bits2
     volatile int *abort_flag;
     int *status;
 };
@@ -591,6 +646,39 @@ template <class C> __device__ __forceinline__ int feature_of(int row, int pos)
     return (row & 16 ? C::HC / 2 : 0) + (pos < C::HC / 2 ? pos : pos - C::HC / 2 + C::CH / 2);
 }
 
+// One group: G positions of every chunk.
+template <class C> __device__ __forceinline__ void load_group(uint32_t taddr, uint32_t (&u)[C::NCH][C::G])
+{
+#pragma unroll
+    for (int ch = 0; ch < C::NCH; ++ch) tmem_ld<C::G>(taddr + ch * C::CH, u[ch]);
+    ptx::tmem_wait_ld();
+}
+// Butterfly stages with strides CH, 2 CH, ...: the chunk index is the butterfly index; two columns per instruction.
+template <class C, bool ROT> __device__ __forceinline__ void across_chunks(uint32_t (&u)[C::NCH][C::G])
+{
+#pragma unroll
+    for (int h = 1; h < (ROT ? C::NCH : 1); h <<= 1) {
+#pragma unroll
+        for (int ch = 0; ch < C::NCH; ++ch) {
+            if ((ch & h) == 0) {
+#pragma unroll
+                for (int i = 0; i < C::G; i += 2) {
+                    f32x2 a = pack2u(u[ch][i], u[ch][i + 1]), b = pack2u(u[ch + h][i], u[ch + h][i + 1]);
+                    bfly2(a, b);
+                    unpack2u(a, u[ch][i], u[ch][i + 1]);
+                    unpack2u(b, u[ch + h][i], u[ch + h][i + 1]);
+                }
+            }
+        }
+    }
+}
+template <int G> __device__ __forceinline__ float max_abs(float m, const uint32_t (&u)[G])
+{
+#pragma unroll
+    for (int i = 0; i < G; i += 2) m = max_abs(m, __uint_as_float(u[i]), __uint_as_float(u[i + 1]));
+    return m;
+}
+
 // Passes 2 and 3: remaining butterfly stages across chunks, quantizer, store of the codes, and the
 // arrival on the "codes ready" barrier.  Returns false if a wait ran out.  s_out receives the
 // token's activation scale of the next layer.
@@ -602,49 +690,41 @@ __device__ __forceinline__ bool finish_layer(SlotCtx &c, float static_s, float s
     ptx::tc_fence_before();
     if (!slot_barrier<PER_TOKEN>(c)) return false;
     ptx::tc_fence_after();
-    float amax = 0.f;
+    if constexpr (!PER_TOKEN) {
+        s_out = static_s;
 #pragma unroll 1
-    for (int gg = 0; gg < C::GPT; ++gg) {
-        const int g = c.sub * C::GPT + gg;
-        uint32_t u[NCH][G];
+        for (int gg = 0; gg < C::GPT; ++gg) {
+            const int g = c.sub * C::GPT + gg;
+            uint32_t u[NCH][G];
+            load_group<C>(c.taddr + g * G, u);
+            across_chunks<C, ROT>(u);
 #pragma unroll
-        for (int ch = 0; ch < NCH; ++ch) tmem_ld<G>(c.taddr + ch * CH + g * G, u[ch]);
-        ptx::tmem_wait_ld();
-        // strides CH, 2 CH, ...: the chunk index is the butterfly index; two columns per instruction
-#pragma unroll
-        for (int h = 1; h < (ROT ? NCH : 1); h <<= 1) {
-#pragma unroll
-            for (int ch = 0; ch < NCH; ++ch) {
-                if ((ch & h) == 0) {
-#pragma unroll
-                    for (int i = 0; i < G; i += 2) {
-                        f32x2 a = pack2u(u[ch][i], u[ch][i + 1]), b = pack2u(u[ch + h][i], u[ch + h][i + 1]);
-                        bfly2(a, b);
-                        unpack2u(a, u[ch][i], u[ch][i + 1]);
-                        unpack2u(b, u[ch + h][i], u[ch + h][i + 1]);
-                    }
-                }
-            }
+            for (int ch = 0; ch < NCH; ++ch) quantize_store<G, true, DUMP, C::DUP>(c.a_tile, c.row, ch * CH + feature_of<C>(c.row, g * G), u[ch], static_inv, c.qmaxf, c.one2, dump_codes);
         }
-        if (PER_TOKEN) {
+    } else {
+        // The row's absmax is combined over the threads that share it before anything can be quantized.  A thread's last
+        // group waits for that in registers, the ones before it in tensor memory.
+        float amax = 0.f;
+        uint32_t u[NCH][G];
+#pragma unroll 1
+        for (int gg = 0; gg < C::GPT - 1; ++gg) {
+            const int g = c.sub * C::GPT + gg;
+            load_group<C>(c.taddr + g * G, u);
+            across_chunks<C, ROT>(u);
 #pragma unroll
             for (int ch = 0; ch < NCH; ++ch) {
-#pragma unroll
-                for (int i = 0; i < G; ++i) amax = fmaxf(amax, fabsf(__uint_as_float(u[ch][i])));
+                amax = max_abs<G>(amax, u[ch]);
                 tmem_st<G>(c.taddr + ch * CH + g * G, u[ch]);
             }
-        } else {
-#pragma unroll
-            for (int ch = 0; ch < NCH; ++ch) quantize_store<G, true, DUMP, C::DUP>(c.a_tile, c.row, ch * CH + feature_of<C>(c.row, g * G), u[ch], static_inv, c.qmaxf, dump_codes);
         }
-    }
-    if (!PER_TOKEN) {
-        s_out = static_s;
-    } else {
-        // combine the row's absmax over the threads that share it
+        const int last = c.sub * C::GPT + C::GPT - 1;
+        load_group<C>(c.taddr + last * G, u);
+        across_chunks<C, ROT>(u);
+#pragma unroll
+        for (int ch = 0; ch < NCH; ++ch) amax = max_abs<G>(amax, u[ch]);
         if constexpr (C::DUP) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, 16));
         asm volatile("st.shared.f32 [%0], %1;" ::"r"(c.amax_addr + (c.sub * kTile + c.row) * 4), "f"(amax) : "memory");
-        ptx::tmem_wait_st();
+        if constexpr (C::GPT > 1) ptx::tmem_wait_st();
         ptx::tc_fence_before();
         if (!slot_barrier<PER_TOKEN>(c)) return false;
         ptx::tc_fence_after();
@@ -654,18 +734,16 @@ __device__ __forceinline__ bool finish_layer(SlotCtx &c, float static_s, float s
             asm volatile("ld.shared.f32 %0, [%1];" : "=f"(o) : "r"(c.amax_addr + (r * kTile + c.row) * 4));
             amax = fmaxf(amax, o);
         }
-        float s, inv;
-        scales_of(amax, c.qmaxf, s, inv);
-        s_out = s;
+        float inv;
+        scales_of(amax, c.qmaxf, s_out, inv);
+#pragma unroll
+        for (int ch = 0; ch < NCH; ++ch) quantize_store<G, false, DUMP, C::DUP>(c.a_tile, c.row, ch * CH + feature_of<C>(c.row, last * G), u[ch], inv, c.qmaxf, c.one2, dump_codes);
 #pragma unroll 1
-        for (int gg = 0; gg < C::GPT; ++gg) {
+        for (int gg = 0; gg < C::GPT - 1; ++gg) {
             const int g = c.sub * C::GPT + gg;
-            uint32_t u[NCH][G];
+            load_group<C>(c.taddr + g * G, u);
 #pragma unroll
-            for (int ch = 0; ch < NCH; ++ch) tmem_ld<G>(c.taddr + ch * CH + g * G, u[ch]);
-            ptx::tmem_wait_ld();
-#pragma unroll
-            for (int ch = 0; ch < NCH; ++ch) quantize_store<G, false, DUMP, C::DUP>(c.a_tile, c.row, ch * CH + feature_of<C>(c.row, g * G), u[ch], inv, c.qmaxf, dump_codes);
+            for (int ch = 0; ch < NCH; ++ch) quantize_store<G, false, DUMP, C::DUP>(c.a_tile, c.row, ch * CH + feature_of<C>(c.row, g * G), u[ch], inv, c.qmaxf, c.one2, dump_codes);
         }
     }
     ptx::fence_proxy_async();
@@ -680,7 +758,6 @@ __device__ __forceinline__ bool finish_layer(SlotCtx &c, float static_s, float s
 // integers).  Same barrier, loads and butterfly stages as finish_layer up to that point.
 template <class C, bool ROT> __device__ __forceinline__ bool calib_finish(SlotCtx &c, bool valid, float *act)
 {
-    constexpr int NCH = C::NCH, G = C::G, CH = C::CH;
     ptx::tmem_wait_st();
     ptx::tc_fence_before();
     if (!slot_barrier<false>(c)) return false;
@@ -688,31 +765,11 @@ template <class C, bool ROT> __device__ __forceinline__ bool calib_finish(SlotCt
     float amax = 0.f;
 #pragma unroll 1
     for (int gg = 0; gg < C::GPT; ++gg) {
-        const int g = c.sub * C::GPT + gg;
-        uint32_t u[NCH][G];
+        uint32_t u[C::NCH][C::G];
+        load_group<C>(c.taddr + (c.sub * C::GPT + gg) * C::G, u);
+        across_chunks<C, ROT>(u);
 #pragma unroll
-        for (int ch = 0; ch < NCH; ++ch) tmem_ld<G>(c.taddr + ch * CH + g * G, u[ch]);
-        ptx::tmem_wait_ld();
-#pragma unroll
-        for (int h = 1; h < (ROT ? NCH : 1); h <<= 1) {
-#pragma unroll
-            for (int ch = 0; ch < NCH; ++ch) {
-                if ((ch & h) == 0) {
-#pragma unroll
-                    for (int i = 0; i < G; i += 2) {
-                        f32x2 a = pack2u(u[ch][i], u[ch][i + 1]), b = pack2u(u[ch + h][i], u[ch + h][i + 1]);
-                        bfly2(a, b);
-                        unpack2u(a, u[ch][i], u[ch][i + 1]);
-                        unpack2u(b, u[ch + h][i], u[ch + h][i + 1]);
-                    }
-                }
-            }
-        }
-#pragma unroll
-        for (int ch = 0; ch < NCH; ++ch) {
-#pragma unroll
-            for (int i = 0; i < G; ++i) amax = fmaxf(amax, fabsf(__uint_as_float(u[ch][i])));
-        }
+        for (int ch = 0; ch < C::NCH; ++ch) amax = max_abs<C::G>(amax, u[ch]);
     }
     if (!valid) amax = 0.f; // rows past the end of the coordinate set do not count
 #pragma unroll
@@ -842,6 +899,7 @@ __device__ void epilogue_role(const ParamsOf<DUMP, CALIB> &p, const SmemMap &sm,
     c.amax_addr = smem_base + sm.amax + slot * (4 * kTile * 4);
     c.sync_parity = 0;
     c.qmaxf = p.qmaxf;
+    c.one2 = pack2(p.one2.x, p.one2.y);
     c.abort_flag = abort_flag;
     c.status = p.status;
     const uint32_t bar_acc = smem_base + sm.acc_full + 8 * (slot * 4);

@@ -69,17 +69,16 @@ __device__ __forceinline__ float sin_approx(float x)
 // sin(x) for |x| up to a few thousand: k = nearest integer to x / (2 pi), r = x - k * 2 pi with
 // 2 pi split into fl32(2 pi) and the remainder (two fused multiply-adds, each exact before its
 // single rounding), then the hardware approximation on |r| <= pi.
-__device__ __forceinline__ float sin_wide(float x)
+__device__ __forceinline__ float wide_reduced(float x)
 {
     const float inv_two_pi = 0.15915494309189535f;
     const float two_pi_hi = 6.2831854820251465f;   // fl32(2 pi)
     const float two_pi_lo = -1.7484555e-07f;       // 2 pi - fl32(2 pi)
     // nearest integer by adding and subtracting 1.5 * 2^23 (ties to even; |x / 2 pi| < 2^22)
-    float k = __fsub_rn(__fadd_rn(__fmul_rn(x, inv_two_pi), 12582912.0f), 12582912.0f);
-    float r = __fmaf_rn(k, -two_pi_hi, x);
-    r = __fmaf_rn(k, -two_pi_lo, r);
-    return sin_approx(r);
+    const float k = __fsub_rn(__fmaf_rn(x, inv_two_pi, 12582912.0f), 12582912.0f);
+    return __fmaf_rn(k, -two_pi_lo, __fmaf_rn(k, -two_pi_hi, x));
 }
+__device__ __forceinline__ float sin_wide(float x) { return sin_approx(wide_reduced(x)); }
 
 // Per-(token, channel) epilogue.  accf = (float)acc is exact (|acc| < 2^24).
 //   c_hi, c_lo : the dequantization constant omega0 * s_w * s_x (or s_w * s_x for the last
@@ -98,21 +97,25 @@ __device__ __forceinline__ float epilogue(int mode, float accf, float c_hi, floa
 __device__ __forceinline__ float epilogue_mixed(float accf, float c_hi, float c_lo, float cb, float limit)
 {
     const float x = __fmaf_rn(accf, c_hi, cb);
-    if (fabsf(x) <= limit) return sin_approx(x);
-    return sin_wide(__fmaf_rn(accf, c_lo, x));
+    return sin_approx(fabsf(x) <= limit ? x : wide_reduced(__fmaf_rn(accf, c_lo, x)));
 }
 
 // Wavelet activation (reading of the paper's WIRE experiments, Section IV): the real Gabor wavelet
 // psi(z) = sin(omega0 z) exp(-(s0 z)^2), from the compensated phase x = omega0 z and c = s0 / omega0.
 // The envelope's exponent carries a relative error of a few 2^-24, the result stays within the
 // sine's own error.
+// (.ftz: an envelope below 2^-126 is zero, which saves the four instructions that scale such arguments and results.)
+__device__ __forceinline__ float gabor_envelope(float t)
+{
+    float e;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(t));
+    return e;
+}
 __device__ __forceinline__ float gabor_epilogue(float accf, float c_hi, float c_lo, float cb, float c)
 {
     const float x = __fmaf_rn(accf, c_lo, __fmaf_rn(accf, c_hi, cb));
     const float g = __fmul_rn(x, c);
-    float e;
-    asm("ex2.approx.f32 %0, %1;" : "=f"(e) : "f"(__fmul_rn(__fmul_rn(g, g), -1.4426950408889634f)));
-    return __fmul_rn(sin_wide(x), e);
+    return __fmul_rn(sin_wide(x), gabor_envelope(__fmul_rn(__fmul_rn(g, g), -1.4426950408889634f)));
 }
 
 // First layer, per-tensor activation scale.  The rotated padded coordinate [x, y, 0, 0] has the
