@@ -20,11 +20,11 @@
 // of the next layer's input can run through it (stages 1, 2, 4 inside a block, 8 .. W/8 in a thread's
 // chunk, W/4 and W/2 across chunks).  The weights stream from L2 in pieces of 16 KB.
 //
-// What bounds it: issue slots of the epilogue, about 38 per element (14 of them the phase, carried as if in
-// fp64: digit_phase), beside 32 x 51 cycles of MMAs per block of 64 outputs.  A block's sums are released as
+// What bounds it: issue slots of the epilogue, about 29 per element (7 of them the phase, carried as if in
+// fp64: digit_phase_pair), beside 32 x 51 cycles of MMAs per block of 64 outputs.  A block's sums are released as
 // soon as they are in registers, so that the next block's MMAs run beside its phases; the first block's MMAs
 // and the stages across chunks are exposed (one tile fills tensor memory).  Measured: 2 -> 256 x 5 -> 3,
-// per-channel / per-token, 262,144 coordinates 9.79 -> 0.77 ms (one dp4a pass and an fp64 butterfly per layer
+// per-channel / per-token, 262,144 coordinates 9.79 -> 0.67 ms (one dp4a pass and an fp64 butterfly per layer
 // before).
 #include "dhq_fused.cuh"
 
@@ -91,6 +91,19 @@ __host__ __device__ inline DigitMap digit_map(int W, int n_stages, int L)
     m.abort_flag = off; off += 16;
     m.total = off;
     return m;
+}
+
+// digit_phase of dhq_math.cuh for two outputs: the same operations, packed, and the same bits (one value at a time: width
+// 256, 262,144 coordinates, 5 layers, per-channel / per-token 757 us, packed 667).
+__device__ __forceinline__ f32x2 digit_phase_pair(f32x2 f0, f32x2 f1, f32x2 c_hi, f32x2 c_lo, f32x2 cb, f32x2 cb_lo, f32x2 &s, f32x2 &lo)
+{
+    const f32x2 two_pi = pack2(6.2831853071795865f, 6.2831853071795865f), two_pi_lo = pack2(-1.7484555e-07f, -1.7484555e-07f);
+    const f32x2 grid = pack2(6144.0f, 6144.0f), magic = pack2(12582912.0f, 12582912.0f);
+    const f32x2 nq = sub2(grid, fma2(f0, c_hi, grid)); // minus the product's part on the grid
+    s = sub2(cb, nq);
+    lo = add2(fma2(f0, c_hi, nq), fma2(f0, c_lo, fma2(f1, c_hi, cb_lo)));
+    const f32x2 t = sub2(s, sub2(add2(add2(s, lo), magic), magic));
+    return fma2(t, two_pi, fma2(lo, two_pi, mul2(t, two_pi_lo)));
 }
 
 // Rotated activations of this thread's quarter of the row -> codes (and, per token, their scale).
@@ -176,15 +189,21 @@ __device__ void digit_epilogue(const DigitParams &p, const DigitMap &sm, uint32_
         const float4 ca = lds128(at), cl = lds128(at + W * 4), cb = lds128(at + 2 * W * 4), cbl = lds128(at + 3 * W * 4);
         float4 cn = make_float4(0.f, 0.f, 0.f, 0.f);
         if (GABOR) cn = lds128(at + 4 * W * 4);
-        const float av[4] = {ca.x, ca.y, ca.z, ca.w}, lv[4] = {cl.x, cl.y, cl.z, cl.w}, bv[4] = {cb.x, cb.y, cb.z, cb.w}, blv[4] = {cbl.x, cbl.y, cbl.z, cbl.w},
-                    nv[4] = {cn.x, cn.y, cn.z, cn.w};
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            float c_hi = av[e], c_lo = lv[e];
-            if (PER_TOKEN) token_const(av[e], lv[e], s_x, c_hi, c_lo);
-            float s, lo;
-            y[e] = sin_approx(digit_phase(f0[e], f1[e], c_hi, c_lo, bv[e], blv[e], s, lo));
-            if constexpr (GABOR) y[e] = __fmul_rn(y[e], digit_envelope(s, lo, nv[e], p.gabor_c));
+        for (int h = 0; h < 2; ++h) {
+            f32x2 c_hi = h ? pack2(ca.z, ca.w) : pack2(ca.x, ca.y), c_lo = h ? pack2(cl.z, cl.w) : pack2(cl.x, cl.y);
+            if (PER_TOKEN) token_const2(c_hi, c_lo, pack2(s_x, s_x), pack2(-s_x, -s_x), c_hi, c_lo);
+            f32x2 s, lo;
+            const f32x2 x = digit_phase_pair(pack2(f0[2 * h], f0[2 * h + 1]), pack2(f1[2 * h], f1[2 * h + 1]), c_hi, c_lo,
+                                             h ? pack2(cb.z, cb.w) : pack2(cb.x, cb.y), h ? pack2(cbl.z, cbl.w) : pack2(cbl.x, cbl.y), s, lo);
+            unpack2(sine2(x), y[2 * h], y[2 * h + 1]);
+            if constexpr (GABOR) {
+                float sv[2], lv[2];
+                unpack2(s, sv[0], sv[1]);
+                unpack2(lo, lv[0], lv[1]);
+#pragma unroll
+                for (int e = 0; e < 2; ++e) y[2 * h + e] = __fmul_rn(y[2 * h + e], digit_envelope(sv[e], lv[e], h ? (e ? cn.w : cn.z) : (e ? cn.y : cn.x), p.gabor_c));
+            }
         }
     };
     // stages 1, 2, 4 of 16 finished activations, and into the row's columns
