@@ -236,7 +236,7 @@ struct BlobHeader {
     float phase_bound[kMaxLayers];
     uint64_t payload_bytes, payload_fnv1a;
 };
-constexpr uint32_t kBlobVersion = 6;
+constexpr uint32_t kBlobVersion = 7, kOldestBlob = 6; // 6: another order of the two-sided digits' image, formed anew on import
 const char kBlobMagic[8] = {'D', 'H', 'Q', 'B', '2', '0', '0', 0};
 
 uint64_t fnv1a(const uint8_t *p, size_t n)
@@ -917,7 +917,7 @@ dhq_status_t dhq_import(const void *host_buf, int64_t bytes, void *stream, dhq_h
     *out = nullptr;
     BlobHeader hd;
     memcpy(&hd, host_buf, sizeof(hd));
-    if (memcmp(hd.magic, kBlobMagic, 8) != 0 || hd.version != kBlobVersion || hd.header_bytes != sizeof(BlobHeader))
+    if (memcmp(hd.magic, kBlobMagic, 8) != 0 || hd.version < kOldestBlob || hd.version > kBlobVersion || hd.header_bytes != sizeof(BlobHeader))
         return DHQ_ERR_INVALID_ARG;
     if (hd.n_layers < 2 || hd.n_layers > kMaxLayers) return DHQ_ERR_INVALID_ARG;
     dhq_config_t cfg;
@@ -974,6 +974,8 @@ dhq_status_t dhq_import(const void *host_buf, int64_t bytes, void *stream, dhq_h
             }
         }
         if (rc != DHQ_OK) break;
+        for (int l = 2; l <= h->L && h->layer[0].has_digits; ++l)
+            if (launch_repack_digits(h->layer[l - 1], h->w, l == h->L, st, &h->launches) != cudaSuccess) rc = DHQ_ERR_CUDA;
         // (the same constants again from the same scales: a block of an earlier build splits the bias differently)
         for (int l = 1; l <= h->L && h->layer[0].has_digits && hd.calibrated; ++l)
             if (launch_finalize(h->layer[l - 1], cfg.a_bits, cfg.a_gran == DHQ_GRAN_CHANNEL_OR_TOKEN, l < h->L, (double)cfg.omega0, st, &h->launches) != cudaSuccess) rc = DHQ_ERR_CUDA;

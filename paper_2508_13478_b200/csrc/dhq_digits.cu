@@ -15,17 +15,18 @@
 //
 // Layout: one tile of 128 coordinates at a time, 16 epilogue warps; a token is a tensor-memory lane
 // and the four threads of a row own a chunk of W/4 features each.  The outputs come in blocks of 64:
-// block b holds 16 features of every chunk, so that all warps work on every block, the four digits' sums
-// in columns 0-255; activations wait in columns 256-511 until the whole row is there and the rotation
-// of the next layer's input can run through it (stages 1, 2, 4 inside a block, 8 .. W/8 in a thread's
-// chunk, W/4 and W/2 across chunks).  The weights stream from L2 in pieces of 16 KB.
+// block b holds 16 features of every chunk, so that all warps work on every block, in two halves whose sums
+// (32 outputs by four digits) have a set of 128 columns each; activations wait in columns 256-511 until the
+// whole row is there and the rotation of the next layer's input can run through it (stages 1, 2, 4 inside a
+// block, 8 .. W/8 in a thread's chunk, W/4 and W/2 across chunks).  The weights stream from L2 in pieces of 16 KB.
 //
 // What bounds it: issue slots of the epilogue, about 29 per element (7 of them the phase, carried as if in
-// fp64: digit_phase_pair), beside 32 x 51 cycles of MMAs per block of 64 outputs.  A block's sums are released as
-// soon as they are in registers, so that the next block's MMAs run beside its phases; the first block's MMAs
-// and the stages across chunks are exposed (one tile fills tensor memory).  Measured: 2 -> 256 x 5 -> 3,
-// per-channel / per-token, 262,144 coordinates 9.79 -> 0.67 ms (one dp4a pass and an fp64 butterfly per layer
-// before).
+// fp64: digit_phase_pair), beside 8 x 67 cycles of MMAs per half block of 32 outputs (N = 128, all four
+// digits' rows in one MMA; digit by digit with N = 64 the same outputs took 16 x 51, because operands leave shared
+// memory at 128 B per cycle).  Two sets of sums: one half's MMAs run while the other's sums are read and worked on;
+// the first half block's MMAs and the stages across chunks are exposed (activations fill the rest of tensor memory).
+// Measured: 2 -> 256 x 5 -> 3, per-channel / per-token, 262,144 coordinates 604 us (667 with one set of 4 x 64 sums and
+// an MMA per digit; 9.79 ms with one dp4a pass and an fp64 butterfly per layer).
 #include "dhq_fused.cuh"
 
 namespace dhq {
@@ -44,8 +45,18 @@ __host__ __device__ inline int digit_feature(int W, int b, int sub, int i)
     return sub * ch + b * 8 + (i >> 1) + (i & 1) * (ch / 2);
 }
 
+// Place of weight digit d of output m at input k in a layer's image.  Hidden layers: [block][half][K/16][128][16], a half block's
+// rows being 32 of each digit (8 per thread of a row), so that one MMA with N = 128 takes all four digits; last
+// layer: [K/16][16][16], row 4 d + m.
+__host__ __device__ inline size_t digit_image_offset(int W, bool last, int m, int k, int d)
+{
+    if (last) return (size_t)(k >> 4) * 256 + (4 * d + m) * 16 + (k & 15);
+    const int ch = W / 4, sub = m / ch, q = m % ch, pos = q % (ch / 2), b = pos / 8, i = 2 * (pos % 8) + q / (ch / 2);
+    return ((size_t)(b * 2 + (i >> 3)) * (W / 16) + (k >> 4)) * 2048 + (d * 32 + sub * 8 + (i & 7)) * 16 + (k & 15);
+}
+
 struct DigitLayer {
-    const uint8_t *img;              // [block][digit][K/16][64][16]; last layer: [K/16][16][16], row 4 * digit + output
+    const uint8_t *img;              // see digit_image_offset
     const float *c, *c_lo, *cb, *cb_lo, *cn; // per output: see digit_phase
     const float *act;
 };
@@ -81,8 +92,8 @@ __host__ __device__ inline DigitMap digit_map(int W, int n_stages, int L)
     m.w_full = off; off += 8 * kDMaxStages;
     m.w_empty = off; off += 8 * kDMaxStages;
     m.codes_full = off; off += 8;
-    m.acc_full = off; off += 8;
-    m.acc_empty = off; off += 8;
+    m.acc_full = off; off += 16;
+    m.acc_empty = off; off += 16;
     m.acc_last = off; off += 8;
     m.last_full = off; off += 8;
     m.quad_sync = off; off += 8 * 4;
@@ -180,7 +191,7 @@ __device__ void digit_epilogue(const DigitParams &p, const DigitMap &sm, uint32_
     c.one2 = pack2(p.one2.x, p.one2.y);
     c.abort_flag = abort_flag;
     c.status = p.status;
-    const uint32_t acc = tmem + ((uint32_t)(quad * 32) << 16) + sub * 16;
+    const uint32_t acc = tmem + ((uint32_t)(quad * 32) << 16) + sub * 8;
     uint32_t use = 0, last_parity = 0;
     float s_x = 1.0f;
 
@@ -284,22 +295,20 @@ __device__ void digit_epilogue(const DigitParams &p, const DigitMap &sm, uint32_
                                        __dp4a(qx, (int)__float_as_uint(wv[2][e]), 0), __dp4a(qx, (int)__float_as_uint(wv[3][e]), 0), f0[4 * q + e], f1[4 * q + e]);
                     }
                 } else {
-                    if (!wait_bar_warp<true>(base + sm.acc_full, use & 1, abort_flag, p.status)) return;
-                    ++use;
-                    ptx::tc_fence_after();
 #pragma unroll
                     for (int hf = 0; hf < 2; ++hf) {
+                        if (!wait_bar_warp<true>(base + sm.acc_full + 8 * hf, use & 1, abort_flag, p.status)) return;
+                        ptx::tc_fence_after();
                         uint32_t D[4][8];
 #pragma unroll
-                        for (int d = 0; d < 4; ++d) ptx::tmem_ld8(acc + d * kDBlock + hf * 8, D[d]);
+                        for (int d = 0; d < 4; ++d) ptx::tmem_ld8(acc + hf * 128 + d * 32, D[d]);
                         ptx::tmem_wait_ld();
-                        if (hf == 1) { // the sums are free for the next block
-                            ptx::tc_fence_before();
-                            ptx::mbar_arrive(base + sm.acc_empty);
-                        }
+                        ptx::tc_fence_before();
+                        ptx::mbar_arrive(base + sm.acc_empty + 8 * hf); // the sums are free for the next block
 #pragma unroll
                         for (int i = 0; i < 8; ++i) digit_sums((int)D[0][i], (int)D[1][i], (int)D[2][i], (int)D[3][i], f0[hf * 8 + i], f1[hf * 8 + i]);
                     }
+                    ++use;
                 }
                 float y[16];
 #pragma unroll
@@ -333,9 +342,9 @@ __device__ void digit_mma(const DigitParams &p, const DigitMap &sm, uint32_t bas
 {
     constexpr int NB = W / kDBlock, PIECE = kDBlock * W;
     ptx::wait_for_previous_kernels(); // before the first bounded wait
-    const uint32_t idesc = ptx::idesc_i8(kTile, kDBlock), idesc_last = ptx::idesc_i8(kTile, 16);
+    const uint32_t idesc = ptx::idesc_i8(kTile, 128), idesc_last = ptx::idesc_i8(kTile, 16);
     constexpr uint32_t kDescHi = (128u >> 4) | (1u << 14);
-    const uint32_t a0 = ((base + sm.a) >> 4) | ((kTile * 16u >> 4) << 16), b0 = ((base + sm.ring) >> 4) | ((kDBlock * 16u >> 4) << 16);
+    const uint32_t a0 = ((base + sm.a) >> 4) | ((kTile * 16u >> 4) << 16), b0 = ((base + sm.ring) >> 4) | ((128 * 16u >> 4) << 16);
     const uint32_t l0 = ((base + sm.last_w) >> 4) | ((16u * 16u >> 4) << 16);
     uint32_t use = 0, codes = 0, wpar = 0;
     int stage = 0;
@@ -344,19 +353,21 @@ __device__ void digit_mma(const DigitParams &p, const DigitMap &sm, uint32_t bas
         for (int l = 2; l < p.L && ok; ++l) {
             ok = wait_bar<0, kHintNs>(base + sm.codes_full, codes & 1, abort_flag, p.status);
             ++codes;
-            for (int b = 0; b < NB && ok; ++b, ++use) {
-                if (!wait_bar<0, kHintNs>(base + sm.acc_empty, (use & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
+            for (int hb = 0; hb < 2 * NB && ok; ++hb, ++use) { // half blocks; set hb & 1 of the sums
+                const uint32_t set = hb & 1;
+                if (!wait_bar<0, kHintNs>(base + sm.acc_empty + 8 * set, ((use >> 1) & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
                 ptx::tc_fence_after();
-                for (int d = 0; d < 4; ++d) {
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
                     if (!wait_bar<0, kHintNs>(base + sm.w_full + 8 * stage, wpar, abort_flag, p.status)) { ok = false; break; }
                     const uint32_t bk = b0 + (uint32_t)stage * (PIECE >> 4);
 #pragma unroll
-                    for (int ks = 0; ks < W / 32; ++ks)
-                        ptx::mma_i8_words(tmem + (uint32_t)d * kDBlock, a0 + (ks * 2 * kTile * 16 >> 4), bk + (ks * 2 * kDBlock * 16 >> 4), kDescHi, idesc, ks > 0 ? 1u : 0u);
+                    for (int ks = 0; ks < W / 64; ++ks)
+                        ptx::mma_i8_words(tmem + set * 128, a0 + ((q * (W / 64) + ks) * 2 * kTile * 16 >> 4), bk + (ks * 2 * 128 * 16 >> 4), kDescHi, idesc, q > 0 || ks > 0 ? 1u : 0u);
                     ptx::mma_commit(base + sm.w_empty + 8 * stage);
                     if (++stage == p.n_stages) { stage = 0; wpar ^= 1; }
                 }
-                if (ok) ptx::mma_commit(base + sm.acc_full);
+                if (ok) ptx::mma_commit(base + sm.acc_full + 8 * set);
             }
         }
         if (!ok) break;
@@ -428,8 +439,10 @@ __global__ void __launch_bounds__(kDThreads, 1) digit_kernel(const __grid_consta
             ptx::mbar_init(base + sm.w_empty + 8 * i, 1);
         }
         ptx::mbar_init(base + sm.codes_full, kEpiWarps * 32);
-        ptx::mbar_init(base + sm.acc_full, 1);
-        ptx::mbar_init(base + sm.acc_empty, kEpiWarps * 32);
+        for (int i = 0; i < 2; ++i) {
+            ptx::mbar_init(base + sm.acc_full + 8 * i, 1);
+            ptx::mbar_init(base + sm.acc_empty + 8 * i, kEpiWarps * 32);
+        }
         ptx::mbar_init(base + sm.acc_last, 1);
         ptx::mbar_init(base + sm.last_full, 1);
         for (int i = 0; i < 4; ++i) ptx::mbar_init(base + sm.quad_sync + 8 * i, 128);
@@ -513,24 +526,13 @@ __global__ void __launch_bounds__(128) prep_digit_rows_kernel(const __grid_const
     __syncthreads();
     g = fmax(fmax(red[0], red[1]), fmax(red[2], red[3]));
     const double f = g > 0.0 ? 2139062143.0 / g : 0.0; // 127 in every digit
-    size_t at = 0; // place of (m, k = 0, digit 0) in the tensor-core image, and the distance of digits
-    size_t digit_bytes = 0;
-    if (l > 0 && l < a.L - 1) {
-        const int CH = a.w / 4, sub = m / CH, q = m % CH, pr = q % (CH / 2), b = pr / 8, i = 2 * (pr % 8) + q / (CH / 2);
-        digit_bytes = (size_t)kDBlock * K;
-        at = (size_t)b * 4 * digit_bytes + (sub * 16 + i) * 16;
-    }
-    const int rows = l == a.L - 1 ? 16 : kDBlock;
     for (int k = tid; k < K; k += 128) {
         const uint32_t v = (uint32_t)((long long)rint(row[k] * f) + 0x80808080ll) ^ 0x80808080u;
 #pragma unroll
         for (int d = 0; d < 4; ++d) {
             const uint8_t byte = (uint8_t)(v >> (24 - 8 * d));
             reinterpret_cast<uint8_t *>(dev.gd_k4m)[(size_t)d * M * K + ((size_t)(k >> 2) * M + m) * 4 + (k & 3)] = byte;
-            if (l > 0) {
-                const size_t o = l == a.L - 1 ? (size_t)(4 * d + m) * 16 : at + d * digit_bytes;
-                dev.gd_img[o + (size_t)(k >> 4) * rows * 16 + (k & 15)] = byte;
-            }
+            if (l > 0) dev.gd_img[digit_image_offset(a.w, l == a.L - 1, m, k, d)] = byte;
         }
     }
     if (tid == 0) {
@@ -538,6 +540,22 @@ __global__ void __launch_bounds__(128) prep_digit_rows_kernel(const __grid_const
         dev.g_scale[m] = f > 0.0 ? (sine ? a.omega0 * 0.15915494309189533576888 * 16777216.0 : 1.0) / f : 0.0;
         if (a.finalize) finalize_row(dev, m, 1.0f, 0.f, sine, a.omega0);
     }
+}
+
+// The image again from the digits in [4][K/4][M] words: a saved block may hold it in the order of an earlier build.
+__global__ void __launch_bounds__(256) repack_digits_kernel(LayerDev dev, int w, int last)
+{
+    const int K = dev.K, M = dev.M, words = M * K; // four digits of M K / 4 words
+    for (int i = blockIdx.x * 256 + threadIdx.x; i < words; i += gridDim.x * 256) {
+        const int d = i / (words / 4), r = i % (words / 4), k = r / M * 4, m = r % M;
+        *reinterpret_cast<uint32_t *>(dev.gd_img + digit_image_offset(w, last != 0, m, k, d)) = dev.gd_k4m[i];
+    }
+}
+cudaError_t launch_repack_digits(const LayerDev &dev, int w, bool last, cudaStream_t st, int64_t *launches)
+{
+    repack_digits_kernel<<<148, 256, 0, st>>>(dev, w, last ? 1 : 0);
+    *launches += 1;
+    return cudaGetLastError();
 }
 
 cudaError_t launch_prep_digits(const DigitPrep &a, cudaStream_t st, int64_t *launches)

@@ -200,6 +200,7 @@ struct DigitPrep {
     LayerDev dev[kMaxLayers];
 };
 cudaError_t launch_prep_digits(const DigitPrep &a, cudaStream_t st, int64_t *launches);
+cudaError_t launch_repack_digits(const LayerDev &dev, int w, bool last, cudaStream_t st, int64_t *launches);
 dhq_status_t digit_create(dhq_handle_s *h);
 void digit_destroy(dhq_handle_s *h);
 dhq_status_t digit_forward(dhq_handle_s *h, const float *coords, int64_t n, float *out, cudaStream_t st);

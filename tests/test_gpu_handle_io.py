@@ -140,3 +140,55 @@ def test_exported_bytes_hold_this_network_only(kw, other):
         for _ in range(3):
             export(nets[1], options)
         assert export(nets[0], kw) == first
+
+
+def as_format_6(blob, start):
+    """The block with its version set back and the checksum of its arrays (which begin at `start`) renewed."""
+    blob = bytearray(blob)
+    blob[8:12] = np.uint32(6).tobytes()
+    fnv = 1469598103934665603
+    for b in blob[start:]:
+        fnv = ((fnv ^ b) * 1099511628211) & 0xFFFFFFFFFFFFFFFF
+    blob[start - 8:start] = fnv.to_bytes(8, "little")
+    return bytes(blob)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("width", [128, 256])
+def test_import_forms_the_two_sided_digit_images_anew(width):
+    # a block of format 6 holds the tensor-core images of the two-sided per-channel network in another order: whatever
+    # its bytes are, the import has to give the same network
+    from paper_2508_13478_b200 import build
+    build.build()
+    dims = (2, width, width, width, 3)
+    weights, biases = dhq_inputs.siren_init(dims, 30.0, 71)
+    h = dhq.dhq_prepare(dims, [to_dev(x) for x in weights], [to_dev(x) for x in biases], 30.0, w_gran=dhq.DHQ_GRAN_CHANNEL_OR_TOKEN,
+                        a_gran=dhq.DHQ_GRAN_CHANNEL_OR_TOKEN, rotation=dhq.DHQ_ROT_BOTH)
+    h2 = None
+    try:
+        blob = bytearray(dhq.dhq_export(h))
+        images, sizes = [], []
+        for l in range(1, len(dims)):
+            K, M, rows = (4 if l == 1 else width), (4 if l == len(dims) - 1 else width), (16 if l == len(dims) - 1 else width)
+            sizes += [4 * M * K, 4 * M, 4 * M, M * K, M * K, rows * max(K, 16)] + [4 * M] * 9 + [16, 4 * M * K]
+            if l > 1:
+                images.append((sum(sizes), 4 * M * K))
+                sizes += [4 * M * K]
+            sizes += [8 * M, 4 * M, 4 * M] + ([4 * M, 4 * M] if l == 1 else [])
+        start = len(blob) - sum(sizes)
+        assert blob[start - 16:start - 8] == np.uint64(sum(sizes)).tobytes()
+        for at, n in images:
+            blob[start + at:start + at + n] = bytes(reversed(blob[start + at:start + at + n]))
+        h2 = dhq.dhq_import(as_format_6(blob, start))
+        coords = to_dev(dhq_inputs.grid_coords(40, 25))
+        out1 = torch.empty((coords.shape[0], 3), device="cuda")
+        out2 = torch.full_like(out1, float("nan"))
+        dhq.dhq_forward(h, coords, out1)
+        dhq.dhq_forward(h2, coords, out2)
+        torch.cuda.synchronize()
+        assert dhq.dhq_last_status(h2) == 0
+        assert torch.equal(out1.view(torch.int32), out2.view(torch.int32))
+    finally:
+        dhq.dhq_destroy(h)
+        if h2:
+            dhq.dhq_destroy(h2)
