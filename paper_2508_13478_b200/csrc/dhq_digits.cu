@@ -341,6 +341,7 @@ template <int W>
 __device__ void digit_mma(const DigitParams &p, const DigitMap &sm, uint32_t base, uint32_t tmem, volatile int *abort_flag)
 {
     constexpr int NB = W / kDBlock, PIECE = kDBlock * W;
+    tmem = __shfl_sync(0xffffffffu, tmem, 0); // uniform for the compiler, see mma_i8
     ptx::wait_for_previous_kernels(); // before the first bounded wait
     const uint32_t idesc = ptx::idesc_i8(kTile, 128), idesc_last = ptx::idesc_i8(kTile, 16);
     constexpr uint32_t kDescHi = (128u >> 4) | (1u << 14);
@@ -351,15 +352,15 @@ __device__ void digit_mma(const DigitParams &p, const DigitMap &sm, uint32_t bas
     bool ok = true;
     for (long long tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
         for (int l = 2; l < p.L && ok; ++l) {
-            ok = wait_bar<0, kHintNs>(base + sm.codes_full, codes & 1, abort_flag, p.status);
+            ok = wait_bar_warp<true>(base + sm.codes_full, codes & 1, abort_flag, p.status);
             ++codes;
             for (int hb = 0; hb < 2 * NB && ok; ++hb, ++use) { // half blocks; set hb & 1 of the sums
                 const uint32_t set = hb & 1;
-                if (!wait_bar<0, kHintNs>(base + sm.acc_empty + 8 * set, ((use >> 1) & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
+                if (!wait_bar_warp<true>(base + sm.acc_empty + 8 * set, ((use >> 1) & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
                 ptx::tc_fence_after();
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
-                    if (!wait_bar<0, kHintNs>(base + sm.w_full + 8 * stage, wpar, abort_flag, p.status)) { ok = false; break; }
+                    if (!wait_bar_warp<true>(base + sm.w_full + 8 * stage, wpar, abort_flag, p.status)) { ok = false; break; }
                     const uint32_t bk = b0 + (uint32_t)stage * (PIECE >> 4);
 #pragma unroll
                     for (int ks = 0; ks < W / 64; ++ks)
@@ -371,8 +372,8 @@ __device__ void digit_mma(const DigitParams &p, const DigitMap &sm, uint32_t bas
             }
         }
         if (!ok) break;
-        if (!wait_bar<0, kHintNs>(base + sm.last_full, 0, abort_flag, p.status) ||
-            !wait_bar<0, kHintNs>(base + sm.codes_full, codes & 1, abort_flag, p.status)) { ok = false; break; }
+        if (!wait_bar_warp<true>(base + sm.last_full, 0, abort_flag, p.status) ||
+            !wait_bar_warp<true>(base + sm.codes_full, codes & 1, abort_flag, p.status)) { ok = false; break; }
         ++codes;
         ptx::tc_fence_after();
 #pragma unroll
@@ -392,8 +393,8 @@ __device__ void digit_load(const DigitParams &p, const DigitMap &sm, uint32_t ba
 {
     constexpr int PIECE = kDBlock * W, PIECES = W / kDBlock * 4;
     if (!p.skip_last_weights) {
-        ptx::mbar_expect_tx(base + sm.last_full, 16 * W);
-        ptx::bulk_g2s(base + sm.last_w, p.layer[p.L - 1].img, 16 * W, base + sm.last_full);
+        ptx::mbar_expect_tx_warp(base + sm.last_full, 16 * W);
+        ptx::bulk_g2s_warp(base + sm.last_w, p.layer[p.L - 1].img, 16 * W, base + sm.last_full);
     }
     int stage = 0;
     uint32_t par = 1, issued = 0;
@@ -402,9 +403,9 @@ __device__ void digit_load(const DigitParams &p, const DigitMap &sm, uint32_t ba
         for (int l = 2; l < p.L && ok; ++l) {
             for (int i = 0; i < PIECES; ++i) {
                 if (issued == (uint32_t)p.n_stages) ptx::wait_for_previous_kernels();
-                if (!wait_bar<0, kHintNs>(base + sm.w_empty + 8 * stage, par, abort_flag, p.status)) { ok = false; break; }
-                ptx::mbar_expect_tx(base + sm.w_full + 8 * stage, PIECE);
-                ptx::bulk_g2s(base + sm.ring + (uint32_t)stage * PIECE, p.layer[l - 1].img + (size_t)i * PIECE, PIECE, base + sm.w_full + 8 * stage);
+                if (!wait_bar_warp<true>(base + sm.w_empty + 8 * stage, par, abort_flag, p.status)) { ok = false; break; }
+                ptx::mbar_expect_tx_warp(base + sm.w_full + 8 * stage, PIECE);
+                ptx::bulk_g2s_warp(base + sm.ring + (uint32_t)stage * PIECE, p.layer[l - 1].img + (size_t)i * PIECE, PIECE, base + sm.w_full + 8 * stage);
                 ++issued;
                 if (++stage == p.n_stages) { stage = 0; par ^= 1; }
             }
@@ -472,10 +473,8 @@ __global__ void __launch_bounds__(kDThreads, 1) digit_kernel(const __grid_consta
     ptx::tc_fence_after();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(gen + sm.holder);
     if (warp < kEpiWarps) digit_epilogue<W, PER_TOKEN, GABOR>(p, sm, base, warp, lane, tmem, abort_flag);
-    else if (lane == 0) {
-        if (warp == kMmaWarp) digit_mma<W>(p, sm, base, tmem, abort_flag);
-        else digit_load<W>(p, sm, base, abort_flag);
-    }
+    else if (warp == kMmaWarp) digit_mma<W>(p, sm, base, tmem, abort_flag);
+    else digit_load<W>(p, sm, base, abort_flag);
     ptx::tc_fence_before();
     __syncthreads();
     if (warp == kMmaWarp) {

@@ -353,13 +353,14 @@ __device__ void float_epilogue(const FloatParams &p, const FloatMap &sm, uint32_
     }
 }
 
-// One thread issues the MMAs and has about 67 cycles for each, so the descriptors are kept as 32-bit
+// One warp issues the MMAs and has about 67 cycles for each, so the descriptors are kept as 32-bit
 // words to which constants are added: the low word holds the operand's address in units of 16 bytes and
 // the distance of core matrices along K, the high word is the same for every operand here.
 template <int W, int WL>
 __device__ void float_mma(const FloatParams &p, const FloatMap &sm, uint32_t base, uint32_t tmem, volatile int *abort_flag)
 {
     constexpr int FB = float_block(W), KC = float_kc(W), NB = W / FB, NKC = W / KC, PIECE = FB * KC;
+    tmem = __shfl_sync(0xffffffffu, tmem, 0); // uniform for the compiler, see mma_i8
     ptx::wait_for_previous_kernels(); // before the first bounded wait
     const uint32_t idesc = ptx::idesc_i8(kTile, FB);
     constexpr uint32_t kDescHi = (128u >> 4) | (1u << 14);
@@ -373,22 +374,22 @@ __device__ void float_mma(const FloatParams &p, const FloatMap &sm, uint32_t bas
     for (long long tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
         for (int l = 2; l < p.L && ok; ++l, ++layers) {
             for (int b = 0; b < NB && ok; ++b, ++use) {
-                if (!wait_bar<0, kHintNs>(base + sm.acc_empty, (use & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
+                if (!wait_bar_warp<true>(base + sm.acc_empty, (use & 1) ^ 1, abort_flag, p.status)) { ok = false; break; }
                 ptx::tc_fence_after();
                 uint32_t ak = a0;
                 for (int kc = 0; kc < NKC; ++kc, ak += (KC / 16) * (kTile * 16) >> 4) {
                     if constexpr (XS) {
                         static_assert(KC == FB && NB <= 2, "a part is a weight piece's k range; see float_x_in_smem");
                         ak = a0 + (((layers * NB + kc) % (NB + 1) * float_part_bytes(W)) >> 4);
-                        if (b == 0) ok = wait_bar<0, kHintNs>(base + sm.a_full + 8 * kc, layers & 1, abort_flag, p.status);
+                        if (b == 0) ok = wait_bar_warp<true>(base + sm.a_full + 8 * kc, layers & 1, abort_flag, p.status);
                         if (b == 0 && ok) ptx::tc_fence_after();
                     } else
                     for (int c = 0; b == 0 && c < KC / 64 && ok; ++c)
-                        ok = wait_bar<0, kHintNs>(base + sm.a_full + 8 * (kc * (KC / 64) + c), layers & 1, abort_flag, p.status);
+                        ok = wait_bar_warp<true>(base + sm.a_full + 8 * (kc * (KC / 64) + c), layers & 1, abort_flag, p.status);
                     if (!ok) break;
 #pragma unroll
                     for (int j = 0; j < WL; ++j) {
-                        if (!wait_bar<0, kHintNs>(base + sm.w_full + 8 * stage, wpar, abort_flag, p.status)) { ok = false; break; }
+                        if (!wait_bar_warp<true>(base + sm.w_full + 8 * stage, wpar, abort_flag, p.status)) { ok = false; break; }
                         const uint32_t bk = b0 + (uint32_t)stage * (PIECE >> 4);
 #pragma unroll
                         for (int i = 0; i + j < 3; ++i) {
@@ -413,9 +414,8 @@ __device__ void float_mma(const FloatParams &p, const FloatMap &sm, uint32_t bas
     }
 }
 
-// Waiting for a stage, arming its barrier and issuing the copy take one thread about 270 cycles,
-// whatever the size of the copy (8 KB pieces from one thread: 15 to 30 B per cycle; the SM can take 59).
-// So kFLoaders warps take the pieces in turn.
+// kFLoaders warps take the pieces in turn: waiting for a stage, arming its barrier and issuing the copy take one
+// warp longer than a piece's MMAs.
 template <int W, int WL>
 __device__ void float_load_weights(const FloatParams &p, const FloatMap &sm, uint32_t base, int which, volatile int *abort_flag)
 {
@@ -428,9 +428,9 @@ __device__ void float_load_weights(const FloatParams &p, const FloatMap &sm, uin
                 if ((int)(i % kFLoaders) != which || (p.skip_first_weights && i == 0)) continue;
                 if (i >= (uint32_t)p.n_stages && i < (uint32_t)p.n_stages + kFLoaders) ptx::wait_for_previous_kernels();
                 const uint32_t stage = i % (uint32_t)p.n_stages, par = ((i / (uint32_t)p.n_stages) & 1) ^ 1;
-                if (!wait_bar<0, kHintNs>(base + sm.w_empty + 8 * stage, par, abort_flag, p.status)) { ok = false; break; }
-                ptx::mbar_expect_tx(base + sm.w_full + 8 * stage, PIECE);
-                ptx::bulk_g2s(base + sm.ring + stage * PIECE, p.wimg[l - 1] + (size_t)q * PIECE, PIECE, base + sm.w_full + 8 * stage);
+                if (!wait_bar_warp<true>(base + sm.w_empty + 8 * stage, par, abort_flag, p.status)) { ok = false; break; }
+                ptx::mbar_expect_tx_warp(base + sm.w_full + 8 * stage, PIECE);
+                ptx::bulk_g2s_warp(base + sm.ring + stage * PIECE, p.wimg[l - 1] + (size_t)q * PIECE, PIECE, base + sm.w_full + 8 * stage);
                 mine = i;
                 ++issued;
             }
@@ -457,13 +457,13 @@ __device__ void float_load_x(const FloatParams &p, const FloatMap &sm, uint32_t 
     bool ok = true;
     for (long long tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
         for (int l = 2; l < p.L; ++l, ++layers) {
-            if (!wait_bar<0, kHintNs>(base + sm.x_ready, layers & 1, abort_flag, p.status)) { ok = false; break; }
+            if (!wait_bar_warp<true>(base + sm.x_ready, layers & 1, abort_flag, p.status)) { ok = false; break; }
             asm volatile("fence.proxy.async;" ::: "memory");
             for (int c = 0; c < W / 64; ++c) {
-                ptx::mbar_expect_tx(base + sm.a_full + 8 * c, 3 * 64 * kTile);
+                ptx::mbar_expect_tx_warp(base + sm.a_full + 8 * c, 3 * 64 * kTile);
                 for (int i = 0; i < 3; ++i) {
                     const uint32_t off = (uint32_t)(i * kTile * W + c * 64 * kTile);
-                    ptx::bulk_g2s(base + sm.a + off, src + off, 64 * kTile, base + sm.a_full + 8 * c);
+                    ptx::bulk_g2s_warp(base + sm.a + off, src + off, 64 * kTile, base + sm.a_full + 8 * c);
                 }
             }
         }
@@ -526,11 +526,9 @@ __global__ void __launch_bounds__(kFThreads, 1) float_kernel(const __grid_consta
     if (warp < kEpiWarps) ptx::take_registers<kEpiRegs>(); // see splits_registers
     else ptx::give_registers<kRoleRegs>();
     if (warp < kEpiWarps) float_epilogue<W, WL, DUMP>(p, sm, base, warp, lane, tmem, abort_flag);
-    else if (lane == 0) {
-        if (warp == kMmaWarp) float_mma<W, WL>(p, sm, base, tmem, abort_flag);
-        else if (warp < kLoadWarp + kFLoaders) float_load_weights<W, WL>(p, sm, base, warp - kLoadWarp, abort_flag);
-        else if constexpr (!float_x_in_smem(W)) float_load_x<W>(p, sm, base, abort_flag);
-    }
+    else if (warp == kMmaWarp) float_mma<W, WL>(p, sm, base, tmem, abort_flag);
+    else if (warp < kLoadWarp + kFLoaders) float_load_weights<W, WL>(p, sm, base, __shfl_sync(0xffffffffu, warp - kLoadWarp, 0), abort_flag);
+    else if constexpr (!float_x_in_smem(W)) float_load_x<W>(p, sm, base, abort_flag);
     ptx::tc_fence_before();
     __syncthreads();
     if (warp == kMmaWarp) {

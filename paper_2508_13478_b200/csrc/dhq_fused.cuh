@@ -214,7 +214,7 @@ __host__ __device__ inline SmemMap smem_map(int W, int n_stages, int const_words
 // tries the thread either sleeps (SLEEP_NS), so that a waiting warp leaves the issue slots to the
 // working ones, or, with HINT_NS > 0, stays suspended inside the try itself for up to that long;
 // the time limit and the abort flag are looked at every 64 tries.  Which form is faster was
-// measured per role: the single-thread MMA and copy roles and the epilogue warps of the
+// measured per role: the one-warp MMA and copy roles and the epilogue warps of the
 // per-token kernels (two more barriers per layer) do better suspended, the epilogue warps of the
 // per-tensor kernels sleeping.
 constexpr int kHintNs = 2000;
@@ -1202,6 +1202,7 @@ __device__ void mma_role(const FusedParams &p, const SmemMap &sm, uint32_t smem_
                          volatile int *abort_flag)
 {
     constexpr int W = C::W;
+    tmem_base = __shfl_sync(0xffffffffu, tmem_base, 0); // uniform for the compiler, see mma_i8
     // (before the first bounded wait: a kernel before this one may run for longer than the limit)
     ptx::wait_for_previous_kernels();
     uint32_t codes_parity[2] = {0, 0};
@@ -1223,9 +1224,9 @@ __device__ void mma_role(const FusedParams &p, const SmemMap &sm, uint32_t smem_
                     const int half = pc / C::KSLABS, ksl = pc % C::KSLABS;
                     const int stage = (int)(use % p.n_stages);
                     const uint32_t par = (uint32_t)((use / p.n_stages) & 1);
-                    if (!wait_bar<0, kHintNs>(smem_base + sm.w_full + 8 * stage, par, abort_flag, p.status)) { ok = false; break; }
+                    if (!wait_bar_warp<true>(smem_base + sm.w_full + 8 * stage, par, abort_flag, p.status)) { ok = false; break; }
                     if (pc == 0) {
-                        if (!wait_bar<0, kHintNs>(smem_base + sm.codes_full, codes_parity[0], abort_flag, p.status)) { ok = false; break; }
+                        if (!wait_bar_warp<true>(smem_base + sm.codes_full, codes_parity[0], abort_flag, p.status)) { ok = false; break; }
                         codes_parity[0] ^= 1;
                         ptx::tc_fence_after();
                     }
@@ -1247,11 +1248,11 @@ __device__ void mma_role(const FusedParams &p, const SmemMap &sm, uint32_t smem_
                 const int slab_id = (l - 2) * C::KSLABS + ksl;
                 const int stage = p.resident ? slab_id : (int)(use % p.n_stages);
                 const uint32_t par = p.resident ? 0u : (uint32_t)((use / p.n_stages) & 1);
-                if (!wait_bar<0, kHintNs>(smem_base + sm.w_full + 8 * stage, par, abort_flag, p.status)) { ok = false; break; }
+                if (!wait_bar_warp<true>(smem_base + sm.w_full + 8 * stage, par, abort_flag, p.status)) { ok = false; break; }
                 const uint32_t b_addr = smem_base + sm.ring + (uint32_t)stage * slab;
                 for (int s = 0; s < active; ++s) {
                     if (ksl == 0) {
-                        if (!wait_bar<0, kHintNs>(smem_base + sm.codes_full + 8 * s, codes_parity[s], abort_flag, p.status)) { ok = false; break; }
+                        if (!wait_bar_warp<true>(smem_base + sm.codes_full + 8 * s, codes_parity[s], abort_flag, p.status)) { ok = false; break; }
                         codes_parity[s] ^= 1;
                         ptx::tc_fence_after();
                     }
@@ -1277,9 +1278,9 @@ __device__ void mma_role(const FusedParams &p, const SmemMap &sm, uint32_t smem_
         if (!ok) break;
         if constexpr (CALIB) continue; // the calibrated layer itself is not computed
         // last layer: N = 16, its weights stay in shared memory
-        if (!wait_bar<0, kHintNs>(smem_base + sm.last_full, 0, abort_flag, p.status)) { ok = false; break; }
+        if (!wait_bar_warp<true>(smem_base + sm.last_full, 0, abort_flag, p.status)) { ok = false; break; }
         for (int s = 0; s < active; ++s) {
-            if (!wait_bar<0, kHintNs>(smem_base + sm.codes_full + 8 * s, codes_parity[s], abort_flag, p.status)) { ok = false; break; }
+            if (!wait_bar_warp<true>(smem_base + sm.codes_full + 8 * s, codes_parity[s], abort_flag, p.status)) { ok = false; break; }
             codes_parity[s] ^= 1;
             ptx::tc_fence_after();
             const uint32_t d = tmem_base + (uint32_t)(s * C::TMEM_COLS_PER_SLOT);
@@ -1307,8 +1308,8 @@ __device__ void load_role(const FusedParams &p, const SmemMap &sm, uint32_t smem
     // (test hook: with skip_last_weights set the copy is left out and nothing ever completes
     // last_full, so the waits for it run out, the abort path runs and the kernel returns)
     if (!p.skip_last_weights && !CALIB) {
-        ptx::mbar_expect_tx(smem_base + sm.last_full, 16 * W);
-        ptx::bulk_g2s(smem_base + sm.last_w, p.layer[p.L - 1].qw_umma, 16 * W, smem_base + sm.last_full);
+        ptx::mbar_expect_tx_warp(smem_base + sm.last_full, 16 * W);
+        ptx::bulk_g2s_warp(smem_base + sm.last_w, p.layer[p.L - 1].qw_umma, 16 * W, smem_base + sm.last_full);
     }
     const int slabs = (p.L - 2) * C::PIECES; // per tile round
     if (slabs <= 0) return;
@@ -1325,15 +1326,15 @@ __device__ void load_role(const FusedParams &p, const SmemMap &sm, uint32_t smem
         if (i >= p.n_stages) {
             if (i == p.n_stages) ptx::wait_for_previous_kernels(); // the first pieces may come early: weights do not change
             uint32_t par = (uint32_t)(((i / p.n_stages) - 1) & 1);
-            if (!wait_bar<0, kHintNs>(smem_base + sm.w_empty + 8 * stage, par, abort_flag, p.status)) { ok = false; break; }
+            if (!wait_bar_warp<true>(smem_base + sm.w_empty + 8 * stage, par, abort_flag, p.status)) { ok = false; break; }
         }
         const int id = (int)(i % slabs);
         const int l = 2 + id / C::PIECES, pc = id % C::PIECES;
-        ptx::mbar_expect_tx(smem_base + sm.w_full + 8 * stage, slab);
+        ptx::mbar_expect_tx_warp(smem_base + sm.w_full + 8 * stage, slab);
         // several copies in flight per slab: one large bulk copy did not reach the L2 bandwidth
         for (uint32_t off = 0; off < slab; off += kCopyBytes) {
             const uint32_t bytes = slab - off < kCopyBytes ? slab - off : kCopyBytes;
-            ptx::bulk_g2s(smem_base + sm.ring + (uint32_t)stage * slab + off,
+            ptx::bulk_g2s_warp(smem_base + sm.ring + (uint32_t)stage * slab + off,
                           p.layer[l - 1].qw_umma + (size_t)pc * slab + off, bytes, smem_base + sm.w_full + 8 * stage);
         }
         ++issued;
@@ -1461,9 +1462,9 @@ __global__ void __launch_bounds__(fused_threads(W, BOTH, GABOR), 1) fused_kernel
     if (warp < kEpiWarps) {
         epilogue_role<C, PER_TOKEN, ROT, SPREAD, AHEAD, DUMP, BOTH, CALIB, GABOR, MIXED>(p, sm, smem_base, warp, lane, tmem_base, abort_flag);
     } else if (warp == kMmaWarp) {
-        if (lane == 0) mma_role<C, SPREAD, CALIB>(p, sm, smem_base, tmem_base, abort_flag);
+        mma_role<C, SPREAD, CALIB>(p, sm, smem_base, tmem_base, abort_flag);
     } else if (warp == kLoadWarp) {
-        if (lane == 0) load_role<C, SPREAD, CALIB>(p, sm, smem_base, abort_flag);
+        load_role<C, SPREAD, CALIB>(p, sm, smem_base, abort_flag);
         if constexpr (DUMP) {
             // Observing instantiation only (in the timed kernels these few instructions cost 3-4 %): an
             // otherwise idle lane of CTA 0 notes the SM's cycle counter and the global nanosecond timer

@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(128) tensor_i8_kernel(int iters, int *status)
     __syncthreads();
     ptx::tc_fence_after();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(gen + holder_off);
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32) {
         const uint32_t idesc = ptx::idesc_i8(128, 256);
         uint32_t parity = 0;
         bool ok = true;
@@ -86,6 +86,7 @@ __global__ void __launch_bounds__(128) tensor_i8_kernel(int iters, int *status)
             while (!ptx::mbar_try_wait(base + bar_off, parity)) {
                 if (ptx::globaltimer() - t0 > 1000000000ull) { ok = false; atomicExch(status, 1); break; }
             }
+            ok = __all_sync(0xffffffffu, ok);
             parity ^= 1;
         }
     }

@@ -71,6 +71,21 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
+// The same, and the arrival that announces its bytes, called by a whole warp and issued by one elected thread: see mma_i8.
+__device__ __forceinline__ void bulk_g2s_warp(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile("{\n\t.reg .pred q;\n\t"
+                 "elect.sync _|q, 0xffffffff;\n\t"
+                 "@q cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n\t}"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+__device__ __forceinline__ void mbar_expect_tx_warp(uint32_t bar, uint32_t bytes)
+{
+    asm volatile("{\n\t.reg .pred q;\n\t"
+                 "elect.sync _|q, 0xffffffff;\n\t"
+                 "@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}" ::"r"(bar), "r"(bytes) : "memory");
+}
+
 // Bulk copy shared -> global of `bytes` (multiple of 16, both addresses 16-byte aligned), tracked
 // by the issuing thread's bulk async-group.
 __device__ __forceinline__ void bulk_s2g(void *dst, uint32_t src, uint32_t bytes)
@@ -99,27 +114,36 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, int8 x int8 -> int32, one CTA.  Issued by one thread.
+// D[tmem] (+)= A[smem] * B[smem]^T, int8 x int8 -> int32, one CTA.  Called by a whole warp, which stays together, and
+// issued by the thread that elect.sync picks (always the same one).  Its operands have to be in uniform registers: in code
+// that only one lane of a warp runs, the compiler has to move each of them there for every instruction, and an MMA took
+// about 105 cycles whatever its size.  With the weight copies issued the same way: width 512, 4,194,304 coordinates 7,416
+// -> 7,022 us; two-sided per channel at width 256 604 -> 569; 8-bit weights with fp32 activations at width 512
+// 1,105 -> 1,047; width 256 with streamed weights 243 -> 238.
 __device__ __forceinline__ void mma_i8(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
 {
-    asm volatile("{\n\t.reg .pred p;\n\t"
+    asm volatile("{\n\t.reg .pred p, q;\n\t"
                  "setp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
+                 "elect.sync _|q, 0xffffffff;\n\t"
+                 "@q tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
                  ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
 // The same with the descriptors as 32-bit words; both operands share the high word.
 __device__ __forceinline__ void mma_i8_words(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t accumulate)
 {
-    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
+    asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t"
                  "mov.b64 a, {%1, %3};\n\tmov.b64 b, {%2, %3};\n\t"
                  "setp.ne.b32 p, %5, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %4, p;\n\t}"
+                 "elect.sync _|q, 0xffffffff;\n\t"
+                 "@q tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %4, p;\n\t}"
                  ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate) : "memory");
 }
-// All MMAs issued so far by this thread arrive on the mbarrier when they have completed.
+// All MMAs issued so far arrive on the mbarrier when they have completed (a whole warp's call, see mma_i8).
 __device__ __forceinline__ void mma_commit(uint32_t bar)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+    asm volatile("{\n\t.reg .pred q;\n\t"
+                 "elect.sync _|q, 0xffffffff;\n\t"
+                 "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar) : "memory");
 }
 
 // Shared-memory operand descriptor, K-major, no swizzle: 8-row x 16-byte core matrices;
