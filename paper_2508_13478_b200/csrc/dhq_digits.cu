@@ -341,7 +341,6 @@ template <int W>
 __device__ void digit_mma(const DigitParams &p, const DigitMap &sm, uint32_t base, uint32_t tmem, volatile int *abort_flag)
 {
     constexpr int NB = W / kDBlock, PIECE = kDBlock * W;
-    tmem = __shfl_sync(0xffffffffu, tmem, 0); // uniform for the compiler, see mma_i8
     ptx::wait_for_previous_kernels(); // before the first bounded wait
     const uint32_t idesc = ptx::idesc_i8(kTile, 128), idesc_last = ptx::idesc_i8(kTile, 16);
     constexpr uint32_t kDescHi = (128u >> 4) | (1u << 14);
@@ -429,7 +428,7 @@ __global__ void __launch_bounds__(kDThreads, 1) digit_kernel(const __grid_consta
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *gen = smem_raw + (base - raw);
     const DigitMap sm = digit_map(W, p.n_stages, p.L);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     volatile int *abort_flag = reinterpret_cast<volatile int *>(gen + sm.abort_flag);
     ptx::launch_dependents();
     if (threadIdx.x == 0) {
@@ -471,7 +470,7 @@ __global__ void __launch_bounds__(kDThreads, 1) digit_kernel(const __grid_consta
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(gen + sm.holder);
+    const uint32_t tmem = ptx::uniform(*reinterpret_cast<volatile uint32_t *>(gen + sm.holder));
     if (warp < kEpiWarps) digit_epilogue<W, PER_TOKEN, GABOR>(p, sm, base, warp, lane, tmem, abort_flag);
     else if (warp == kMmaWarp) digit_mma<W>(p, sm, base, tmem, abort_flag);
     else digit_load<W>(p, sm, base, abort_flag);

@@ -23,12 +23,12 @@
 // (192 KB at width 512; below that from layer to layer), the weights stream past them from L2.  An MMA takes
 // 67 cycles at N = 128 and 51 at N = 64 (operands leave shared memory at 128 B per cycle), hence blocks of 128 outputs
 // and a single set of 3 x 128 accumulator columns: the epilogue releases it as soon as the phases
-// are in registers and computes sines and digits beside the next block's MMAs.  At width 512 the
-// remaining 32 KB of shared memory keep too few weight bytes in flight (105 cycles per MMA); at
-// width 256 the sines and digits of the block behind take as long as the MMAs.
-// Measured: 2 -> 256 x 3 -> 3, fp32, 65,536 coordinates 940 -> 68 us (88 with the digits through L2); 2 -> 512 x 4 -> 3, 8-bit
-// weights, 262,144 coordinates 17.2 -> 1.11 ms (one fp32 CUDA-core pass per layer before; 1.21 ms without the
-// register split of the warpgroups).
+// are in registers and computes sines and digits beside the next block's MMAs.  The sines
+// and digits of a block take as long as the next block's MMAs or longer.
+// Measured: 2 -> 256 x 3 -> 3, fp32, 65,536 coordinates 940 -> 65 us (88 with the digits through L2); 2 -> 512 x 4 -> 3, 8-bit
+// weights, 262,144 coordinates 17.2 -> 1.01 ms (one fp32 CUDA-core pass per layer before).  Blocks of 64 outputs with the weight
+// digits stacked in one operand and two sets of accumulators were slower (70.6 us, 1.16 ms): fewer outputs at a
+// time hide less of the epilogue's latency.
 #include "dhq_fused.cuh"
 
 namespace dhq {
@@ -360,7 +360,6 @@ template <int W, int WL>
 __device__ void float_mma(const FloatParams &p, const FloatMap &sm, uint32_t base, uint32_t tmem, volatile int *abort_flag)
 {
     constexpr int FB = float_block(W), KC = float_kc(W), NB = W / FB, NKC = W / KC, PIECE = FB * KC;
-    tmem = __shfl_sync(0xffffffffu, tmem, 0); // uniform for the compiler, see mma_i8
     ptx::wait_for_previous_kernels(); // before the first bounded wait
     const uint32_t idesc = ptx::idesc_i8(kTile, FB);
     constexpr uint32_t kDescHi = (128u >> 4) | (1u << 14);
@@ -483,7 +482,7 @@ __global__ void __launch_bounds__(kFThreads, 1) float_kernel(const __grid_consta
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *gen = smem_raw + (base - raw);
     const FloatMap sm = float_map(W, p.n_stages, p.L);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     volatile int *abort_flag = reinterpret_cast<volatile int *>(gen + sm.abort_flag);
     ptx::launch_dependents();
     if (threadIdx.x == 0) {
@@ -522,12 +521,12 @@ __global__ void __launch_bounds__(kFThreads, 1) float_kernel(const __grid_consta
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(gen + sm.holder);
+    const uint32_t tmem = ptx::uniform(*reinterpret_cast<volatile uint32_t *>(gen + sm.holder));
     if (warp < kEpiWarps) ptx::take_registers<kEpiRegs>(); // see splits_registers
     else ptx::give_registers<kRoleRegs>();
     if (warp < kEpiWarps) float_epilogue<W, WL, DUMP>(p, sm, base, warp, lane, tmem, abort_flag);
     else if (warp == kMmaWarp) float_mma<W, WL>(p, sm, base, tmem, abort_flag);
-    else if (warp < kLoadWarp + kFLoaders) float_load_weights<W, WL>(p, sm, base, __shfl_sync(0xffffffffu, warp - kLoadWarp, 0), abort_flag);
+    else if (warp < kLoadWarp + kFLoaders) float_load_weights<W, WL>(p, sm, base, warp - kLoadWarp, abort_flag);
     else if constexpr (!float_x_in_smem(W)) float_load_x<W>(p, sm, base, abort_flag);
     ptx::tc_fence_before();
     __syncthreads();

@@ -1202,7 +1202,6 @@ __device__ void mma_role(const FusedParams &p, const SmemMap &sm, uint32_t smem_
                          volatile int *abort_flag)
 {
     constexpr int W = C::W;
-    tmem_base = __shfl_sync(0xffffffffu, tmem_base, 0); // uniform for the compiler, see mma_i8
     // (before the first bounded wait: a kernel before this one may run for longer than the limit)
     ptx::wait_for_previous_kernels();
     uint32_t codes_parity[2] = {0, 0};
@@ -1388,7 +1387,7 @@ __global__ void __launch_bounds__(fused_threads(W, BOTH, GABOR), 1) fused_kernel
     const uint32_t smem_base = (raw + 1023u) & ~1023u;
     uint8_t *smem_gen = smem_raw + (smem_base - raw);
     const SmemMap sm = smem_map(W, p.n_stages, p.const_words);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem_gen + sm.abort_flag);
     volatile uint32_t *tmem_holder = reinterpret_cast<volatile uint32_t *>(smem_gen + sm.tmem_holder);
     // Repeated calls: the next launch's blocks set themselves up - barriers, tensor memory, constants and first
@@ -1453,7 +1452,7 @@ __global__ void __launch_bounds__(fused_threads(W, BOTH, GABOR), 1) fused_kernel
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    const uint32_t tmem_base = *tmem_holder;
+    const uint32_t tmem_base = ptx::uniform(*tmem_holder);
 
     if constexpr (splits_registers(W, BOTH, GABOR)) {
         if (warp < kEpiWarps) ptx::take_registers<kEpiRegs>();
