@@ -20,13 +20,13 @@
 // activations or weights use little of that range go to dhq_float_layers.cu (fixed_point_serves).
 //
 // What bounds it.  The digits of a tile of 128 activations stay in shared memory for a whole layer
-// (192 KB at width 512; below that from layer to layer), the weights stream past them from L2.  An MMA takes
+// (128 KB and a quarter of tensor memory at width 512; below that from layer to layer), the weights stream past them from L2.  An MMA takes
 // 67 cycles at N = 128 and 51 at N = 64 (operands leave shared memory at 128 B per cycle), hence blocks of 128 outputs
 // and a single set of 3 x 128 accumulator columns: the epilogue releases it as soon as the phases
 // are in registers and computes sines and digits beside the next block's MMAs.  The sines
 // and digits of a block take as long as the next block's MMAs or longer.
 // Measured: 2 -> 256 x 3 -> 3, fp32, 65,536 coordinates 940 -> 65 us (88 with the digits through L2); 2 -> 512 x 4 -> 3, 8-bit
-// weights, 262,144 coordinates 17.2 -> 1.01 ms (one fp32 CUDA-core pass per layer before).  Blocks of 64 outputs with the weight
+// weights, 262,144 coordinates 17.2 -> 0.94 ms (one fp32 CUDA-core pass per layer before).  Blocks of 64 outputs with the weight
 // digits stacked in one operand and two sets of accumulators were slower (70.6 us, 1.16 ms): fewer outputs at a
 // time hide less of the epilogue's latency.
 #include "dhq_fused.cuh"
@@ -65,26 +65,36 @@ struct FloatParams {
 // sums.  So the next layer's MMAs begin on part 0 while block 1's outputs are still being formed.  At width 512 one layer's
 // digits fill 192 KB and go through L2 instead.
 __host__ __device__ constexpr bool float_x_in_smem(int W) { return W < 512; }
+// Width 512: the third digit, which meets the first weight digit only, is an operand in tensor memory (columns 384-511,
+// four consecutive k to a column) instead of shared memory.  That leaves room for the epilogue constants, which were read
+// through an L1 cache of a few KB, and for seven weight pieces in flight instead of four: 262,144 coordinates, 5 layers, 8-bit
+// weights 1,011 -> 940 us (the third digit alone, without the constants: no gain).
+constexpr int kFX2Col = 3 * 128;
+__host__ __device__ constexpr int float_smem_digits(int W) { return W == 512 ? 2 : 3; }
 __host__ __device__ constexpr uint32_t float_part_bytes(int W) { return 3u * kTile * (W < 128 ? W : 128); }
 
-// At width 512 the activations leave no room for the epilogue constants: they are read through L1.
-__host__ __device__ constexpr bool float_consts_in_smem(int W) { return W < 512; }
+// At width 512 there is room for the first layer's epilogue constants and those of two hidden layers: a layer's three arrays
+// are brought by bulk copies while the layer before is worked on.
+__host__ __device__ constexpr bool float_consts_resident(int W) { return W < 512; }
 __host__ __device__ constexpr int float_areas(int W) { return W <= 128 ? 4 : 3; } // per hidden layer, see digit_phase2
 
 struct FloatMap {
-    uint32_t a, ring, consts, w_full, w_empty, a_full, x_ready, acc_full, acc_empty, quad_sync, drain, holder, abort_flag, total;
+    uint32_t a, ring, consts, part, w_full, w_empty, a_full, x_ready, x2_ready, c_full, acc_full, acc_empty, quad_sync, drain, holder, abort_flag, total;
 };
 __host__ __device__ inline FloatMap float_map(int W, int n_stages, int L)
 {
     FloatMap m;
     uint32_t off = 0;
-    m.a = off; off += float_x_in_smem(W) ? (uint32_t)(W / float_block(W) + 1) * float_part_bytes(W) : 3u * kTile * W;
+    m.a = off; off += float_x_in_smem(W) ? (uint32_t)(W / float_block(W) + 1) * float_part_bytes(W) : (uint32_t)float_smem_digits(W) * kTile * W;
     m.ring = off; off += (uint32_t)n_stages * float_block(W) * float_kc(W);
-    m.consts = off; off += float_consts_in_smem(W) ? (uint32_t)(4 + float_areas(W) * (L - 2)) * W * 4 : 0; // first layer, then c0 | c0_lo | cb (| cb_lo) per hidden layer
+    m.consts = off; off += (uint32_t)(4 + float_areas(W) * (float_consts_resident(W) ? L - 2 : 2)) * W * 4; // first layer, then c0 | c0_lo | cb (| cb_lo) per hidden layer
+    m.part = off; off += float_x_in_smem(W) ? 0 : 2 * 4 * kTile * 16; // width 512: the last layer's partial sums
     m.w_full = off; off += 8 * kFMaxStages;
     m.w_empty = off; off += 8 * kFMaxStages;
     m.a_full = off; off += 8 * 8;
     m.x_ready = off; off += 8;
+    m.x2_ready = off; off += 8;
+    m.c_full = off; off += 8 * 2;
     m.acc_full = off; off += 8;
     m.acc_empty = off; off += 8;
     m.quad_sync = off; off += 8 * 4;
@@ -224,7 +234,7 @@ __device__ void float_epilogue(const FloatParams &p, const FloatMap &sm, uint32_
             float y[16];
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
-                const float4 w = float_consts_in_smem(W) ? lds128(base + sm.consts + (k0 + j) * 16) : __ldg(p.l1 + k0 + j);
+                const float4 w = lds128(base + sm.consts + (k0 + j) * 16);
                 const float t = __fmaf_rn(x, w.x, __fmaf_rn(yc, w.y, w.z));
                 y[j] = sine_of_turns(__fsub_rn(t, __fsub_rn(__fadd_rn(t, 12582912.0f), 12582912.0f)));
             }
@@ -259,10 +269,25 @@ __device__ void float_epilogue(const FloatParams &p, const FloatMap &sm, uint32_
         coords_of(tile + gridDim.x, x, yc);
         for (int l = 2; l < p.L; ++l) {
             ++tlayer;
+            const uint32_t cbase = base + sm.consts + (uint32_t)((4 + float_areas(W) * (float_consts_resident(W) ? (uint32_t)(l - 2) : (tlayer - 1) & 1)) * W * 4);
             if constexpr (!XS) {
                 // the activations in device memory become visible to the bulk copies of this CTA
                 asm volatile("fence.proxy.async;" ::: "memory");
                 ptx::mbar_arrive(base + sm.x_ready);
+                // this thread's part of the third digit to tensor memory: the MMAs of the layer before, which read that
+                // operand, completed with its last block's sums
+                uint4 v[2 * NB];
+#pragma unroll
+                for (int q = 0; q < 2 * NB; ++q) v[q] = __ldcg(reinterpret_cast<const uint4 *>(xrow + 2 * (kTile * W) + (q / 2 * 8 + sub * 2 + q % 2) * (kTile * 16)));
+#pragma unroll
+                for (int b = 0; b < NB; ++b) {
+                    const uint32_t u[8] = {v[2 * b].x, v[2 * b].y, v[2 * b].z, v[2 * b].w, v[2 * b + 1].x, v[2 * b + 1].y, v[2 * b + 1].z, v[2 * b + 1].w};
+                    ptx::tmem_st8(taddr + kFX2Col + (b * 8 + sub * 2) * 4, u);
+                }
+                ptx::tmem_wait_st();
+                ptx::tc_fence_before();
+                ptx::mbar_arrive(base + sm.x2_ready);
+                if (!wait_bar_warp<true>(base + sm.c_full + 8 * ((tlayer - 1) & 1), ((tlayer - 1) >> 1) & 1, abort_flag, p.status)) return;
             }
 #pragma unroll 1
             for (int b = 0; b < NB; ++b, ++use) {
@@ -285,15 +310,9 @@ __device__ void float_epilogue(const FloatParams &p, const FloatMap &sm, uint32_
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         float4 c, e, o, ol = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if constexpr (float_consts_in_smem(W)) {
-                            const uint32_t at = base + sm.consts + (uint32_t)(((4 + float_areas(W) * (l - 2)) * W + k0 + g * 16 + 4 * q) * 4);
-                            c = lds128(at); e = lds128(at + W * 4); o = lds128(at + 2 * W * 4);
-                            if constexpr (float_rounds_once(W)) ol = lds128(at + 3 * W * 4);
-                        } else {
-                            c = __ldg(reinterpret_cast<const float4 *>(p.c0[l - 1] + k0 + g * 16) + q);
-                            e = __ldg(reinterpret_cast<const float4 *>(p.c0_lo[l - 1] + k0 + g * 16) + q);
-                            o = __ldg(reinterpret_cast<const float4 *>(p.cb[l - 1] + k0 + g * 16) + q);
-                        }
+                        const uint32_t at = cbase + (uint32_t)((k0 + g * 16 + 4 * q) * 4);
+                        c = lds128(at); e = lds128(at + W * 4); o = lds128(at + 2 * W * 4);
+                        if constexpr (float_rounds_once(W)) ol = lds128(at + 3 * W * 4);
                         r[g * 8 + 2 * q] = digit_phase2<W>(&D[0][4 * q], &D[1][4 * q], &D[2][4 * q], pack2(c.x, c.y), pack2(e.x, e.y), pack2(o.x, o.y), pack2(ol.x, ol.y));
                         r[g * 8 + 2 * q + 1] = digit_phase2<W>(&D[0][4 * q + 2], &D[1][4 * q + 2], &D[2][4 * q + 2], pack2(c.z, c.w), pack2(e.z, e.w), pack2(o.z, o.w), pack2(ol.z, ol.w));
                     }
@@ -322,19 +341,32 @@ __device__ void float_epilogue(const FloatParams &p, const FloatMap &sm, uint32_
         // layers and one block of outputs nothing else orders the two), but to come back to this set it has to pass the
         // next tile's barrier, where the reader arrives after its reads.
         {
-            const uint32_t part_col = taddr + kFPartCol + 16 * qpar;
             const uint32_t u[4] = {__float_as_uint(part[0]), __float_as_uint(part[1]), __float_as_uint(part[2]), __float_as_uint(part[3])};
-            ptx::tmem_st4(part_col + 4 * sub, u);
-            ptx::tmem_wait_st();
-            ptx::tc_fence_before();
+            const uint32_t part_col = taddr + kFPartCol + 16 * qpar;
+            const uint32_t part_at = base + sm.part + qpar * (4 * kTile * 16) + row * 16; // (width 512: in shared memory)
+            if constexpr (XS) {
+                ptx::tmem_st4(part_col + 4 * sub, u);
+                ptx::tmem_wait_st();
+                ptx::tc_fence_before();
+            } else {
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(part_at + sub * (kTile * 16)), "r"(u[0]), "r"(u[1]), "r"(u[2]), "r"(u[3]) : "memory");
+            }
             ptx::mbar_arrive(base + sm.quad_sync + 8 * quad);
             if (!wait_bar_warp<true>(base + sm.quad_sync + 8 * quad, qpar, abort_flag, p.status)) return;
             qpar ^= 1;
             ptx::tc_fence_after();
             if (sub == 0) {
                 uint32_t v[16];
-                ptx::tmem_ld16(part_col, v);
-                ptx::tmem_wait_ld();
+                if constexpr (XS) {
+                    ptx::tmem_ld16(part_col, v);
+                    ptx::tmem_wait_ld();
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float4 f = lds128(part_at + q * (kTile * 16));
+                        v[4 * q] = __float_as_uint(f.x); v[4 * q + 1] = __float_as_uint(f.y); v[4 * q + 2] = __float_as_uint(f.z); v[4 * q + 3] = __float_as_uint(f.w);
+                    }
+                }
                 if (valid) {
 #pragma unroll
                     for (int m = 0; m < 4; ++m) {
@@ -392,11 +424,24 @@ __device__ void float_mma(const FloatParams &p, const FloatMap &sm, uint32_t bas
                         const uint32_t bk = b0 + (uint32_t)stage * (PIECE >> 4);
 #pragma unroll
                         for (int i = 0; i + j < 3; ++i) {
+                            if (!XS && i == 2 && b == 0 && kc == 0) { // the third digit is in tensor memory
+                                ok = wait_bar_warp<true>(base + sm.x2_ready, layers & 1, abort_flag, p.status);
+                                if (!ok) break;
+                                ptx::tc_fence_after();
+                            }
 #pragma unroll
-                            for (int ks = 0; ks < KC / 32; ++ks)
+                            for (int ks = 0; ks < KC / 32; ++ks) {
+                                if constexpr (!XS) {
+                                    if (i == 2) {
+                                        ptx::mma_i8_tmem(tmem + (uint32_t)(i + j) * FB, tmem + kFX2Col + (uint32_t)((kc * (KC / 32) + ks) * 8), bk + (ks * 2 * FB * 16 >> 4), kDescHi, idesc, (j > 0 || ks > 0) ? 1u : (uint32_t)kc);
+                                        continue;
+                                    }
+                                }
                                 ptx::mma_i8_words(tmem + (uint32_t)(i + j) * FB, ak + ((i * DIGIT + ks * 2 * kTile * 16) >> 4), bk + (ks * 2 * FB * 16 >> 4),
                                                   kDescHi, idesc, (j > 0 || ks > 0) ? 1u : (uint32_t)kc);
+                            }
                         }
+                        if (!ok) break;
                         ptx::mma_commit(base + sm.w_empty + 8 * stage);
                         if (++stage == p.n_stages) { stage = 0; wpar ^= 1; }
                     }
@@ -451,6 +496,17 @@ template <int W>
 __device__ void float_load_x(const FloatParams &p, const FloatMap &sm, uint32_t base, volatile int *abort_flag)
 {
     const uint8_t *src = p.x + (size_t)blockIdx.x * (3 * kTile * W);
+    // the constants of layer l for the CTA's t-th tensor-core layer, into set t & 1
+    uint32_t asked = 0;
+    auto load_consts = [&](int l, uint32_t t) {
+        asked = t + 1;
+        const uint32_t at = base + sm.consts + (4 + 3 * (t & 1)) * W * 4, bar = base + sm.c_full + 8 * (t & 1);
+        ptx::mbar_expect_tx_warp(bar, 3 * W * 4);
+        ptx::bulk_g2s_warp(at, p.c0[l - 1], W * 4, bar);
+        ptx::bulk_g2s_warp(at + W * 4, p.c0_lo[l - 1], W * 4, bar);
+        ptx::bulk_g2s_warp(at + 2 * W * 4, p.cb[l - 1], W * 4, bar);
+    };
+    if (p.L > 2) load_consts(2, 0);
     ptx::wait_for_previous_kernels();
     uint32_t layers = 0;
     bool ok = true;
@@ -459,17 +515,22 @@ __device__ void float_load_x(const FloatParams &p, const FloatMap &sm, uint32_t 
             if (!wait_bar_warp<true>(base + sm.x_ready, layers & 1, abort_flag, p.status)) { ok = false; break; }
             asm volatile("fence.proxy.async;" ::: "memory");
             for (int c = 0; c < W / 64; ++c) {
-                ptx::mbar_expect_tx_warp(base + sm.a_full + 8 * c, 3 * 64 * kTile);
-                for (int i = 0; i < 3; ++i) {
+                ptx::mbar_expect_tx_warp(base + sm.a_full + 8 * c, float_smem_digits(W) * 64 * kTile);
+                for (int i = 0; i < float_smem_digits(W); ++i) {
                     const uint32_t off = (uint32_t)(i * kTile * W + c * 64 * kTile);
                     ptx::bulk_g2s_warp(base + sm.a + off, src + off, 64 * kTile, base + sm.a_full + 8 * c);
                 }
             }
+            // all threads are done with the layer before: the next one's constants take the place of that one's
+            if (l + 1 < p.L || tile + gridDim.x < p.n_tiles) load_consts(l + 1 < p.L ? l + 1 : 2, layers + 1);
         }
     }
-    if ((!ok || *abort_flag) && layers > 0) {
+    if (!ok || *abort_flag) { // let copies in flight land before the CTA may exit
         const unsigned long long t0 = ptx::globaltimer();
-        for (int c = 0; c < W / 64; ++c)
+        // (set t & 1 holds the constants of layer t; the last copies were those for `asked` - 1 and the one before)
+        for (uint32_t t = asked > 2 ? asked - 2 : 0; t < asked; ++t)
+            while (!ptx::mbar_try_wait(base + sm.c_full + 8 * (t & 1), (t >> 1) & 1) && ptx::globaltimer() - t0 < wait_limit_of(abort_flag)) {}
+        for (int c = 0; layers > 0 && c < W / 64; ++c)
             while (!ptx::mbar_try_wait(base + sm.a_full + 8 * c, (layers - 1) & 1) && ptx::globaltimer() - t0 < wait_limit_of(abort_flag)) {}
     }
 }
@@ -494,6 +555,8 @@ __global__ void __launch_bounds__(kFThreads, 1) float_kernel(const __grid_consta
         }
         for (int i = 0; i < 8; ++i) ptx::mbar_init(base + sm.a_full + 8 * i, float_x_in_smem(W) ? kEpiWarps : 1);
         ptx::mbar_init(base + sm.x_ready, kEpiWarps * 32);
+        ptx::mbar_init(base + sm.x2_ready, kEpiWarps * 32);
+        for (int i = 0; i < 2; ++i) ptx::mbar_init(base + sm.c_full + 8 * i, 1);
         ptx::mbar_init(base + sm.acc_full, 1);
         ptx::mbar_init(base + sm.acc_empty, kEpiWarps * 32);
         for (int i = 0; i < 4; ++i) ptx::mbar_init(base + sm.quad_sync + 8 * i, 128);
@@ -504,10 +567,10 @@ __global__ void __launch_bounds__(kFThreads, 1) float_kernel(const __grid_consta
         ptx::tmem_alloc(base + sm.holder, 512);
         ptx::tmem_relinquish();
     }
-    if constexpr (float_consts_in_smem(W)) {
+    {
         float4 *dst = reinterpret_cast<float4 *>(gen + sm.consts);
         for (int i = threadIdx.x; i < W; i += kFThreads) dst[i] = __ldg(p.l1 + i);
-        for (int l = 1; l < p.L - 1; ++l) {
+        for (int l = 1; float_consts_resident(W) && l < p.L - 1; ++l) {
             float *c = reinterpret_cast<float *>(dst) + (4 + float_areas(W) * (l - 1)) * W;
             for (int i = threadIdx.x; i < W; i += kFThreads) {
                 c[i] = __ldg(p.c0[l] + i);

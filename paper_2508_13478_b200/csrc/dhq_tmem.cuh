@@ -145,6 +145,16 @@ __device__ __forceinline__ void mma_i8_words(uint32_t d_tmem, uint32_t a_lo, uin
                  "@q tcgen05.mma.cta_group::1.kind::i8 [%0], a, b, %4, p;\n\t}"
                  ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate) : "memory");
 }
+// The same with A in tensor memory: lane = row, four consecutive k of a row to a column.
+__device__ __forceinline__ void mma_i8_tmem(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b64 b;\n\t"
+                 "mov.b64 b, {%2, %3};\n\t"
+                 "setp.ne.b32 p, %5, 0;\n\t"
+                 "elect.sync _|q, 0xffffffff;\n\t"
+                 "@q tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], b, %4, p;\n\t}"
+                 ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accumulate) : "memory");
+}
 // All MMAs issued so far arrive on the mbarrier when they have completed (a whole warp's call, see mma_i8).
 __device__ __forceinline__ void mma_commit(uint32_t bar)
 {

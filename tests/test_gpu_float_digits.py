@@ -83,6 +83,29 @@ def test_tiles_of_one_block_do_not_disturb_each_other(width, n_linear):
         dhq.dhq_destroy(h)
 
 
+@pytest.mark.parametrize("n_linear,w_bits", [(3, 32), (3, 8), (4, 8), (6, 32)])
+def test_tiles_of_one_block_at_width_512(n_linear, w_bits):
+    # the same for the width whose third digit, constants and last-layer sums pass from tile to tile through tensor and
+    # shared memory: one and several tensor-core layers, two and three weight digits
+    dims = (2,) + (512,) * (n_linear - 1) + (3,)
+    weights, biases = dhq_inputs.siren_init(dims, 30.0, 950 + n_linear)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n = 128 * (2 * sms + 1) + 77
+    cd = to_dev(dhq_inputs.grid_coords(n // 240 + 1, 240)[:n])
+    h = dhq.dhq_prepare(dims, [to_dev(x) for x in weights], [to_dev(x) for x in biases], 30.0, w_bits, dhq.DHQ_BITS_FLOAT)
+    try:
+        want = torch.empty((n, 3), device="cuda")
+        for t in range(0, n, 128 * sms):   # one tile per block
+            dhq.dhq_forward(h, cd[t:t + 128 * sms], want[t:t + 128 * sms])
+        for _ in range(5):
+            got = torch.full((n, 3), float("nan"), device="cuda")
+            dhq.dhq_forward(h, cd, got)
+            assert torch.equal(got.view(torch.int32), want.view(torch.int32))
+        assert dhq.dhq_last_status(h) == 0
+    finally:
+        dhq.dhq_destroy(h)
+
+
 @pytest.mark.parametrize("width", [64, 256, 512])
 def test_dump_buffers_and_coordinates_need_no_more_than_float_alignment(width):
     dims, n = (2, width, width, width, 3), 300
