@@ -1463,17 +1463,18 @@ __global__ void __launch_bounds__(fused_threads(W, BOTH, GABOR), 1) fused_kernel
     } else if (warp == kMmaWarp) {
         mma_role<C, SPREAD, CALIB>(p, sm, smem_base, tmem_base, abort_flag);
     } else if (warp == kLoadWarp) {
-        load_role<C, SPREAD, CALIB>(p, sm, smem_base, abort_flag);
         if constexpr (DUMP) {
-            // Observing instantiation only (in the timed kernels these few instructions cost 3-4 %): an
-            // otherwise idle lane of CTA 0 notes the SM's cycle counter and the global nanosecond timer
-            // before the work (status words 2-5); the MMA warp notes them again after it (words 6-9).
+            // Observing instantiation only (in the timed kernels these few instructions cost 3-4 %): the copy
+            // warp of CTA 0 notes the SM's cycle counter and the global nanosecond timer before it begins
+            // (status words 2-5); the MMA warp notes them again after the work (words 6-9).
             // The ratio of the differences is the SM clock the launch really ran at.
-            if (lane == 1 && blockIdx.x == 0) {
+            if (lane == 0 && blockIdx.x == 0) {
                 reinterpret_cast<long long *>(p.status)[1] = clock64();
                 reinterpret_cast<unsigned long long *>(p.status)[2] = ptx::globaltimer();
             }
+            __syncwarp();
         }
+        load_role<C, SPREAD, CALIB>(p, sm, smem_base, abort_flag);
     } else {
         if constexpr (C::BULK_XY) {
             if (warp == kXyWarp && lane == 0) xy_role<C, SPREAD>(p, sm, smem_base, abort_flag);
