@@ -294,7 +294,7 @@ __device__ __forceinline__ float max_abs(float m, float a, float b)
 // The epilogues of dhq_math.cuh on two columns at once: packed multiplies, additions and fused multiply-adds in the
 // same order give the same bits with half the issue slots.  Per-token scales at width 256, with the one-instruction maxima
 // and the group kept in registers by finish_layer: 262,144 coordinates, 5 layers 260 -> 244 us, 1,048,576 in 4-bit
-// codes 1,031 -> 972; wavelet without rotation at width 128, 267,007 coordinates, 4 layers 147 -> 126.
+// codes 1,031 -> 972.
 __device__ __forceinline__ f32x2 sine2(f32x2 x)
 {
     float a, b;

@@ -104,11 +104,13 @@ __device__ __forceinline__ float epilogue_mixed(float accf, float c_hi, float c_
 // psi(z) = sin(omega0 z) exp(-(s0 z)^2), from the compensated phase x = omega0 z and c = s0 / omega0.
 // The envelope's exponent carries a relative error of a few 2^-24, the result stays within the
 // sine's own error.
-// (.ftz: an envelope below 2^-126 is zero, which saves the four instructions that scale such arguments and results.)
+// (Not ex2.approx.ftz, which makes envelopes below 2^-126 zero: the scaling that ex2.approx spends on them costs 16 us of 134,
+// width 128, 267,007 coordinates, 4 layers, without rotation.  With .ftz and a vote per four columns on whether any is
+// that small it is 130 us, but 139 where many are.)
 __device__ __forceinline__ float gabor_envelope(float t)
 {
     float e;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(t));
+    asm("ex2.approx.f32 %0, %1;" : "=f"(e) : "f"(t));
     return e;
 }
 __device__ __forceinline__ float gabor_epilogue(float accf, float c_hi, float c_lo, float cb, float c)
