@@ -53,6 +53,11 @@ constexpr int kMmaWarp = 16, kLoadWarp = 17, kXyWarp = 18;
 // width 512 lost 2 to 5 % and those of width 64 2 %, so they keep 18 warps (19 at width 512).
 __host__ __device__ constexpr bool splits_registers(int W, bool both, bool gabor) { return W == 128 || W == 256 || (W == 512 && (both || gabor)); }
 __host__ __device__ constexpr int fused_threads(int W, bool both, bool gabor) { return splits_registers(W, both, gabor) ? 20 * 32 : W == 512 ? 19 * 32 : 18 * 32; }
+// Whether a kernel makes its warp's number a uniform value (ptx::uniform): not the observing ones, where it took the registers of
+// the row pointers (spilled bytes stored / loaded 40-176 / 50-310 -> 490-820 / 1,740-3,570, 70,000 coordinates at width 128
+// with all dumps 585 -> 665 us), nor calibration without rotation at width 512 (88 / 240 -> 528 / 920, 65,536 coordinates
+// 323 -> 425 us) and at width 64 (79 -> 82 us); at the other widths calibration gains (256: 0.90 x).
+__host__ __device__ constexpr bool uniform_warp(int W, bool rot, bool dump, bool calib, bool gabor) { return !dump && !(calib && (W == 64 || (W == 512 && !rot && !gabor))); }
 constexpr int kEpiRegs = 104, kRoleRegs = 56, kLaunchRegs = 96;
 static_assert(kEpiWarps * kEpiRegs + (20 - kEpiWarps) * kRoleRegs <= 20 * kLaunchRegs, "more registers than the launch has");
 constexpr int kMaxStages = 32;
@@ -1387,7 +1392,7 @@ __global__ void __launch_bounds__(fused_threads(W, BOTH, GABOR), 1) fused_kernel
     const uint32_t smem_base = (raw + 1023u) & ~1023u;
     uint8_t *smem_gen = smem_raw + (smem_base - raw);
     const SmemMap sm = smem_map(W, p.n_stages, p.const_words);
-    const int warp = ptx::uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int warp = uniform_warp(W, ROT, DUMP, CALIB, GABOR) ? ptx::uniform(threadIdx.x >> 5) : threadIdx.x >> 5, lane = threadIdx.x & 31;
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem_gen + sm.abort_flag);
     volatile uint32_t *tmem_holder = reinterpret_cast<volatile uint32_t *>(smem_gen + sm.tmem_holder);
     // Repeated calls: the next launch's blocks set themselves up - barriers, tensor memory, constants and first
