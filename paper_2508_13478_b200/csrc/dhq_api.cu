@@ -236,7 +236,7 @@ struct BlobHeader {
     float phase_bound[kMaxLayers];
     uint64_t payload_bytes, payload_fnv1a;
 };
-constexpr uint32_t kBlobVersion = 7, kOldestBlob = 6; // 6: another order of the two-sided digits' image, formed anew on import
+constexpr uint32_t kBlobVersion = 7, kOldestBlob = 6; // 6: another order of the two-sided digits' images, which are then formed anew
 const char kBlobMagic[8] = {'D', 'H', 'Q', 'B', '2', '0', '0', 0};
 
 uint64_t fnv1a(const uint8_t *p, size_t n)
@@ -974,7 +974,7 @@ dhq_status_t dhq_import(const void *host_buf, int64_t bytes, void *stream, dhq_h
             }
         }
         if (rc != DHQ_OK) break;
-        for (int l = 2; l <= h->L && h->layer[0].has_digits; ++l)
+        for (int l = 2; l <= h->L && h->layer[0].has_digits && hd.version < kBlobVersion; ++l)
             if (launch_repack_digits(h->layer[l - 1], h->w, l == h->L, st, &h->launches) != cudaSuccess) rc = DHQ_ERR_CUDA;
         // (the same constants again from the same scales: a block of an earlier build splits the bias differently)
         for (int l = 1; l <= h->L && h->layer[0].has_digits && hd.calibrated; ++l)

@@ -540,18 +540,18 @@ __global__ void __launch_bounds__(128) prep_digit_rows_kernel(const __grid_const
     }
 }
 
-// The image again from the digits in [4][K/4][M] words: a saved block may hold it in the order of an earlier build.
+// The image again from the digits in [4][K/4][M] words: a block saved by an earlier build holds it in another order.
 __global__ void __launch_bounds__(256) repack_digits_kernel(LayerDev dev, int w, int last)
 {
     const int K = dev.K, M = dev.M, words = M * K; // four digits of M K / 4 words
-    for (int i = blockIdx.x * 256 + threadIdx.x; i < words; i += gridDim.x * 256) {
-        const int d = i / (words / 4), r = i % (words / 4), k = r / M * 4, m = r % M;
-        *reinterpret_cast<uint32_t *>(dev.gd_img + digit_image_offset(w, last != 0, m, k, d)) = dev.gd_k4m[i];
-    }
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i >= words) return;
+    const int d = i / (words / 4), r = i % (words / 4), k = r / M * 4, m = r % M;
+    *reinterpret_cast<uint32_t *>(dev.gd_img + digit_image_offset(w, last != 0, m, k, d)) = dev.gd_k4m[i];
 }
 cudaError_t launch_repack_digits(const LayerDev &dev, int w, bool last, cudaStream_t st, int64_t *launches)
 {
-    repack_digits_kernel<<<148, 256, 0, st>>>(dev, w, last ? 1 : 0);
+    repack_digits_kernel<<<(dev.M * dev.K + 255) / 256, 256, 0, st>>>(dev, w, last ? 1 : 0);
     *launches += 1;
     return cudaGetLastError();
 }

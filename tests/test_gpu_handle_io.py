@@ -192,3 +192,23 @@ def test_import_forms_the_two_sided_digit_images_anew(width):
         dhq.dhq_destroy(h)
         if h2:
             dhq.dhq_destroy(h2)
+
+
+@pytest.mark.gpu
+def test_import_of_the_present_format_forms_no_images():
+    from paper_2508_13478_b200 import build
+    build.build()
+    dims = (2, 128, 128, 128, 3)
+    weights, biases = dhq_inputs.siren_init(dims, 30.0, 72)
+    fine = dhq.DHQ_GRAN_CHANNEL_OR_TOKEN
+    handles = [dhq.dhq_prepare(dims, [to_dev(x) for x in weights], [to_dev(x) for x in biases], 30.0, w_gran=fine, a_gran=fine, rotation=dhq.DHQ_ROT_BOTH)]
+    try:
+        blob = dhq.dhq_export(handles[0])
+        header = int(np.frombuffer(blob[12:16], np.uint32)[0])
+        handles += [dhq.dhq_import(blob), dhq.dhq_import(as_format_6(blob, header))]
+        launches = [dhq.dhq_launch_count(h) for h in handles]
+        assert launches[2] - launches[1] == len(dims) - 2    # one image per layer but the first
+        assert dhq.dhq_export(handles[1]) == blob and dhq.dhq_export(handles[2]) == blob
+    finally:
+        for h in handles:
+            dhq.dhq_destroy(h)
