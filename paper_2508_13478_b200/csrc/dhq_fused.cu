@@ -457,7 +457,7 @@ template <int WHICH> __global__ void __launch_bounds__(512, 1) pass_rate_kernel(
     constexpr uint32_t kConsts = 2 * kTile * W, kHolder = kConsts + 3 * W * 4; // two A tiles, then cA | cB | cA_lo
     float *cst = reinterpret_cast<float *>(gen + kConsts);
     for (int i = threadIdx.x; i < 3 * W; i += blockDim.x) cst[i] = (i < W) ? 1e-5f : (i < 2 * W ? 0.3f : 0.f);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (warp == 0) {
         ptx::tmem_alloc(base + kHolder, 512);
         ptx::tmem_relinquish();
@@ -465,7 +465,7 @@ template <int WHICH> __global__ void __launch_bounds__(512, 1) pass_rate_kernel(
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(gen + kHolder);
+    const uint32_t tmem = ptx::uniform(*reinterpret_cast<volatile uint32_t *>(gen + kHolder));
     const int quad = warp & 3, slot = warp >> 3, sub = (warp >> 2) & 1;
     const uint32_t taddr = tmem + (uint32_t)(slot * C::TMEM_COLS_PER_SLOT) + ((uint32_t)(quad * 32) << 16);
     {
@@ -480,7 +480,7 @@ template <int WHICH> __global__ void __launch_bounds__(512, 1) pass_rate_kernel(
         if (WHICH & 1) {
 #pragma unroll
             for (int cc = 0; cc < C::CPT; ++cc) {
-                const int ch = sub * C::CPT + cc;
+                const int ch = chunk_of<C>(sub, cc);
                 uint32_t v[CH];
                 tmem_ld<CH>(taddr + ch * CH, v);
                 ptx::tmem_wait_ld();
@@ -494,24 +494,8 @@ template <int WHICH> __global__ void __launch_bounds__(512, 1) pass_rate_kernel(
             for (int gg = 0; gg < C::GPT; ++gg) {
                 const int g = sub * C::GPT + gg;
                 uint32_t u[NCH][G];
-#pragma unroll
-                for (int ch = 0; ch < NCH; ++ch) tmem_ld<G>(taddr + ch * CH + g * G, u[ch]);
-                ptx::tmem_wait_ld();
-#pragma unroll
-                for (int h = 1; h < NCH; h <<= 1) {
-#pragma unroll
-                    for (int ch = 0; ch < NCH; ++ch) {
-                        if ((ch & h) == 0) {
-#pragma unroll
-                            for (int i = 0; i < G; i += 2) {
-                                f32x2 a = pack2u(u[ch][i], u[ch][i + 1]), b = pack2u(u[ch + h][i], u[ch + h][i + 1]);
-                                bfly2(a, b);
-                                unpack2u(a, u[ch][i], u[ch][i + 1]);
-                                unpack2u(b, u[ch + h][i], u[ch + h][i + 1]);
-                            }
-                        }
-                    }
-                }
+                load_group<C>(taddr + g * G, u);
+                across_chunks<C, true>(u);
 #pragma unroll
                 for (int ch = 0; ch < NCH; ++ch)
                     quantize_store<G, true>(base + slot * (kTile * W), quad * 32 + lane, ch * CH + g * G, u[ch], 1e-3f, 127.f, 0);
