@@ -367,7 +367,7 @@ DHQ_API dhq_status_t dhq_last_status(dhq_handle_t h);
  * the global nanosecond timer before and after the work; sm_mhz = cycles / time.  (NVML reports the
  * clock the driver asks for; inside the launches the SMs were seen 4-8 % below it.  The timed
  * instantiations do not carry the probe: a dhq_forward_fused_debug call without dump buffers does
- * the same work at nearly the same speed and serves as the clock measurement.)  milliseconds: that
+ * the same work, up to a fifth slower, and serves as the clock measurement.)  milliseconds: that
  * CTA's run time, close to the launch's.  Synchronizes the device.  Either pointer may be NULL.
  * (No counterpart in the paper: measurement.)
  * Errors: INVALID_ARG (no such launch yet), UNSUPPORTED (handle runs layer by layer), CUDA.

@@ -25,8 +25,9 @@
 // digits' rows in one MMA; digit by digit with N = 64 the same outputs took 16 x 51, because operands leave shared
 // memory at 128 B per cycle).  Two sets of sums: one half's MMAs run while the other's sums are read and worked on;
 // the first half block's MMAs and the stages across chunks are exposed (activations fill the rest of tensor memory).
-// Measured: 2 -> 256 x 5 -> 3, per-channel / per-token, 262,144 coordinates 604 us (667 with one set of 4 x 64 sums and
-// an MMA per digit; 9.79 ms with one dp4a pass and an fp64 butterfly per layer).
+// Measured: 2 -> 256 x 5 -> 3, per-channel / per-token, 262,144 coordinates 535 us (two sets of sums and one MMA for all digits
+// against one set of 4 x 64 and an MMA per digit, both with MMAs issued by one lane: 604 against 667; 9.79 ms with one dp4a
+// pass and an fp64 butterfly per layer).
 #include "dhq_fused.cuh"
 
 namespace dhq {

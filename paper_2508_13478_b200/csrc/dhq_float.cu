@@ -27,8 +27,8 @@
 // and digits of a block take as long as the next block's MMAs or longer.
 // Measured: 2 -> 256 x 3 -> 3, fp32, 65,536 coordinates 940 -> 65 us (88 with the digits through L2); 2 -> 512 x 4 -> 3, 8-bit
 // weights, 262,144 coordinates 17.2 -> 0.94 ms (one fp32 CUDA-core pass per layer before).  Blocks of 64 outputs with the weight
-// digits stacked in one operand and two sets of accumulators were slower (70.6 us, 1.16 ms): fewer outputs at a
-// time hide less of the epilogue's latency.
+// digits stacked in one operand and two sets of accumulators were slower (70.6 against 67.9 us, 1.16 against 1.10 ms, both
+// before the warp's number was a uniform value): fewer outputs at a time hide less of the epilogue's latency.
 #include "dhq_fused.cuh"
 
 namespace dhq {
@@ -63,7 +63,7 @@ struct FloatParams {
 // CTA lies in buffer (t NB + k) mod (NB + 1).  Block 0's outputs go to the buffer that this layer does not
 // read, block 1's (the last) to the one of this layer's part 0, whose MMAs have all completed with that block's
 // sums.  So the next layer's MMAs begin on part 0 while block 1's outputs are still being formed.  At width 512 one layer's
-// digits fill 192 KB and go through L2 instead.
+// digits take 128 KB of shared memory and 128 tensor-memory columns, which leaves no room beside them: they go through L2.
 __host__ __device__ constexpr bool float_x_in_smem(int W) { return W < 512; }
 // Width 512: the third digit, which meets the first weight digit only, is an operand in tensor memory (columns 384-511,
 // four consecutive k to a column) instead of shared memory.  That leaves room for the epilogue constants, which were read
@@ -330,7 +330,9 @@ __device__ void float_epilogue(const FloatParams &p, const FloatMap &sm, uint32_
                     emit(l, k0 + g * 16, y, tok, valid);
                 }
                 // Beside the last tensor-core layer, which writes no activations: the first layer of the CTA's next
-                // tile, whose digits go where this tile's were (at width 512 those are all in shared memory by now).
+                // tile, whose digits go where this tile's were.  At width 512 the first two digits have all been copied to
+                // shared memory by now (this block's sums needed every copy), and each thread read its part of the third,
+                // which it is about to overwrite, at the start of the layer.
                 if (l == p.L - 1 && tile + gridDim.x < p.n_tiles)
                     first_layer(b, x, yc, tok + gridDim.x * (long long)kTile, (tok + gridDim.x * (long long)kTile) < p.n);
                 if (l < p.L - 1 || tile + gridDim.x < p.n_tiles) end_part(b);

@@ -50,7 +50,9 @@ constexpr int kMmaWarp = 16, kLoadWarp = 17, kXyWarp = 18;
 // launch gives every thread 96 registers; the fifth warpgroup then hands 40 of its own back and the other four
 // take 8 more each, 512 * 104 + 128 * 56 <= 640 * 96.  Measured per kernel: width 256, 1,048,576 coordinates, 4
 // layers 515 -> 499 us; width 128 96 -> 85; two-sided at width 512 768 -> 742; but the plain kernels of
-// width 512 lost 2 to 5 % and those of width 64 2 %, so they keep 18 warps (19 at width 512).
+// width 512 lost 2 to 5 % and those of width 64 2 %, so they keep 18 warps (19 at width 512).  All of these were measured before
+// the warp's number was a uniform value (ptx::uniform), which took most spills away; with it the split would gain
+// 0.7 % in the plain kernels of width 512 (4,194,304 coordinates 6,327 -> 6,280 us) and change nothing at width 64.
 __host__ __device__ constexpr bool splits_registers(int W, bool both, bool gabor) { return W == 128 || W == 256 || (W == 512 && (both || gabor)); }
 __host__ __device__ constexpr int fused_threads(int W, bool both, bool gabor) { return splits_registers(W, both, gabor) ? 20 * 32 : W == 512 ? 19 * 32 : 18 * 32; }
 // Whether a kernel makes its warp's number a uniform value (ptx::uniform): not the observing ones, where it took the registers of

@@ -104,9 +104,10 @@ __device__ __forceinline__ float epilogue_mixed(float accf, float c_hi, float c_
 // psi(z) = sin(omega0 z) exp(-(s0 z)^2), from the compensated phase x = omega0 z and c = s0 / omega0.
 // The envelope's exponent carries a relative error of a few 2^-24, the result stays within the
 // sine's own error.
-// (Not ex2.approx.ftz, which makes envelopes below 2^-126 zero: the scaling that ex2.approx spends on them costs 16 us of 134,
+// (Not ex2.approx.ftz, which makes envelopes below 2^-126 zero: the scaling that ex2.approx spends on them costs 17 us of 135,
 // width 128, 267,007 coordinates, 4 layers, without rotation.  With .ftz and a vote per four columns on whether any is
-// that small it is 130 us, but 139 where many are.)
+// that small it is 130 us, but 139 where many are; with a second look at a chunk of 64 that met one, 130 too, and 3 %
+// more than now at width 64.)
 __device__ __forceinline__ float gabor_envelope(float t)
 {
     float e;

@@ -99,8 +99,8 @@ __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wa
 
 // A value that is the same in all lanes, in a form that the compiler knows to be.  Tensor-memory addresses and MMA operands
 // live in uniform registers; with the warp's number and the tensor-memory base made uniform, what is computed from them
-// stays there instead of being moved for every access, and the epilogue warps' spills (100 to 200 bytes a thread)
-// are gone.  Width 512, 4,194,304 coordinates 7,022 -> 6,349 us; width 256, 65,536 coordinates 39.1 -> 36.8, per token
+// stays there instead of being moved for every access, and most of the epilogue warps' spills (100 to 200 bytes a thread)
+// are gone: width 512 keeps 24 to 40 bytes, the two-sided per-channel kernel 24 to 44.  Width 512, 4,194,304 coordinates 7,022 -> 6,349 us; width 256, 65,536 coordinates 39.1 -> 36.8, per token
 // 238 -> 225; two-sided per channel 570 -> 535; wavelet at width 128 127 -> 118; fp32 at width 256 68.2 -> 65.1.
 __device__ __forceinline__ uint32_t uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
 
